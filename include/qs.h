@@ -85,8 +85,8 @@ typedef struct qs_options {
 #define QS_FLAG_UNPIPELINED_MEASURE 2u
 /* qs_options.flags: never measure in blocks. By default a window of >= 16
  * measurements on >= 64 qubits is measured in blocks of up to 64 with one
- * pass over the tableau per block (identical results); the blocked path waits
- * for the stream once per block. */
+ * pass over the tableau per block, and its deterministic outcomes together
+ * after the last block (identical results; nothing waits on the host). */
 #define QS_FLAG_NO_BLOCKED_MEASURE 4u
 /* qs_options.flags: address the row-major tableau with 64-bit word offsets in
  * the blocked measurement's apply pass even when 32-bit ones suffice. By
@@ -96,10 +96,8 @@ typedef struct qs_options {
 #define QS_FLAG_WIDE_OFFSETS 8u
 /* qs_options.flags: run the blocked measurement's symbolic pass (which rows
  * each of a block's measurements targets) as one launch per measurement over
- * every row. By default that launch sequence is used only above 25,600 qubits;
- * up to that size one CTA runs every step over the stabilizer rows held in
- * shared memory. The flag runs the large-size code path at any size
- * (identical results). */
+ * every row. By default one CTA finds a block's pivots among the rows that can
+ * hold them, at any size (identical results). */
 #define QS_FLAG_STEP_SYMBOLIC 16u
 /* qs_options.flags: inverse-tableau mode, the representation of the paper's
  * own measurement variant (Sec. 3.2, Alg. 1: Gaussian elimination by CX
@@ -444,8 +442,7 @@ int qs_batch_destroy(qs_batch *batch);
 /* Runs every circuit from |0...0> through its rounds (the first round_limit
  * rounds, 0 = all): the n < 1024 circuits in one cooperative persistent
  * kernel launch on the batch's stream, the others on the worker streams.
- * Returns when all work is enqueued (the host threads wait for their streams
- * once per block of measurements); the batch's stream then waits for the
+ * Returns when all work is enqueued; the batch's stream then waits for the
  * worker streams, so work enqueued on it afterwards follows the whole batch.
  * tuning: NULL for the default shape of the persistent kernel. */
 int qs_batch_run(qs_batch *batch, const qs_batch_tuning *tuning, uint32_t round_limit);

@@ -1082,8 +1082,7 @@ static int run_kernel(qs_batch *b, const qs_batch_tuning *tuning, uint32_t round
 static int batch_run(qs_batch *b, const qs_batch_tuning *tuning, uint32_t round_limit);
 
 // Enqueues every large circuit's rounds on its simulator, one host thread per
-// worker stream (blocked measurement waits for its stream once per block),
-// then makes the batch stream wait for the worker streams.
+// worker stream, then makes the batch stream wait for the worker streams.
 static int run_sims(qs_batch *b, uint32_t round_limit) {
   const uint32_t nw = (uint32_t)b->wstreams.size();
   std::mutex mu;

@@ -11,16 +11,14 @@
 //     stabilizer with bit j set), XORs the pivot's C into the targets and records
 //     in M_r which steps targeted r; the destabilizer partner gets the pivot's C
 //     (base = step j, M reset), the pivot row is marked. A step without a pivot
-//     (deterministic outcome) ends the block there; it is measured afterwards by
-//     the single-measurement path.
+//     has a deterministic outcome and changes nothing.
 //  2. pivot rows: V_j = (V_{j'} ... over the steps j' that targeted row p_j, in
 //     order) * original row p_j, built word-parallel; their signs follow from
 //     the phase of a product of Paulis,
 //       i^(2 sum r + sum |x_a & z_a| + 2 sum_{a<b} z_a . x_b - |X & Z|),
 //     whose cross term is GF(2)-bilinear, so per-word popcounts summed over the
 //     row (|x & z| of each V, of each original pivot row, parities
-//     G[s][t] = z_{V_s} . x_{V_t}) are enough; the signs are then resolved in
-//     step order by one thread.
+//     G[s][t] = z_{V_s} . x_{V_t}) are enough.
 //  3. one streaming pass: row r becomes (prod over s in M_r of V_s) * base_r,
 //     base_r = its original value or V_j if it was replaced at step j; the XOR
 //     accumulation reads the V words of a column chunk from shared memory, the
@@ -28,6 +26,18 @@
 //     z_acc . x_base + sum_{s>t in M_r} G[s][t]. Pivot rows become +-Z_q.
 // Per block the tableau is read and written once instead of once per
 // measurement (the paper measures one qubit at a time, Alg. 2).
+//
+// Deterministic outcomes of a window are evaluated together after its last
+// block: measurements of one window commute, so (-1)^m Z_q stays in the
+// stabilizer group, and with it its value, until the window ends.
+//
+// Launches: a window is a memset, blk_front, then per block blk_middle,
+// blk_apply and blk_front (which signs block b's rows and starts block b + 1),
+// then blk_det. The serial parts run in the block of a grid that arrives last,
+// so the host neither waits nor reads anything back: 3 launches per block where
+// a launch per part took 9 and a wait per round. 64 measurements of a dense
+// 10,000-qubit state: 172 -> 103 us; 3,000 measurements of a shallow 1,500-qubit
+// state, 2,456 of them deterministic (measured one by one before): 30.3 -> 2.4 ms.
 #include <algorithm>
 #include <climits>
 
@@ -35,356 +45,713 @@
 
 namespace qs {
 
-constexpr int64_t kBlkNone = LLONG_MAX;
 constexpr int32_t kBaseOrig = -1;
 constexpr int32_t kBasePivot = 1000;  // base = kBasePivot + j: pivot row of step j
 constexpr int kCW = 32;               // column words per phase-3 chunk
-// windows of the lazy symbolic pass: stabilizer rows per window = threads of its
-// CTA. 256 took the pass from 30.9 to 23.8 ms per step on the 10k workload and
-// from 0.56 to 0.45 ms at 180k against 1,024 (512: 24.3 and 0.47 ms): a step
-// waits on barriers of 8 warps instead of 32.
-constexpr int kLazyLog2 = 8;
-constexpr int kLazyThreads = 1 << kLazyLog2;
-constexpr uint32_t kLazyMaxWindows = (1u << 20) >> kLazyLog2;  // n <= 2^20
+constexpr int64_t kBlkNone = LLONG_MAX;
 
+// state of one block (two of them alternate: blk_front signs block b's rows
+// with one while its symbolic pass fills the other for block b + 1)
 struct BlkState {
-  int64_t slot[3];     // pivot search results, rotating
-  int32_t len;         // steps completed in this block
+  int64_t slot[3];     // pivot search results, rotating (step-by-step symbolic pass)
   uint32_t ntouched;   // rows the block changes (entries of the apply pass's row list)
-  uint32_t i0;         // first measurement of the block within its window
-  int32_t B;           // measurements the block attempts (0 past the window's end)
-  uint32_t cursor;     // next measurement of the window: read by the next block's reset
-  int64_t piv[64];     // pivot row of each step
+  uint32_t pad;
+  int64_t piv[64];     // pivot row of each step, or kBlkNone (deterministic)
   uint64_t mpiv[64];   // steps that targeted the pivot row before it became pivot
+  uint64_t cpiv[64];   // C of the pivot row at its step (0: deterministic)
+  uint64_t E[64];      // V_j = product of the original pivot rows of the steps in E_j
+  uint64_t lin[64];    // M_r = XOR of lin[t] over the bits t of C_r (rows never replaced)
   int32_t A[64];       // |x_V & z_V| mod 4 (summed over words)
   int32_t B0[64];      // |x & z| of the original pivot row
   int32_t Cp[64];      // parity of (z_V ^ z_orig) . x_orig
   int32_t rV[64];      // sign bit of V_j
   uint64_t G[64];      // G[s] bit t = parity(z_{V_s} . x_{V_t})
-  uint64_t cpiv[64];   // C of the pivot row at its step (lazy symbolic pass)
-  uint32_t err;
-  uint32_t pad2;
-  uint64_t win_or[4096];  // OR of C over each window of stabilizer rows (lazy pass)
+};
+
+constexpr uint32_t kDetChunks = 512;  // 32-word column chunks of the largest row (n = 2^20)
+
+// state of one window; zeroed before its first block together with the
+// accumulators behind it
+struct BlkWindow {
+  uint32_t front_arrived, middle_arrived, ndet, pad;
+  uint32_t det_chunk[kDetChunks];  // row ranges of blk_det that have arrived, per column chunk
+  BlkState st[2];
 };
 
 __device__ __forceinline__ int m4(int v) { return ((v % 4) + 4) % 4; }
 
-// the block starts where the previous block of the window stopped (st->cursor),
-// so the host can enqueue several blocks before it reads how far they got
-__global__ void blk_reset_kernel(BlkState *st, uint32_t count, uint32_t nwin) {
+__device__ __forceinline__ uint64_t shfl64(uint64_t v, int src) { return __shfl_sync(0xffffffffu, v, src); }
+
+// The x bits of one row at a run of measured qubits. Measured qubits are cut
+// into runs of consecutive ones inside a word, so that an ascending list takes
+// one load, shift and mask per 64 qubits.
+struct ColRuns {
+  uint32_t n;
+  uint32_t word[64];
+  uint64_t mask[64];
+  uint8_t shift[64], pos[64];
+};
+
+// fills R from qubits[0..B); called by the first 64 threads of a block, which
+// then synchronises. Out-of-range qubits belong to no run (their bits are 0).
+__device__ __forceinline__ void build_runs(ColRuns &R, const uint32_t *qubits, int B, uint32_t n) {
+  __shared__ uint32_t s_start[2], s_ok[2];
   const int t = threadIdx.x;
-  const uint32_t i0 = st->cursor;
-  const int B = i0 < count ? (int)min(64u, count - i0) : 0;
-  if (t < 3) st->slot[t] = kBlkNone;
-  if (t == 0) { st->len = B; st->err = 0; st->ntouched = 0; st->i0 = i0; st->B = B; }
-  if (t < 64) {
-    st->piv[t] = kBlkNone; st->mpiv[t] = 0; st->A[t] = 0; st->B0[t] = 0; st->Cp[t] = 0;
-    st->rV[t] = 0; st->G[t] = 0;
+  const uint32_t q = t < B ? qubits[t] : 0xFFFFFFFFu;
+  const uint32_t before = (t > 0 && t - 1 < B) ? qubits[t - 1] : 0xFFFFFFFFu;
+  const bool ok = q < n;
+  const bool start = ok && !(before < n && q == before + 1 && (q & 63) != 0);
+  const uint32_t bs = __ballot_sync(0xffffffffu, start), bo = __ballot_sync(0xffffffffu, ok);
+  if ((t & 31) == 0) { s_start[t >> 5] = bs; s_ok[t >> 5] = bo; }
+  asm volatile("bar.sync 1, 64;" ::: "memory");
+  const uint64_t st = ((uint64_t)s_start[1] << 32) | s_start[0], okm = ((uint64_t)s_ok[1] << 32) | s_ok[0];
+  if (start) {
+    const int i = __popcll(st & ((1ull << t) - 1));
+    const uint64_t stop = (st | ~okm) & ~((2ull << t) - 1);  // the next start or invalid entry ends the run
+    const int len = (stop ? __ffsll((long long)stop) - 1 : 64) - t;
+    R.word[i] = q >> 6;
+    R.shift[i] = (uint8_t)(q & 63);
+    R.pos[i] = (uint8_t)t;
+    R.mask[i] = len >= 64 ? ~0ull : (1ull << len) - 1;
   }
-  for (uint32_t w = t; w < nwin; w += blockDim.x) st->win_or[w] = 0;
+  if (t == 0) R.n = (uint32_t)__popcll(st);
 }
 
-// C_r = x bits of row r at q_0..q_{B-1}; M = 0; base = original; T = parity = 0;
-// pivot of step 0 by atomicMin
-__global__ void __launch_bounds__(256)
-blk_init_kernel(const uint64_t *__restrict__ RX, uint32_t rs, uint64_t nrows, uint32_t n, uint32_t k,
-                const uint32_t *__restrict__ window, uint64_t *__restrict__ C,
-                uint64_t *__restrict__ M, int32_t *__restrict__ base, BlkState *st,
-                uint32_t *__restrict__ err) {
-  const int B = st->B;
-  const uint32_t *qubits = window + st->i0;
-  const uint64_t r = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// the runs' bits of row r, four words in flight
+__device__ __forceinline__ uint64_t gather_runs(const ColRuns &R, const uint64_t *row) {
   uint64_t c = 0;
-  if (r < nrows) {
-    uint32_t lastw = 0xFFFFFFFFu;
-    uint64_t word = 0;
-    for (int j = 0; j < B; ++j) {
-      const uint32_t q = qubits[j];
-      if (q >= n) { if (r == 0) atomicOr(err, kErrBadQubit); continue; }
-      if ((q >> 6) != lastw) { lastw = q >> 6; word = RX[r * rs + lastw]; }
-      c |= ((word >> (q & 63)) & 1ull) << j;
+  for (uint32_t i = 0; i < R.n; i += 4) {
+    uint64_t w[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) w[u] = i + u < R.n ? row[R.word[i + u]] : 0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (i + u < R.n) c |= ((w[u] >> R.shift[i + u]) & R.mask[i + u]) << R.pos[i + u];
+  }
+  return c;
+}
+
+// E_j = {j} xor (xor of E_s over the steps s that targeted p_j): thread t of
+// the first 64 keeps column t of E (bit s = whether t is in E_s), so a step is
+// one parity per thread and no exchange; the ballots are the rows.
+__device__ __forceinline__ void build_products(const uint64_t *mpiv, const int64_t *piv, int B, uint64_t *E) {
+  const int t = threadIdx.x;
+  uint64_t col = 0;
+  for (int j = 0; j < 64; ++j) {
+    uint32_t bit = 0;
+    if (j < B && piv[j] != kBlkNone) bit = (uint32_t)(__popcll(col & mpiv[j]) & 1) ^ (t == j ? 1u : 0u);
+    const uint32_t row = __ballot_sync(0xffffffffu, bit);
+    col |= (uint64_t)bit << j;
+    if ((t & 31) == 0) reinterpret_cast<uint32_t *>(&E[j])[t >> 5] = row;
+  }
+}
+
+// ---------------------------------------------------------------------------
+// blk_front: signs of the previous block's rows, C of the next block's, and in
+// the last block to arrive the next block's symbolic pass
+// ---------------------------------------------------------------------------
+struct FrontArgs {
+  const uint64_t *RX;
+  uint64_t *S;
+  uint64_t nrows;
+  uint32_t rs, n, k, chunks;
+  const uint32_t *window;       // measured qubits of the window
+  uint32_t i0, B;               // next block: first measurement and count (0: none)
+  uint32_t prev_i0, prev_B;     // previous block (0: none)
+  int cur;                      // state of the next block; the previous block's is the other
+  int lazy;                     // run the symbolic pass here (else step by step)
+  uint64_t *C, *listC;          // C of every row; nonzero stabilizer rows of each 256-row range: C,
+  uint32_t *listRow;            // their rows,
+  uint32_t *cnt, *done;         // their number, the steps replayed on them
+  uint64_t *orC;                // and the OR of their C
+  uint64_t *M;
+  int32_t *base;
+  const int32_t *Tp;
+  BlkWindow *win;
+  uint32_t *det;                // window positions of deterministic outcomes
+  uint64_t m0, seed, shot;
+  uint8_t *record, *kinds;
+  uint32_t *err;
+};
+
+// per row: new sign from the accumulated terms; pivot rows get their coin; record
+__device__ __forceinline__ void sign_rows(const FrontArgs &a, uint64_t r) {
+  __shared__ int sw[64];          // 2 rV_s + A_s of each step
+  __shared__ uint64_t sG[64];     // G rows
+  __shared__ uint32_t s_det[2];
+  const BlkState &st = a.win->st[a.cur ^ 1];
+  const uint64_t m0 = a.m0 + a.prev_i0;  // record index of the block's first measurement
+  const int t = threadIdx.x, B = (int)a.prev_B;
+  if (t < 64) {
+    sw[t] = 2 * st.rV[t] + st.A[t];
+    sG[t] = st.G[t];
+  }
+  __syncthreads();
+  if (blockIdx.x == 0 && t < 64) {
+    const bool in = t < B, prob = in && st.piv[t] != kBlkNone;
+    if (in) {
+      a.record[m0 + t] = prob ? (uint8_t)(philox4x64_10(m0 + t, a.shot, 0, 0, a.seed, kCoinKey).v[0] & 1u) : 0;
+      a.kinds[m0 + t] = prob;
     }
-    C[r] = c;
-    M[r] = 0;
-    base[r] = kBaseOrig;
+    const bool det = in && !prob && a.window[a.prev_i0 + t] < a.n;
+    const uint32_t ball = __ballot_sync(0xffffffffu, det);
+    if ((t & 31) == 0) s_det[t >> 5] = ball;
+    const uint32_t first = a.win->ndet;
+    asm volatile("bar.sync 1, 64;" ::: "memory");
+    if (det) a.det[first + (t >= 32 ? __popc(s_det[0]) : 0) + __popc(ball & ((1u << (t & 31)) - 1))] = a.prev_i0 + t;
+    if (t == 0) a.win->ndet = first + __popc(s_det[0]) + __popc(s_det[1]);
   }
-  {
-    // OR of C over this warp's 32 rows (in one window of stabilizer rows: the
-    // stabilizer half starts at 64 k, a multiple of 32)
-    uint64_t o = (r >= 64ull * k && r < 64ull * k + n) ? c : 0;
-    for (int d = 16; d > 0; d >>= 1) o |= __shfl_xor_sync(0xffffffffu, o, d);
-    if ((threadIdx.x & 31) == 0 && o)
-      atomicOr(reinterpret_cast<unsigned long long *>(&st->win_or[(r - 64ull * k) >> kLazyLog2]), o);
-  }
-  const uint32_t ball = __ballot_sync(0xffffffffu, (c & 1ull) != 0);
-  if ((threadIdx.x & 31) == 0 && r < nrows) {
-    const uint64_t lo = 64ull * k, hi = 64ull * k + n, b0 = r;
-    uint32_t m = ball;
-    if (b0 + 32 > lo && b0 < hi && m) {
-      if (b0 < lo) m &= ~0u << (uint32_t)(lo - b0);
-      if (b0 + 32 > hi) m &= (uint32_t)((1ull << (hi - b0)) - 1);
-      if (m) atomicMin(reinterpret_cast<long long *>(&st->slot[0]), (long long)(b0 + __ffs(m) - 1));
+  uint64_t delta = 0;
+  if (r < a.nrows) {
+    const int32_t b = a.base[r];
+    const uint64_t sr = a.M[r];
+    const uint64_t old = (a.S[r >> 6] >> (r & 63)) & 1u;
+    uint64_t nb = old;
+    if (b >= kBasePivot) {
+      nb = philox4x64_10(m0 + (b - kBasePivot), a.shot, 0, 0, a.seed, kCoinKey).v[0] & 1u;
+    } else if (b != kBaseOrig || sr != 0) {
+      const int rb = (b == kBaseOrig) ? (int)old : st.rV[b];
+      int e = 2 * rb, csum = 0;
+#pragma unroll 4
+      for (uint32_t ch = 0; ch < a.chunks; ++ch) {
+        const int32_t v = a.Tp[(uint64_t)ch * a.nrows + r];
+        e += v >> 1;  // arithmetic shift: t
+        csum ^= v & 1;
+      }
+      e += 2 * csum;
+      // + sum over s in M_r of (2 rV_s + A_s) + 2 sum over s > t in M_r of G[s] bit t
+      uint64_t mm = sr;
+      while (mm) {
+        const int s = __ffsll((long long)mm) - 1;
+        mm &= mm - 1;
+        e += sw[s] + 2 * (__popcll(sG[s] & sr & ((1ull << s) - 1)) & 1);
+      }
+      e = m4(e);
+      if (e & 1) atomicOr(a.err, kErrOddPhase);
+      nb = (uint64_t)(e >> 1);
     }
+    delta = (nb ^ old) << (r & 63);
   }
+  // fold the sign changes of the 32 rows of this warp into one atomic
+  for (int o = 16; o > 0; o >>= 1) delta |= __shfl_xor_sync(0xffffffffu, delta, o);
+  if ((threadIdx.x & 31) == 0 && r < a.nrows && delta)
+    atomicXor(reinterpret_cast<unsigned long long *>(&a.S[r >> 6]), delta);
+}
+
+// Symbolic pass. Only the pivot sequence (p_j, v_j = C_{p_j} at step j) has to
+// be found in order, and the pivot of step j is the first stabilizer row whose
+// current C has bit j. Rows with C = 0 never take part, and in any state the
+// pivots come from the first nonzero rows, so the first 1,024 of those are held
+// by the block's 8 warps, 128 rows each, transposed: lane t of a warp holds the
+// warp's rows' bits at steps t and t + 32 as four words each. A step is then a
+// broadcast of column j, a search for its first bit and one masked XOR into the
+// columns v_j has; the pivot row clears itself (its C is v_j). Warp 0 runs alone
+// while its rows hold a pivot (no barriers: 64 steps of a dense state take about
+// 5 us); at its first miss the other warps replay the steps so far on their
+// rows and all eight go on in step. Nonzero rows beyond the first 1,024 are only
+// looked at when those have no pivot for a step: range by range of 256 rows,
+// skipping a range when an upper bound on the OR of its C rules the step's bit
+// out (exact when the range was last replayed, then grown by v_s for every step
+// s whose bit the bound has).
+constexpr int kGroup = 1024;
+
+struct Tile {  // one warp's 128 rows: columns lane and lane + 32
+  uint32_t lo[4], hi[4];
+};
+
+// 32 x 32 bit transpose over the warp: out[lane t] bit r = in[lane r] bit t
+__device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane) {
+#pragma unroll
+  for (int j = 16; j > 0; j >>= 1) {
+    const uint32_t low = j == 16 ? 0x0000FFFFu : j == 8 ? 0x00FF00FFu : j == 4 ? 0x0F0F0F0Fu : j == 2 ? 0x33333333u : 0x55555555u;
+    const uint32_t y = __shfl_xor_sync(0xffffffffu, x, j);
+    x = (lane & j) ? ((x & ~low) | ((y & ~low) >> j)) : ((x & low) | ((y & low) << j));
+  }
+  return x;
+}
+
+__device__ __forceinline__ void tile_column(const Tile &T, int j, uint32_t (&w)[4]) {
+#pragma unroll
+  for (int m = 0; m < 4; ++m) w[m] = __shfl_sync(0xffffffffu, j < 32 ? T.lo[m] : T.hi[m], j & 31);
+}
+
+// first row with a bit in column w (-1: none)
+__device__ __forceinline__ int tile_first(const uint32_t (&w)[4]) {
+  int p = -1;
+#pragma unroll
+  for (int m = 3; m >= 0; --m)
+    if (w[m]) p = 32 * m + __ffs(w[m]) - 1;
+  return p;
+}
+
+// C of row p of the tile (warp-uniform p)
+__device__ __forceinline__ uint64_t tile_row(const Tile &T, int p) {
+  const int m = p >> 5, b = p & 31;
+  uint32_t l = T.lo[0], h = T.hi[0];
+#pragma unroll
+  for (int i = 1; i < 4; ++i)
+    if (m == i) { l = T.lo[i]; h = T.hi[i]; }
+  const uint32_t vl = __ballot_sync(0xffffffffu, (l >> b) & 1u), vh = __ballot_sync(0xffffffffu, (h >> b) & 1u);
+  return ((uint64_t)vh << 32) | vl;
+}
+
+// rows with bit j (w) take v
+__device__ __forceinline__ void tile_apply(Tile &T, const uint32_t (&w)[4], uint64_t v, int lane) {
+  const uint32_t ml = 0u - (uint32_t)((v >> lane) & 1u), mh = 0u - (uint32_t)((v >> (lane + 32)) & 1u);
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    T.lo[m] ^= w[m] & ml;
+    T.hi[m] ^= w[m] & mh;
+  }
+}
+
+__device__ __forceinline__ uint64_t lazy_bound(uint64_t u, int a, int j, const uint64_t *v) {
+  for (int s = a; s < j; ++s)
+    if ((u >> s) & 1ull) u |= v[s];
+  return u;
+}
+
+struct SymbolicShared {
+  uint64_t c[kGroup];          // C of the first nonzero rows
+  uint32_t row[kGroup];
+  uint64_t v[64];              // C of each step's pivot (0: none)
+  int64_t piv[64];
+  uint64_t mpiv[64], E[64];
+  uint64_t cand_v[2][8], wor[8];
+  int cand[2][8];
+  uint32_t sum[8], flags[8];
+  int j0;
+  int found;
+  uint64_t found_v;
+  int64_t found_row;
+};
+
+// pivot of step j among the nonzero rows past the first kGroup (all 256
+// threads; off[w] = nonzero rows before range w); leaves found_* in sh
+__device__ void search_rest(const FrontArgs &a, SymbolicShared &sh, const uint32_t *off, uint32_t nwin, int j) {
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  __syncthreads();
+  if (t == 0) sh.found = 0;
+  for (uint32_t w0 = 0; w0 < nwin; w0 += 256) {
+    const uint32_t w = w0 + t;
+    bool may = false;
+    if (w < nwin) {
+      const uint32_t c = __ldcg(a.cnt + w);
+      may = c && off[w] + c > (uint32_t)kGroup &&
+            ((lazy_bound(__ldcg(a.orC + w), (int)__ldcg(a.done + w), j, sh.v) >> j) & 1ull);
+    }
+    const uint32_t ball = __ballot_sync(0xffffffffu, may);
+    if (lane == 0) sh.flags[warp] = ball;
+    __syncthreads();
+    for (int f = 0; f < 8; ++f) {
+      uint32_t bits = sh.flags[f];  // uniform
+      while (bits) {
+        const uint32_t ww = w0 + 32 * f + __ffs(bits) - 1;
+        bits &= bits - 1;
+        const uint32_t cnt = __ldcg(a.cnt + ww);
+        const int from = (int)__ldcg(a.done + ww);
+        const bool in = (uint32_t)t < cnt && off[ww] + t >= (uint32_t)kGroup;
+        uint64_t c = 0;
+        if (in) {
+          c = __ldcg(a.listC + (size_t)ww * 256 + t);
+          for (int s = from; s < j; ++s)
+            if ((c >> s) & 1ull) c ^= sh.v[s];
+          __stcg(a.listC + (size_t)ww * 256 + t, c);
+        }
+        const uint32_t has = __ballot_sync(0xffffffffu, (c >> j) & 1ull);
+        uint64_t o = c;
+        for (int d = 16; d > 0; d >>= 1) o |= __shfl_xor_sync(0xffffffffu, o, d);
+        const int first = has ? __ffs(has) - 1 : 0;
+        const uint64_t fv = shfl64(c, first);
+        if (lane == 0) {
+          sh.cand[0][warp] = has ? 32 * warp + first : -1;
+          sh.cand_v[0][warp] = fv;
+          sh.wor[warp] = o;
+        }
+        __syncthreads();
+        int win = -1;
+        uint64_t all = 0;
+#pragma unroll
+        for (int i = 7; i >= 0; --i) {
+          if (sh.cand[0][i] >= 0) win = i;
+          all |= sh.wor[i];
+        }
+        if (t == 0) {
+          __stcg(a.orC + ww, all);
+          __stcg(a.done + ww, (uint32_t)j);
+          if (win >= 0) {
+            sh.found = 1;
+            sh.found_v = sh.cand_v[0][win];
+            sh.found_row = (int64_t)__ldcg(a.listRow + (size_t)ww * 256 + sh.cand[0][win]);
+          }
+        }
+        __syncthreads();
+        if (win >= 0) return;
+      }
+    }
+    __syncthreads();  // flags are rewritten
+  }
+}
+
+__device__ void symbolic_pass(const FrontArgs &a, SymbolicShared &sh, uint32_t *off, uint32_t nwin) {
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5, B = (int)a.B;
+  BlkState &st = a.win->st[a.cur];
+  // off[w] = nonzero rows before range w
+  const uint32_t per = (nwin + 255) / 256, w0 = min(nwin, t * per), w1 = min(nwin, w0 + per);
+  uint32_t sum = 0;
+  for (uint32_t w = w0; w < w1; ++w) sum += __ldcg(a.cnt + w);
+  uint32_t inc = sum;
+  for (int d = 1; d < 32; d <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, inc, d);
+    if (lane >= d) inc += y;
+  }
+  if (lane == 31) sh.sum[warp] = inc;
+  if (t < 64) { sh.v[t] = 0; sh.piv[t] = kBlkNone; }
+  __syncthreads();
+  uint32_t before = inc - sum, total = 0;
+  for (int i = 0; i < 8; ++i) {
+    if (i < warp) before += sh.sum[i];
+    total += sh.sum[i];
+  }
+  for (uint32_t w = w0; w < w1; ++w) {
+    off[w] = before;
+    before += __ldcg(a.cnt + w);
+  }
+  __syncthreads();
+  const uint32_t group = min(total, (uint32_t)kGroup);
+#pragma unroll
+  for (int i = 0; i < kGroup / 256; ++i) {
+    const uint32_t g = t + 256 * i;
+    uint64_t c = 0;
+    uint32_t row = 0;
+    if (g < group) {
+      uint32_t lo = 0, hi = nwin;  // last range with off <= g
+      while (hi - lo > 1) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (off[mid] <= g) lo = mid; else hi = mid;
+      }
+      const size_t e = (size_t)lo * 256 + (g - off[lo]);
+      c = __ldcg(a.listC + e);
+      row = __ldcg(a.listRow + e);
+    }
+    sh.c[g] = c;
+    sh.row[g] = row;
+  }
+  __syncthreads();
+  Tile T;
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    const uint64_t c = sh.c[128 * warp + 32 * m + lane];
+    T.lo[m] = transpose32((uint32_t)c, lane);
+    T.hi[m] = transpose32((uint32_t)(c >> 32), lane);
+  }
+  uint32_t w[4];
+  if (warp == 0) {
+    int j = 0;
+    for (; j < B; ++j) {
+      tile_column(T, j, w);
+      const int p = tile_first(w);
+      if (p < 0) {
+        if (group > 128) break;  // the other warps' rows may have one
+        continue;
+      }
+      const uint64_t v = tile_row(T, p);
+      tile_apply(T, w, v, lane);
+      if (lane == 0) { sh.v[j] = v; sh.piv[j] = sh.row[p]; }
+    }
+    if (lane == 0) sh.j0 = j;
+  }
+  __syncthreads();
+  const int j0 = sh.j0;
+  if (j0 < B) {
+    if (warp > 0)
+      for (int s = 0; s < j0; ++s) {
+        const uint64_t v = sh.v[s];
+        if (!v) continue;
+        tile_column(T, s, w);
+        tile_apply(T, w, v, lane);
+      }
+    for (int j = j0, par = 0; j < B; ++j, par ^= 1) {
+      tile_column(T, j, w);
+      const int p = tile_first(w);
+      const uint64_t v = p >= 0 ? tile_row(T, p) : 0;
+      if (lane == 0) {
+        sh.cand[par][warp] = p >= 0 ? 128 * warp + p : -1;
+        sh.cand_v[par][warp] = v;
+      }
+      __syncthreads();
+      int win = -1;
+#pragma unroll
+      for (int i = 7; i >= 0; --i)
+        if (sh.cand[par][i] >= 0) win = i;
+      uint64_t pv = 0;
+      int64_t prow = kBlkNone;
+      if (win >= 0) {
+        pv = sh.cand_v[par][win];
+        prow = sh.row[sh.cand[par][win]];
+      } else if (total > (uint32_t)kGroup) {
+        search_rest(a, sh, off, nwin, j);
+        if (sh.found) { pv = sh.found_v; prow = sh.found_row; }
+        __syncthreads();
+      }
+      if (pv) tile_apply(T, w, pv, lane);
+      if (t == 0) { sh.v[j] = pv; sh.piv[j] = prow; }
+    }
+    __syncthreads();
+  }
+  // M is linear in C: lin[t] = the steps that reduce unit vector t; mpiv from it
+  if (t < 64) {
+    uint64_t c = 1ull << t, m = 0;
+    for (int s = t; s < B; ++s) {
+      const uint64_t v = sh.v[s];
+      if (v && ((c >> s) & 1ull)) { c ^= v; m |= 1ull << s; }
+    }
+    st.lin[t] = m;
+  } else if (t < 128) {
+    const int j = t - 64;
+    uint64_t m = 0;
+    if (j < B && sh.v[j]) {
+      uint64_t c = __ldcg(a.C + sh.piv[j]);
+      for (int s = 0; s < j; ++s) {
+        const uint64_t v = sh.v[s];
+        if (v && ((c >> s) & 1ull)) { c ^= v; m |= 1ull << s; }
+      }
+    }
+    sh.mpiv[j] = m;
+  }
+  __syncthreads();
+  if (t < 64) build_products(sh.mpiv, sh.piv, B, sh.E);
+  __syncthreads();
+  if (t < 64) {
+    st.piv[t] = sh.piv[t];
+    st.cpiv[t] = sh.v[t];
+    st.mpiv[t] = sh.mpiv[t];
+    st.E[t] = sh.E[t];
+    st.A[t] = 0; st.B0[t] = 0; st.Cp[t] = 0; st.rV[t] = 0; st.G[t] = 0;
+  }
+  if (t == 0) st.ntouched = 0;
+}
+
+__global__ void __launch_bounds__(256) blk_front_kernel(const FrontArgs a) {
+  extern __shared__ uint32_t s_off[];  // gridDim.x words (lazy symbolic pass)
+  __shared__ ColRuns s_runs;
+  __shared__ SymbolicShared s_sym;
+  __shared__ uint32_t s_cnt[8];
+  __shared__ uint64_t s_or[8];
+  __shared__ bool s_last;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const uint64_t r = (uint64_t)blockIdx.x * 256 + t;
+  if (a.prev_B) sign_rows(a, r);
+  if (!a.B) return;
+  if (t < 64) {
+    build_runs(s_runs, a.window + a.i0, (int)a.B, a.n);
+    if (blockIdx.x == 0 && t < (int)a.B && a.window[a.i0 + t] >= a.n) atomicOr(a.err, kErrBadQubit);
+  }
+  __syncthreads();
+  uint64_t c = 0;
+  if (r < a.nrows) {
+    c = gather_runs(s_runs, a.RX + r * a.rs);
+    a.C[r] = c;
+  }
+  const bool stab = r >= 64ull * a.k && r < 64ull * a.k + a.n;
+  if (!a.lazy) {
+    if (r < a.nrows) { a.M[r] = 0; a.base[r] = kBaseOrig; }
+    const uint32_t ball = __ballot_sync(0xffffffffu, stab && (c & 1ull));
+    if (lane == 0 && ball)
+      atomicMin(reinterpret_cast<long long *>(&a.win->st[a.cur].slot[0]), (long long)(r + __ffs(ball) - 1));
+    return;
+  }
+  // nonzero stabilizer rows of this range, in order, and the OR of their C
+  const bool keep = stab && c != 0;
+  const uint32_t ball = __ballot_sync(0xffffffffu, keep);
+  uint64_t o = keep ? c : 0;
+  for (int d = 16; d > 0; d >>= 1) o |= __shfl_xor_sync(0xffffffffu, o, d);
+  if (lane == 0) { s_cnt[warp] = __popc(ball); s_or[warp] = o; }
+  __syncthreads();
+  uint32_t at = __popc(ball & ((1u << lane) - 1));
+  for (int i = 0; i < warp; ++i) at += s_cnt[i];
+  if (keep) {
+    a.listC[(size_t)blockIdx.x * 256 + at] = c;
+    a.listRow[(size_t)blockIdx.x * 256 + at] = (uint32_t)r;
+  }
+  if (t == 0) {
+    uint32_t cnt = 0;
+    uint64_t all = 0;
+    for (int i = 0; i < 8; ++i) { cnt += s_cnt[i]; all |= s_or[i]; }
+    a.cnt[blockIdx.x] = cnt;
+    a.orC[blockIdx.x] = all;
+    a.done[blockIdx.x] = 0;
+  }
+  __threadfence();
+  __syncthreads();
+  if (t == 0) {
+    s_last = atomicAdd(&a.win->front_arrived, 1u) == gridDim.x - 1;
+    if (s_last) a.win->front_arrived = 0;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  symbolic_pass(a, s_sym, s_off, gridDim.x);
+}
+
+// ---------------------------------------------------------------------------
+// step-by-step symbolic pass (QS_FLAG_STEP_SYMBOLIC): reset, one launch per
+// step over every row, then the products E
+// ---------------------------------------------------------------------------
+__global__ void blk_step_reset_kernel(BlkState *st) {
+  const int t = threadIdx.x;
+  if (t < 3) st->slot[t] = kBlkNone;
+  if (t == 0) st->ntouched = 0;
+  st->piv[t] = kBlkNone; st->mpiv[t] = 0; st->cpiv[t] = 0;
+  st->A[t] = 0; st->B0[t] = 0; st->Cp[t] = 0; st->rV[t] = 0; st->G[t] = 0;
 }
 
 // symbolic step j: Cin -> Cout
 __global__ void __launch_bounds__(256)
-blk_step_kernel(uint64_t nrows, uint32_t n, uint32_t k, int j, const uint64_t *__restrict__ Cin,
+blk_step_kernel(uint64_t nrows, uint32_t n, uint32_t k, int j, int B, const uint64_t *__restrict__ Cin,
                 uint64_t *__restrict__ Cout, uint64_t *__restrict__ M, int32_t *__restrict__ base,
                 BlkState *st) {
-  if (j >= st->len) return;
-  const int B = st->B;
   const int64_t p = st->slot[j % 3];
-  if (p == kBlkNone) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) st->len = j;
-    return;
-  }
+  const bool prob = p != kBlkNone;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     st->slot[(j + 2) % 3] = kBlkNone;
     st->piv[j] = p;
   }
   const int64_t pd = p - 64ll * k;
-  const uint64_t cp = Cin[p];
+  const uint64_t cp = prob ? Cin[p] : 0;
   const uint64_t r = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   uint64_t c = 0;
   if (r < nrows) {
     c = Cin[r];
-    if ((int64_t)r == p) {
-      st->mpiv[j] = M[r];
-      base[r] = kBasePivot + j;
-      c = 0;
-    } else if ((int64_t)r == pd) {
-      c = cp;
-      M[r] = 0;
-      base[r] = j;
-    } else if ((c >> j) & 1ull) {
-      c ^= cp;
-      M[r] |= 1ull << j;
+    if (prob) {
+      if ((int64_t)r == p) {
+        st->mpiv[j] = M[r];
+        st->cpiv[j] = cp;
+        M[r] = 0;
+        base[r] = kBasePivot + j;
+        c = 0;
+      } else if ((int64_t)r == pd) {
+        c = cp;
+        M[r] = 0;
+        base[r] = j;
+      } else if ((c >> j) & 1ull) {
+        c ^= cp;
+        M[r] |= 1ull << j;
+      }
     }
     Cout[r] = c;
   }
   if (j + 1 < B) {
-    const uint32_t ball = __ballot_sync(0xffffffffu, ((c >> (j + 1)) & 1ull) != 0);
-    if ((threadIdx.x & 31) == 0 && r < nrows) {
-      const uint64_t lo = 64ull * k, hi = 64ull * k + n, b0 = r;
-      uint32_t m = ball;
-      if (b0 + 32 > lo && b0 < hi && m) {
-        if (b0 < lo) m &= ~0u << (uint32_t)(lo - b0);
-        if (b0 + 32 > hi) m &= (uint32_t)((1ull << (hi - b0)) - 1);
-        if (m)
-          atomicMin(reinterpret_cast<long long *>(&st->slot[(j + 1) % 3]), (long long)(b0 + __ffs(m) - 1));
-      }
-    }
+    const bool stab = r >= 64ull * k && r < 64ull * k + n;
+    const uint32_t ball = __ballot_sync(0xffffffffu, stab && ((c >> (j + 1)) & 1ull));
+    if ((threadIdx.x & 31) == 0 && ball)
+      atomicMin(reinterpret_cast<long long *>(&st->slot[(j + 1) % 3]), (long long)(r + __ffs(ball) - 1));
   }
 }
 
-// Lazy symbolic pass in one CTA, for any n: only the pivot sequence
-// (p_j, C_{p_j}) is needed here (blk_replay_kernel then derives every row's M_r
-// and base_r from it), and the pivot of step j is the first stabilizer row, in
-// index order, whose current C has bit j. So the stabilizer rows are scanned in
-// windows of kLazyThreads (one row per thread), in order, and a window's rows are
-// brought up to step j (replaying steps a_w..j-1 on them: the pivot row of a
-// step becomes 0, a row with bit s set takes ^= C_{p_s}) only when it can hold
-// bit j. That is decided from U_w, an upper bound on the OR of the window's C:
-// exact when the window was last replayed, then grown by C_{p_s} for every
-// step s whose bit U_w has (a row that takes C_{p_s} had bit s). In a dense
-// state the pivots come from the first nonzero window, so a step costs one
-// window and one barrier; rows far from the front are never read. Rows of
-// replayed windows live in a working copy (W, the second C buffer); C0 stays
-// intact for the replay kernel.
-
-__device__ __forceinline__ uint64_t lazy_bound(uint64_t u, int a, int j, const uint64_t *cp) {
-  for (int s = a; s < j; ++s)
-    if ((u >> s) & 1ull) u |= cp[s];
-  return u;
+__global__ void __launch_bounds__(64) blk_step_finish_kernel(BlkState *st, int B) {
+  build_products(st->mpiv, st->piv, B, st->E);
 }
 
-__global__ void __launch_bounds__(kLazyThreads)
-blk_lazy_symbolic_kernel(uint32_t n, uint32_t k, const uint64_t *__restrict__ C0,
-                         uint64_t *__restrict__ W, BlkState *st) {
-  const int B = st->B;
-  __shared__ uint64_t su[kLazyMaxWindows];   // U_w
-  __shared__ uint8_t sa[kLazyMaxWindows];    // a_w: steps replayed on the window's rows
-  __shared__ uint8_t sinit[kLazyMaxWindows]; // rows already in the working copy
-  __shared__ int32_t spiv[64];               // stabilizer index of each step's pivot
-  __shared__ uint64_t scp[64];               // its C at that step
-  __shared__ uint32_t srow[2][32];           // per warp: first row with bit j (or ~0u)
-  __shared__ uint64_t sval[2][32], sor[2][32];
-  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const uint32_t nwin = (n + kLazyThreads - 1) >> kLazyLog2;
-  const uint64_t lo = 64ull * k;
-  for (uint32_t w = tid; w < nwin; w += kLazyThreads) {
-    su[w] = st->win_or[w];
-    sa[w] = 0;
-    sinit[w] = 0;
-  }
-  if (tid < 64) {  // slots of warps the block does not have stay empty
-    srow[tid >> 5][tid & 31] = 0xFFFFFFFFu;
-    sval[tid >> 5][tid & 31] = 0;
-    sor[tid >> 5][tid & 31] = 0;
-  }
-  __syncthreads();
-  uint32_t front = 0;  // first window that may hold a nonzero row (uniform)
-  while (front < nwin && su[front] == 0) ++front;
-  int len = B, par = 0;
-  uint32_t cw = 0xFFFFFFFFu;  // window whose row this thread holds in cc
-  uint64_t cc = 0;
-  for (int j = 0; j < B; ++j) {
-    uint32_t hit = 0xFFFFFFFFu;
-    uint64_t hitc = 0;
-    for (uint32_t w = front; w < nwin; ++w) {
-      const int a = sa[w];
-      if (!((lazy_bound(su[w], a, j, scp) >> j) & 1ull)) continue;  // no row can have bit j
-      // bring row kLazyThreads w + tid up to step j
-      const uint32_t i = w * kLazyThreads + tid;
-      uint64_t c = 0;
-      if (i < n) {
-        if (cw == w) c = cc;
-        else c = sinit[w] ? W[lo + i] : C0[lo + i];
-        for (int s2 = a; s2 < j; ++s2) {
-          if ((int32_t)i == spiv[s2]) c = 0;
-          else if ((c >> s2) & 1ull) c ^= scp[s2];
-        }
-        if (cw != w && cw != 0xFFFFFFFFu) W[lo + cw * kLazyThreads + tid] = cc;  // evict the held row
-        cw = w;
-        cc = c;
-      }
-      const bool has = i < n && ((c >> j) & 1ull);
-      const uint32_t ball = __ballot_sync(0xffffffffu, has);
-      const uint32_t first = ball ? (uint32_t)(__ffs(ball) - 1) : 32u;
-      const uint64_t fc = __shfl_sync(0xffffffffu, c, first & 31);
-      uint64_t o = c;
-      for (int d = 16; d > 0; d >>= 1) o |= __shfl_xor_sync(0xffffffffu, o, d);
-      if (lane == 0) {
-        srow[par][warp] = ball ? warp * 32 + first : 0xFFFFFFFFu;
-        sval[par][warp] = fc;
-        sor[par][warp] = o;
-      }
-      __syncthreads();
-      // every warp reduces the 32 per-warp slots lane-parallel (lane v reads slot v)
-      const uint32_t rv = srow[par][lane];
-      const uint64_t vv = sval[par][lane], ov = sor[par][lane];
-      const uint32_t best = __reduce_min_sync(0xffffffffu, rv);
-      const uint32_t bl = __ffs(__ballot_sync(0xffffffffu, rv == best)) - 1;
-      const uint64_t bc = __shfl_sync(0xffffffffu, vv, bl);
-      const uint64_t wor = ((uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)(ov >> 32)) << 32) |
-                           __reduce_or_sync(0xffffffffu, (uint32_t)ov);
-      par ^= 1;
-      if (tid == 0) {
-        su[w] = wor;
-        sa[w] = (uint8_t)j;
-        sinit[w] = 1;
-      }
-      if (best != 0xFFFFFFFFu) {
-        hit = w * kLazyThreads + best;
-        hitc = bc;
-        break;
-      }
-    }
-    if (hit == 0xFFFFFFFFu) { len = j; break; }  // deterministic: the block ends before step j
-    if (tid == 0) {
-      spiv[j] = (int32_t)hit;
-      scp[j] = hitc;
-      st->piv[j] = (int64_t)(lo + hit);
-      st->cpiv[j] = hitc;
-    }
-    __syncthreads();  // su/sa/sinit and the new pivot are visible to every thread
-  }
-  if (tid == 0) st->len = len;
-}
-
-__global__ void __launch_bounds__(256)
-blk_replay_kernel(uint64_t nrows, uint32_t k, const uint64_t *__restrict__ C0,
-                  uint64_t *__restrict__ M, int32_t *__restrict__ base, BlkState *st) {
-  __shared__ int64_t sp[64];
-  __shared__ uint64_t sc[64];
-  const int L = st->len;
-  if (threadIdx.x < 64 && (int)threadIdx.x < L) {
-    sp[threadIdx.x] = st->piv[threadIdx.x];
-    sc[threadIdx.x] = st->cpiv[threadIdx.x];
-  }
-  __syncthreads();
-  const uint64_t r = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= nrows) return;
-  const int64_t lo = 64ll * k;
-  uint64_t c = C0[r], m = 0;
-  int32_t b = kBaseOrig;
-  for (int j = 0; j < L; ++j) {
-    const int64_t p = sp[j];
-    if ((int64_t)r == p) {
-      st->mpiv[j] = m;
-      b = kBasePivot + j;
-      c = 0;
-    } else if ((int64_t)r == p - lo) {
-      c = sc[j];
-      m = 0;
-      b = j;
-    } else if ((c >> j) & 1ull) {
-      c ^= sc[j];
-      m |= 1ull << j;
-    }
-  }
-  M[r] = m;
-  base[r] = b;
-}
-
-// pivot rows V_j and their phase sums for one chunk of 32 column words.
-// V_j is the product of the original pivot rows p_s over a set E_j of steps:
-// E_j = {j} xor (xor of E_s over the steps s that targeted p_j before step j),
-// built by one warp in step order; every V_j of the chunk is then independent.
-// Lane = column word; warp w takes steps w, w + 32; four blocks per chunk
-// share the pairwise parities G.
-constexpr int kVrowThreads = 1024;
+// ---------------------------------------------------------------------------
+// blk_middle: the pivot rows V_j with their phase sums (and in the last of
+// those blocks their signs), next to the blocks that turn C into M, the bases
+// and the list of rows the block changes
+// ---------------------------------------------------------------------------
+constexpr int kMidThreads = 1024;
 constexpr int kVrowSplit = 4;  // blocks per chunk; block y computes G rows 16 y .. 16 y + 15
 constexpr size_t kVrowSmem = 4ull * 64 * 32 * sizeof(uint64_t);  // original and V rows, x and z
 
-__global__ void __launch_bounds__(kVrowThreads)
-blk_vrows_kernel(const uint64_t *__restrict__ RX, const uint64_t *__restrict__ RZ, uint32_t rs,
-                 uint64_t *__restrict__ VX, uint64_t *__restrict__ VZ, BlkState *st) {
+struct MiddleArgs {
+  const uint64_t *RX, *RZ, *S, *C;
+  uint64_t nrows;
+  uint32_t rs, k, chunks, B;
+  int lazy;
+  uint64_t *VX, *VZ, *M;
+  int32_t *base;
+  uint4 *list;
+  BlkWindow *win;
+  BlkState *st;
+  uint32_t *err;
+};
+
+// signs of V_j (first 64 x 16 threads of the block). The phase exponent of step j is
+//   e_j = 2 r(p_j) + B0_j - A_j + 2 Cp_j + sum_{s in m_j} (2 rV_s + A_s) + 2 cross(m_j)
+// (mod 4), cross(m) = sum over s > t in m of G[s] bit t; everything but the
+// 2 rV_s terms is independent of the other steps. With b_j = e'_j / 2 the signs
+// solve rV = b + m rV (m strictly lower triangular), so rV_j = parity(E_j & b).
+__device__ __forceinline__ void pivot_signs(const MiddleArgs &a) {
+  __shared__ int sA[64];
+  __shared__ uint64_t sm[64], sG[64];
+  __shared__ uint32_t s_b[64];
+  BlkState *st = a.st;
+  const int t = threadIdx.x;
+  if (t < 64) {
+    sm[t] = t < (int)a.B ? __ldcg(&st->mpiv[t]) : 0;
+    sA[t] = __ldcg(&st->A[t]);
+    sG[t] = __ldcg(&st->G[t]);
+  }
+  __syncthreads();
+  const int j = t >> 4, part = t & 15;  // 16 threads per step, 4 bits of m each
+  const uint64_t m = sm[j];
+  int e = 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int s = 4 * part + i;
+    if ((m >> s) & 1ull) e += sA[s] + 2 * (__popcll(sG[s] & m & ((1ull << s) - 1)) & 1);
+  }
+  for (int o = 8; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+  if (part == 0) {
+    uint32_t b = 0;
+    const int64_t p = j < (int)a.B ? st->piv[j] : kBlkNone;
+    if (p != kBlkNone) {
+      e += 2 * (int)((a.S[p >> 6] >> (p & 63)) & 1u) + __ldcg(&st->B0[j]) - sA[j] + 2 * __ldcg(&st->Cp[j]);
+      e = m4(e);
+      if (e & 1) atomicOr(a.err, kErrOddPhase);
+      b = (uint32_t)(e >> 1);
+    }
+    s_b[j] = b;
+  }
+  __syncthreads();
+  if (t < 64) {
+    const uint64_t E = st->E[t];
+    int rv = 0;
+    for (int s = 0; s < 64; ++s) rv ^= (int)((E >> s) & s_b[s] & 1u);
+    st->rV[t] = rv;
+  }
+}
+
+__device__ __forceinline__ void pivot_rows(const MiddleArgs &a, uint32_t chunk, int y) {
   extern __shared__ uint64_t vsm[];
   uint64_t(*ox)[32] = reinterpret_cast<uint64_t(*)[32]>(vsm);
   uint64_t(*oz)[32] = reinterpret_cast<uint64_t(*)[32]>(vsm + 64 * 32);
   uint64_t(*vx)[32] = reinterpret_cast<uint64_t(*)[32]>(vsm + 2 * 64 * 32);
   uint64_t(*vz)[32] = reinterpret_cast<uint64_t(*)[32]>(vsm + 3 * 64 * 32);
   __shared__ uint64_t sE[64];
-  const int L = st->len;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const bool lead = blockIdx.y == 0;  // writes the V rows and the per-step sums
+  __shared__ bool s_last;
+  BlkState *st = a.st;
+  const uint32_t rs = a.rs;
+  const int L = (int)a.B;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = kMidThreads >> 5;
+  const bool lead = y == 0;  // writes the V rows and the per-step sums
   // every word of the padded row (u < rs): padding qubit words are zero in the
   // tableau and come out zero in the V rows too
-  const uint32_t u = blockIdx.x * 32 + lane;
+  const uint32_t u = chunk * 32 + lane;
   const bool in = u < rs;
   for (int j = w; j < L; j += nw) {
-    const uint64_t p = (uint64_t)st->piv[j];
-    ox[j][lane] = in ? RX[p * rs + u] : 0;
-    oz[j][lane] = in ? RZ[p * rs + u] : 0;
+    const int64_t p = st->piv[j];
+    const bool ld = in && p != kBlkNone;
+    ox[j][lane] = ld ? a.RX[(uint64_t)p * rs + u] : 0;
+    oz[j][lane] = ld ? a.RZ[(uint64_t)p * rs + u] : 0;
   }
-  if (w == 0) {
-    // E_j = {j} + sum of E_s over the steps s < j that targeted p_j (m_j), one
-    // step after another: lane l keeps E_l and E_{l+32} in registers and each
-    // step is one XOR reduction over the warp; the masks are loaded once
-    const uint64_t mlo = lane < L ? st->mpiv[lane] : 0, mhi = lane + 32 < L ? st->mpiv[lane + 32] : 0;
-    uint64_t elo = 0, ehi = 0;
-    for (int j = 0; j < L; ++j) {
-      const uint64_t m = __shfl_sync(0xffffffffu, j < 32 ? mlo : mhi, j & 31);  // only steps before j
-      const uint64_t acc = (((m >> lane) & 1u) ? elo : 0) ^ (((m >> (lane + 32)) & 1u) ? ehi : 0);
-      const uint64_t ej = (((uint64_t)__reduce_xor_sync(0xffffffffu, (uint32_t)(acc >> 32)) << 32) |
-                           __reduce_xor_sync(0xffffffffu, (uint32_t)acc)) ^ (1ull << j);
-      if (lane == (j & 31)) {
-        if (j < 32) elo = ej;
-        else ehi = ej;
-      }
-    }
-    if (lane < L) sE[lane] = elo;
-    if (lane + 32 < L) sE[lane + 32] = ehi;
-  }
+  if (threadIdx.x < 64) sE[threadIdx.x] = st->E[threadIdx.x];
   __syncthreads();
   // every block builds all V rows of its chunk (G needs them); the lead block
-  // also stores them and adds the per-step popcount sums
+  // also stores them and adds the per-step popcount sums. Deterministic steps
+  // have an empty E: their V row is zero.
   for (int j = w; j < L; j += nw) {
     const uint64_t x0 = ox[j][lane], z0 = oz[j][lane];
-    uint64_t ax = x0, az = z0, e = sE[j] & ~(1ull << j);
+    uint64_t ax = 0, az = 0, e = sE[j];
     while (e) {
       const int s2 = __ffsll((long long)e) - 1;
       e &= e - 1;
@@ -395,17 +762,14 @@ blk_vrows_kernel(const uint64_t *__restrict__ RX, const uint64_t *__restrict__ R
     vz[j][lane] = az;
     if (!lead) continue;
     if (in) {
-      VX[(uint64_t)j * rs + u] = ax;
-      VZ[(uint64_t)j * rs + u] = az;
+      a.VX[(uint64_t)j * rs + u] = ax;
+      a.VZ[(uint64_t)j * rs + u] = az;
     }
-    int a = __popcll(ax & az), b = __popcll(x0 & z0);
+    const int av = __reduce_add_sync(0xffffffffu, __popcll(ax & az));
+    const int b = __reduce_add_sync(0xffffffffu, __popcll(x0 & z0));
     const uint32_t c = __ballot_sync(0xffffffffu, __popcll((az ^ z0) & x0) & 1);
-    for (int o = 16; o > 0; o >>= 1) {
-      a += __shfl_xor_sync(0xffffffffu, a, o);
-      b += __shfl_xor_sync(0xffffffffu, b, o);
-    }
     if (lane == 0) {
-      if (a) atomicAdd(&st->A[j], a);
+      if (av) atomicAdd(&st->A[j], av);
       if (b) atomicAdd(&st->B0[j], b);
       if (__popc(c) & 1) atomicXor(&st->Cp[j], 1);
     }
@@ -413,7 +777,7 @@ blk_vrows_kernel(const uint64_t *__restrict__ RX, const uint64_t *__restrict__ R
   __syncthreads();
   // G[s] bit t = parity of z_{V_s} . x_{V_t} over the chunk: block y takes
   // s = 16 y + w / 2, each warp half of the t range
-  const int sg = 16 * (int)blockIdx.y + (w >> 1), t0 = 32 * (w & 1);
+  const int sg = 16 * y + (w >> 1), t0 = 32 * (w & 1);
   if (sg < L) {
     const uint64_t zs = vz[sg][lane];
     uint64_t row = 0;
@@ -423,60 +787,80 @@ blk_vrows_kernel(const uint64_t *__restrict__ RX, const uint64_t *__restrict__ R
     }
     if (lane == 0 && row) atomicXor(reinterpret_cast<unsigned long long *>(&st->G[sg]), row);
   }
-}
-
-__device__ __forceinline__ int cross_pairs(const uint64_t *G, uint64_t m) {
-  // parity of sum over s > t, both in m, of G[s] bit t
-  int par = 0;
-  uint64_t mm = m;
-  while (mm) {
-    const int s = __ffsll((long long)mm) - 1;
-    mm &= mm - 1;
-    par ^= __popcll(G[s] & m & ((1ull << s) - 1)) & 1;
-  }
-  return par;
-}
-
-// signs of V_j. The phase exponent of step j is
-//   e_j = 2 r(p_j) + B0_j - A_j + 2 Cp_j + sum_{s in m_j} (2 rV_s + A_s) + 2 cross(m_j)
-// (mod 4); everything but the 2 rV_s terms is independent of the other steps and
-// is computed by one thread per step, then one thread resolves the signs in
-// step order: rV_j = (e'_j >> 1) ^ parity(m_j & {s : rV_s = 1}).
-__global__ void __launch_bounds__(64) blk_signs_kernel(const uint64_t *__restrict__ S, BlkState *st,
-                                                       uint32_t *err) {
-  __shared__ int sb[64], sA[64];
-  __shared__ uint64_t sm[64], sG[64];
-  const int L = st->len, j = threadIdx.x;
-  if (j < L) {
-    sm[j] = st->mpiv[j];
-    sA[j] = st->A[j];
-    sG[j] = st->G[j];
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    s_last = atomicAdd(&a.win->middle_arrived, 1u) == a.chunks * kVrowSplit - 1;
+    if (s_last) a.win->middle_arrived = 0;
   }
   __syncthreads();
-  if (j < L) {
-    const int64_t p = st->piv[j];
-    const uint64_t m = sm[j];
-    int e = 2 * (int)((S[p >> 6] >> (p & 63)) & 1u) + st->B0[j] - sA[j] + 2 * st->Cp[j];
-    uint64_t mm = m;
-    while (mm) {
-      const int s = __ffsll((long long)mm) - 1;
-      mm &= mm - 1;
-      e += sA[s];
+  if (!s_last) return;
+  __threadfence();
+  pivot_signs(a);
+}
+
+// M, base and the row list of 1,024 rows. A row that is neither a pivot nor a
+// replaced destabilizer has M_r = XOR of lin[t] over the bits of C_r: 16
+// lookups in tables of 4 bits each instead of replaying 64 steps. The partner
+// of step j starts from C = v_j with only the later steps left. The list holds
+// every row the block changes with its pattern and base (one atomic per warp);
+// rows left alone (M_r = 0, original base: e.g. the +-Z_q pivot rows of earlier
+// blocks) are neither listed, read nor written by the apply pass.
+__device__ __forceinline__ void list_rows(const MiddleArgs &a, uint32_t blk) {
+  __shared__ uint64_t tab[16 * 16];
+  __shared__ int16_t special[kMidThreads];
+  const int t = threadIdx.x, lane = t & 31;
+  const uint64_t r0 = (uint64_t)blk * kMidThreads, r = r0 + t;
+  uint64_t m = 0;
+  int32_t b = kBaseOrig;
+  if (a.lazy) {
+    special[t] = -1;
+    if (t < 256) {
+      const int g = t >> 4, pat = t & 15;
+      uint64_t x = 0;
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if ((pat >> i) & 1) x ^= a.st->lin[4 * g + i];
+      tab[t] = x;
     }
-    e += 2 * cross_pairs(sG, m);
-    sb[j] = m4(e);
-  }
-  __syncthreads();
-  if (j == 0) {
-    uint64_t R = 0;
-    for (int i = 0; i < L; ++i) {
-      const int e = sb[i];
-      if (e & 1) atomicOr(err, kErrOddPhase);
-      const int rv = (e >> 1) ^ (__popcll(sm[i] & R) & 1);
-      R |= (uint64_t)rv << i;
+    __syncthreads();
+    if (t < (int)a.B) {
+      const int64_t p = a.st->piv[t];
+      if (p != kBlkNone) {
+        const int64_t dp = p - (int64_t)r0, dd = dp - 64ll * a.k;
+        if (dp >= 0 && dp < kMidThreads) special[dp] = (int16_t)(kBasePivot + t);
+        if (dd >= 0 && dd < kMidThreads) special[dd] = (int16_t)t;
+      }
     }
-    for (int i = 0; i < L; ++i) st->rV[i] = (int)((R >> i) & 1u);
+    __syncthreads();
+    if (r < a.nrows) {
+      b = special[t];
+      uint64_t c = 0;
+      if (b == kBaseOrig) c = a.C[r];
+      else if (b < kBasePivot) c = a.st->cpiv[b] & ~((2ull << b) - 1);
+#pragma unroll
+      for (int g = 0; g < 16; ++g) m ^= tab[16 * g + ((c >> (4 * g)) & 15)];
+      a.M[r] = m;
+      a.base[r] = b;
+    }
+  } else if (r < a.nrows) {
+    m = a.M[r];
+    b = a.base[r];
   }
+  const bool touched = r < a.nrows && (b != kBaseOrig || m != 0);
+  const uint32_t ball = __ballot_sync(0xffffffffu, touched);
+  uint32_t at = 0;
+  if (lane == 0 && ball) at = atomicAdd(&a.st->ntouched, (uint32_t)__popc(ball));
+  at = __shfl_sync(0xffffffffu, at, 0);
+  if (touched)
+    a.list[at + __popc(ball & ((1u << lane) - 1))] =
+        make_uint4((uint32_t)r, (uint32_t)b, (uint32_t)m, (uint32_t)(m >> 32));
+}
+
+__global__ void __launch_bounds__(kMidThreads) blk_middle_kernel(const MiddleArgs a) {
+  const uint32_t nv = a.chunks * kVrowSplit;
+  if (blockIdx.x < nv) pivot_rows(a, blockIdx.x / kVrowSplit, (int)(blockIdx.x % kVrowSplit));
+  else list_rows(a, blockIdx.x - nv);
 }
 
 // phase 3: block = one chunk of kCW (32) column words x a range of rows.
@@ -529,32 +913,6 @@ __device__ __forceinline__ void apply_meta(ApplyMeta &m, uint32_t j, uint32_t cn
     m.lo = e.z;
     m.hi = e.w;
   }
-}
-
-// the row list: every row the block changes (a step targeted it, or its base
-// changed: replaced destabilizers and the new pivots) with its pattern and
-// base, in groups of consecutive rows (one atomic per warp). Rows left alone
-// (M_r = 0, original base: e.g. the +-Z_q pivot rows of earlier blocks) are
-// neither listed, read nor written.
-__global__ void __launch_bounds__(256)
-blk_list_kernel(uint64_t nrows, const uint64_t *__restrict__ M, const int32_t *__restrict__ base,
-                uint4 *__restrict__ list, BlkState *st) {
-  const uint64_t r = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  uint64_t m = 0;
-  int32_t b = kBaseOrig;
-  if (r < nrows) {
-    m = M[r];
-    b = base[r];
-  }
-  const bool touched = r < nrows && (b != kBaseOrig || m != 0);
-  const uint32_t ball = __ballot_sync(0xffffffffu, touched);
-  const uint32_t lane = threadIdx.x & 31;
-  uint32_t at = 0;
-  if (lane == 0 && ball) at = atomicAdd(&st->ntouched, (uint32_t)__popc(ball));
-  at = __shfl_sync(0xffffffffu, at, 0);
-  if (touched)
-    list[at + __popc(ball & ((1u << lane) - 1))] =
-        make_uint4((uint32_t)r, (uint32_t)b, (uint32_t)m, (uint32_t)(m >> 32));
 }
 
 // the row's words, fetched only when the row changes: a row that no step
@@ -659,7 +1017,7 @@ __device__ __forceinline__ void apply_row(const ApplyRow &a, uint32_t nrows, uin
   if (r >= nrows) return;  // uniform over the warp
   const Idx off = (Idx)r * rs + word;
   uint2 *px = reinterpret_cast<uint2 *>(RX), *pz = reinterpret_cast<uint2 *>(RZ);
-  if (a.b >= kBasePivot) {  // pivot row of step j: +-Z_q (sign set by blk_rows_kernel)
+  if (a.b >= kBasePivot) {  // pivot row of step j: +-Z_q (sign set by blk_front_kernel)
     const uint32_t q = qubits[a.b - kBasePivot];
     if (ok) {
       px[off] = make_uint2(0, 0);
@@ -716,14 +1074,13 @@ constexpr int kApplyWaves = 32;
 template <typename Idx>
 __global__ void __launch_bounds__(kApplyThreads, 1)
 blk_apply_kernel(uint64_t *__restrict__ RX, uint64_t *__restrict__ RZ, uint32_t rs, uint32_t nrows,
-                 const uint32_t *__restrict__ window, const uint64_t *__restrict__ VX,
+                 const uint32_t *__restrict__ qubits, int L, const uint64_t *__restrict__ VX,
                  const uint64_t *__restrict__ VZ, const uint4 *__restrict__ list,
                  int32_t *__restrict__ Tp, const BlkState *st) {
   extern __shared__ ulonglong2 T[];  // [kSmemEntries][kCW] of (x word, z word)
   __shared__ uint32_t s_tmem;
-  const int L = st->len;
-  if (L == 0) return;  // a block enqueued past the window's end or behind a deterministic step
-  const uint32_t *qubits = window + st->i0;
+  const uint32_t cnt = st->ntouched;
+  if (cnt == 0) return;  // every outcome of the block is deterministic
   const uint32_t u0 = blockIdx.x * kCW;  // first column word of the chunk
   const uint32_t nw = min((uint32_t)kCW, rs - u0);
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -796,8 +1153,7 @@ blk_apply_kernel(uint64_t *__restrict__ RX, uint64_t *__restrict__ RZ, uint32_t 
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t cnt = st->ntouched;
-  if (L > 0) {
+  {
     const bool ok = lane < nw;
     const uint32_t word = u0 + lane;
     const char *tb = reinterpret_cast<const char *>(T);
@@ -833,163 +1189,331 @@ blk_apply_kernel(uint64_t *__restrict__ RX, uint64_t *__restrict__ RZ, uint32_t 
   }
 }
 
-// per row: new sign from the accumulated terms; pivot rows get their coin; record
-__global__ void __launch_bounds__(256)
-blk_rows_kernel(uint64_t *__restrict__ S, uint64_t nrows, const uint64_t *__restrict__ M,
-                const int32_t *__restrict__ base, const int32_t *__restrict__ Tp, uint32_t chunks,
-                BlkState *st, uint64_t window_m0, uint64_t seed, uint64_t shot,
-                uint8_t *__restrict__ record, uint8_t *__restrict__ kinds, uint32_t *__restrict__ err) {
-  __shared__ int sw[64];          // 2 rV_s + A_s of each step
-  __shared__ uint64_t sG[64];     // G rows
-  const int L = st->len;
-  const uint64_t m0 = window_m0 + st->i0;  // record index of the block's first measurement
-  const uint64_t r = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if ((int)threadIdx.x < L) {  // blockDim >= 64 >= L
-    sw[threadIdx.x] = 2 * st->rV[threadIdx.x] + st->A[threadIdx.x];
-    sG[threadIdx.x] = st->G[threadIdx.x];
-  }
-  __syncthreads();
-  if (r == 0) st->cursor = st->i0 + (uint32_t)L;  // the next block starts here
-  if (r < (uint64_t)L) {
-    const uint32_t b = (uint32_t)(philox4x64_10(m0 + r, shot, 0, 0, seed, kCoinKey).v[0] & 1u);
-    record[m0 + r] = (uint8_t)b;
-    kinds[m0 + r] = 1;  // every step of a block had a pivot
-  }
-  uint64_t delta = 0;
-  if (r < nrows && L > 0) {
-    const int32_t b = base[r];
-    const uint64_t sr = M[r];
-    const uint64_t old = (S[r >> 6] >> (r & 63)) & 1u;
-    uint64_t nb = old;
-    if (b >= kBasePivot) {
-      const int j = b - kBasePivot;
-      nb = philox4x64_10(m0 + j, shot, 0, 0, seed, kCoinKey).v[0] & 1u;
-    } else if (b != kBaseOrig || sr != 0) {
-      const int rb = (b == kBaseOrig) ? (int)old : st->rV[b];
-      int tsum = 0, csum = 0;
-      for (uint32_t ch = 0; ch < chunks; ++ch) {
-        const int32_t v = Tp[(uint64_t)ch * nrows + r];
-        tsum += v >> 1;  // arithmetic shift: t
-        csum ^= v & 1;
+// ---------------------------------------------------------------------------
+// blk_det: the deterministic outcomes of a window, after its last block.
+// (-1)^m Z_q = prod of S_i over the destabilizers D_i with x_iq = 1 (Sec. 2.5);
+// the phase of the product P_1 ... P_t is 2 sum r + sum |x_a & z_a| +
+// 2 sum_{a<b} z_a . x_b (mod 4), in any order of the rows since they commute.
+// An item is (up to 32 outcomes) x (32 column words) x (a range of rows): a
+// block gathers the outcomes' column bits of 128 destabilizer rows at a time,
+// keeps the rows that belong to any of them, and each of its four warps folds
+// those rows into 8 outcomes (lane = word; XOR totals X, Z and the cross term
+// in registers). With one group of outcomes the rows are split over blocks
+// (about 152 (range, outcome) pairs, as one outcome per launch had), whose
+// totals the last block of a column chunk merges: cross ^= X_range . Z_before.
+// The last block of a group of outcomes writes their record entries.
+// ---------------------------------------------------------------------------
+constexpr int kDetThreads = 128;
+constexpr int kDetGroup = 32;
+
+struct DetArgs {
+  const uint64_t *RX, *RZ, *S;
+  uint32_t rs, n, k, chunks;
+  const uint32_t *window, *det;
+  BlkWindow *win;
+  int32_t *acc;         // phase exponent per outcome
+  uint32_t *arrived;    // items of a group that are done
+  uint64_t *det_x, *det_z;
+  uint64_t m0;
+  uint8_t *record;
+  uint32_t *err;
+};
+
+__global__ void __launch_bounds__(kDetThreads) blk_det_kernel(const DetArgs a) {
+  __shared__ uint32_t s_q[kDetGroup];
+  __shared__ uint32_t s_row[kDetThreads], s_d[kDetThreads];
+  __shared__ uint32_t s_cnt[4];
+  __shared__ int s_flag;
+  const uint32_t nd = a.win->ndet;
+  if (nd == 0) return;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const uint32_t groups = (nd + kDetGroup - 1) / kDetGroup;
+  const uint32_t R = groups > 1 ? 1u : max(1u, min((uint32_t)kDetBlocks / nd, (a.n + kDetThreads - 1) / kDetThreads));
+  const uint32_t per = ((a.n + R - 1) / R + kDetThreads - 1) / kDetThreads * kDetThreads;
+  const uint64_t items = (uint64_t)groups * a.chunks * R;
+  for (uint64_t it = blockIdx.x; it < items; it += gridDim.x) {
+    const uint32_t range = (uint32_t)(it % R), ch = (uint32_t)(it / R % a.chunks), g = (uint32_t)(it / R / a.chunks);
+    const uint32_t d = min((uint32_t)kDetGroup, nd - g * kDetGroup);
+    __syncthreads();
+    if (t < kDetGroup) s_q[t] = (uint32_t)t < d ? a.window[a.det[g * kDetGroup + t]] : 0;
+    __syncthreads();
+    const uint32_t u = ch * 32 + lane;
+    const bool in = u < a.k;
+    uint64_t X[8], Z[8], cross[8];
+    int cnt[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) { X[j] = Z[j] = cross[j] = 0; cnt[j] = 0; }
+    const uint32_t i1 = min(a.n, (range + 1) * per);
+    for (uint32_t i0 = range * per; i0 < i1; i0 += kDetThreads) {
+      const uint32_t i = i0 + t;
+      uint32_t D = 0;
+      if (i < i1) {
+        const uint64_t *row = a.RX + (uint64_t)i * a.rs;
+        uint32_t lastw = 0xFFFFFFFFu;
+        uint64_t word = 0;
+        for (uint32_t j = 0; j < d; ++j) {
+          const uint32_t q = s_q[j];
+          if ((q >> 6) != lastw) { lastw = q >> 6; word = row[lastw]; }
+          D |= (uint32_t)((word >> (q & 63)) & 1u) << j;
+        }
       }
-      int e = 2 * rb + tsum + 2 * csum;
-      uint64_t mm = sr;
-      while (mm) {
-        const int s = __ffsll((long long)mm) - 1;
-        mm &= mm - 1;
-        e += sw[s];
+      const uint32_t ball = __ballot_sync(0xffffffffu, D != 0);
+      if (lane == 0) s_cnt[warp] = __popc(ball);
+      __syncthreads();
+      uint32_t at = __popc(ball & ((1u << lane) - 1)), rows = 0;
+      for (int w = 0; w < 4; ++w) {
+        if (w < warp) at += s_cnt[w];
+        rows += s_cnt[w];
       }
-      e += 2 * cross_pairs(sG, sr);
-      e = m4(e);
-      if (e & 1) atomicOr(err, kErrOddPhase);
-      nb = (uint64_t)(e >> 1);
+      if (D) { s_row[at] = i; s_d[at] = D; }
+      __syncthreads();
+      for (uint32_t e0 = 0; e0 < rows; e0 += 4) {
+        uint64_t x[4], z[4];
+        uint32_t m[4], rb[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+          const uint32_t e = e0 + v;
+          m[v] = e < rows ? (s_d[e] >> (8 * warp)) & 0xFFu : 0u;
+          x[v] = z[v] = 0;
+          rb[v] = 0;
+          if (m[v]) {
+            const uint64_t row = 64ull * a.k + s_row[e];
+            if (in) { x[v] = a.RX[row * a.rs + u]; z[v] = a.RZ[row * a.rs + u]; }
+            if (ch == 0 && lane == 0) rb[v] = (uint32_t)(a.S[row >> 6] >> (row & 63)) & 1u;
+          }
+        }
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+          if (!m[v]) continue;
+          const int pc = __popcll(x[v] & z[v]) + 2 * (int)rb[v];
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+            if ((m[v] >> j) & 1u) {  // uniform over the warp
+              cross[j] ^= x[v] & Z[j];
+              X[j] ^= x[v];
+              Z[j] ^= z[v];
+              cnt[j] += pc;
+            }
+        }
+      }
+      __syncthreads();  // the row list is rewritten
     }
-    delta = (nb ^ old) << (r & 63);
+    bool bad = false;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const uint32_t o = 8 * warp + j;
+      if (o >= d) break;
+      const int v = __reduce_add_sync(0xffffffffu, cnt[j] + 2 * (__popcll(cross[j]) & 1));
+      if (lane == 0 && v) atomicAdd(a.acc + g * kDetGroup + o, v);
+      if (R == 1) {
+        const uint32_t q = s_q[o];
+        bad |= in && (X[j] != 0 || Z[j] != (u == (q >> 6) ? 1ull << (q & 63) : 0ull));
+      } else if (in) {
+        a.det_x[((uint64_t)range * d + o) * a.rs + u] = X[j];
+        a.det_z[((uint64_t)range * d + o) * a.rs + u] = Z[j];
+      }
+    }
+    __threadfence();
+    __syncthreads();
+    if (R > 1) {
+      if (t == 0) s_flag = atomicAdd(&a.win->det_chunk[ch], 1u) == R - 1;
+      __syncthreads();
+      if (!s_flag) continue;
+      __threadfence();
+      for (uint32_t o = warp; o < d; o += 4) {  // last range of this chunk: merge the ranges
+        uint64_t c = 0, xb = 0, zb = 0;
+        if (in)
+#pragma unroll 4
+          for (uint32_t q = 0; q < R; ++q) {
+            const uint64_t x = __ldcg(a.det_x + ((uint64_t)q * d + o) * a.rs + u),
+                           z = __ldcg(a.det_z + ((uint64_t)q * d + o) * a.rs + u);
+            c ^= x & zb;
+            xb ^= x;
+            zb ^= z;
+          }
+        const int v = __reduce_add_sync(0xffffffffu, 2 * (__popcll(c) & 1));
+        if (lane == 0 && v) atomicAdd(a.acc + o, v);
+        const uint32_t q = s_q[o];
+        bad |= in && (xb != 0 || zb != (u == (q >> 6) ? 1ull << (q & 63) : 0ull));
+      }
+      __threadfence();
+    }
+    if (bad) atomicOr(a.err, kErrDetProduct);
+    __syncthreads();
+    if (t == 0) s_flag = atomicAdd(a.arrived + g, 1u) == a.chunks - 1;
+    __syncthreads();
+    if (!s_flag) continue;
+    __threadfence();
+    if ((uint32_t)t < d) {
+      const int e = m4(__ldcg(a.acc + g * kDetGroup + t));
+      if (e & 1) atomicOr(a.err, kErrOddPhase);
+      a.record[a.m0 + a.det[g * kDetGroup + t]] = (uint8_t)(e >> 1);
+    }
   }
-  // fold the sign changes of the 32 rows of this warp into one atomic
-  for (int o = 16; o > 0; o >>= 1) delta |= __shfl_xor_sync(0xffffffffu, delta, o);
-  if ((threadIdx.x & 31) == 0 && r < nrows && delta)
-    atomicXor(reinterpret_cast<unsigned long long *>(&S[r >> 6]), delta);
 }
 
+// ---------------------------------------------------------------------------
+// launches
+// ---------------------------------------------------------------------------
 static uint32_t blk_chunks(const Layout &L) { return (L.rs + kCW - 1) / kCW; }
 
-size_t blocked_scratch_bytes(const Layout &L) {
-  auto al = [](size_t b) { return (b + 255) & ~size_t(255); };
-  return 3 * al(L.nrows * 8) + al(L.nrows * 4) + al((size_t)blk_chunks(L) * L.nrows * 4) +
-         2 * al(64ull * L.rs * 8) + al(sizeof(BlkState)) + al(L.nrows * 16);
-}
+// device scratch of the blocked measurement
+struct BlkScratch {
+  uint8_t *zero;       // start of the part zeroed per window: win, acc, arrived
+  size_t zero_bytes;
+  BlkWindow *win;
+  int32_t *acc;
+  uint32_t *arrived;
+  uint64_t *C0, *C1, *M, *orC, *VX, *VZ;
+  uint32_t *listRow, *cnt, *done, *det;
+  int32_t *base, *Tp;
+  uint4 *list;
+  size_t total;
+};
 
-static std::atomic<uint64_t> g_apply_attr_set{0};
+// measurements per window (the capacity of det and acc)
+static uint32_t blk_window_cap(const Layout &L) { return (uint32_t)L.nrows; }
 
-// Enqueues one block of up to 64 measurements; the number actually done is
-// st->len (read by the host after the stream is synchronised).
-cudaError_t launch_measure_block(const Dev &d, void *scratch, const uint32_t *window, uint32_t count,
-                                 uint64_t m0, qs_key key, cudaStream_t s, int *launches) {
-  const Layout &L = d.L;
+static BlkScratch blk_scratch(const Layout &L, void *scratch) {
+  BlkScratch b;
+  size_t off = 0;
   uint8_t *p = static_cast<uint8_t *>(scratch);
-  auto take = [&](size_t bytes) { uint8_t *q = p; p += (bytes + 255) & ~size_t(255); return q; };
-  uint64_t *C0 = reinterpret_cast<uint64_t *>(take(L.nrows * 8));
-  uint64_t *C1 = reinterpret_cast<uint64_t *>(take(L.nrows * 8));
-  uint64_t *M = reinterpret_cast<uint64_t *>(take(L.nrows * 8));
-  int32_t *base = reinterpret_cast<int32_t *>(take(L.nrows * 4));
-  const uint32_t chunks = blk_chunks(L);
-  int32_t *Tp = reinterpret_cast<int32_t *>(take((size_t)chunks * L.nrows * 4));
-  uint64_t *VX = reinterpret_cast<uint64_t *>(take(64ull * L.rs * 8));
-  uint64_t *VZ = reinterpret_cast<uint64_t *>(take(64ull * L.rs * 8));
-  BlkState *st = reinterpret_cast<BlkState *>(take(sizeof(BlkState)));
-  uint4 *list = reinterpret_cast<uint4 *>(take(L.nrows * 16));
-  const unsigned rb = (unsigned)((L.nrows + 255) / 256);
+  auto take = [&](size_t bytes) {
+    uint8_t *q = p + off;
+    off += (bytes + 255) & ~size_t(255);
+    return q;
+  };
+  const size_t cap = blk_window_cap(L), ranges = (L.nrows + 255) / 256;
+  b.zero = p;
+  b.win = reinterpret_cast<BlkWindow *>(take(sizeof(BlkWindow)));
+  b.acc = reinterpret_cast<int32_t *>(take(cap * 4));
+  b.arrived = reinterpret_cast<uint32_t *>(take((cap / kDetGroup + 1) * 4));
+  b.zero_bytes = off;
+  b.C0 = reinterpret_cast<uint64_t *>(take(L.nrows * 8));
+  b.C1 = reinterpret_cast<uint64_t *>(take(ranges * 256 * 8));
+  b.M = reinterpret_cast<uint64_t *>(take(L.nrows * 8));
+  b.base = reinterpret_cast<int32_t *>(take(L.nrows * 4));
+  b.Tp = reinterpret_cast<int32_t *>(take((size_t)blk_chunks(L) * L.nrows * 4));
+  b.VX = reinterpret_cast<uint64_t *>(take(64ull * L.rs * 8));
+  b.VZ = reinterpret_cast<uint64_t *>(take(64ull * L.rs * 8));
+  b.list = reinterpret_cast<uint4 *>(take(L.nrows * 16));
+  b.listRow = reinterpret_cast<uint32_t *>(take(ranges * 256 * 4));
+  b.cnt = reinterpret_cast<uint32_t *>(take(ranges * 4));
+  b.done = reinterpret_cast<uint32_t *>(take(ranges * 4));
+  b.orC = reinterpret_cast<uint64_t *>(take(ranges * 8));
+  b.det = reinterpret_cast<uint32_t *>(take(cap * 4));
+  b.total = off;
+  return b;
+}
+
+size_t blocked_scratch_bytes(const Layout &L) { return blk_scratch(L, nullptr).total; }
+
+static std::atomic<uint64_t> g_blk_attr_set{0};
+
+// about kApplyWaves waves of one block per SM (the tables take 226 KB of
+// shared memory and all of TMEM), but at least 512 rows per block so that
+// building the tables stays small next to the rows they serve
+static uint32_t apply_rows_y(const Dev &d, uint32_t chunks) {
+  return std::max<uint32_t>(1, (uint32_t)std::min<uint64_t>(((uint64_t)d.sms * kApplyWaves + chunks - 1) / chunks,
+                                                            d.L.nrows / 512));
+}
+
+static cudaError_t measure_window_cap(const Dev &d, void *scratch, const uint32_t *window, uint32_t count,
+                                      uint64_t m0, qs_key key, cudaStream_t s, int *launches) {
+  const Layout &L = d.L;
+  const BlkScratch b = blk_scratch(L, scratch);
+  const uint32_t chunks = blk_chunks(L), ranges = (uint32_t)((L.nrows + 255) / 256);
   const size_t smem = (size_t)kSmemEntries * kEntryBytes;
-  cudaError_t ea = once_per_device(g_apply_attr_set, [&]() {
-    cudaError_t e = cudaFuncSetAttribute(blk_apply_kernel<uint32_t>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(blk_apply_kernel<uint64_t>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)smem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(blk_vrows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)kVrowSmem);
-    return e;
+  cudaError_t e = once_per_device(g_blk_attr_set, [&]() {
+    cudaError_t x = cudaFuncSetAttribute(blk_apply_kernel<uint32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
+    if (x == cudaSuccess)
+      x = cudaFuncSetAttribute(blk_apply_kernel<uint64_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (x == cudaSuccess)
+      x = cudaFuncSetAttribute(blk_middle_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kVrowSmem);
+    if (x == cudaSuccess)  // 4 bytes per range of 256 rows: 32 KB at n = 2^20, next to 17 KB of static arrays
+      x = cudaFuncSetAttribute(blk_front_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
+    return x;
   });
-  if (ea != cudaSuccess) return ea;
-  tbegin(d.timer, QS_TIME_BLK_SYMBOLIC, s);
-  const uint32_t nwin = (L.n + kLazyThreads - 1) >> kLazyLog2;
-  blk_reset_kernel<<<1, 256, 0, s>>>(st, count, nwin);
-  blk_init_kernel<<<rb, 256, 0, s>>>(d.RX, L.rs, L.nrows, L.n, L.k, window, C0, M, base, st, d.err);
-  int sym_launches = 64;
-  if (!d.step_symbolic) {
-    blk_lazy_symbolic_kernel<<<1, kLazyThreads, 0, s>>>(L.n, L.k, C0, C1, st);
-    blk_replay_kernel<<<rb, 256, 0, s>>>(L.nrows, L.k, C0, M, base, st);
-    sym_launches = 2;
-  } else {
-    for (int j = 0; j < 64; ++j)  // steps past the block's length return at once
-      blk_step_kernel<<<rb, 256, 0, s>>>(L.nrows, L.n, L.k, j, (j & 1) ? C1 : C0, (j & 1) ? C0 : C1, M,
-                                         base, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(b.zero, 0, b.zero_bytes, s);
+  if (e != cudaSuccess) return e;
+  FrontArgs f{};
+  f.RX = d.RX; f.S = d.S; f.nrows = L.nrows; f.rs = L.rs; f.n = L.n; f.k = L.k; f.chunks = chunks;
+  f.window = window;
+  f.lazy = !d.step_symbolic;
+  f.C = b.C0; f.listC = b.C1; f.listRow = b.listRow; f.cnt = b.cnt; f.done = b.done; f.orC = b.orC;
+  f.M = b.M; f.base = b.base; f.Tp = b.Tp; f.win = b.win; f.det = b.det;
+  f.m0 = m0; f.seed = key.seed; f.shot = key.shot;
+  f.record = d.record; f.kinds = d.kinds; f.err = d.err;
+  MiddleArgs m{};
+  m.RX = d.RX; m.RZ = d.RZ; m.S = d.S; m.C = b.C0; m.nrows = L.nrows; m.rs = L.rs; m.k = L.k; m.chunks = chunks;
+  m.lazy = f.lazy;
+  m.VX = b.VX; m.VZ = b.VZ; m.M = b.M; m.base = b.base; m.list = b.list; m.win = b.win; m.err = d.err;
+  const uint32_t mid_blocks = chunks * kVrowSplit + (uint32_t)((L.nrows + kMidThreads - 1) / kMidThreads);
+  const uint32_t rows_y = apply_rows_y(d, chunks);
+  const bool narrow = !d.wide_offsets && (uint64_t)L.nrows * L.rs < (1ull << 32);
+  int nl = 0;
+  for (uint32_t i0 = 0, cur = 0;; i0 += 64, cur ^= 1) {
+    // signs of the block before i0, symbolic pass of the block at i0
+    f.prev_i0 = f.i0; f.prev_B = f.B;
+    f.i0 = i0;
+    f.B = i0 < count ? std::min<uint32_t>(64, count - i0) : 0;
+    f.cur = (int)cur;
+    BlkState *st = &b.win->st[cur];
+    const int kind = f.B ? QS_TIME_BLK_SYMBOLIC : QS_TIME_BLK_SIGNS;
+    tbegin(d.timer, kind, s);
+    if (!f.lazy && f.B) {
+      blk_step_reset_kernel<<<1, 64, 0, s>>>(st);
+      ++nl;
+    }
+    blk_front_kernel<<<ranges, 256, f.lazy ? ranges * 4 : 0, s>>>(f);
+    ++nl;
+    if (!f.lazy && f.B) {
+      // C0 -> C1 -> C0 ...; nothing reads C after the last step
+      for (int j = 0; j < (int)f.B; ++j)
+        blk_step_kernel<<<ranges, 256, 0, s>>>(L.nrows, L.n, L.k, j, (int)f.B, (j & 1) ? b.C1 : b.C0,
+                                               (j & 1) ? b.C0 : b.C1, b.M, b.base, st);
+      blk_step_finish_kernel<<<1, 64, 0, s>>>(st, (int)f.B);
+      nl += (int)f.B + 1;
+    }
+    tend(d.timer, kind, s);
+    if (!f.B) break;
+    m.B = f.B;
+    m.st = st;
+    tbegin(d.timer, QS_TIME_BLK_PIVOT_ROWS, s);
+    blk_middle_kernel<<<mid_blocks, kMidThreads, kVrowSmem, s>>>(m);
+    tend(d.timer, QS_TIME_BLK_PIVOT_ROWS, s);
+    tbegin(d.timer, QS_TIME_BLK_APPLY, s);
+    if (narrow)
+      blk_apply_kernel<uint32_t><<<dim3(chunks, rows_y), kApplyThreads, smem, s>>>(
+          d.RX, d.RZ, L.rs, (uint32_t)L.nrows, window + i0, (int)f.B, b.VX, b.VZ, b.list, b.Tp, st);
+    else
+      blk_apply_kernel<uint64_t><<<dim3(chunks, rows_y), kApplyThreads, smem, s>>>(
+          d.RX, d.RZ, L.rs, (uint32_t)L.nrows, window + i0, (int)f.B, b.VX, b.VZ, b.list, b.Tp, st);
+    tend(d.timer, QS_TIME_BLK_APPLY, s);
+    nl += 2;
+    if (d.timer && (i0 & 4095) == 4032) d.timer->resolve();  // completed event pairs go back to the pool
   }
-  tend(d.timer, QS_TIME_BLK_SYMBOLIC, s);
-  tbegin(d.timer, QS_TIME_BLK_PIVOT_ROWS, s);
-  blk_vrows_kernel<<<dim3(chunks, kVrowSplit), kVrowThreads, kVrowSmem, s>>>(d.RX, d.RZ, L.rs, VX,
-                                                                              VZ, st);
-  blk_signs_kernel<<<1, 64, 0, s>>>(d.S, st, d.err);
-  blk_list_kernel<<<rb, 256, 0, s>>>(L.nrows, M, base, list, st);
-  tend(d.timer, QS_TIME_BLK_PIVOT_ROWS, s);
-  // about kApplyWaves waves of one block per SM (the tables take 226 KB of
-  // shared memory and all of TMEM), but at least 512 rows per block so that
-  // building the tables stays small next to the rows they serve
-  const uint32_t rows_y = std::max<uint32_t>(
-      1, (uint32_t)std::min<uint64_t>(((uint64_t)d.sms * kApplyWaves + chunks - 1) / chunks, L.nrows / 512));
-  tbegin(d.timer, QS_TIME_BLK_APPLY, s);
-  if (!d.wide_offsets && (uint64_t)L.nrows * L.rs < (1ull << 32))
-    blk_apply_kernel<uint32_t><<<dim3(chunks, rows_y), kApplyThreads, smem, s>>>(
-        d.RX, d.RZ, L.rs, (uint32_t)L.nrows, window, VX, VZ, list, Tp, st);
-  else
-    blk_apply_kernel<uint64_t><<<dim3(chunks, rows_y), kApplyThreads, smem, s>>>(
-        d.RX, d.RZ, L.rs, (uint32_t)L.nrows, window, VX, VZ, list, Tp, st);
-  tend(d.timer, QS_TIME_BLK_APPLY, s);
-  tbegin(d.timer, QS_TIME_BLK_SIGNS, s);
-  blk_rows_kernel<<<rb, 256, 0, s>>>(d.S, L.nrows, M, base, Tp, chunks, st, m0, key.seed, key.shot,
-                                     d.record, d.kinds, d.err);
-  tend(d.timer, QS_TIME_BLK_SIGNS, s);
-  if (launches) *launches += 7 + sym_launches;
+  DetArgs t{};
+  t.RX = d.RX; t.RZ = d.RZ; t.S = d.S; t.rs = L.rs; t.n = L.n; t.k = L.k; t.chunks = (L.k + 31) / 32;
+  t.window = window; t.det = b.det; t.win = b.win; t.acc = b.acc; t.arrived = b.arrived;
+  t.det_x = d.det_x; t.det_z = d.det_z; t.m0 = m0; t.record = d.record; t.err = d.err;
+  // enough blocks for one outcome's ranges and for every group; blocks without an item leave at once
+  const uint64_t most = std::max<uint64_t>(kDetBlocks, (count + kDetGroup - 1) / kDetGroup) * t.chunks;
+  blk_det_kernel<<<(unsigned)std::min<uint64_t>(most, 12ull * d.sms), kDetThreads, 0, s>>>(t);
+  if (launches) *launches += nl + 2;
   return cudaGetLastError();
 }
 
-__global__ void blk_set_cursor_kernel(BlkState *st, uint32_t v) { st->cursor = v; }
-
-static BlkState *blk_state(const Layout &L, void *scratch) {
-  auto al = [](size_t b) { return (b + 255) & ~size_t(255); };
-  return reinterpret_cast<BlkState *>(static_cast<uint8_t *>(scratch) + 3 * al(L.nrows * 8) +
-                                      al(L.nrows * 4) + al((size_t)blk_chunks(L) * L.nrows * 4) +
-                                      2 * al(64ull * L.rs * 8));
+cudaError_t launch_measure_blocks(const Dev &d, void *scratch, const uint32_t *window, uint32_t count, uint64_t m0,
+                                  qs_key key, cudaStream_t s, int *launches) {
+  const uint32_t cap = blk_window_cap(d.L);
+  for (uint32_t off = 0; off < count; off += cap) {
+    const cudaError_t e = measure_window_cap(d, scratch, window + off, std::min(cap, count - off), m0 + off, key, s,
+                                             launches);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
-
-cudaError_t set_block_cursor(const Layout &L, void *scratch, uint32_t v, cudaStream_t s) {
-  blk_set_cursor_kernel<<<1, 1, 0, s>>>(blk_state(L, scratch), v);
-  return cudaGetLastError();
-}
-
-const uint32_t *block_cursor(const Layout &L, void *scratch) { return &blk_state(L, scratch)->cursor; }
-
 
 }  // namespace qs

@@ -1,0 +1,55 @@
+"""Measurement windows with deterministic outcomes in them: they are evaluated together after the
+window's last block, and the symbolic pass looks past the rows it holds when those have no pivot."""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_2603_14641_gb300 import qs
+from workloads import circuits as C
+
+pytestmark = pytest.mark.gpu
+
+
+def _check(sim, o, rec, orec, okinds):
+    assert np.array_equal(rec, orec)
+    assert np.array_equal(sim.record_kinds(), okinds)
+    for a, b in zip(sim.export(), o.get()):
+        assert np.array_equal(a, b)
+    sim.sync()
+
+
+# 2,100 qubits: two 32-word column chunks. depth 2: sparse columns, most outcomes of the second pass
+# deterministic. 2,600 dense qubits with repeats: more than 1,024 nonzero rows and steps without a
+# pivot among them, so the symbolic pass scans the rest. One repeat only: the rows of its product are
+# split over blocks. 97 repeats: several groups of 32, the last one short.
+@pytest.mark.parametrize("flags", [0, qs.QS_FLAG_STEP_SYMBOLIC])
+@pytest.mark.parametrize("n,depth,first,again", [(70, 3, 70, 33), (300, 2, 150, 97), (2100, 2, 130, 97),
+                                                 (2600, 60, 40, 1), (2600, 60, 40, 97), (1030, 40, 64, 64)])
+def test_window_with_deterministic_outcomes(n, depth, first, again, flags):
+    circ = C.random_circuit(n, depth, 0.5, seed=n + depth, final_measure_all=False)
+    rng = np.random.default_rng(n + again)
+    q = rng.permutation(n)[:first].astype(np.uint32)
+    # repeats of measured qubits between and after the first measurements of others
+    q = np.concatenate([q[:first // 2], rng.choice(q[:first // 2], again // 2), q[first // 2:],
+                        rng.choice(q, again - again // 2)]).astype(np.uint32)
+    sim = qs.Simulator(n, flags=flags)
+    dc = sim.upload(circ)
+    sim.apply_layers_dev(dc, 0, depth)
+    rec = sim.measure(q, seed=5, shot=3)
+    o = O.Oracle(n)
+    o.apply(circ.gates)
+    orec, okinds = o.measure(q, seed=5, shot=3)
+    _check(sim, o, rec, orec, okinds)
+
+
+def test_out_of_range_device_qubit_in_a_window():
+    """A device list is not checked on the host: the outcome is 0 and the next sync reports it."""
+    import torch
+    sim = qs.Simulator(100)
+    q = np.arange(40, dtype=np.int32)
+    q[7] = 100
+    dev = torch.from_numpy(q).cuda()
+    sim.measure_dev(dev, seed=1)
+    with pytest.raises(qs.QsError) as e:
+        sim.sync()
+    assert e.value.code == -7
