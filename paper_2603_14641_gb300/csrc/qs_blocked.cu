@@ -36,8 +36,8 @@
 // then blk_det. The serial parts run in the block of a grid that arrives last,
 // so the host neither waits nor reads anything back: 3 launches per block where
 // a launch per part took 9 and a wait per round. 64 measurements of a dense
-// 10,000-qubit state: 172 -> 103 us; 3,000 measurements of a shallow 1,500-qubit
-// state, 2,456 of them deterministic (measured one by one before): 30.3 -> 2.4 ms.
+// 10,000-qubit state: 172 -> 70 us; 3,000 measurements of a shallow 1,500-qubit
+// state, 2,456 of them deterministic (measured one by one before): 30.3 -> 1.6 ms.
 #include <algorithm>
 #include <climits>
 
@@ -45,7 +45,7 @@
 
 namespace qs {
 
-constexpr int32_t kBaseOrig = -1;
+constexpr int32_t kBaseOrig = -1;    // all bits set
 constexpr int32_t kBasePivot = 1000;  // base = kBasePivot + j: pivot row of step j
 constexpr int kCW = 32;               // column words per phase-3 chunk
 constexpr int64_t kBlkNone = LLONG_MAX;
@@ -61,9 +61,8 @@ struct BlkState {
   uint64_t cpiv[64];   // C of the pivot row at its step (0: deterministic)
   uint64_t E[64];      // V_j = product of the original pivot rows of the steps in E_j
   uint64_t lin[64];    // M_r = XOR of lin[t] over the bits t of C_r (rows never replaced)
-  int32_t A[64];       // |x_V & z_V| mod 4 (summed over words)
-  int32_t B0[64];      // |x & z| of the original pivot row
-  int32_t Cp[64];      // parity of (z_V ^ z_orig) . x_orig
+  uint32_t AD[64];     // sums over 4-word chunks of two values mod 4: |x_V & z_V| (low half) and
+                       // |x_o & z_o| - |x_V & z_V| + 2 parity((z_V ^ z_o) . x_o), o = the original pivot row
   int32_t rV[64];      // sign bit of V_j
   uint64_t G[64];      // G[s] bit t = parity(z_{V_s} . x_{V_t})
 };
@@ -79,8 +78,6 @@ struct BlkWindow {
 };
 
 __device__ __forceinline__ int m4(int v) { return ((v % 4) + 4) % 4; }
-
-__device__ __forceinline__ uint64_t shfl64(uint64_t v, int src) { return __shfl_sync(0xffffffffu, v, src); }
 
 // The x bits of one row at a run of measured qubits. Measured qubits are cut
 // into runs of consecutive ones inside a word, so that an ascending list takes
@@ -117,33 +114,57 @@ __device__ __forceinline__ void build_runs(ColRuns &R, const uint32_t *qubits, i
   if (t == 0) R.n = (uint32_t)__popcll(st);
 }
 
-// the runs' bits of row r, four words in flight
-__device__ __forceinline__ uint64_t gather_runs(const ColRuns &R, const uint64_t *row) {
+// part `part` of `parts` of the runs' bits of a row, four words in flight
+__device__ __forceinline__ uint64_t gather_runs(const ColRuns &R, const uint64_t *row, uint32_t part, uint32_t parts) {
   uint64_t c = 0;
-  for (uint32_t i = 0; i < R.n; i += 4) {
+  for (uint32_t i = part; i < R.n; i += 4 * parts) {
     uint64_t w[4];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) w[u] = i + u < R.n ? row[R.word[i + u]] : 0;
+    for (int u = 0; u < 4; ++u) w[u] = i + u * parts < R.n ? row[R.word[i + u * parts]] : 0;
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
-      if (i + u < R.n) c |= ((w[u] >> R.shift[i + u]) & R.mask[i + u]) << R.pos[i + u];
+    for (int u = 0; u < 4; ++u) {
+      const uint32_t x = i + u * parts;
+      if (x < R.n) c |= ((w[u] >> R.shift[x]) & R.mask[x]) << R.pos[x];
+    }
   }
   return c;
 }
 
-// E_j = {j} xor (xor of E_s over the steps s that targeted p_j): thread t of
-// the first 64 keeps column t of E (bit s = whether t is in E_s), so a step is
-// one parity per thread and no exchange; the ballots are the rows.
-__device__ __forceinline__ void build_products(const uint64_t *mpiv, const int64_t *piv, int B, uint64_t *E) {
-  const int t = threadIdx.x;
-  uint64_t col = 0;
-  for (int j = 0; j < 64; ++j) {
-    uint32_t bit = 0;
-    if (j < B && piv[j] != kBlkNone) bit = (uint32_t)(__popcll(col & mpiv[j]) & 1) ^ (t == j ? 1u : 0u);
+// E_j = {j} xor (xor of E_s over the steps s that targeted p_j), for the steps
+// of half h (32 h .. 32 h + 31) among themselves; one warp. Lane t keeps column
+// t (bit s = whether t is in E_s), so a step is one parity per lane and no
+// exchange; the ballots are the rows. prob: bit j set where step j has a pivot.
+__device__ __forceinline__ void half_products(const uint64_t *mpiv, uint64_t prob, int h, uint32_t *E) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t m = (uint32_t)(mpiv[32 * h + lane] >> (32 * h)), pm = (uint32_t)(prob >> (32 * h));
+  uint32_t col = 0, mine = 0;
+#pragma unroll 8
+  for (int j = 0; j < 32; ++j) {
+    const uint32_t mj = __shfl_sync(0xffffffffu, m, j);
+    const uint32_t bit = ((__popc(col & mj) & 1u) ^ (lane == j)) & (pm >> j);
+    col |= bit << j;
     const uint32_t row = __ballot_sync(0xffffffffu, bit);
-    col |= (uint64_t)bit << j;
-    if ((t & 31) == 0) reinterpret_cast<uint32_t *>(&E[j])[t >> 5] = row;
+    if (lane == j) mine = row;
   }
+  E[lane] = mine;
+}
+
+// the two halves joined by one warp: with the steps' targets m split into
+// halves, E_low = E1, E_high = E2 and below the diagonal E2 (m E1); tmp: 32 words
+__device__ __forceinline__ void join_products(const uint64_t *mpiv, const uint32_t *E1, const uint32_t *E2,
+                                              uint32_t *tmp, uint64_t *E) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t m = (uint32_t)mpiv[32 + lane], e2 = E2[lane];
+  uint32_t x = 0;
+#pragma unroll 8
+  for (int s = 0; s < 32; ++s) x ^= E1[s] & (0u - ((m >> s) & 1u));
+  tmp[lane] = x;
+  __syncwarp();
+  uint32_t y = 0;
+#pragma unroll 8
+  for (int s = 0; s < 32; ++s) y ^= tmp[s] & (0u - ((e2 >> s) & 1u));
+  E[lane] = E1[lane];
+  E[32 + lane] = ((uint64_t)e2 << 32) | y;
 }
 
 // ---------------------------------------------------------------------------
@@ -160,10 +181,10 @@ struct FrontArgs {
   uint32_t prev_i0, prev_B;     // previous block (0: none)
   int cur;                      // state of the next block; the previous block's is the other
   int lazy;                     // run the symbolic pass here (else step by step)
-  uint64_t *C, *listC;          // C of every row; nonzero stabilizer rows of each 256-row range: C,
-  uint32_t *listRow;            // their rows,
-  uint32_t *cnt, *done;         // their number, the steps replayed on them
-  uint64_t *orC;                // and the OR of their C
+  uint64_t *C, *listC;          // C of every row; nonzero stabilizer rows of each range (the rows of one
+  uint32_t *listRow;            // block): C, row,
+  uint32_t *cnt, *done;         // number, steps replayed on them
+  uint64_t *orC;                // and OR of their C
   uint64_t *M;
   int32_t *base;
   const int32_t *Tp;
@@ -174,136 +195,184 @@ struct FrontArgs {
   uint32_t *err;
 };
 
-// per row: new sign from the accumulated terms; pivot rows get their coin; record
-__device__ __forceinline__ void sign_rows(const FrontArgs &a, uint64_t r) {
-  __shared__ int sw[64];          // 2 rV_s + A_s of each step
-  __shared__ uint64_t sG[64];     // G rows
-  __shared__ uint32_t s_det[2];
+// Threads per row: 8 where blocks of 256 rows would leave SMs idle (up to 32,768
+// rows), which then share a row's column words, chunk sums and table lookups;
+// else 1. At 4,000 qubits with 64 scattered measured qubits the gather alone
+// took 21,000 cycles with one thread per row.
+constexpr uint64_t kFrontSplitRows = 32768;
+
+template <int P>
+__device__ __forceinline__ uint64_t or_parts(uint64_t v) {
+#pragma unroll
+  for (int d = 1; d < P; d <<= 1) v |= __shfl_xor_sync(0xffffffffu, v, d);
+  return v;
+}
+
+// what signing a row reads of it
+struct SignIn {
+  int32_t b;
+  uint64_t m, word;
+  int e, csum;  // this part's chunk sums
+};
+
+template <int P>
+__device__ __forceinline__ SignIn sign_load(const FrontArgs &a, uint64_t r, int part) {
+  SignIn in;
+  in.b = a.base[r];
+  in.m = a.M[r];
+  in.word = a.S[r >> 6];
+  in.e = in.csum = 0;
+  // with several threads per row the sums are few and are loaded
+  // beside the rest; rows the block left alone have stale ones, which nothing uses
+  if (P == 1 && (in.b >= kBasePivot || (in.b == kBaseOrig && in.m == 0))) return in;
+#pragma unroll 4
+  for (uint32_t ch = part; ch < a.chunks; ch += P) {
+    const int32_t v = a.Tp[(uint64_t)ch * a.nrows + r];
+    in.e += v >> 1;  // arithmetic shift: t
+    in.csum ^= v & 1;
+  }
+  return in;
+}
+
+struct SignShared {
+  uint64_t x[256];
+  int sum[256];
+  int rV[64];
+  uint32_t det[2];
+};
+
+// Over the steps s of M_r: the sum of 2 rV_s + A_s, and the XOR X of G[s]
+// restricted to earlier steps, whose parity with M_r is the sum over s > t in
+// M_r of G[s] bit t. Both come from tables over 4 steps each, 16 lookups a row
+// (a loop over the steps of M_r took most of the 7 us this part needed on its own).
+__device__ __forceinline__ void sign_tables(const FrontArgs &a, SignShared &sh) {
+  const BlkState &st = a.win->st[a.cur ^ 1];
+  const int t = threadIdx.x, g = t >> 4, pat = t & 15;
+  uint64_t x = 0;
+  int sum = 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int s = 4 * g + i;
+    const uint64_t gs = st.G[s] & ((1ull << s) - 1);
+    const int ws = 2 * st.rV[s] + (int)(st.AD[s] & 3u);
+    if ((pat >> i) & 1) { x ^= gs; sum += ws; }
+  }
+  sh.x[t] = x;
+  sh.sum[t] = sum;
+  if (t < 64) sh.rV[t] = st.rV[t];
+}
+
+// the block's record entries; its deterministic outcomes are listed for blk_det
+__device__ __forceinline__ void sign_record(const FrontArgs &a, SignShared &sh) {
   const BlkState &st = a.win->st[a.cur ^ 1];
   const uint64_t m0 = a.m0 + a.prev_i0;  // record index of the block's first measurement
   const int t = threadIdx.x, B = (int)a.prev_B;
-  if (t < 64) {
-    sw[t] = 2 * st.rV[t] + st.A[t];
-    sG[t] = st.G[t];
+  const bool in = t < B, prob = in && st.piv[t] != kBlkNone;
+  if (in) {
+    a.record[m0 + t] = prob ? (uint8_t)(philox4x64_10(m0 + t, a.shot, 0, 0, a.seed, kCoinKey).v[0] & 1u) : 0;
+    a.kinds[m0 + t] = prob;
   }
-  __syncthreads();
-  if (blockIdx.x == 0 && t < 64) {
-    const bool in = t < B, prob = in && st.piv[t] != kBlkNone;
-    if (in) {
-      a.record[m0 + t] = prob ? (uint8_t)(philox4x64_10(m0 + t, a.shot, 0, 0, a.seed, kCoinKey).v[0] & 1u) : 0;
-      a.kinds[m0 + t] = prob;
+  const bool det = in && !prob && a.window[a.prev_i0 + t] < a.n;
+  const uint32_t ball = __ballot_sync(0xffffffffu, det);
+  if ((t & 31) == 0) sh.det[t >> 5] = ball;
+  const uint32_t first = a.win->ndet;
+  asm volatile("bar.sync 1, 64;" ::: "memory");
+  if (det) a.det[first + (t >= 32 ? __popc(sh.det[0]) : 0) + __popc(ball & ((1u << (t & 31)) - 1))] = a.prev_i0 + t;
+  if (t == 0) a.win->ndet = first + __popc(sh.det[0]) + __popc(sh.det[1]);
+}
+
+// new sign of a row from the accumulated terms; pivot rows get their coin
+template <int P>
+__device__ __forceinline__ void sign_row(const FrontArgs &a, const SignShared &sh, const SignIn &in, uint64_t r,
+                                         int part) {
+  const int32_t b = in.b;
+  const uint64_t sr = in.m, old = (in.word >> (r & 63)) & 1u;
+  uint64_t nb = old;
+  const bool product = b < kBasePivot && (b != kBaseOrig || sr != 0);
+  int e = 0;
+  if (product) {
+    uint64_t x = 0;
+#pragma unroll
+    for (int q = 0; q < 16 / P; ++q) {
+      const int g = part + P * q, i = 16 * g + (int)((sr >> (4 * g)) & 15);
+      x ^= sh.x[i];
+      e += sh.sum[i];
     }
-    const bool det = in && !prob && a.window[a.prev_i0 + t] < a.n;
-    const uint32_t ball = __ballot_sync(0xffffffffu, det);
-    if ((t & 31) == 0) s_det[t >> 5] = ball;
-    const uint32_t first = a.win->ndet;
-    asm volatile("bar.sync 1, 64;" ::: "memory");
-    if (det) a.det[first + (t >= 32 ? __popc(s_det[0]) : 0) + __popc(ball & ((1u << (t & 31)) - 1))] = a.prev_i0 + t;
-    if (t == 0) a.win->ndet = first + __popc(s_det[0]) + __popc(s_det[1]);
+    // parities of an XOR: the parts may be counted apart
+    e += in.e + 2 * in.csum + 2 * (__popcll(x & sr) & 1);
   }
-  uint64_t delta = 0;
-  if (r < a.nrows) {
-    const int32_t b = a.base[r];
-    const uint64_t sr = a.M[r];
-    const uint64_t old = (a.S[r >> 6] >> (r & 63)) & 1u;
-    uint64_t nb = old;
-    if (b >= kBasePivot) {
-      nb = philox4x64_10(m0 + (b - kBasePivot), a.shot, 0, 0, a.seed, kCoinKey).v[0] & 1u;
-    } else if (b != kBaseOrig || sr != 0) {
-      const int rb = (b == kBaseOrig) ? (int)old : st.rV[b];
-      int e = 2 * rb, csum = 0;
-#pragma unroll 4
-      for (uint32_t ch = 0; ch < a.chunks; ++ch) {
-        const int32_t v = a.Tp[(uint64_t)ch * a.nrows + r];
-        e += v >> 1;  // arithmetic shift: t
-        csum ^= v & 1;
-      }
-      e += 2 * csum;
-      // + sum over s in M_r of (2 rV_s + A_s) + 2 sum over s > t in M_r of G[s] bit t
-      uint64_t mm = sr;
-      while (mm) {
-        const int s = __ffsll((long long)mm) - 1;
-        mm &= mm - 1;
-        e += sw[s] + 2 * (__popcll(sG[s] & sr & ((1ull << s) - 1)) & 1);
-      }
-      e = m4(e);
-      if (e & 1) atomicOr(a.err, kErrOddPhase);
-      nb = (uint64_t)(e >> 1);
-    }
-    delta = (nb ^ old) << (r & 63);
+#pragma unroll
+  for (int d = 1; d < P; d <<= 1) e += __shfl_xor_sync(0xffffffffu, e, d);
+  if (b >= kBasePivot) {
+    nb = philox4x64_10(a.m0 + a.prev_i0 + (b - kBasePivot), a.shot, 0, 0, a.seed, kCoinKey).v[0] & 1u;
+  } else if (product) {
+    e = m4(e + 2 * ((b == kBaseOrig) ? (int)old : sh.rV[b]));
+    if (e & 1) atomicOr(a.err, kErrOddPhase);
+    nb = (uint64_t)(e >> 1);
   }
-  // fold the sign changes of the 32 rows of this warp into one atomic
-  for (int o = 16; o > 0; o >>= 1) delta |= __shfl_xor_sync(0xffffffffu, delta, o);
-  if ((threadIdx.x & 31) == 0 && r < a.nrows && delta)
-    atomicXor(reinterpret_cast<unsigned long long *>(&a.S[r >> 6]), delta);
+  uint64_t delta = (nb ^ old) << (r & 63);
+  // fold the sign changes of this warp's rows (at most 32, in one word) into one atomic
+  for (int o = 16; o >= P; o >>= 1) delta |= __shfl_xor_sync(0xffffffffu, delta, o);
+  if ((threadIdx.x & 31) == 0 && delta) atomicXor(reinterpret_cast<unsigned long long *>(&a.S[r >> 6]), delta);
 }
 
 // Symbolic pass. Only the pivot sequence (p_j, v_j = C_{p_j} at step j) has to
 // be found in order, and the pivot of step j is the first stabilizer row whose
 // current C has bit j. Rows with C = 0 never take part, and in any state the
-// pivots come from the first nonzero rows, so the first 1,024 of those are held
-// by the block's 8 warps, 128 rows each, transposed: lane t of a warp holds the
-// warp's rows' bits at steps t and t + 32 as four words each. A step is then a
-// broadcast of column j, a search for its first bit and one masked XOR into the
-// columns v_j has; the pivot row clears itself (its C is v_j). Warp 0 runs alone
-// while its rows hold a pivot (no barriers: 64 steps of a dense state take about
-// 5 us); at its first miss the other warps replay the steps so far on their
-// rows and all eight go on in step. Nonzero rows beyond the first 1,024 are only
-// looked at when those have no pivot for a step: range by range of 256 rows,
-// skipping a range when an upper bound on the OR of its C rules the step's bit
-// out (exact when the range was last replayed, then grown by v_s for every step
-// s whose bit the bound has).
-constexpr int kGroup = 1024;
+// pivots come from the first nonzero rows, so the first 768 of those are held in
+// registers by the block's 8 warps, 96 rows each, three a lane (64 steps of a
+// random state miss a pivot among 96 rows once in 2^32). A step is a
+// ballot, a shuffle of the pivot's C and one XOR per row that has the bit. The
+// registers rotate right by one per step, so that step j always looks at bit 0;
+// a row is done with that bit and keeps it as it was, so the bits that went
+// round are the row's M, and the pivot brings the steps that targeted it along.
+// Warp 0 first runs all steps alone, without branches (312 cycles a step with
+// them and four rows a lane); if its rows lack a pivot for a step and there are more rows, all eight
+// warps replay the steps before it and go on in step. Nonzero rows beyond the first 768 are only looked at when those have
+// no pivot for a step: 256 rows at a time, skipping those that an upper bound on
+// the OR of their C rules out (exact when they were last replayed, then grown by
+// v_s for every step s whose bit the bound has).
+constexpr int kLaneRows = 3, kTileRows = 32 * kLaneRows, kGroup = 8 * kTileRows;
 
-struct Tile {  // one warp's 128 rows: columns lane and lane + 32
-  uint32_t lo[4], hi[4];
+// 0 or all ones by bit b
+__device__ __forceinline__ uint64_t spread(uint64_t x, int b) { return 0ull - ((x >> b) & 1ull); }
+
+// one warp's rows, lane l holding rows 3 l .. 3 l + 2, rotated right by the
+// step; above: bits of the rotated word past bit 0 that have not gone round yet
+struct Tile {
+  uint32_t lo[kLaneRows], hi[kLaneRows];
+  uint32_t above_lo, above_hi;
 };
 
-// 32 x 32 bit transpose over the warp: out[lane t] bit r = in[lane r] bit t
-__device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane) {
+// the warp's first row with bit 0: raw_* (without bit 0 if there is none) and
+// its index, without branches, in every lane
+__device__ __forceinline__ void tile_first(const Tile &T, uint32_t &raw_lo, uint32_t &raw_hi, int &index) {
+  const bool p0 = T.lo[0] & 1u, p1 = T.lo[1] & 1u, p2 = T.lo[2] & 1u;
+  const uint32_t b = __ballot_sync(0xffffffffu, p0 | p1 | p2);
+  const uint32_t sl = p0 ? T.lo[0] : p1 ? T.lo[1] : T.lo[2];
+  const uint32_t sh = p0 ? T.hi[0] : p1 ? T.hi[1] : T.hi[2];
+  const int m = p0 ? 0 : p1 ? 1 : 2;
+  const int l = __ffs(b) - 1;  // -1 reads lane 31, whose row 2 has no bit 0 then
+  raw_lo = __shfl_sync(0xffffffffu, sl, l);
+  raw_hi = __shfl_sync(0xffffffffu, sh, l);
+  index = kLaneRows * l + __shfl_sync(0xffffffffu, m, l);
+}
+
+// rows with bit 0 take the pivot's bits above (raw 0: no pivot); on to the next step
+__device__ __forceinline__ void tile_step(Tile &T, uint32_t raw_lo, uint32_t raw_hi) {
+  const uint32_t vl = raw_lo & T.above_lo & ~1u, vh = raw_hi & T.above_hi;
 #pragma unroll
-  for (int j = 16; j > 0; j >>= 1) {
-    const uint32_t low = j == 16 ? 0x0000FFFFu : j == 8 ? 0x00FF00FFu : j == 4 ? 0x0F0F0F0Fu : j == 2 ? 0x33333333u : 0x55555555u;
-    const uint32_t y = __shfl_xor_sync(0xffffffffu, x, j);
-    x = (lane & j) ? ((x & ~low) | ((y & ~low) >> j)) : ((x & low) | ((y & low) << j));
+  for (int m = 0; m < kLaneRows; ++m) {
+    uint32_t l = T.lo[m], h = T.hi[m];
+    if (l & 1u) { l ^= vl; h ^= vh; }
+    T.lo[m] = __funnelshift_r(l, h, 1);
+    T.hi[m] = __funnelshift_r(h, l, 1);
   }
-  return x;
+  T.above_lo = __funnelshift_r(T.above_lo, T.above_hi, 1);
+  T.above_hi >>= 1;
 }
 
-__device__ __forceinline__ void tile_column(const Tile &T, int j, uint32_t (&w)[4]) {
-#pragma unroll
-  for (int m = 0; m < 4; ++m) w[m] = __shfl_sync(0xffffffffu, j < 32 ? T.lo[m] : T.hi[m], j & 31);
-}
-
-// first row with a bit in column w (-1: none)
-__device__ __forceinline__ int tile_first(const uint32_t (&w)[4]) {
-  int p = -1;
-#pragma unroll
-  for (int m = 3; m >= 0; --m)
-    if (w[m]) p = 32 * m + __ffs(w[m]) - 1;
-  return p;
-}
-
-// C of row p of the tile (warp-uniform p)
-__device__ __forceinline__ uint64_t tile_row(const Tile &T, int p) {
-  const int m = p >> 5, b = p & 31;
-  uint32_t l = T.lo[0], h = T.hi[0];
-#pragma unroll
-  for (int i = 1; i < 4; ++i)
-    if (m == i) { l = T.lo[i]; h = T.hi[i]; }
-  const uint32_t vl = __ballot_sync(0xffffffffu, (l >> b) & 1u), vh = __ballot_sync(0xffffffffu, (h >> b) & 1u);
-  return ((uint64_t)vh << 32) | vl;
-}
-
-// rows with bit j (w) take v
-__device__ __forceinline__ void tile_apply(Tile &T, const uint32_t (&w)[4], uint64_t v, int lane) {
-  const uint32_t ml = 0u - (uint32_t)((v >> lane) & 1u), mh = 0u - (uint32_t)((v >> (lane + 32)) & 1u);
-#pragma unroll
-  for (int m = 0; m < 4; ++m) {
-    T.lo[m] ^= w[m] & ml;
-    T.hi[m] ^= w[m] & mh;
-  }
-}
+__device__ __forceinline__ uint64_t rotl64(uint64_t x, int b) { return (x << b) | (x >> ((64 - b) & 63)); }
 
 __device__ __forceinline__ uint64_t lazy_bound(uint64_t u, int a, int j, const uint64_t *v) {
   for (int s = a; s < j; ++s)
@@ -312,33 +381,41 @@ __device__ __forceinline__ uint64_t lazy_bound(uint64_t u, int a, int j, const u
 }
 
 struct SymbolicShared {
-  uint64_t c[kGroup];          // C of the first nonzero rows
-  uint32_t row[kGroup];
-  uint64_t v[64];              // C of each step's pivot (0: none)
-  int64_t piv[64];
-  uint64_t mpiv[64], E[64];
+  uint32_t row[kGroup];        // rows of the group
+  uint64_t raw[64];            // each step's pivot: its bits rotated right by the step (0: none),
+  int index[64];               // index in warp 0's rows (first run),
+  int64_t piv[64];             // row,
+  uint64_t v[64], mpiv[64];    // C, and steps that targeted it
   uint64_t cand_v[2][8], wor[8];
   int cand[2][8];
   uint32_t sum[8], flags[8];
-  int j0;
+  uint32_t E1[32], E2[32], tmp[32];
   int found;
   uint64_t found_v;
   int64_t found_row;
 };
 
 // pivot of step j among the nonzero rows past the first kGroup (all 256
-// threads; off[w] = nonzero rows before range w); leaves found_* in sh
-__device__ void search_rest(const FrontArgs &a, SymbolicShared &sh, const uint32_t *off, uint32_t nwin, int j) {
+// threads; off[w] = nonzero rows before range w, P ranges per 256 rows); leaves
+// found_* in sh
+template <int P>
+__device__ __forceinline__ void search_rest(const FrontArgs &a, SymbolicShared &sh, const uint32_t *off, uint32_t ranges, int j) {
+  constexpr int kRange = 256 / P;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const uint32_t chunks = ranges / P;
   __syncthreads();
   if (t == 0) sh.found = 0;
-  for (uint32_t w0 = 0; w0 < nwin; w0 += 256) {
+  for (uint32_t w0 = 0; w0 < chunks; w0 += 256) {
     const uint32_t w = w0 + t;
     bool may = false;
-    if (w < nwin) {
-      const uint32_t c = __ldcg(a.cnt + w);
-      may = c && off[w] + c > (uint32_t)kGroup &&
-            ((lazy_bound(__ldcg(a.orC + w), (int)__ldcg(a.done + w), j, sh.v) >> j) & 1ull);
+    if (w < chunks) {
+      uint64_t o = 0;
+      uint32_t end = 0;
+      for (int i = 0; i < P; ++i) {
+        const uint32_t c = __ldcg(a.cnt + w * P + i);
+        if (c) { o |= __ldcg(a.orC + w * P + i); end = off[w * P + i] + c; }
+      }
+      may = end > (uint32_t)kGroup && ((lazy_bound(o, (int)__ldcg(a.done + w * P), j, sh.v) >> j) & 1ull);
     }
     const uint32_t ball = __ballot_sync(0xffffffffu, may);
     if (lane == 0) sh.flags[warp] = ball;
@@ -348,21 +425,21 @@ __device__ void search_rest(const FrontArgs &a, SymbolicShared &sh, const uint32
       while (bits) {
         const uint32_t ww = w0 + 32 * f + __ffs(bits) - 1;
         bits &= bits - 1;
-        const uint32_t cnt = __ldcg(a.cnt + ww);
-        const int from = (int)__ldcg(a.done + ww);
-        const bool in = (uint32_t)t < cnt && off[ww] + t >= (uint32_t)kGroup;
+        const uint32_t range = ww * P + t / kRange, e = t % kRange;
+        const int from = (int)__ldcg(a.done + ww * P);
+        const bool in = e < __ldcg(a.cnt + range) && off[range] + e >= (uint32_t)kGroup;
         uint64_t c = 0;
         if (in) {
           c = __ldcg(a.listC + (size_t)ww * 256 + t);
           for (int s = from; s < j; ++s)
-            if ((c >> s) & 1ull) c ^= sh.v[s];
+            if ((c >> s) & 1ull) c ^= sh.v[s] & ~(1ull << s);
           __stcg(a.listC + (size_t)ww * 256 + t, c);
         }
         const uint32_t has = __ballot_sync(0xffffffffu, (c >> j) & 1ull);
         uint64_t o = c;
         for (int d = 16; d > 0; d >>= 1) o |= __shfl_xor_sync(0xffffffffu, o, d);
         const int first = has ? __ffs(has) - 1 : 0;
-        const uint64_t fv = shfl64(c, first);
+        const uint64_t fv = __shfl_sync(0xffffffffu, c, first);
         if (lane == 0) {
           sh.cand[0][warp] = has ? 32 * warp + first : -1;
           sh.cand_v[0][warp] = fv;
@@ -376,9 +453,9 @@ __device__ void search_rest(const FrontArgs &a, SymbolicShared &sh, const uint32
           if (sh.cand[0][i] >= 0) win = i;
           all |= sh.wor[i];
         }
+        if (t < P) __stcg(a.orC + ww * P + t, all);
         if (t == 0) {
-          __stcg(a.orC + ww, all);
-          __stcg(a.done + ww, (uint32_t)j);
+          __stcg(a.done + ww * P, (uint32_t)j);
           if (win >= 0) {
             sh.found = 1;
             sh.found_v = sh.cand_v[0][win];
@@ -393,7 +470,8 @@ __device__ void search_rest(const FrontArgs &a, SymbolicShared &sh, const uint32
   }
 }
 
-__device__ void symbolic_pass(const FrontArgs &a, SymbolicShared &sh, uint32_t *off, uint32_t nwin) {
+template <int P>
+__device__ __forceinline__ void symbolic_pass(const FrontArgs &a, SymbolicShared &sh, uint32_t *off, uint32_t nwin) {
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5, B = (int)a.B;
   BlkState &st = a.win->st[a.cur];
   // off[w] = nonzero rows before range w
@@ -406,7 +484,7 @@ __device__ void symbolic_pass(const FrontArgs &a, SymbolicShared &sh, uint32_t *
     if (lane >= d) inc += y;
   }
   if (lane == 31) sh.sum[warp] = inc;
-  if (t < 64) { sh.v[t] = 0; sh.piv[t] = kBlkNone; }
+  if (t < 64) { sh.raw[t] = 0; sh.v[t] = 0; sh.mpiv[t] = 0; sh.piv[t] = kBlkNone; }
   __syncthreads();
   uint32_t before = inc - sum, total = 0;
   for (int i = 0; i < 8; ++i) {
@@ -419,160 +497,195 @@ __device__ void symbolic_pass(const FrontArgs &a, SymbolicShared &sh, uint32_t *
   }
   __syncthreads();
   const uint32_t group = min(total, (uint32_t)kGroup);
-#pragma unroll
-  for (int i = 0; i < kGroup / 256; ++i) {
-    const uint32_t g = t + 256 * i;
-    uint64_t c = 0;
-    uint32_t row = 0;
-    if (g < group) {
-      uint32_t lo = 0, hi = nwin;  // last range with off <= g
-      while (hi - lo > 1) {
-        const uint32_t mid = (lo + hi) >> 1;
-        if (off[mid] <= g) lo = mid; else hi = mid;
-      }
-      const size_t e = (size_t)lo * 256 + (g - off[lo]);
-      c = __ldcg(a.listC + e);
-      row = __ldcg(a.listRow + e);
-    }
-    sh.c[g] = c;
-    sh.row[g] = row;
-  }
-  __syncthreads();
   Tile T;
+  T.above_lo = T.above_hi = ~0u;
+  uint64_t c0[kLaneRows];
+  {
+    // last range with off <= g, for the lane's rows side by side
+    uint32_t lo[kLaneRows], hi[kLaneRows];
+    const uint32_t g0 = kTileRows * warp + kLaneRows * lane;
 #pragma unroll
-  for (int m = 0; m < 4; ++m) {
-    const uint64_t c = sh.c[128 * warp + 32 * m + lane];
-    T.lo[m] = transpose32((uint32_t)c, lane);
-    T.hi[m] = transpose32((uint32_t)(c >> 32), lane);
-  }
-  uint32_t w[4];
-  if (warp == 0) {
-    int j = 0;
-    for (; j < B; ++j) {
-      tile_column(T, j, w);
-      const int p = tile_first(w);
-      if (p < 0) {
-        if (group > 128) break;  // the other warps' rows may have one
-        continue;
+    for (int m = 0; m < kLaneRows; ++m) { lo[m] = 0; hi[m] = nwin; }
+    for (uint32_t left = nwin; left > 1; left = (left + 1) >> 1)
+#pragma unroll
+      for (int m = 0; m < kLaneRows; ++m) {
+        const uint32_t mid = (lo[m] + hi[m]) >> 1;
+        const bool up = mid > lo[m] && off[mid] <= g0 + m;
+        lo[m] = up ? mid : lo[m];
+        hi[m] = up ? hi[m] : mid;
       }
-      const uint64_t v = tile_row(T, p);
-      tile_apply(T, w, v, lane);
-      if (lane == 0) { sh.v[j] = v; sh.piv[j] = sh.row[p]; }
+    uint32_t row[kLaneRows];
+#pragma unroll
+    for (int m = 0; m < kLaneRows; ++m) {
+      const bool in = g0 + m < group;
+      const size_t e = in ? (size_t)lo[m] * (256 / P) + (g0 + m - off[lo[m]]) : 0;
+      c0[m] = in ? __ldcg(a.listC + e) : 0;
+      row[m] = in ? __ldcg(a.listRow + e) : 0;
     }
-    if (lane == 0) sh.j0 = j;
+#pragma unroll
+    for (int m = 0; m < kLaneRows; ++m) {
+      sh.row[g0 + m] = row[m];
+      T.lo[m] = (uint32_t)c0[m];
+      T.hi[m] = (uint32_t)(c0[m] >> 32);
+    }
   }
   __syncthreads();
-  const int j0 = sh.j0;
+  if (warp == 0) {
+#pragma unroll 8
+    for (int j = 0; j < 64; ++j) {
+      uint32_t rl, rh;
+      int index;
+      tile_first(T, rl, rh, index);
+      tile_step(T, rl, rh);
+      sh.raw[j] = ((uint64_t)rh << 32) | rl;  // every lane, the same value; no bit 0: no pivot
+      sh.index[j] = index;
+    }
+  }
+  __syncthreads();
+  // the first step warp 0 has no pivot for, if other rows may have one
+  int j0 = B;
+  {
+    const uint32_t lo = __ballot_sync(0xffffffffu, !(sh.raw[lane] & 1u)),
+                   hi = __ballot_sync(0xffffffffu, !(sh.raw[lane + 32] & 1u));
+    const uint64_t none = ((uint64_t)hi << 32) | lo;
+    if (group > (uint32_t)kTileRows && none) j0 = min(B, __ffsll((long long)none) - 1);
+  }
+  // from the rotated frame: C and the steps that targeted the pivot
+  auto unrotate = [&](int j) {
+    const uint64_t raw = rotl64(sh.raw[j], j), low = (1ull << j) - 1;
+    sh.v[j] = raw & ~low;
+    sh.mpiv[j] = raw & low;
+  };
+  if (t < j0 && (sh.raw[t] & 1u)) {
+    unrotate(t);
+    sh.piv[t] = sh.row[sh.index[t]];
+  }
   if (j0 < B) {
-    if (warp > 0)
-      for (int s = 0; s < j0; ++s) {
-        const uint64_t v = sh.v[s];
-        if (!v) continue;
-        tile_column(T, s, w);
-        tile_apply(T, w, v, lane);
-      }
+    __syncthreads();
+    if (warp == 0) {
+      T.above_lo = T.above_hi = ~0u;
+#pragma unroll
+      for (int m = 0; m < kLaneRows; ++m) { T.lo[m] = (uint32_t)c0[m]; T.hi[m] = (uint32_t)(c0[m] >> 32); }
+    }
+    for (int s = 0; s < j0; ++s) tile_step(T, (uint32_t)sh.raw[s], (uint32_t)(sh.raw[s] >> 32));
     for (int j = j0, par = 0; j < B; ++j, par ^= 1) {
-      tile_column(T, j, w);
-      const int p = tile_first(w);
-      const uint64_t v = p >= 0 ? tile_row(T, p) : 0;
+      uint32_t rl, rh;
+      int index;
+      tile_first(T, rl, rh, index);
       if (lane == 0) {
-        sh.cand[par][warp] = p >= 0 ? 128 * warp + p : -1;
-        sh.cand_v[par][warp] = v;
+        sh.cand[par][warp] = (rl & 1u) ? kTileRows * warp + index : -1;
+        sh.cand_v[par][warp] = ((uint64_t)rh << 32) | rl;
       }
       __syncthreads();
       int win = -1;
 #pragma unroll
       for (int i = 7; i >= 0; --i)
         if (sh.cand[par][i] >= 0) win = i;
-      uint64_t pv = 0;
+      uint64_t raw = 0;
       int64_t prow = kBlkNone;
       if (win >= 0) {
-        pv = sh.cand_v[par][win];
+        raw = sh.cand_v[par][win];
         prow = sh.row[sh.cand[par][win]];
       } else if (total > (uint32_t)kGroup) {
-        search_rest(a, sh, off, nwin, j);
-        if (sh.found) { pv = sh.found_v; prow = sh.found_row; }
+        search_rest<P>(a, sh, off, nwin, j);
+        if (sh.found) { raw = rotl64(sh.found_v, (64 - j) & 63); prow = sh.found_row; }
         __syncthreads();
       }
-      if (pv) tile_apply(T, w, pv, lane);
-      if (t == 0) { sh.v[j] = pv; sh.piv[j] = prow; }
-    }
-    __syncthreads();
-  }
-  // M is linear in C: lin[t] = the steps that reduce unit vector t; mpiv from it
-  if (t < 64) {
-    uint64_t c = 1ull << t, m = 0;
-    for (int s = t; s < B; ++s) {
-      const uint64_t v = sh.v[s];
-      if (v && ((c >> s) & 1ull)) { c ^= v; m |= 1ull << s; }
-    }
-    st.lin[t] = m;
-  } else if (t < 128) {
-    const int j = t - 64;
-    uint64_t m = 0;
-    if (j < B && sh.v[j]) {
-      uint64_t c = __ldcg(a.C + sh.piv[j]);
-      for (int s = 0; s < j; ++s) {
-        const uint64_t v = sh.v[s];
-        if (v && ((c >> s) & 1ull)) { c ^= v; m |= 1ull << s; }
+      tile_step(T, (uint32_t)raw, (uint32_t)(raw >> 32));
+      if (t == 0) {
+        sh.raw[j] = raw;
+        sh.piv[j] = prow;
+        unrotate(j);
       }
     }
-    sh.mpiv[j] = m;
   }
   __syncthreads();
-  if (t < 64) build_products(sh.mpiv, sh.piv, B, sh.E);
-  __syncthreads();
+  uint64_t prob = 0;  // steps with a pivot
+  {
+    const uint32_t lo = __ballot_sync(0xffffffffu, sh.v[lane] != 0), hi = __ballot_sync(0xffffffffu, sh.v[lane + 32] != 0);
+    prob = ((uint64_t)hi << 32) | lo;
+  }
+  // M is linear in C: lin[t] = the steps that reduce unit vector t (bits stay
+  // behind as above); next to it the products, the two halves of steps apart
   if (t < 64) {
-    st.piv[t] = sh.piv[t];
-    st.cpiv[t] = sh.v[t];
-    st.mpiv[t] = sh.mpiv[t];
-    st.E[t] = sh.E[t];
-    st.A[t] = 0; st.B0[t] = 0; st.Cp[t] = 0; st.rV[t] = 0; st.G[t] = 0;
+    uint32_t lo = t < 32 ? 1u << t : 0, hi = t < 32 ? 0 : 1u << (t - 32);
+#pragma unroll 8
+    for (int s = 0; s < 32; ++s) {
+      const uint64_t v = sh.v[s];
+      const uint32_t on = 0u - ((lo >> s) & 1u);
+      lo ^= (uint32_t)v & ~(1u << s) & on;
+      hi ^= (uint32_t)(v >> 32) & on;
+    }
+#pragma unroll 8
+    for (int s = 0; s < 32; ++s) hi ^= (uint32_t)(sh.v[s + 32] >> 32) & ~(1u << s) & (0u - ((hi >> s) & 1u));
+    st.lin[t] = (((uint64_t)hi << 32) | lo) & prob;
+  } else if (warp == 2) {
+    half_products(sh.mpiv, prob, 0, sh.E1);
+  } else if (warp == 3) {
+    half_products(sh.mpiv, prob, 1, sh.E2);
+  } else if (warp >= 6) {
+    const int i = t - 192;
+    st.piv[i] = sh.piv[i];
+    st.cpiv[i] = sh.v[i];
+    st.mpiv[i] = sh.mpiv[i];
+    st.AD[i] = 0;
+    st.G[i] = 0;
+    if (i == 0) st.ntouched = 0;
   }
-  if (t == 0) st.ntouched = 0;
+  __syncthreads();
+  if (warp == 0) join_products(sh.mpiv, sh.E1, sh.E2, sh.tmp, st.E);
 }
 
-__global__ void __launch_bounds__(256) blk_front_kernel(const FrontArgs a) {
-  extern __shared__ uint32_t s_off[];  // gridDim.x words (lazy symbolic pass)
+template <int P>
+__global__ void __launch_bounds__(256, 4) blk_front_kernel(const FrontArgs a) {
+  extern __shared__ uint32_t s_off[];  // a word per range (lazy symbolic pass)
   __shared__ ColRuns s_runs;
   __shared__ SymbolicShared s_sym;
+  __shared__ SignShared s_sign;
   __shared__ uint32_t s_cnt[8];
   __shared__ uint64_t s_or[8];
   __shared__ bool s_last;
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const uint64_t r = (uint64_t)blockIdx.x * 256 + t;
-  if (a.prev_B) sign_rows(a, r);
-  if (!a.B) return;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5, part = t % P;
+  // the first blocks gather the next block's columns, the others sign the rows
+  // of the previous one (nothing of which the symbolic pass needs)
+  const uint32_t ranges = (uint32_t)(a.nrows / (256 / P));  // nrows is a multiple of 256
+  const bool signs = blockIdx.x >= (a.B ? ranges : 0);
+  const uint32_t range = signs && a.B ? blockIdx.x - ranges : blockIdx.x;
+  const uint64_t r = (uint64_t)range * (256 / P) + t / P;
+  if (signs) {
+    const SignIn in = sign_load<P>(a, r, part);
+    sign_tables(a, s_sign);
+    __syncthreads();
+    if (range == 0 && t < 64) sign_record(a, s_sign);
+    sign_row<P>(a, s_sign, in, r, part);
+    return;
+  }
   if (t < 64) {
     build_runs(s_runs, a.window + a.i0, (int)a.B, a.n);
-    if (blockIdx.x == 0 && t < (int)a.B && a.window[a.i0 + t] >= a.n) atomicOr(a.err, kErrBadQubit);
+    if (range == 0 && t < (int)a.B && a.window[a.i0 + t] >= a.n) atomicOr(a.err, kErrBadQubit);
   }
   __syncthreads();
-  uint64_t c = 0;
-  if (r < a.nrows) {
-    c = gather_runs(s_runs, a.RX + r * a.rs);
-    a.C[r] = c;
-  }
-  const bool stab = r >= 64ull * a.k && r < 64ull * a.k + a.n;
+  const uint64_t c = or_parts<P>(gather_runs(s_runs, a.RX + r * a.rs, part, P));
+  const bool stab = part == 0 && r >= 64ull * a.k && r < 64ull * a.k + a.n;
+  if (part == 0) a.C[r] = c;
   if (!a.lazy) {
-    if (r < a.nrows) { a.M[r] = 0; a.base[r] = kBaseOrig; }
     const uint32_t ball = __ballot_sync(0xffffffffu, stab && (c & 1ull));
     if (lane == 0 && ball)
-      atomicMin(reinterpret_cast<long long *>(&a.win->st[a.cur].slot[0]), (long long)(r + __ffs(ball) - 1));
+      atomicMin(reinterpret_cast<long long *>(&a.win->st[a.cur].slot[0]), (long long)(r + (__ffs(ball) - 1) / P));
     return;
   }
   // nonzero stabilizer rows of this range, in order, and the OR of their C
   const bool keep = stab && c != 0;
   const uint32_t ball = __ballot_sync(0xffffffffu, keep);
   uint64_t o = keep ? c : 0;
-  for (int d = 16; d > 0; d >>= 1) o |= __shfl_xor_sync(0xffffffffu, o, d);
+  for (int d = 16; d >= P; d >>= 1) o |= __shfl_xor_sync(0xffffffffu, o, d);
   if (lane == 0) { s_cnt[warp] = __popc(ball); s_or[warp] = o; }
   __syncthreads();
   uint32_t at = __popc(ball & ((1u << lane) - 1));
   for (int i = 0; i < warp; ++i) at += s_cnt[i];
   if (keep) {
-    a.listC[(size_t)blockIdx.x * 256 + at] = c;
-    a.listRow[(size_t)blockIdx.x * 256 + at] = (uint32_t)r;
+    a.listC[(size_t)blockIdx.x * (256 / P) + at] = c;
+    a.listRow[(size_t)blockIdx.x * (256 / P) + at] = (uint32_t)r;
   }
   if (t == 0) {
     uint32_t cnt = 0;
@@ -582,28 +695,28 @@ __global__ void __launch_bounds__(256) blk_front_kernel(const FrontArgs a) {
     a.orC[blockIdx.x] = all;
     a.done[blockIdx.x] = 0;
   }
-  __threadfence();
   __syncthreads();
   if (t == 0) {
-    s_last = atomicAdd(&a.win->front_arrived, 1u) == gridDim.x - 1;
+    __threadfence();
+    s_last = atomicAdd(&a.win->front_arrived, 1u) == ranges - 1;
     if (s_last) a.win->front_arrived = 0;
   }
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  symbolic_pass(a, s_sym, s_off, gridDim.x);
+  symbolic_pass<P>(a, s_sym, s_off, ranges);
 }
 
 // ---------------------------------------------------------------------------
 // step-by-step symbolic pass (QS_FLAG_STEP_SYMBOLIC): reset, one launch per
 // step over every row, then the products E
 // ---------------------------------------------------------------------------
-__global__ void blk_step_reset_kernel(BlkState *st) {
+__global__ void __launch_bounds__(64) blk_step_reset_kernel(BlkState *st) {
   const int t = threadIdx.x;
   if (t < 3) st->slot[t] = kBlkNone;
   if (t == 0) st->ntouched = 0;
   st->piv[t] = kBlkNone; st->mpiv[t] = 0; st->cpiv[t] = 0;
-  st->A[t] = 0; st->B0[t] = 0; st->Cp[t] = 0; st->rV[t] = 0; st->G[t] = 0;
+  st->AD[t] = 0; st->G[t] = 0;
 }
 
 // symbolic step j: Cin -> Cout
@@ -649,8 +762,17 @@ blk_step_kernel(uint64_t nrows, uint32_t n, uint32_t k, int j, int B, const uint
   }
 }
 
-__global__ void __launch_bounds__(64) blk_step_finish_kernel(BlkState *st, int B) {
-  build_products(st->mpiv, st->piv, B, st->E);
+__global__ void __launch_bounds__(64) blk_step_finish_kernel(BlkState *st) {
+  __shared__ uint64_t s_m[64];
+  __shared__ uint32_t s_prob[2], E1[32], E2[32], tmp[32];
+  const int t = threadIdx.x;
+  s_m[t] = st->mpiv[t];
+  const uint32_t ball = __ballot_sync(0xffffffffu, st->piv[t] != kBlkNone);
+  if ((t & 31) == 0) s_prob[t >> 5] = ball;
+  __syncthreads();
+  half_products(s_m, ((uint64_t)s_prob[1] << 32) | s_prob[0], t >> 5, t < 32 ? E1 : E2);
+  __syncthreads();
+  if (t < 32) join_products(s_m, E1, E2, tmp, st->E);
 }
 
 // ---------------------------------------------------------------------------
@@ -658,9 +780,8 @@ __global__ void __launch_bounds__(64) blk_step_finish_kernel(BlkState *st, int B
 // those blocks their signs), next to the blocks that turn C into M, the bases
 // and the list of rows the block changes
 // ---------------------------------------------------------------------------
-constexpr int kMidThreads = 1024;
-constexpr int kVrowSplit = 4;  // blocks per chunk; block y computes G rows 16 y .. 16 y + 15
-constexpr size_t kVrowSmem = 4ull * 64 * 32 * sizeof(uint64_t);  // original and V rows, x and z
+constexpr int kMidThreads = 256;
+constexpr int kVW = 4;  // column words per chunk of pivot rows: a thread per (step, word)
 
 struct MiddleArgs {
   const uint64_t *RX, *RZ, *S, *C;
@@ -675,122 +796,118 @@ struct MiddleArgs {
   uint32_t *err;
 };
 
-// signs of V_j (first 64 x 16 threads of the block). The phase exponent of step j is
-//   e_j = 2 r(p_j) + B0_j - A_j + 2 Cp_j + sum_{s in m_j} (2 rV_s + A_s) + 2 cross(m_j)
-// (mod 4), cross(m) = sum over s > t in m of G[s] bit t; everything but the
-// 2 rV_s terms is independent of the other steps. With b_j = e'_j / 2 the signs
-// solve rV = b + m rV (m strictly lower triangular), so rV_j = parity(E_j & b).
+// signs of V_j, four threads per step. The phase exponent of step j is
+//   e_j = 2 r(p_j) + D_j + sum_{s in m_j} (2 rV_s + A_s) + 2 cross(m_j)   (mod 4),
+// A and D the halves of AD, cross(m) = sum over s > t in m of G[s] bit t;
+// everything but the 2 rV_s terms is independent of the other steps. With
+// b_j = e'_j / 2 the signs solve rV = b + m rV (m strictly lower triangular), so
+// rV_j = parity(E_j & b).
 __device__ __forceinline__ void pivot_signs(const MiddleArgs &a) {
-  __shared__ int sA[64];
-  __shared__ uint64_t sm[64], sG[64];
-  __shared__ uint32_t s_b[64];
+  __shared__ uint32_t sAD[64];
+  __shared__ uint64_t sG[64];
+  __shared__ uint32_t s_b[8];
   BlkState *st = a.st;
-  const int t = threadIdx.x;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int j = t >> 2, part = t & 3;  // 16 bits of m each
+  const int64_t p = j < (int)a.B ? st->piv[j] : kBlkNone;
+  const uint64_t m = p != kBlkNone ? st->mpiv[j] : 0;
+  const int rp = p != kBlkNone ? (int)((a.S[p >> 6] >> (p & 63)) & 1u) : 0;
   if (t < 64) {
-    sm[t] = t < (int)a.B ? __ldcg(&st->mpiv[t]) : 0;
-    sA[t] = __ldcg(&st->A[t]);
-    sG[t] = __ldcg(&st->G[t]);
+    sAD[t] = __ldcg(&st->AD[t]);
+    sG[t] = __ldcg(&st->G[t]) & ((1ull << t) - 1);
   }
   __syncthreads();
-  const int j = t >> 4, part = t & 15;  // 16 threads per step, 4 bits of m each
-  const uint64_t m = sm[j];
   int e = 0;
+  uint64_t x = 0;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int s = 4 * part + i;
-    if ((m >> s) & 1ull) e += sA[s] + 2 * (__popcll(sG[s] & m & ((1ull << s) - 1)) & 1);
+  for (int i = 0; i < 16; ++i) {
+    const int sidx = 16 * part + i;
+    if ((m >> sidx) & 1ull) { e += (int)(sAD[sidx] & 3u); x ^= sG[sidx]; }
   }
-  for (int o = 8; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
-  if (part == 0) {
+  e += 2 * (__popcll(x & m) & 1);
+  e += __shfl_xor_sync(0xffffffffu, e, 1);
+  e += __shfl_xor_sync(0xffffffffu, e, 2);
+  e = p != kBlkNone ? m4(e + 2 * rp + (int)(sAD[j] >> 16)) : 0;
+  if (e & 1) atomicOr(a.err, kErrOddPhase);
+  const uint32_t ball = __ballot_sync(0xffffffffu, part == 0 && (e >> 1));  // steps 8 warp .. + 7 at lanes 0, 4, ..
+  if (lane == 0) {
     uint32_t b = 0;
-    const int64_t p = j < (int)a.B ? st->piv[j] : kBlkNone;
-    if (p != kBlkNone) {
-      e += 2 * (int)((a.S[p >> 6] >> (p & 63)) & 1u) + __ldcg(&st->B0[j]) - sA[j] + 2 * __ldcg(&st->Cp[j]);
-      e = m4(e);
-      if (e & 1) atomicOr(a.err, kErrOddPhase);
-      b = (uint32_t)(e >> 1);
-    }
-    s_b[j] = b;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) b |= ((ball >> (4 * i)) & 1u) << i;
+    s_b[warp] = b;
   }
   __syncthreads();
   if (t < 64) {
-    const uint64_t E = st->E[t];
-    int rv = 0;
-    for (int s = 0; s < 64; ++s) rv ^= (int)((E >> s) & s_b[s] & 1u);
-    st->rV[t] = rv;
+    uint64_t b = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) b |= (uint64_t)s_b[i] << (8 * i);
+    st->rV[t] = __popcll(st->E[t] & b) & 1;
   }
 }
 
-__device__ __forceinline__ void pivot_rows(const MiddleArgs &a, uint32_t chunk, int y) {
-  extern __shared__ uint64_t vsm[];
-  uint64_t(*ox)[32] = reinterpret_cast<uint64_t(*)[32]>(vsm);
-  uint64_t(*oz)[32] = reinterpret_cast<uint64_t(*)[32]>(vsm + 64 * 32);
-  uint64_t(*vx)[32] = reinterpret_cast<uint64_t(*)[32]>(vsm + 2 * 64 * 32);
-  uint64_t(*vz)[32] = reinterpret_cast<uint64_t(*)[32]>(vsm + 3 * 64 * 32);
-  __shared__ uint64_t sE[64];
+// Pivot rows of one chunk of 4 column words: thread = (step j, word). The V rows
+// are products over E_j of the original rows in shared memory (64 predicated
+// XORs), and G[s][t] = z_{V_s} . x_{V_t} is one bit per word, thread (s, word)
+// walking the 64 steps t; the four words of a step meet by shuffles. With 32-word
+// chunks, lane = word and loops over the bits of E, the kernel took 21 us at 256
+// qubits (4 of 32 lanes busy) and 22 us at 10,000 (5 chunks); now 4-word chunks
+// fill the lanes at any size.
+__device__ __forceinline__ void pivot_rows(const MiddleArgs &a, uint32_t chunk) {
+  __shared__ ulonglong2 so[64][kVW], sv[64][kVW];  // (x, z) of the original and the V rows
   __shared__ bool s_last;
   BlkState *st = a.st;
   const uint32_t rs = a.rs;
-  const int L = (int)a.B;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = kMidThreads >> 5;
-  const bool lead = y == 0;  // writes the V rows and the per-step sums
-  // every word of the padded row (u < rs): padding qubit words are zero in the
-  // tableau and come out zero in the V rows too
-  const uint32_t u = chunk * 32 + lane;
-  const bool in = u < rs;
-  for (int j = w; j < L; j += nw) {
-    const int64_t p = st->piv[j];
-    const bool ld = in && p != kBlkNone;
-    ox[j][lane] = ld ? a.RX[(uint64_t)p * rs + u] : 0;
-    oz[j][lane] = ld ? a.RZ[(uint64_t)p * rs + u] : 0;
-  }
-  if (threadIdx.x < 64) sE[threadIdx.x] = st->E[threadIdx.x];
+  const int t = threadIdx.x, j = t >> 2, w = t & 3;
+  const uint32_t u = chunk * kVW + w;  // rs is a multiple of 4
+  // deterministic steps have no row and an empty E: their V row is zero
+  const int64_t p = j < (int)a.B ? st->piv[j] : kBlkNone;
+  const uint64_t E = st->E[j];
+  ulonglong2 o = make_ulonglong2(0, 0);
+  if (p != kBlkNone) o = make_ulonglong2(a.RX[(uint64_t)p * rs + u], a.RZ[(uint64_t)p * rs + u]);
+  so[j][w] = o;
   __syncthreads();
-  // every block builds all V rows of its chunk (G needs them); the lead block
-  // also stores them and adds the per-step popcount sums. Deterministic steps
-  // have an empty E: their V row is zero.
-  for (int j = w; j < L; j += nw) {
-    const uint64_t x0 = ox[j][lane], z0 = oz[j][lane];
-    uint64_t ax = 0, az = 0, e = sE[j];
-    while (e) {
-      const int s2 = __ffsll((long long)e) - 1;
-      e &= e - 1;
-      ax ^= ox[s2][lane];
-      az ^= oz[s2][lane];
-    }
-    vx[j][lane] = ax;
-    vz[j][lane] = az;
-    if (!lead) continue;
-    if (in) {
-      a.VX[(uint64_t)j * rs + u] = ax;
-      a.VZ[(uint64_t)j * rs + u] = az;
-    }
-    const int av = __reduce_add_sync(0xffffffffu, __popcll(ax & az));
-    const int b = __reduce_add_sync(0xffffffffu, __popcll(x0 & z0));
-    const uint32_t c = __ballot_sync(0xffffffffu, __popcll((az ^ z0) & x0) & 1);
-    if (lane == 0) {
-      if (av) atomicAdd(&st->A[j], av);
-      if (b) atomicAdd(&st->B0[j], b);
-      if (__popc(c) & 1) atomicXor(&st->Cp[j], 1);
-    }
+  uint64_t x = 0, z = 0;
+#pragma unroll 16
+  for (int s = 0; s < 64; ++s) {
+    const ulonglong2 q = so[s][w];
+    const uint64_t on = spread(E, s);
+    x ^= q.x & on;
+    z ^= q.y & on;
   }
-  __syncthreads();
-  // G[s] bit t = parity of z_{V_s} . x_{V_t} over the chunk: block y takes
-  // s = 16 y + w / 2, each warp half of the t range
-  const int sg = 16 * y + (w >> 1), t0 = 32 * (w & 1);
-  if (sg < L) {
-    const uint64_t zs = vz[sg][lane];
-    uint64_t row = 0;
-    for (int t = t0; t < t0 + 32 && t < L; ++t) {
-      const uint32_t bal = __ballot_sync(0xffffffffu, __popcll(zs & vx[t][lane]) & 1);
-      row |= (uint64_t)(__popc(bal) & 1) << t;
-    }
-    if (lane == 0 && row) atomicXor(reinterpret_cast<unsigned long long *>(&st->G[sg]), row);
+  sv[j][w] = make_ulonglong2(x, z);
+  if (j < (int)a.B) {
+    a.VX[(uint64_t)j * rs + u] = x;
+    a.VZ[(uint64_t)j * rs + u] = z;
   }
-  __threadfence();
+  int av = __popcll(x & z), dv = __popcll(o.x & o.y) - av + 2 * (__popcll((z ^ o.y) & o.x) & 1);
+#pragma unroll
+  for (int d = 1; d < 4; d <<= 1) {
+    av += __shfl_xor_sync(0xffffffffu, av, d);
+    dv += __shfl_xor_sync(0xffffffffu, dv, d);
+  }
+  const uint32_t ad = (uint32_t)m4(av) | ((uint32_t)m4(dv) << 16);
+  if (w == 0 && ad) atomicAdd(&st->AD[j], ad);
   __syncthreads();
-  if (threadIdx.x == 0) {
-    s_last = atomicAdd(&a.win->middle_arrived, 1u) == a.chunks * kVrowSplit - 1;
+  // bits t = 0..31 enter glo at the top and move down, then 32..63 ghi
+  const uint32_t zl = (uint32_t)z, zh = (uint32_t)(z >> 32);
+  uint32_t glo = 0, ghi = 0;
+#pragma unroll 16
+  for (int q = 0; q < 32; ++q) {
+    const uint64_t x0 = sv[q][w].x, x1 = sv[q + 32][w].x;
+    glo = __funnelshift_r(glo, __popc((zl & (uint32_t)x0) ^ (zh & (uint32_t)(x0 >> 32))), 1);
+    ghi = __funnelshift_r(ghi, __popc((zl & (uint32_t)x1) ^ (zh & (uint32_t)(x1 >> 32))), 1);
+  }
+#pragma unroll
+  for (int d = 1; d < 4; d <<= 1) {
+    glo ^= __shfl_xor_sync(0xffffffffu, glo, d);
+    ghi ^= __shfl_xor_sync(0xffffffffu, ghi, d);
+  }
+  const uint64_t g = ((uint64_t)ghi << 32) | glo;
+  if (w == 0 && g) atomicXor(reinterpret_cast<unsigned long long *>(&st->G[j]), g);
+  __syncthreads();
+  if (t == 0) {
+    __threadfence();
+    s_last = atomicAdd(&a.win->middle_arrived, 1u) == a.chunks - 1;
     if (s_last) a.win->middle_arrived = 0;
   }
   __syncthreads();
@@ -799,7 +916,7 @@ __device__ __forceinline__ void pivot_rows(const MiddleArgs &a, uint32_t chunk, 
   pivot_signs(a);
 }
 
-// M, base and the row list of 1,024 rows. A row that is neither a pivot nor a
+// M, base and the row list of 256 rows. A row that is neither a pivot nor a
 // replaced destabilizer has M_r = XOR of lin[t] over the bits of C_r: 16
 // lookups in tables of 4 bits each instead of replaying 64 steps. The partner
 // of step j starts from C = v_j with only the later steps left. The list holds
@@ -858,9 +975,8 @@ __device__ __forceinline__ void list_rows(const MiddleArgs &a, uint32_t blk) {
 }
 
 __global__ void __launch_bounds__(kMidThreads) blk_middle_kernel(const MiddleArgs a) {
-  const uint32_t nv = a.chunks * kVrowSplit;
-  if (blockIdx.x < nv) pivot_rows(a, blockIdx.x / kVrowSplit, (int)(blockIdx.x % kVrowSplit));
-  else list_rows(a, blockIdx.x - nv);
+  if (blockIdx.x < a.chunks) pivot_rows(a, blockIdx.x);
+  else list_rows(a, blockIdx.x - a.chunks);
 }
 
 // phase 3: block = one chunk of kCW (32) column words x a range of rows.
@@ -1374,6 +1490,9 @@ struct BlkScratch {
 // measurements per window (the capacity of det and acc)
 static uint32_t blk_window_cap(const Layout &L) { return (uint32_t)L.nrows; }
 
+// rows per block of blk_front
+static uint32_t front_range(const Layout &L) { return L.nrows <= kFrontSplitRows ? 32 : 256; }
+
 static BlkScratch blk_scratch(const Layout &L, void *scratch) {
   BlkScratch b;
   size_t off = 0;
@@ -1383,21 +1502,21 @@ static BlkScratch blk_scratch(const Layout &L, void *scratch) {
     off += (bytes + 255) & ~size_t(255);
     return q;
   };
-  const size_t cap = blk_window_cap(L), ranges = (L.nrows + 255) / 256;
+  const size_t cap = blk_window_cap(L), ranges = L.nrows / front_range(L);
   b.zero = p;
   b.win = reinterpret_cast<BlkWindow *>(take(sizeof(BlkWindow)));
   b.acc = reinterpret_cast<int32_t *>(take(cap * 4));
   b.arrived = reinterpret_cast<uint32_t *>(take((cap / kDetGroup + 1) * 4));
   b.zero_bytes = off;
   b.C0 = reinterpret_cast<uint64_t *>(take(L.nrows * 8));
-  b.C1 = reinterpret_cast<uint64_t *>(take(ranges * 256 * 8));
+  b.C1 = reinterpret_cast<uint64_t *>(take(L.nrows * 8));
   b.M = reinterpret_cast<uint64_t *>(take(L.nrows * 8));
   b.base = reinterpret_cast<int32_t *>(take(L.nrows * 4));
   b.Tp = reinterpret_cast<int32_t *>(take((size_t)blk_chunks(L) * L.nrows * 4));
   b.VX = reinterpret_cast<uint64_t *>(take(64ull * L.rs * 8));
   b.VZ = reinterpret_cast<uint64_t *>(take(64ull * L.rs * 8));
   b.list = reinterpret_cast<uint4 *>(take(L.nrows * 16));
-  b.listRow = reinterpret_cast<uint32_t *>(take(ranges * 256 * 4));
+  b.listRow = reinterpret_cast<uint32_t *>(take(L.nrows * 4));
   b.cnt = reinterpret_cast<uint32_t *>(take(ranges * 4));
   b.done = reinterpret_cast<uint32_t *>(take(ranges * 4));
   b.orC = reinterpret_cast<uint64_t *>(take(ranges * 8));
@@ -1422,17 +1541,16 @@ static cudaError_t measure_window_cap(const Dev &d, void *scratch, const uint32_
                                       uint64_t m0, qs_key key, cudaStream_t s, int *launches) {
   const Layout &L = d.L;
   const BlkScratch b = blk_scratch(L, scratch);
-  const uint32_t chunks = blk_chunks(L), ranges = (uint32_t)((L.nrows + 255) / 256);
+  const uint32_t chunks = blk_chunks(L), ranges = (uint32_t)(L.nrows / front_range(L)),
+                 row_blocks = (uint32_t)(L.nrows / 256);  // nrows is a multiple of 256
   const size_t smem = (size_t)kSmemEntries * kEntryBytes;
   cudaError_t e = once_per_device(g_blk_attr_set, [&]() {
     cudaError_t x = cudaFuncSetAttribute(blk_apply_kernel<uint32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (x == cudaSuccess)
       x = cudaFuncSetAttribute(blk_apply_kernel<uint64_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (x == cudaSuccess)
-      x = cudaFuncSetAttribute(blk_middle_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kVrowSmem);
-    if (x == cudaSuccess)  // 4 bytes per range of 256 rows: 32 KB at n = 2^20, next to 17 KB of static arrays
-      x = cudaFuncSetAttribute(blk_front_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
+    if (x == cudaSuccess)  // 4 bytes per range of 256 rows: 32 KB at n = 2^20, next to the static arrays
+      x = cudaFuncSetAttribute(blk_front_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
     return x;
   });
   if (e == cudaSuccess) e = cudaMemsetAsync(b.zero, 0, b.zero_bytes, s);
@@ -1446,10 +1564,11 @@ static cudaError_t measure_window_cap(const Dev &d, void *scratch, const uint32_
   f.m0 = m0; f.seed = key.seed; f.shot = key.shot;
   f.record = d.record; f.kinds = d.kinds; f.err = d.err;
   MiddleArgs m{};
-  m.RX = d.RX; m.RZ = d.RZ; m.S = d.S; m.C = b.C0; m.nrows = L.nrows; m.rs = L.rs; m.k = L.k; m.chunks = chunks;
+  m.RX = d.RX; m.RZ = d.RZ; m.S = d.S; m.C = b.C0; m.nrows = L.nrows; m.rs = L.rs; m.k = L.k;
+  m.chunks = L.rs / kVW;
   m.lazy = f.lazy;
   m.VX = b.VX; m.VZ = b.VZ; m.M = b.M; m.base = b.base; m.list = b.list; m.win = b.win; m.err = d.err;
-  const uint32_t mid_blocks = chunks * kVrowSplit + (uint32_t)((L.nrows + kMidThreads - 1) / kMidThreads);
+  const uint32_t mid_blocks = m.chunks + row_blocks;  // kMidThreads rows each
   const uint32_t rows_y = apply_rows_y(d, chunks);
   const bool narrow = !d.wide_offsets && (uint64_t)L.nrows * L.rs < (1ull << 32);
   int nl = 0;
@@ -1466,14 +1585,19 @@ static cudaError_t measure_window_cap(const Dev &d, void *scratch, const uint32_
       blk_step_reset_kernel<<<1, 64, 0, s>>>(st);
       ++nl;
     }
-    blk_front_kernel<<<ranges, 256, f.lazy ? ranges * 4 : 0, s>>>(f);
+    const uint32_t blocks = (f.B ? ranges : 0) + (f.prev_B ? ranges : 0);
+    const size_t off_bytes = f.lazy ? ranges * 4 : 0;
+    if (L.nrows <= kFrontSplitRows) blk_front_kernel<8><<<blocks, 256, off_bytes, s>>>(f);
+    else blk_front_kernel<1><<<blocks, 256, off_bytes, s>>>(f);
     ++nl;
     if (!f.lazy && f.B) {
-      // C0 -> C1 -> C0 ...; nothing reads C after the last step
+      // the previous block's M and base are signed; C0 -> C1 -> C0 ...
+      if ((e = cudaMemsetAsync(b.M, 0, L.nrows * 8, s)) != cudaSuccess) return e;
+      if ((e = cudaMemsetAsync(b.base, 0xFF, L.nrows * 4, s)) != cudaSuccess) return e;  // kBaseOrig
       for (int j = 0; j < (int)f.B; ++j)
-        blk_step_kernel<<<ranges, 256, 0, s>>>(L.nrows, L.n, L.k, j, (int)f.B, (j & 1) ? b.C1 : b.C0,
+        blk_step_kernel<<<row_blocks, 256, 0, s>>>(L.nrows, L.n, L.k, j, (int)f.B, (j & 1) ? b.C1 : b.C0,
                                                (j & 1) ? b.C0 : b.C1, b.M, b.base, st);
-      blk_step_finish_kernel<<<1, 64, 0, s>>>(st, (int)f.B);
+      blk_step_finish_kernel<<<1, 64, 0, s>>>(st);
       nl += (int)f.B + 1;
     }
     tend(d.timer, kind, s);
@@ -1481,7 +1605,7 @@ static cudaError_t measure_window_cap(const Dev &d, void *scratch, const uint32_
     m.B = f.B;
     m.st = st;
     tbegin(d.timer, QS_TIME_BLK_PIVOT_ROWS, s);
-    blk_middle_kernel<<<mid_blocks, kMidThreads, kVrowSmem, s>>>(m);
+    blk_middle_kernel<<<mid_blocks, kMidThreads, 0, s>>>(m);
     tend(d.timer, QS_TIME_BLK_PIVOT_ROWS, s);
     tbegin(d.timer, QS_TIME_BLK_APPLY, s);
     if (narrow)
