@@ -187,7 +187,7 @@ struct FrontArgs {
   uint64_t *orC;                // and OR of their C
   uint64_t *M;
   int32_t *base;
-  const int32_t *Tp;
+  const uint8_t *Tp;            // phase sums mod 4 of the apply pass, per column chunk and row
   BlkWindow *win;
   uint32_t *det;                // window positions of deterministic outcomes
   uint64_t m0, seed, shot;
@@ -212,7 +212,7 @@ __device__ __forceinline__ uint64_t or_parts(uint64_t v) {
 struct SignIn {
   int32_t b;
   uint64_t m, word;
-  int e, csum;  // this part's chunk sums
+  int e;  // this part's chunk sums
 };
 
 template <int P>
@@ -221,16 +221,12 @@ __device__ __forceinline__ SignIn sign_load(const FrontArgs &a, uint64_t r, int 
   in.b = a.base[r];
   in.m = a.M[r];
   in.word = a.S[r >> 6];
-  in.e = in.csum = 0;
+  in.e = 0;
   // with several threads per row the sums are few and are loaded
   // beside the rest; rows the block left alone have stale ones, which nothing uses
   if (P == 1 && (in.b >= kBasePivot || (in.b == kBaseOrig && in.m == 0))) return in;
 #pragma unroll 4
-  for (uint32_t ch = part; ch < a.chunks; ch += P) {
-    const int32_t v = a.Tp[(uint64_t)ch * a.nrows + r];
-    in.e += v >> 1;  // arithmetic shift: t
-    in.csum ^= v & 1;
-  }
+  for (uint32_t ch = part; ch < a.chunks; ch += P) in.e += a.Tp[(uint64_t)ch * a.nrows + r];
   return in;
 }
 
@@ -298,8 +294,8 @@ __device__ __forceinline__ void sign_row(const FrontArgs &a, const SignShared &s
       x ^= sh.x[i];
       e += sh.sum[i];
     }
-    // parities of an XOR: the parts may be counted apart
-    e += in.e + 2 * in.csum + 2 * (__popcll(x & sr) & 1);
+    // the parity of an XOR: the parts may be counted apart
+    e += in.e + 2 * (__popcll(x & sr) & 1);
   }
 #pragma unroll
   for (int d = 1; d < P; d <<= 1) e += __shfl_xor_sync(0xffffffffu, e, d);
@@ -1050,6 +1046,20 @@ __device__ __forceinline__ void apply_fetch(ApplyRow &a, const ApplyMeta &m, con
   }
 }
 
+// Phase terms of one word (mod 4, summed over the row's words): with base row
+// (xb, zb) and result (xf, zf) = V product * base,
+//   |xb & zb| - |xf & zf| + 2 parity((zf ^ zb) & xb).
+// -|b| = |~b| - 32 makes it a sum of four popcounts, which a full adder and a
+// half adder fold into a ones and a twos word: two popcounts instead of five
+// (a quarter-rate instruction).
+__device__ __forceinline__ int phase_word(uint2 xb, uint2 zb, uint2 xf, uint2 zf) {
+  const uint32_t a0 = xb.x & zb.x, a1 = xb.y & zb.y, n0 = ~(xf.x & zf.x), n1 = ~(xf.y & zf.y);
+  const uint32_t d0 = xb.x & (zf.x ^ zb.x), d1 = xb.y & (zf.y ^ zb.y);
+  const uint32_t s = a0 ^ a1 ^ n0, cy = (a0 & a1) | (a0 & n0) | (a1 & n0);
+  const uint32_t t = ((s & n1) ^ cy) ^ d0 ^ d1;
+  return __popc(s ^ n1) + 2 * __popc(t);
+}
+
 // a ^ b ^ c in one three-input logic operation
 __device__ __forceinline__ uint32_t xor3(uint32_t a, uint32_t b, uint32_t c) {
   uint32_t d;
@@ -1127,7 +1137,7 @@ template <typename Idx>
 __device__ __forceinline__ void apply_row(const ApplyRow &a, uint32_t nrows, uint64_t *RX, uint64_t *RZ,
                                           bool ok, uint32_t word, const uint32_t *qubits,
                                           const uint64_t *VX, const uint64_t *VZ, uint32_t rs,
-                                          uint32_t lane, const char *tb, uint32_t tq, int32_t *Tp,
+                                          uint32_t lane, const char *tb, uint32_t tq, uint8_t *Tp,
                                           uint64_t tp0) {
   const uint32_t r = a.r;
   if (r >= nrows) return;  // uniform over the warp
@@ -1176,23 +1186,21 @@ __device__ __forceinline__ void apply_row(const ApplyRow &a, uint32_t nrows, uin
   const int t = __popc(xb.x & zb.x) + __popc(xb.y & zb.y) - __popc(xf.x & zf.x) - __popc(xf.y & zf.y);
   const int c = __popc((acc.z & xb.x) ^ (acc.w & xb.y)) & 1;  // parity of z_acc . x_b
   const int v = __reduce_add_sync(0xffffffffu, 64 * t + c);
-  if (lane == 0) Tp[tp0 + r] = (v >> 6) * 2 + (v & 1);
+  if (lane == 0) Tp[tp0 + r] = (uint8_t)(((v >> 6) + 2 * (v & 1)) & 3);
 }
 
 // 1,024 threads at 64 registers: 6.80 ms per dense block at 180k, against
-// 7.46 ms with 768 threads (80 registers) and 9.55 ms with 512 (100)
+// 7.46 ms with 768 threads (80 registers) and 9.55 ms with 512 (100). Fewer
+// instructions per row do not help (measured: 64-bit multiply-adds for the row
+// addresses, two popcounts instead of five): the pass waits on memory.
 constexpr int kApplyThreads = 1024;
-// blocks per SM over the grid: 6.41 ms per dense 180k block with 32 waves of
-// one block per SM, 6.43 with 24, 6.49 with 16, 6.79 with 8, 7.46 with 4 (the
-// tails of the last wave shrink; a block's table build stays small)
-constexpr int kApplyWaves = 32;
 
 template <typename Idx>
 __global__ void __launch_bounds__(kApplyThreads, 1)
 blk_apply_kernel(uint64_t *__restrict__ RX, uint64_t *__restrict__ RZ, uint32_t rs, uint32_t nrows,
                  const uint32_t *__restrict__ qubits, int L, const uint64_t *__restrict__ VX,
                  const uint64_t *__restrict__ VZ, const uint4 *__restrict__ list,
-                 int32_t *__restrict__ Tp, const BlkState *st) {
+                 uint8_t *__restrict__ Tp, const BlkState *st) {
   extern __shared__ ulonglong2 T[];  // [kSmemEntries][kCW] of (x word, z word)
   __shared__ uint32_t s_tmem;
   const uint32_t cnt = st->ntouched;
@@ -1302,6 +1310,114 @@ blk_apply_kernel(uint64_t *__restrict__ RX, uint64_t *__restrict__ RZ, uint32_t 
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_tmem), "r"(kTmemCols)
                  : "memory");
+  }
+}
+
+// The same pass for small tableaus, where building 226 KB of tables for a few
+// hundred rows a block is most of the work and few blocks would run: 16 groups
+// of 4 steps (256 entries) over chunks of CW = 4 or 8 column words, 16 or 32 KB
+// of shared memory, 256 threads. CW lanes share a row, a warp has 32 / CW rows.
+// Twice the lookups per word of the large variant, an eighth of its table build.
+// Up to 6,144 qubits: 5,000 qubits take 14.7 us (large variant 16.2), 10,000 take
+// 38.7 (28.5); 256 qubits 19 -> 6.1 us, 1,500 qubits 22.7 -> 7.2 us.
+constexpr uint32_t kSmallApplyQubits = 6144;
+constexpr int kSmallThreads = 256;
+
+// the words of a listed row. bx, bz: this lane's word of row 0; a row is one
+// 32 x 32 -> 64-bit multiply-add away from it
+__device__ __forceinline__ void apply_fetch_small(ApplyRow &a, const ApplyMeta &m, const uint64_t *bx, const uint64_t *bz,
+                                            uint32_t row_bytes, uint32_t nrows, bool ok) {
+  a.r = m.r;
+  a.b = m.b;
+  a.lo = m.lo;
+  a.hi = m.hi;
+  a.x = a.z = make_uint2(0, 0);
+  if (ok && m.r < nrows) {
+    const uint64_t off = (uint64_t)m.r * row_bytes;
+    a.x = *reinterpret_cast<const uint2 *>(reinterpret_cast<const char *>(bx) + off);
+    a.z = *reinterpret_cast<const uint2 *>(reinterpret_cast<const char *>(bz) + off);
+  }
+}
+
+template <int CW>
+__global__ void __launch_bounds__(kSmallThreads)
+blk_apply_small_kernel(uint64_t *__restrict__ RX, uint64_t *__restrict__ RZ, uint32_t rs, uint32_t nrows,
+                       const uint32_t *__restrict__ qubits, int L, const uint64_t *__restrict__ VX,
+                       const uint64_t *__restrict__ VZ, const uint4 *__restrict__ list, uint8_t *__restrict__ Tp,
+                       const BlkState *st) {
+  __shared__ ulonglong2 T[16 * 16][CW];
+  const uint32_t cnt = st->ntouched;
+  const uint32_t t = threadIdx.x, w = t % CW, word = blockIdx.x * CW + w;
+  const uint32_t group = t / CW, units = gridDim.y * (kSmallThreads / CW);
+  if (cnt == 0) return;  // every outcome of the block is deterministic
+  const bool ok = word < rs;
+  // entry p of step group g = XOR of the V rows of p's bits; a thread builds its
+  // word's entries of one group, each one row away from an earlier one
+  for (uint32_t g = group; g < 16; g += kSmallThreads / CW) {
+    ulonglong2 v[4];
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      const int s = 4 * (int)g + b;
+      v[b] = make_ulonglong2(0, 0);
+      if (ok && s < L) v[b] = make_ulonglong2(VX[(uint64_t)s * rs + word], VZ[(uint64_t)s * rs + word]);
+    }
+    ulonglong2 e[16];
+    e[0] = make_ulonglong2(0, 0);
+#pragma unroll
+    for (int p = 1; p < 16; ++p) {
+      const int b = p & 8 ? 3 : p & 4 ? 2 : p & 2 ? 1 : 0;
+      e[p] = make_ulonglong2(e[p ^ (1 << b)].x ^ v[b].x, e[p ^ (1 << b)].y ^ v[b].y);
+    }
+#pragma unroll
+    for (int p = 0; p < 16; ++p) T[16 * g + p][w] = e[p];
+  }
+  __syncthreads();
+  const uint32_t row_bytes = rs * 8;
+  uint64_t *bx = RX + word, *bz = RZ + word;
+  uint8_t *tp = Tp + (uint64_t)blockIdx.x * nrows;
+  const char *tw = reinterpret_cast<const char *>(&T[0][w]);
+  ApplyRow a, nx;
+  ApplyMeta m;
+  // rows of a warp in step (the shuffles below), so the loop runs to the warp's last
+  const uint32_t first = blockIdx.y * (kSmallThreads / CW), lane0 = first + (t & ~31u) / CW;
+  uint32_t j = first + group;
+  apply_meta(m, j, cnt, nrows, list);
+  apply_fetch_small(a, m, bx, bz, row_bytes, nrows, ok);
+  for (uint32_t j0 = lane0; j0 < cnt; j0 += units, j += units) {
+    apply_meta(m, j + units, cnt, nrows, list);
+    apply_fetch_small(nx, m, bx, bz, row_bytes, nrows, ok);
+    uint2 xb = a.x, zb = a.z;
+    if (a.b != kBaseOrig && a.b < kBasePivot && ok) {  // destabilizer replaced by V_b at step b
+      xb = reinterpret_cast<const uint2 *>(VX)[(uint64_t)a.b * rs + word];
+      zb = reinterpret_cast<const uint2 *>(VZ)[(uint64_t)a.b * rs + word];
+    }
+    uint4 f = make_uint4(xb.x, xb.y, zb.x, zb.y);
+#pragma unroll
+    for (int g = 0; g < 16; g += 2) {
+      const uint32_t mw = g < 8 ? a.lo : a.hi;
+      const int sh = 4 * (g & 7);
+      const uint4 e0 = *reinterpret_cast<const uint4 *>(tw + (16 * g + ((mw >> sh) & 15)) * (16 * CW));
+      const uint4 e1 = *reinterpret_cast<const uint4 *>(tw + (16 * (g + 1) + ((mw >> (sh + 4)) & 15)) * (16 * CW));
+      acc3(f, e0, e1);
+    }
+    uint2 xf = make_uint2(f.x, f.y), zf = make_uint2(f.z, f.w);
+    int v = phase_word(xb, zb, xf, zf);
+    if (!ok) v = 0;
+    if (a.b >= kBasePivot) {  // pivot row of step b: +-Z_q (sign set by blk_front_kernel)
+      const uint32_t q = qubits[a.b - kBasePivot];
+      const uint32_t bit = ((q >> 6) == word) ? 1u << (q & 31) : 0u;
+      xf = make_uint2(0, 0);
+      zf = (q & 32) ? make_uint2(0, bit) : make_uint2(bit, 0);
+    }
+    if (ok && a.r < nrows) {
+      const uint64_t off = (uint64_t)a.r * row_bytes;
+      *reinterpret_cast<uint2 *>(reinterpret_cast<char *>(bx) + off) = xf;
+      *reinterpret_cast<uint2 *>(reinterpret_cast<char *>(bz) + off) = zf;
+    }
+#pragma unroll
+    for (int d = 1; d < CW; d <<= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+    if (w == 0 && a.r < nrows) tp[a.r] = (uint8_t)(v & 3);
+    a = nx;
   }
 }
 
@@ -1471,7 +1587,12 @@ __global__ void __launch_bounds__(kDetThreads) blk_det_kernel(const DetArgs a) {
 // ---------------------------------------------------------------------------
 // launches
 // ---------------------------------------------------------------------------
-static uint32_t blk_chunks(const Layout &L) { return (L.rs + kCW - 1) / kCW; }
+// column words per chunk of the apply pass: 4 or 8 (small variant) or 32
+static uint32_t apply_words(const Layout &L) {
+  if (L.n > kSmallApplyQubits) return kCW;
+  return L.rs <= 4 ? 4 : 8;
+}
+static uint32_t apply_chunks(const Layout &L) { return (L.rs + apply_words(L) - 1) / apply_words(L); }
 
 // device scratch of the blocked measurement
 struct BlkScratch {
@@ -1482,7 +1603,8 @@ struct BlkScratch {
   uint32_t *arrived;
   uint64_t *C0, *C1, *M, *orC, *VX, *VZ;
   uint32_t *listRow, *cnt, *done, *det;
-  int32_t *base, *Tp;
+  int32_t *base;
+  uint8_t *Tp;
   uint4 *list;
   size_t total;
 };
@@ -1512,7 +1634,7 @@ static BlkScratch blk_scratch(const Layout &L, void *scratch) {
   b.C1 = reinterpret_cast<uint64_t *>(take(L.nrows * 8));
   b.M = reinterpret_cast<uint64_t *>(take(L.nrows * 8));
   b.base = reinterpret_cast<int32_t *>(take(L.nrows * 4));
-  b.Tp = reinterpret_cast<int32_t *>(take((size_t)blk_chunks(L) * L.nrows * 4));
+  b.Tp = take((size_t)apply_chunks(L) * L.nrows);
   b.VX = reinterpret_cast<uint64_t *>(take(64ull * L.rs * 8));
   b.VZ = reinterpret_cast<uint64_t *>(take(64ull * L.rs * 8));
   b.list = reinterpret_cast<uint4 *>(take(L.nrows * 16));
@@ -1529,19 +1651,38 @@ size_t blocked_scratch_bytes(const Layout &L) { return blk_scratch(L, nullptr).t
 
 static std::atomic<uint64_t> g_blk_attr_set{0};
 
-// about kApplyWaves waves of one block per SM (the tables take 226 KB of
-// shared memory and all of TMEM), but at least 512 rows per block so that
-// building the tables stays small next to the rows they serve
-static uint32_t apply_rows_y(const Dev &d, uint32_t chunks) {
-  return std::max<uint32_t>(1, (uint32_t)std::min<uint64_t>(((uint64_t)d.sms * kApplyWaves + chunks - 1) / chunks,
-                                                            d.L.nrows / 512));
+// Row ranges of the apply pass's grid. The large variant runs one block per SM
+// (its tables fill shared memory and TMEM), so a grid just past a whole number
+// of waves leaves SMs idle for one: at 10,000 qubits 195 blocks of 518 rows took
+// 42 us and one wave of 150 takes 28.5. A wave costs a table build (about 4 us)
+// and more waves even out the SMs (about 1.3 % at one, 0.4 % at three): with
+// u_k the filled share of k waves, k minimises (1 + 0.013 / k) / u_k + 4 us k / T,
+// T = 31 ns per row and chunk over the SMs. Dense blocks of 64, before (at least
+// 512 rows per block, at most 32 waves) and after: 20,000 qubits 127 -> 97 us,
+// 60,000 918 -> 845, 90,000 1,729 -> 1,570, 180,000 6,310 -> 6,180.
+// The small variant holds several blocks per SM: three measured best at 3,000
+// and 5,000 qubits (10.0 and 14.7 us; 24 us with the large variant's old grid).
+static uint32_t apply_rows_y(const Dev &d, uint32_t chunks, uint32_t words) {
+  const uint64_t nrows = d.L.nrows, sms = d.sms;
+  if (words < kCW)
+    return (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(3 * sms / chunks, nrows / (kSmallThreads / words)));
+  const double total_us = 0.031 * (double)nrows * chunks / (double)sms;
+  uint32_t best = 1;
+  double least = 1e30;
+  for (uint32_t k = 1; k <= 12; ++k) {
+    const uint64_t ry = k * sms / chunks;
+    if (ry == 0) continue;
+    const double cost = (1 + 0.013 / k) * (double)(k * sms) / (double)(ry * chunks) + 4.0 * k / total_us;
+    if (cost < least) { least = cost; best = (uint32_t)ry; }
+  }
+  return best;
 }
 
 static cudaError_t measure_window_cap(const Dev &d, void *scratch, const uint32_t *window, uint32_t count,
                                       uint64_t m0, qs_key key, cudaStream_t s, int *launches) {
   const Layout &L = d.L;
   const BlkScratch b = blk_scratch(L, scratch);
-  const uint32_t chunks = blk_chunks(L), ranges = (uint32_t)(L.nrows / front_range(L)),
+  const uint32_t words = apply_words(L), chunks = apply_chunks(L), ranges = (uint32_t)(L.nrows / front_range(L)),
                  row_blocks = (uint32_t)(L.nrows / 256);  // nrows is a multiple of 256
   const size_t smem = (size_t)kSmemEntries * kEntryBytes;
   cudaError_t e = once_per_device(g_blk_attr_set, [&]() {
@@ -1569,8 +1710,7 @@ static cudaError_t measure_window_cap(const Dev &d, void *scratch, const uint32_
   m.lazy = f.lazy;
   m.VX = b.VX; m.VZ = b.VZ; m.M = b.M; m.base = b.base; m.list = b.list; m.win = b.win; m.err = d.err;
   const uint32_t mid_blocks = m.chunks + row_blocks;  // kMidThreads rows each
-  const uint32_t rows_y = apply_rows_y(d, chunks);
-  const bool narrow = !d.wide_offsets && (uint64_t)L.nrows * L.rs < (1ull << 32);
+  const uint32_t rows_y = apply_rows_y(d, chunks, words);
   int nl = 0;
   for (uint32_t i0 = 0, cur = 0;; i0 += 64, cur ^= 1) {
     // signs of the block before i0, symbolic pass of the block at i0
@@ -1608,7 +1748,13 @@ static cudaError_t measure_window_cap(const Dev &d, void *scratch, const uint32_
     blk_middle_kernel<<<mid_blocks, kMidThreads, 0, s>>>(m);
     tend(d.timer, QS_TIME_BLK_PIVOT_ROWS, s);
     tbegin(d.timer, QS_TIME_BLK_APPLY, s);
-    if (narrow)
+    if (words == 4)
+      blk_apply_small_kernel<4><<<dim3(chunks, rows_y), kSmallThreads, 0, s>>>(
+          d.RX, d.RZ, L.rs, (uint32_t)L.nrows, window + i0, (int)f.B, b.VX, b.VZ, b.list, b.Tp, st);
+    else if (words == 8)
+      blk_apply_small_kernel<8><<<dim3(chunks, rows_y), kSmallThreads, 0, s>>>(
+          d.RX, d.RZ, L.rs, (uint32_t)L.nrows, window + i0, (int)f.B, b.VX, b.VZ, b.list, b.Tp, st);
+    else if (!d.wide_offsets && (uint64_t)L.nrows * L.rs < (1ull << 32))
       blk_apply_kernel<uint32_t><<<dim3(chunks, rows_y), kApplyThreads, smem, s>>>(
           d.RX, d.RZ, L.rs, (uint32_t)L.nrows, window + i0, (int)f.B, b.VX, b.VZ, b.list, b.Tp, st);
     else

@@ -53,3 +53,23 @@ def test_out_of_range_device_qubit_in_a_window():
     with pytest.raises(qs.QsError) as e:
         sim.sync()
     assert e.value.code == -7
+
+
+# 255..257 and 511..513: 4- and 8-word chunks of the small apply pass (row strides 4, 8 and 12 words,
+# the last with a half-empty chunk); 6,144 / 6,145: the last small and the first large size
+@pytest.mark.parametrize("n,flags", [(255, 0), (257, 0), (512, 0), (513, 0), (6144, 0), (6145, 0),
+                                     (6145, qs.QS_FLAG_WIDE_OFFSETS)])
+def test_apply_variants_match_single_measurements(n, flags):
+    """Blocks of 64 (the second one short) against measurements one by one, on a dense state."""
+    circ = C.random_circuit(n, 30, 0.5, seed=n, final_measure_all=False)
+    q = np.random.default_rng(n).permutation(n)[:100].astype(np.uint32)
+    out = []
+    for f in (flags, qs.QS_FLAG_NO_BLOCKED_MEASURE):
+        sim = qs.Simulator(n, flags=f)
+        dc = sim.upload(circ)
+        sim.apply_layers_dev(dc, 0, 30)
+        rec = sim.measure(q, seed=2)
+        out.append((rec, sim.record_kinds(), qs.qs_sim_tableau_export(sim.sim)))
+        sim.sync()
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
