@@ -389,12 +389,14 @@ int qs_sim_sample_noalloc(qs_sim *sim, uint64_t shots, uint64_t seed, uint64_t *
  * tableau are the same alone (qs_sim_*) and in a batch. All arrays are host
  * memory and are copied at qs_batch_create. 1 <= n <= 2^20.
  *
- * Circuits of n < 1024 qubits run in one cooperative persistent kernel on the
- * batch's stream (their cost is per-launch overhead when they run alone);
- * circuits of n >= 1024 run through one qs_sim each (blocked measurement),
- * spread over up to 16 worker streams that host threads drive during
- * qs_batch_run. The paper has no batch mode; this follows the batched
- * workload's shape (many small and some large circuits).
+ * Circuits of up to 640 qubits run with one thread block each, their tableau
+ * in shared memory for the whole program (their cost is per-launch overhead
+ * when they run alone); larger ones run through one qs_sim each (blocked
+ * measurement), spread over up to 16 worker streams that host threads drive
+ * during qs_batch_run. With a launch shape (qs_batch_tuning) the circuits of
+ * n < 1024 run in one cooperative persistent kernel instead. The paper has no
+ * batch mode; this follows the batched workload's shape (many small and some
+ * large circuits).
  */
 typedef struct qs_batch_circuit {
   uint32_t n;
@@ -410,7 +412,8 @@ typedef struct qs_batch_circuit {
 } qs_batch_circuit;
 
 /* Launch shape of the persistent kernel (qs_batch_autotune picks one).
- *   threads:         256, 512 or 1024 per CTA
+ *   threads:         256, 512 or 1024 per CTA; 0 = the default path, without
+ *                    the persistent kernel (the other members are not read)
  *   blocks_per_sm:   CTAs per SM (0 = as many as fit)
  *   words_per_block: 64-row column words per shared-memory slice in the gate phase (1 or 2)
  *   fuse_depth:      layers per shared-memory pass in the gate phase (0 = whole round)
@@ -426,25 +429,28 @@ typedef struct qs_batch_tuning {
 
 typedef struct qs_batch qs_batch;
 
-/* Device bytes of a batch's persistent-kernel part (0 if the description is
- * invalid); the simulators of the n >= 1024 circuits allocate their own. */
+/* Device bytes of the batch's own part: every circuit of n < 1024 (0 if the
+ * description is invalid); the simulators of the circuits above 640 qubits
+ * allocate their own. */
 size_t qs_batch_required_bytes(uint32_t count, const qs_batch_circuit *circuits);
 
 /* Validates (as qs_pack_layers; measured qubits < n; offsets in range) and
  * uploads the batch. workspace: caller device memory of >= required bytes,
  * 256-byte aligned, or NULL to let the library cudaMalloc it. Creates the
- * worker streams and the simulators of the n >= 1024 circuits. */
+ * worker streams and the simulators of the circuits above 640 qubits. */
 int qs_batch_create(uint32_t count, const qs_batch_circuit *circuits, void *cuda_stream,
                     void *workspace, size_t workspace_bytes, qs_batch **out);
 
 int qs_batch_destroy(qs_batch *batch);
 
 /* Runs every circuit from |0...0> through its rounds (the first round_limit
- * rounds, 0 = all): the n < 1024 circuits in one cooperative persistent
- * kernel launch on the batch's stream, the others on the worker streams.
+ * rounds, 0 = all): a block per circuit of up to 640 qubits, in up to three
+ * launches by size, the others on the worker streams; with a launch shape the
+ * n < 1024 circuits in one cooperative persistent kernel launch on the batch's
+ * stream.
  * Returns when all work is enqueued; the batch's stream then waits for the
  * worker streams, so work enqueued on it afterwards follows the whole batch.
- * tuning: NULL for the default shape of the persistent kernel. */
+ * tuning: NULL for the default path. */
 int qs_batch_run(qs_batch *batch, const qs_batch_tuning *tuning, uint32_t round_limit);
 
 /* Waits for the batch's stream; QS_ERR_TIMEOUT if a grid barrier ran out,
@@ -458,8 +464,9 @@ int qs_batch_record(qs_batch *batch, uint32_t circuit, uint8_t *dst, size_t coun
 int qs_batch_export_rows(qs_batch *batch, uint32_t circuit, const uint32_t *rows, uint32_t count,
                          uint64_t *dst);
 
-/* Times the candidate launch shapes of the persistent kernel on this batch
- * (the first round_limit rounds; 0 = all; the worker streams are idle
+/* Times the default path and the candidate launch shapes of the persistent
+ * kernel on this batch's circuits of n < 1024 (the first round_limit rounds;
+ * 0 = all; the simulators of the larger ones are idle
  * meanwhile) and returns the fastest. cache_path: NULL, or a text file
  * of "device|batch-signature|rounds threads blocks_per_sm words_per_block
  * fuse_depth" lines that is read first and appended to. Results do not depend

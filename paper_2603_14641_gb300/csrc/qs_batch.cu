@@ -1,9 +1,12 @@
-// Batched persistent launch: many independent circuits of uneven size in ONE
-// kernel launch.
+// Batches of many independent circuits of uneven size.
 //
 // The paper simulates one circuit at a time with one kernel per window and a
 // host loop over measurements (Sec. 4.1, Alg. 2). Small circuits leave most of
-// a GB300 idle and pay a launch per step. Here a cooperative persistent kernel
+// a GB300 idle that way and pay a launch per step. A batch runs circuits of up
+// to 640 qubits with one block each, tableau in shared memory
+// (qs_batch_resident.cu), and the larger ones through one simulator each on
+// worker streams. With a launch shape given (qs_batch_tuning) the circuits of
+// n < 1024 run in the persistent kernel below instead: a cooperative launch that
 // walks every circuit's program in lock-step rounds (a round = a segment of gate
 // layers followed by a list of Z-measurements) and spreads each phase of a round
 // over all CTAs through flattened work lists (a work queue built on the host
@@ -37,35 +40,18 @@
 
 #include <nvtx3/nvToolsExt.h>
 
-#include "qs_internal.cuh"
+#include "qs_batch.cuh"
 #include "qs_rules.cuh"
 
 namespace qs {
 
 constexpr int64_t kBNoPivot = LLONG_MAX;
-constexpr uint32_t kBatchMaxQubits = 8192;  // det partials: <= 4 words per lane
-// Circuits of at least this many qubits run through per-circuit simulators
-// (blocked measurement, 64 measurements per tableau pass) on worker streams;
-// the persistent kernel takes the smaller ones, whose per-launch costs
-// dominate when they run alone.
+// Circuits of at least this many qubits always run through per-circuit
+// simulators (blocked measurement, 64 measurements per tableau pass) on worker
+// streams; the persistent kernel takes the smaller ones.
 constexpr uint32_t kBatchSimMinQubits = 1024;
 constexpr uint32_t kBatchMaxWorkers = 16;
 constexpr uint32_t kBatchLimitQubits = 1u << 20;
-
-struct BCirc {
-  uint32_t n, k, cs, rs, ncols, nrows;
-  uint32_t lpr, pad_;  // lanes per row in the update phase (power of two <= 32)
-  uint64_t *X, *Z, *S, *RX, *RZ;
-  uint32_t *colx;
-  int64_t *mst;
-  uint64_t *det_x, *det_z;  // k chunks x rs words
-  int32_t *det_scal;        // k
-  const uint32_t *gates;    // packed records of this circuit
-  const int64_t *lptr;      // n_layers + 1 offsets into gates
-  const uint32_t *qubits;   // measured qubits in program order
-  uint8_t *record;
-  uint64_t seed, shot;
-};
 
 struct BAct {
   uint32_t c, l0, l1, q0, qn, pad;
@@ -637,6 +623,7 @@ struct Carve2 {
 struct BSim {
   uint32_t index = 0;
   qs_sim *sim = nullptr;
+  bool mid = false;                // n < kBatchSimMinQubits: runs here unless a launch shape is given
   uint32_t *packed_dev = nullptr;  // qs_pack_layers records, device
   std::vector<int64_t> lp;         // layer offsets
   std::vector<uint32_t> rl, rm, qubits;
@@ -662,7 +649,17 @@ struct qs_batch {
   uint32_t built_wpb = 0;
   uint64_t signature = 0;
   int sms = 152;
-  bool any_small = false;               // the persistent kernel has work
+  bool any_small = false;               // circuits of n < kBatchSimMinQubits have work
+  struct Class {                        // circuits of one launch of the resident kernel
+    uint32_t first = 0, count = 0, threads = 0;  // ids [first, first + count), largest first
+    size_t smem = 0;
+    cudaStream_t stream = nullptr;      // classes after the first run beside it
+    cudaEvent_t done = nullptr;
+  };
+  std::vector<Class> classes;
+  uint32_t *d_ids = nullptr;
+  bool pending = false;                 // work enqueued since the last successful qs_batch_sync
+  bool persistent_ran = false;          // the last run gave a launch shape: n < kBatchSimMinQubits ran there
   std::vector<int32_t> sim_of;          // per circuit: index into sims, or -1
   std::vector<BSim> sims;
   std::vector<cudaStream_t> wstreams;   // worker streams of the large circuits
@@ -682,6 +679,11 @@ static void free_sims(qs_batch *b) {
   for (cudaStream_t st : b->wstreams) cudaStreamDestroy(st);
   if (b->start_ev) cudaEventDestroy(b->start_ev);
   b->start_ev = nullptr;
+  for (auto &c : b->classes) {
+    if (c.done) cudaEventDestroy(c.done);
+    if (c.stream) cudaStreamDestroy(c.stream);
+  }
+  b->classes.clear();
   b->wevents.clear();
   b->wstreams.clear();
 }
@@ -694,8 +696,8 @@ static void layout_of(uint32_t n, uint32_t &k, uint32_t &cs, uint32_t &ncols, ui
 
 struct BatchPlan {
   std::vector<size_t> off_X, off_Z, off_S, off_RX, off_RZ, off_colx, off_mst, off_dx, off_dz,
-      off_ds, off_rec, off_g, off_lp, off_q;
-  size_t zero_end = 0, circs = 0, acts = 0, rounds = 0, pre_n = 0, bar = 0, err = 0, total = 0;
+      off_ds, off_rec, off_g, off_lp, off_q, off_rt;
+  size_t zero_end = 0, circs = 0, ids = 0, acts = 0, rounds = 0, pre_n = 0, bar = 0, err = 0, total = 0;
   size_t acts_cap = 0;
 };
 
@@ -716,7 +718,7 @@ static int plan_batch(uint32_t count, const qs_batch_circuit *cc, BatchPlan &P, 
   P.zero_end = c.off;
   P.off_RX.resize(count); P.off_RZ.resize(count); P.off_colx.resize(count); P.off_mst.resize(count);
   P.off_dx.resize(count); P.off_dz.resize(count); P.off_ds.resize(count); P.off_rec.resize(count);
-  P.off_g.resize(count); P.off_lp.resize(count); P.off_q.resize(count);
+  P.off_g.resize(count); P.off_lp.resize(count); P.off_q.resize(count); P.off_rt.resize(count);
   for (uint32_t i = 0; i < count; ++i) {
     uint32_t k, cs, ncols, rs, nrows;
     layout_of(cc[i].n, k, cs, ncols, rs, nrows);
@@ -734,9 +736,11 @@ static int plan_batch(uint32_t count, const qs_batch_circuit *cc, BatchPlan &P, 
     P.off_g[i] = c.take((size_t)std::max<int64_t>(G, 1) * 8);
     P.off_lp[i] = c.take(((size_t)cc[i].n_layers + 1) * 8);
     P.off_q[i] = c.take((size_t)std::max<uint64_t>(M, 1) * 4);
+    P.off_rt[i] = c.take(2 * ((size_t)nrr + 1) * 4);
   }
   P.acts_cap = acts + 2 * (size_t)nrounds + 2;
   P.circs = c.take(count * sizeof(BCirc));
+  P.ids = c.take((size_t)count * 4);
   P.acts = c.take(P.acts_cap * sizeof(BAct));
   P.rounds = c.take((size_t)std::max<uint32_t>(nrounds, 1) * sizeof(BRound));
   P.pre_n = c.take(((size_t)count + 1) * 8);
@@ -945,6 +949,9 @@ int qs_batch_create(uint32_t count, const qs_batch_circuit *cc, void *stream, vo
     C.gates = reinterpret_cast<const uint32_t *>(base + P.off_g[i]);
     C.lptr = reinterpret_cast<const int64_t *>(base + P.off_lp[i]);
     C.qubits = reinterpret_cast<const uint32_t *>(base + P.off_q[i]);
+    C.rl = reinterpret_cast<const uint32_t *>(base + P.off_rt[i]);
+    C.rm = C.rl + c.n_rounds + 1;
+    C.nrounds = c.n_rounds;
     const uint64_t M = c.n_rounds ? c.round_meas[c.n_rounds] : 0;
     e = cudaMemcpy(base + P.off_g[i], packed.data(), packed.size() * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
@@ -958,6 +965,9 @@ int qs_batch_create(uint32_t count, const qs_batch_circuit *cc, void *stream, vo
     b->rm[i].assign(c.round_meas ? c.round_meas : nullptr,
                     c.round_meas ? c.round_meas + c.n_rounds + 1 : nullptr);
     if (b->rl[i].empty()) { b->rl[i].push_back(0); b->rm[i].push_back(0); }
+    const size_t rtb = b->rl[i].size() * 4;
+    if (e == cudaSuccess) e = cudaMemcpy(base + P.off_rt[i], b->rl[i].data(), rtb, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(base + P.off_rt[i] + rtb, b->rm[i].data(), rtb, cudaMemcpyHostToDevice);
     if (orig[i].n < kBatchSimMinQubits && (G > 0 || M > 0)) b->any_small = true;
     pre_n[i + 1] = pre_n[i] + c.n;
     b->n_max = std::max(b->n_max, c.n);
@@ -978,6 +988,28 @@ int qs_batch_create(uint32_t count, const qs_batch_circuit *cc, void *stream, vo
   if (e == cudaSuccess)
     e = cudaMemcpy(b->d_pre_n, pre_n.data(), pre_n.size() * 8, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemset(b->d_err, 0, 64);
+  // resident circuits by size class (threads and shared memory per block), largest first
+  {
+    std::vector<uint32_t> ids;
+    for (uint32_t i = 0; i < count; ++i)
+      if (orig[i].n <= kResidentMaxQubits) ids.push_back(i);
+    std::stable_sort(ids.begin(), ids.end(), [&](uint32_t x, uint32_t y) { return orig[x].n > orig[y].n; });
+    const struct { uint32_t min_n, threads; } kinds[3] = {{449, 1024}, {257, 512}, {0, 256}};
+    uint32_t at = 0;
+    for (const auto &kind : kinds) {
+      qs_batch::Class c;
+      c.first = at;
+      while (at < ids.size() && orig[ids[at]].n >= kind.min_n) ++at;
+      c.count = at - c.first;
+      if (!c.count) continue;
+      c.threads = kind.threads;
+      c.smem = batch_resident_smem(orig[ids[c.first]].n);
+      b->classes.push_back(c);
+    }
+    b->d_ids = reinterpret_cast<uint32_t *>(base + P.ids);
+    if (e == cudaSuccess && !ids.empty())
+      e = cudaMemcpy(b->d_ids, ids.data(), ids.size() * 4, cudaMemcpyHostToDevice);
+  }
   int dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, dev);
@@ -986,16 +1018,20 @@ int qs_batch_create(uint32_t count, const qs_batch_circuit *cc, void *stream, vo
     delete b;
     return bfail(QS_ERR_CUDA, std::string("batch upload: ") + cudaGetErrorString(e));
   }
-  // large circuits: one simulator each, spread over the worker streams by size
+  // the other circuits: one simulator each, spread over the worker streams by size
   b->sim_of.assign(count, -1);
   std::vector<uint32_t> large;
   for (uint32_t i = 0; i < count; ++i)
-    if (orig[i].n >= kBatchSimMinQubits) large.push_back(i);
+    if (orig[i].n > kResidentMaxQubits) large.push_back(i);
   std::stable_sort(large.begin(), large.end(),
                    [&](uint32_t x, uint32_t y) { return orig[x].n > orig[y].n; });
   const uint32_t nw = std::min<uint32_t>(kBatchMaxWorkers, (uint32_t)large.size());
-  if (nw && cudaEventCreateWithFlags(&b->start_ev, cudaEventDisableTiming) != cudaSuccess)
+  if (cudaEventCreateWithFlags(&b->start_ev, cudaEventDisableTiming) != cudaSuccess)
     rc = bfail(QS_ERR_CUDA, "batch event creation failed");
+  for (size_t i = 1; i < b->classes.size() && rc == QS_OK; ++i)
+    if (cudaStreamCreateWithFlags(&b->classes[i].stream, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreateWithFlags(&b->classes[i].done, cudaEventDisableTiming) != cudaSuccess)
+      rc = bfail(QS_ERR_CUDA, "batch stream creation failed");
   for (uint32_t w = 0; w < nw && rc == QS_OK; ++w) {
     cudaStream_t st = nullptr;
     cudaEvent_t ev = nullptr;
@@ -1013,6 +1049,7 @@ int qs_batch_create(uint32_t count, const qs_batch_circuit *cc, void *stream, vo
     const qs_batch_circuit &c = orig[i];
     BSim x;
     x.index = i;
+    x.mid = c.n < kBatchSimMinQubits;
     x.seed = c.seed;
     x.shot = c.shot;
     const uint64_t M = c.n_rounds ? c.round_meas[c.n_rounds] : 0;
@@ -1067,6 +1104,8 @@ int qs_batch_destroy(qs_batch *b) {
 }
 
 static int tuning_ok(const qs_batch *b, const qs_batch_tuning &t, size_t *smem) {
+  *smem = 0;
+  if (t.threads == 0) return QS_OK;  // the default: no persistent kernel
   if (t.threads != 256 && t.threads != 512 && t.threads != 1024)
     return bfail(QS_ERR_ARG, "tuning.threads must be 256, 512 or 1024");
   if (t.words_per_block != 1 && t.words_per_block != 2)
@@ -1078,11 +1117,11 @@ static int tuning_ok(const qs_batch *b, const qs_batch_tuning &t, size_t *smem) 
   return QS_OK;
 }
 
-static int run_kernel(qs_batch *b, const qs_batch_tuning *tuning, uint32_t round_limit);
+static int run_kernel(qs_batch *b, const qs_batch_tuning &tuning, uint32_t round_limit);
 static int batch_run(qs_batch *b, const qs_batch_tuning *tuning, uint32_t round_limit);
 
-// Enqueues every large circuit's rounds on its simulator, one host thread per
-// worker stream, then makes the batch stream wait for the worker streams.
+// Enqueues the rounds of the circuits that run through simulators, one host
+// thread per worker stream, then makes the batch stream wait for the worker streams.
 static int run_sims(qs_batch *b, uint32_t round_limit) {
   const uint32_t nw = (uint32_t)b->wstreams.size();
   std::mutex mu;
@@ -1090,9 +1129,9 @@ static int run_sims(qs_batch *b, uint32_t round_limit) {
   std::string first_msg;
   auto worker = [&](uint32_t w) {
     int rc = QS_OK;
-    if (cudaStreamWaitEvent(b->wstreams[w], b->start_ev, 0) != cudaSuccess) rc = QS_ERR_CUDA;
     for (size_t j = w; j < b->sims.size() && rc == QS_OK; j += nw) {
       BSim &x = b->sims[j];
+      if (x.mid ? b->persistent_ran : b->skip_sims) continue;
       rc = qs_sim_reset(x.sim, nullptr);
       const uint32_t nr = x.rl.empty() ? 0 : (uint32_t)x.rl.size() - 1;
       const uint32_t lim = std::min(nr, round_limit);
@@ -1103,6 +1142,12 @@ static int run_sims(qs_batch *b, uint32_t round_limit) {
           rc = qs_sim_measure(x.sim, x.qubits.data() + x.rm[r], x.rm[r + 1] - x.rm[r],
                               qs_key{x.seed, x.shot}, nullptr);
       }
+      // where qs_batch_sample looks for the records of n < kBatchSimMinQubits
+      const uint64_t M = qs_sim_num_measurements(x.sim);
+      if (rc == QS_OK && x.mid && M &&
+          cudaMemcpyAsync(b->circs[x.index].record, sim_record(x.sim), M, cudaMemcpyDeviceToDevice,
+                          b->wstreams[w]) != cudaSuccess)
+        rc = QS_ERR_CUDA;
       if (rc != QS_OK) {
         std::lock_guard<std::mutex> lock(mu);
         if (first_rc == QS_OK) {
@@ -1141,23 +1186,59 @@ int qs_batch_run(qs_batch *b, const qs_batch_tuning *tuning, uint32_t round_limi
   return rc;
 }
 
+// The resident kernel's launches, one per size class, side by side: a class's
+// blocks run until their circuits are done, so the classes must not queue.
+static int run_resident(qs_batch *b, uint32_t round_limit) {
+  cudaError_t e = cudaMemsetAsync(b->d_err, 0, 64, b->stream);
+  if (e == cudaSuccess && b->classes.size() > 1) e = cudaEventRecord(b->start_ev, b->stream);
+  for (size_t i = 0; i < b->classes.size() && e == cudaSuccess; ++i) {
+    const qs_batch::Class &c = b->classes[i];
+    const cudaStream_t st = c.stream ? c.stream : b->stream;
+    if (c.stream) e = cudaStreamWaitEvent(st, b->start_ev, 0);
+    if (e == cudaSuccess)
+      e = launch_batch_resident(b->d_circs, b->d_ids + c.first, c.count, c.threads, c.smem,
+                                round_limit ? round_limit : 0xFFFFFFFFu, b->d_err, st);
+    if (e == cudaSuccess && c.stream) e = cudaEventRecord(c.done, st);
+  }
+  for (size_t i = 0; i < b->classes.size() && e == cudaSuccess; ++i)
+    if (b->classes[i].stream) e = cudaStreamWaitEvent(b->stream, b->classes[i].done, 0);
+  if (e != cudaSuccess) {
+    b->broken = true;
+    return bfail(QS_ERR_CUDA, std::string("batch launch: ") + cudaGetErrorString(e));
+  }
+  return QS_OK;
+}
+
 static int batch_run(qs_batch *b, const qs_batch_tuning *tuning, uint32_t round_limit) {
   if (!b) return bfail(QS_ERR_ARG, "batch is NULL");
   if (b->broken) return bfail(QS_ERR_STATE, "batch is unusable after an earlier device error");
-  b->ran_full = (round_limit == 0 || round_limit >= b->nrounds) && !b->skip_sims;
+  const bool persistent = tuning && tuning->threads != 0;
+  b->pending = true;
+  size_t smem = 0;
   int rc = QS_OK;
-  const bool sims = !b->skip_sims && !b->sims.empty();
+  if (persistent && (rc = tuning_ok(b, *tuning, &smem))) return rc;
+  b->ran_full = (round_limit == 0 || round_limit >= b->nrounds) && !b->skip_sims;
+  b->persistent_ran = persistent;
+  bool sims = false;
+  for (const BSim &x : b->sims) sims |= !(x.mid ? persistent : b->skip_sims);
+  // the worker streams start after the batch stream's earlier work, beside its kernels
   if (sims && cudaEventRecord(b->start_ev, b->stream) != cudaSuccess)
     return bfail(QS_ERR_CUDA, "batch event record failed");
-  if (b->any_small || b->sims.empty()) {
-    if ((rc = run_kernel(b, tuning, round_limit))) return rc;
+  if (sims)
+    for (cudaStream_t st : b->wstreams)
+      if (cudaStreamWaitEvent(st, b->start_ev, 0) != cudaSuccess)
+        return bfail(QS_ERR_CUDA, "worker stream wait failed");
+  if (persistent) {
+    if ((b->any_small || b->sims.empty()) && (rc = run_kernel(b, *tuning, round_limit))) return rc;
+  } else if ((rc = run_resident(b, round_limit))) {
+    return rc;
   }
   if (sims) rc = run_sims(b, round_limit ? round_limit : 0xFFFFFFFFu);
   return rc;
 }
 
-static int run_kernel(qs_batch *b, const qs_batch_tuning *tuning, uint32_t round_limit) {
-  qs_batch_tuning t = tuning ? *tuning : qs_batch_tuning{512, 0, 1, 0, 0};
+static int run_kernel(qs_batch *b, const qs_batch_tuning &tuning, uint32_t round_limit) {
+  qs_batch_tuning t = tuning;
   if (t.spin_limit == 0) t.spin_limit = 20ull * 1000 * 1000;  // x >=128 ns: several seconds
   size_t smem = 0;
   int rc = tuning_ok(b, t, &smem);
@@ -1206,6 +1287,9 @@ int qs_batch_sync(qs_batch *b) {
   if (!b) return bfail(QS_ERR_ARG, "batch is NULL");
   if (b->broken) return bfail(QS_ERR_STATE, "batch is unusable after an earlier device error");
   cudaError_t e = cudaStreamSynchronize(b->stream);
+  // no batch work since the flags were last read: reading 56 circuits' records
+  // read every simulator's flags 56 times, 5 of the 9 ms of a batch of 56
+  if (e == cudaSuccess && !b->pending) return QS_OK;
   uint32_t flags = 0;
   if (e == cudaSuccess) e = cudaMemcpy(&flags, b->d_err, 4, cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) {
@@ -1222,7 +1306,15 @@ int qs_batch_sync(qs_batch *b) {
     const int rc = qs_sim_sync(x.sim);
     if (rc) return bfail(rc, std::string("circuit ") + std::to_string(x.index) + ": " + qs_last_error());
   }
+  b->pending = false;
   return QS_OK;
+}
+
+// the simulator that holds circuit c's state after the last run, or nullptr
+static BSim *sim_of(qs_batch *b, uint32_t c) {
+  if (b->sim_of[c] < 0) return nullptr;
+  BSim &x = b->sims[b->sim_of[c]];
+  return x.mid && b->persistent_ran ? nullptr : &x;
 }
 
 int qs_batch_record(qs_batch *b, uint32_t circuit, uint8_t *dst, size_t count) {
@@ -1231,8 +1323,8 @@ int qs_batch_record(qs_batch *b, uint32_t circuit, uint8_t *dst, size_t count) {
   if (count && !dst) return bfail(QS_ERR_ARG, "dst is NULL");
   int rc = qs_batch_sync(b);
   if (rc) return rc;
-  if (b->sim_of[circuit] >= 0) {
-    rc = count ? qs_sim_record(b->sims[b->sim_of[circuit]].sim, 0, count, dst) : QS_OK;
+  if (BSim *x = sim_of(b, circuit)) {
+    rc = count ? qs_sim_record(x->sim, 0, count, dst) : QS_OK;
     return rc ? bfail(rc, qs_last_error()) : QS_OK;
   }
   if (count && cudaMemcpy(dst, b->circs[circuit].record, count, cudaMemcpyDeviceToHost) != cudaSuccess)
@@ -1245,8 +1337,8 @@ int qs_batch_export_rows(qs_batch *b, uint32_t circuit, const uint32_t *rows, ui
   if (!b || circuit >= b->count) return bfail(QS_ERR_ARG, "bad batch or circuit index");
   int rc = qs_batch_sync(b);
   if (rc) return rc;
-  if (b->sim_of[circuit] >= 0) {
-    rc = qs_sim_export_rows(b->sims[b->sim_of[circuit]].sim, rows, count, dst);
+  if (BSim *x = sim_of(b, circuit)) {
+    rc = qs_sim_export_rows(x->sim, rows, count, dst);
     return rc ? bfail(rc, qs_last_error()) : QS_OK;
   }
   const BCirc &C = b->circs[circuit];
@@ -1313,19 +1405,33 @@ int qs_batch_autotune(qs_batch *b, uint32_t round_limit, const char *cache_path,
     }
   }
   if (!b->any_small) {  // every circuit runs through a simulator: nothing to tune
-    *best = qs_batch_tuning{512, 0, 1, 0, 0};
+    *best = qs_batch_tuning{0, 0, 0, 0, 0};
     return QS_OK;
   }
-  b->skip_sims = true;  // time the persistent kernel alone
+  b->skip_sims = true;  // time the circuits of n < 1024 alone
   const uint32_t threads[] = {256, 512, 1024};
   const uint32_t bps[] = {1, 2, 4};
   const uint32_t wpbs[] = {1, 2};
   const uint32_t depths[] = {0, 1};
   float best_ms = 1e30f;
-  qs_batch_tuning best_t{512, 0, 1, 0, 0};
+  qs_batch_tuning best_t{0, 0, 0, 0, 0};
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
+  auto consider = [&](const qs_batch_tuning &t) {
+    float ms_min = 1e30f;
+    for (int rep = 0; rep < 2; ++rep) {
+      cudaEventRecord(e0, b->stream);
+      if (qs_batch_run(b, &t, round_limit) != QS_OK) break;
+      cudaEventRecord(e1, b->stream);
+      if (qs_batch_sync(b) != QS_OK) break;
+      float ms = 0;
+      cudaEventElapsedTime(&ms, e0, e1);
+      ms_min = std::min(ms_min, ms);
+    }
+    if (ms_min < best_ms) { best_ms = ms_min; best_t = t; }
+  };
+  consider(best_t);  // the default: a block per small circuit
   for (uint32_t th : threads)
     for (uint32_t bp : bps)
       for (uint32_t w : wpbs)
@@ -1334,17 +1440,7 @@ int qs_batch_autotune(qs_batch *b, uint32_t round_limit, const char *cache_path,
           size_t smem;
           if (tuning_ok(b, t, &smem) != QS_OK) continue;
           if (th * bp > 2048) continue;
-          float ms_min = 1e30f;
-          for (int rep = 0; rep < 2; ++rep) {
-            cudaEventRecord(e0, b->stream);
-            if (qs_batch_run(b, &t, round_limit) != QS_OK) break;
-            cudaEventRecord(e1, b->stream);
-            if (qs_batch_sync(b) != QS_OK) break;
-            float ms = 0;
-            cudaEventElapsedTime(&ms, e0, e1);
-            ms_min = std::min(ms_min, ms);
-          }
-          if (ms_min < best_ms) { best_ms = ms_min; best_t = t; }
+          consider(t);
         }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
@@ -1359,11 +1455,15 @@ int qs_batch_autotune(qs_batch *b, uint32_t round_limit, const char *cache_path,
   return best_ms < 1e29f ? QS_OK : bfail(QS_ERR_INTERNAL, "no tuning candidate ran");
 }
 
+// circuits that only simulators run (n >= kBatchSimMinQubits)
+static bool is_large(const qs_batch *b, uint32_t c) { return b->sim_of[c] >= 0 && !b->sims[b->sim_of[c]].mid; }
+
 int qs_batch_sample(qs_batch *b, const uint64_t *shots, const uint64_t *seeds, uint64_t *const *records) {
   if (!b) return bfail(QS_ERR_ARG, "batch is NULL");
   if (b->broken) return bfail(QS_ERR_STATE, "batch is unusable after an earlier device error");
   if (!shots || !seeds || !records) return bfail(QS_ERR_ARG, "NULL argument");
   if (!b->ran_full) return bfail(QS_ERR_STATE, "sampling needs the records of a complete qs_batch_run");
+  b->pending = true;
   // small circuits: one launch; a table of the sampled circuits, their round
   // tables and the prefix of their shot words
   std::vector<BSampleCirc> sc;
@@ -1374,7 +1474,7 @@ int qs_batch_sample(qs_batch *b, const uint64_t *shots, const uint64_t *seeds, u
     if (shots[c] == 0) continue;
     if (shots[c] > 2000000000ull) return bfail(QS_ERR_ARG, "shots must be at most 2e9");
     if (!records[c] && b->meas_total[c]) return bfail(QS_ERR_ARG, "records[c] is NULL");
-    if (b->sim_of[c] >= 0 || b->meas_total[c] == 0) continue;  // large, or nothing to record
+    if (is_large(b, c) || b->meas_total[c] == 0) continue;  // large, or nothing to record
     BSampleCirc x{};
     x.c = c;
     x.nrounds = (uint32_t)b->rl[c].size() - 1;
@@ -1420,7 +1520,7 @@ int qs_batch_sample(qs_batch *b, const uint64_t *shots, const uint64_t *seeds, u
   }
   // large circuits: their own simulators replay their op logs on the worker streams
   bool any_large = false;
-  for (uint32_t c = 0; c < b->count; ++c) any_large |= shots[c] > 0 && b->sim_of[c] >= 0;
+  for (uint32_t c = 0; c < b->count; ++c) any_large |= shots[c] > 0 && is_large(b, c);
   if (any_large) {
     if (cudaEventRecord(b->start_ev, b->stream) != cudaSuccess)
       return bfail(QS_ERR_CUDA, "batch event record failed");
@@ -1429,7 +1529,7 @@ int qs_batch_sample(qs_batch *b, const uint64_t *shots, const uint64_t *seeds, u
       if (cudaStreamWaitEvent(b->wstreams[w], b->start_ev, 0) != cudaSuccess)
         return bfail(QS_ERR_CUDA, "worker stream wait failed");
     for (uint32_t c = 0; c < b->count; ++c) {
-      if (!(shots[c] > 0 && b->sim_of[c] >= 0)) continue;
+      if (!(shots[c] > 0 && is_large(b, c))) continue;
       BSim &x = b->sims[b->sim_of[c]];
       const uint64_t ow = (shots[c] + 63) / 64;
       const int rc = qs_sim_sample(x.sim, shots[c], seeds[c], records[c], b->meas_total[c] * ow, nullptr, 0);

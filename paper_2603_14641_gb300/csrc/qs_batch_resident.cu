@@ -1,0 +1,301 @@
+// Batched small circuits, one block per circuit with its tableau in shared
+// memory for the whole program (n <= 640).
+//
+// The persistent batch kernel (qs_batch.cu) walks all circuits in lock-step with
+// three grid barriers per measurement: 56 circuits of 50..1,000 qubits with
+// 1,000 measurements each at most took 19 ms, nearly all of it barriers. A
+// circuit of n <= 640 qubits fits one SM (2,080 ceil(n/64)^2 bytes, 208 KB at
+// 640), and there everything is a block barrier away.
+//
+// Layout: the tableau is kept as 64 x 64-bit blocks (u, w), u = qubit / 64, w =
+// packed row / 64, 65 words apart so that neighbouring blocks start one bank
+// later. In gate phases word i of block (u, w) is word w of the column of qubit
+// 64 u + i; in measurement phases it is word u of packed row 64 w + i. The
+// layout switch transposes every block in place.
+//   gates:   thread = (column word w, gate lane): a warp's lanes walk the words
+//            of a gate's columns (conflict-free), signs stay in a register for
+//            the whole run of layers, the next layer's records arrive by cp.async.
+//   measure: thread = packed row (two at most), two barriers per measurement: the
+//            pivot by ballot and a shared-memory minimum, then every target row
+//            multiplies the pivot row into itself and the destabilizer partner
+//            copies it; the pivot row becomes +-Z_q before the next search. Phases
+//            are two-bit counters per bit position, so a row needs two popcounts.
+//            Deterministic outcomes of a round are evaluated after it, one warp
+//            each (measurements of a round commute).
+#include <climits>
+
+#include "qs_batch.cuh"
+#include "qs_rules.cuh"
+
+namespace qs {
+
+constexpr uint32_t kListed = 1024;  // measurements whose qubits and coins are staged at a time
+
+__host__ __device__ constexpr size_t resident_blocks_words(uint32_t k) { return (size_t)k * 2 * k * 65; }
+
+size_t batch_resident_smem(uint32_t n) {
+  const uint32_t k = (n + 63) / 64;
+  return 2 * resident_blocks_words(k) * 8 + 2 * k * 8 + 2 * (size_t)n * 8 + kListed * (2 + 1 + 2) + 64;
+}
+
+// rows lane (lo) and lane + 32 (hi) of a 64 x 64 bit block -> its transpose
+__device__ __forceinline__ void transpose_block(uint64_t &lo, uint64_t &hi, int lane) {
+  {
+    const uint64_t t = ((lo >> 32) ^ hi) & 0x00000000FFFFFFFFull;
+    lo ^= t << 32;
+    hi ^= t;
+  }
+  const uint64_t masks[5] = {0x0000FFFF0000FFFFull, 0x00FF00FF00FF00FFull, 0x0F0F0F0F0F0F0F0Full,
+                             0x3333333333333333ull, 0x5555555555555555ull};
+#pragma unroll
+  for (int s = 0; s < 5; ++s) {
+    const int j = 16 >> s;
+    const uint64_t m = masks[s];
+    const uint64_t pl = __shfl_xor_sync(0xffffffffu, lo, j), ph = __shfl_xor_sync(0xffffffffu, hi, j);
+    if ((lane & j) == 0) {
+      lo ^= (((lo >> j) ^ pl) & m) << j;
+      hi ^= (((hi >> j) ^ ph) & m) << j;
+    } else {
+      lo ^= ((pl >> j) ^ lo) & m;
+      hi ^= ((ph >> j) ^ hi) & m;
+    }
+  }
+}
+
+// two-bit counters, one per bit position: ones + 2 twos (mod 4)
+struct Count4 {
+  uint64_t ones = 0, twos = 0;
+  __device__ __forceinline__ void add(uint64_t v) { twos ^= ones & v; ones ^= v; }
+  __device__ __forceinline__ void add2(uint64_t v) { twos ^= v; }
+  __device__ __forceinline__ void sub(uint64_t v) { add(v); add2(v); }
+  __device__ __forceinline__ int total() const { return (__popcll(ones) + 2 * __popcll(twos)) & 3; }
+};
+
+__global__ void __launch_bounds__(1024)
+batch_resident_kernel(const BCirc *__restrict__ circs, const uint32_t *__restrict__ ids, uint32_t round_limit,
+                      uint32_t *__restrict__ err) {
+  extern __shared__ uint64_t sm[];
+  __shared__ uint32_t s_piv[3], s_ndet;
+  const BCirc &C = circs[ids[blockIdx.x]];
+  const uint32_t n = C.n, k = C.k, KB = 2 * k, T = blockDim.x, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const size_t words = resident_blocks_words(k);
+  uint64_t *X = sm, *Z = X + words;
+  uint32_t *S = reinterpret_cast<uint32_t *>(Z + words);  // 2 KB words of 32 rows
+  uint2 *gbuf = reinterpret_cast<uint2 *>(S + 2 * KB);    // two layers of gate records
+  uint16_t *s_q = reinterpret_cast<uint16_t *>(gbuf + 2 * (size_t)n);
+  uint16_t *s_det = s_q + kListed;
+  uint8_t *s_coin = reinterpret_cast<uint8_t *>(s_det + kListed);
+  auto at = [KB](uint32_t u, uint32_t w, uint32_t i) { return (u * KB + w) * 65 + i; };
+
+  // D_i = X_i, S_i = Z_i, no signs (Alg. 2 init)
+  for (size_t i = t; i < 2 * words; i += T) sm[i] = 0;
+  for (uint32_t i = t; i < 2 * KB; i += T) S[i] = 0;
+  __syncthreads();
+  for (uint32_t q = t; q < n; q += T) {
+    X[at(q >> 6, q >> 6, q & 63)] = 1ull << (q & 63);
+    Z[at(q >> 6, k + (q >> 6), q & 63)] = 1ull << (q & 63);
+  }
+  __syncthreads();
+
+  auto transpose_all = [&]() {
+    for (uint32_t b = warp; b < 2 * k * KB; b += T >> 5) {
+      uint64_t *p = sm + (size_t)b * 65;  // X and Z blocks lie one after the other
+      uint64_t lo = p[lane], hi = p[lane + 32];
+      transpose_block(lo, hi, (int)lane);
+      p[lane] = lo;
+      p[lane + 32] = hi;
+    }
+    __syncthreads();
+  };
+
+  const uint32_t gate_lanes = T / KB, gw = t % KB, gl = t / KB;
+  const uint32_t rounds = min(C.nrounds, round_limit);
+  for (uint32_t r = 0; r < rounds; ++r) {
+    const uint32_t l0 = C.rl[r], l1 = C.rl[r + 1];
+    if (l1 > l0) {
+      // records of a layer: g[a .. b) -> buffer, one 8-byte copy per thread and record
+      auto fetch = [&](int64_t a, int64_t b, uint2 *dst) {
+        for (int64_t g = a + t; g < b; g += T) {
+          const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst + (g - a));
+          asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(C.gates + 2 * g) : "memory");
+        }
+      };
+      int64_t a = C.lptr[l0], b = C.lptr[l0 + 1], c = l0 + 2 <= l1 ? C.lptr[l0 + 2] : b;
+      fetch(a, b, gbuf);
+      uint64_t sacc = 0;
+      for (uint32_t l = l0; l < l1; ++l) {
+        const int64_t after = l + 3 <= l1 ? __ldg(C.lptr + l + 3) : c;
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();  // this layer's records are here; the previous layer is done with its buffer
+        if (l + 1 < l1) fetch(b, c, gbuf + ((l + 1 - l0) & 1) * (size_t)n);
+        const uint2 *rec = gbuf + ((l - l0) & 1) * (size_t)n;
+        const uint32_t cnt = (uint32_t)(b - a);
+        if (gl < gate_lanes)
+          for (uint32_t g = gl; g < cnt; g += gate_lanes) {
+            const uint2 q = rec[g];
+            const uint32_t type = q.x >> 24, qa = q.x & 0xFFFFFFu, qb = q.y;
+            const bool two = type >= QS_CX && type <= QS_ISWAP;
+            if (qa >= n || type >= QS_NUM_GATE_TYPES || (two && (qb >= n || qb == qa))) {
+              atomicOr(err, kErrBadGate);
+              continue;
+            }
+            const uint32_t ia = at(qa >> 6, gw, qa & 63), ib = two ? at(qb >> 6, gw, qb & 63) : ia;
+            uint64_t xa = X[ia], za = Z[ia], xb = 0, zb = 0;
+            if (two) { xb = X[ib]; zb = Z[ib]; }
+            rule<true>(type, xa, za, xb, zb, sacc);
+            if ((kWritesXa >> type) & 1) X[ia] = xa;
+            if ((kWritesZa >> type) & 1) Z[ia] = za;
+            if ((kWritesXb >> type) & 1) X[ib] = xb;
+            if ((kWritesZb >> type) & 1) Z[ib] = zb;
+          }
+        a = b; b = c; c = after;
+      }
+      if (gl < gate_lanes) {
+        if ((uint32_t)sacc) atomicXor(S + 2 * gw, (uint32_t)sacc);
+        if ((uint32_t)(sacc >> 32)) atomicXor(S + 2 * gw + 1, (uint32_t)(sacc >> 32));
+      }
+      __syncthreads();
+    }
+    const uint32_t m0 = C.rm[r], m1 = C.rm[r + 1];
+    if (m1 == m0) continue;
+    transpose_all();
+    for (uint32_t base = m0; base < m1; base += kListed) {
+      const uint32_t cnt = min(kListed, m1 - base);
+      for (uint32_t j = t; j < cnt; j += T) {
+        s_q[j] = (uint16_t)C.qubits[base + j];
+        s_coin[j] = (uint8_t)(philox4x64_10(base + j, C.shot, 0, 0, C.seed, kCoinKey).v[0] & 1u);
+      }
+      if (t < 3) s_piv[t] = UINT_MAX;
+      if (t == 0) s_ndet = 0;
+      __syncthreads();
+      uint32_t p_old = UINT_MAX, q_old = 0, coin_old = 0;  // pivot row still to become +-Z_q
+      for (uint32_t j = 0; j <= cnt; ++j) {
+        const bool last = j == cnt;  // only finishes the last pivot row
+        const uint32_t q = last ? 0 : s_q[j], qu = q >> 6, qi = q & 63;
+        uint32_t bits = 0;  // bit m: own row t + m T has x bit q
+        for (uint32_t r0 = 0, m = 0; r0 < 64 * KB; r0 += T, ++m) {
+          const uint32_t row = r0 + t, w = row >> 6, i = row & 63;
+          if (row - lane >= 64 * KB) break;  // uniform over the warp
+          bool bit = false;
+          uint32_t flip = 0;
+          if (row == p_old) {
+            for (uint32_t u = 0; u < k; ++u) {
+              X[at(u, w, i)] = 0;
+              Z[at(u, w, i)] = u == (q_old >> 6) ? 1ull << (q_old & 63) : 0ull;
+            }
+            flip = ((S[row >> 5] >> (row & 31)) & 1u) ^ coin_old;
+          } else if (!last) {
+            bit = (X[at(qu, w, i)] >> qi) & 1ull;
+          }
+          if (p_old != UINT_MAX && (p_old >> 5) == (row >> 5)) {  // uniform over the warp
+            const uint32_t f = __ballot_sync(0xffffffffu, flip);
+            if (lane == 0 && f) S[row >> 5] ^= f;
+          }
+          const uint32_t ball = __ballot_sync(0xffffffffu, bit);
+          if (lane == 0 && ball && row >= 64 * k) atomicMin(&s_piv[j % 3], row + __ffs(ball) - 1);
+          bits |= (uint32_t)bit << m;
+        }
+        if (last) break;
+        if (t == 0) s_piv[(j + 1) % 3] = UINT_MAX;
+        __syncthreads();
+        const uint32_t p = s_piv[j % 3];
+        p_old = p;
+        if (p == UINT_MAX) {  // deterministic: nothing changes; evaluated after the list
+          if (t == 0) s_det[s_ndet++] = (uint16_t)j;
+          continue;
+        }
+        q_old = q;
+        coin_old = s_coin[j];
+        if (t == 0) C.record[base + j] = (uint8_t)coin_old;
+        const uint32_t pd = p - 64 * k, pw = p >> 6, pi = p & 63;
+        const int rp = (int)((S[p >> 5] >> (p & 31)) & 1u);
+        for (uint32_t r0 = 0, m = 0; r0 < 64 * KB; r0 += T, ++m) {
+          const uint32_t row = r0 + t, w = row >> 6, i = row & 63;
+          if (row - lane >= 64 * KB) break;
+          uint32_t flip = 0;
+          if (row == pd) {  // D_{p-n} <- S_p
+            for (uint32_t u = 0; u < k; ++u) {
+              X[at(u, w, i)] = X[at(u, pw, pi)];
+              Z[at(u, w, i)] = Z[at(u, pw, pi)];
+            }
+            flip = ((S[row >> 5] >> (row & 31)) & 1u) ^ (uint32_t)rp;
+          } else if (((bits >> m) & 1u) && row != p) {
+            Count4 c;
+            for (uint32_t u = 0; u < k; ++u) {
+              const uint64_t x = X[at(u, w, i)], z = Z[at(u, w, i)], ax = X[at(u, pw, pi)], az = Z[at(u, pw, pi)];
+              const uint64_t nx = x ^ ax, nz = z ^ az;
+              c.add(x & z);
+              c.add(ax & az);
+              c.add2(az & x);
+              c.sub(nx & nz);
+              X[at(u, w, i)] = nx;
+              Z[at(u, w, i)] = nz;
+            }
+            const int e = (c.total() + 2 * rp) & 3;
+            if (e & 1) atomicOr(err, kErrOddPhase);
+            flip = (uint32_t)(e >> 1);
+          }
+          const uint32_t f = __ballot_sync(0xffffffffu, flip);
+          if (lane == 0 && f) S[row >> 5] ^= f;  // the warp's own 32 rows; bit p is none of them
+        }
+        __syncthreads();
+      }
+      __syncthreads();
+      // deterministic outcomes: (-1)^m Z_q = prod of S_i over D_i with x_iq = 1, a warp each, lane = word
+      for (uint32_t d = warp; d < s_ndet; d += T >> 5) {
+        const uint32_t j = s_det[d], q = s_q[j];
+        uint64_t px = 0, pz = 0, cross = 0;
+        int cnt4 = 0;
+        for (uint32_t w = 0; w < k; ++w) {
+          const uint64_t *col = X + at(q >> 6, w, 0);
+          const uint32_t lo = __ballot_sync(0xffffffffu, (col[lane] >> (q & 63)) & 1ull);
+          const uint32_t hi = __ballot_sync(0xffffffffu, (col[lane + 32] >> (q & 63)) & 1ull);
+          uint64_t m = ((uint64_t)hi << 32) | lo;
+          if (lane == 0) cnt4 += 2 * (__popc(lo & S[2 * (k + w)]) + __popc(hi & S[2 * (k + w) + 1]));
+          while (m) {
+            const uint32_t i = (uint32_t)__ffsll((long long)m) - 1;
+            m &= m - 1;
+            if (lane < k) {
+              const uint64_t x = X[at(lane, k + w, i)], z = Z[at(lane, k + w, i)];
+              cross ^= x & pz;
+              cnt4 += __popcll(x & z);
+              px ^= x;
+              pz ^= z;
+            }
+          }
+        }
+        const int e = __reduce_add_sync(0xffffffffu, cnt4 + 2 * (__popcll(cross) & 1)) & 3;
+        const uint64_t want = lane == (q >> 6) ? 1ull << (q & 63) : 0ull;
+        if (lane < k && (px != 0 || pz != want)) atomicOr(err, kErrDetProduct);
+        if (lane == 0) {
+          if (e & 1) atomicOr(err, kErrOddPhase);
+          C.record[base + j] = (uint8_t)(e >> 1);
+        }
+      }
+      __syncthreads();
+    }
+    transpose_all();
+  }
+  // the column-major tableau with its zero padding
+  for (size_t i = t; i < (size_t)C.ncols * C.cs; i += T) {
+    const uint32_t q = (uint32_t)(i / C.cs), w = (uint32_t)(i % C.cs);
+    const bool in = q < 64 * k && w < KB;
+    C.X[i] = in ? X[at(q >> 6, w, q & 63)] : 0;
+    C.Z[i] = in ? Z[at(q >> 6, w, q & 63)] : 0;
+  }
+  for (uint32_t w = t; w < C.cs; w += T) C.S[w] = w < KB ? ((uint64_t)S[2 * w + 1] << 32) | S[2 * w] : 0;
+}
+
+cudaError_t launch_batch_resident(const BCirc *circs, const uint32_t *ids, uint32_t count, uint32_t threads,
+                                  size_t smem, uint32_t round_limit, uint32_t *err, cudaStream_t s) {
+  static std::atomic<uint64_t> attr_set{0};
+  cudaError_t e = once_per_device(attr_set, []() {
+    return cudaFuncSetAttribute(batch_resident_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)batch_resident_smem(kResidentMaxQubits));
+  });
+  if (e != cudaSuccess) return e;
+  batch_resident_kernel<<<count, threads, smem, s>>>(circs, ids, round_limit, err);
+  return cudaGetLastError();
+}
+
+}  // namespace qs

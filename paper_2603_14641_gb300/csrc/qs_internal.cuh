@@ -256,4 +256,7 @@ cudaError_t launch_fused_segment(uint64_t *X, uint64_t *Z, uint64_t *S, uint32_t
                                  uint32_t nwords, const uint32_t *packed, const int64_t *lptr,
                                  uint32_t L, uint32_t max_gates, uint32_t *err, cudaStream_t s);
 
+// device record of a simulator (one byte per measurement)
+const uint8_t *sim_record(const qs_sim *sim);
+
 }  // namespace qs

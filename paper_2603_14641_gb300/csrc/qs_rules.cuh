@@ -53,4 +53,11 @@ __device__ __forceinline__ void rule(uint32_t type, uint64_t &xa, uint64_t &za, 
   }
 }
 
+// which words a rule changes: bit t of each mask for gate type t
+constexpr uint32_t kWritesXa = 1u << QS_H | 1u << QS_SWAP | 1u << QS_ISWAP;
+constexpr uint32_t kWritesZa = 1u << QS_H | 1u << QS_S | 1u << QS_SDG | 1u << QS_CX | 1u << QS_CY | 1u << QS_CZ |
+                               1u << QS_SWAP | 1u << QS_ISWAP;
+constexpr uint32_t kWritesXb = 1u << QS_CX | 1u << QS_CY | 1u << QS_SWAP | 1u << QS_ISWAP;
+constexpr uint32_t kWritesZb = 1u << QS_CY | 1u << QS_CZ | 1u << QS_SWAP | 1u << QS_ISWAP;
+
 }  // namespace qs

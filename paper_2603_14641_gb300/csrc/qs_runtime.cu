@@ -276,6 +276,8 @@ int run_dev_layers(qs_sim *s, uint64_t *X, uint64_t *Z, uint64_t *S, uint32_t st
 
 }  // namespace
 
+const uint8_t *qs::sim_record(const qs_sim *sim) { return sim->d.record; }
+
 // device address of the allocation-free sampler's static array on the current
 // device (looked up once per device; defined with the array further below)
 static cudaError_t noalloc_setup(void **addr);
