@@ -14,8 +14,10 @@
 // signs compiled out, evolves the Pauli frames of Sec. 5 (Alg. 9 reuses the
 // gate kernel on frames).
 #include <algorithm>
+#include <vector>
 
 #include "qs_internal.cuh"
+#include "qs_lazy.cuh"
 #include "qs_rules.cuh"
 
 namespace qs {
@@ -240,6 +242,236 @@ cudaError_t launch_frame_layer(uint64_t *FX, uint64_t *FZ, uint32_t n, uint32_t 
   else
     gate_layer_kernel<false, 1><<<g.grid, g.block, 0, s>>>(FX, FZ, nullptr, n, fw, packed, n_gates,
                                                         g.P, g.lanes, g.gpl, err);
+  return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------
+// Layers with deferred one-qubit gates (qs_lazy.cuh), one launch per layer:
+// launch l applies layer l's two-qubit gates with the pending operations of
+// their qubits, and its first blocks turn layer l + 1 into such records (a
+// separate launch for that took as long as the layer itself at 15,000 qubits). After the last layer the operations still pending are listed and
+// applied the same way.
+// At 180,000 qubits (p_cx 0.4) the one-qubit gates are half of a layer's 468,000
+// column accesses; deferred, about 245,000 remain: 3.13 -> 1.71 ms a layer; 30,001 qubits 99 -> 58 us.
+// ---------------------------------------------------------------------
+struct LazyScratch {
+  uint2 *rec0, *rec1;  // records of the layers of even and odd launches
+  uint32_t *count;     // their number: three counters take turns (read, filled, cleared)
+  uint8_t *pend;       // pending operation per qubit
+};
+
+struct LazyArgs {
+  uint64_t *X, *Z, *S;
+  uint32_t cs, n, P, lanes, gx;  // gx: blocks over the layer's gates
+  uint32_t prep_blocks;          // first blocks of the grid: the next layer's records
+  const uint2 *next;             // its gates, or nullptr: list what is pending
+  uint32_t next_gates;
+  uint32_t step;
+  LazyScratch L;
+  uint32_t *err;
+};
+
+constexpr uint32_t kLazyPrepBlocks = 256;
+constexpr int kPrepGates = 2;  // gates per thread and pass, loaded together
+
+// The next layer's records: one-qubit gates compose into their qubit's pending
+// operation, two-qubit gates take both along. One atomic per block and pass.
+__device__ __forceinline__ void lazy_prepare(const LazyArgs &a) {
+  __shared__ uint32_t s_warp[8], s_base;
+  uint2 *rec = a.step & 1 ? a.L.rec0 : a.L.rec1;
+  uint32_t *count = a.L.count + (a.step + 1) % 3;
+  const uint32_t t = threadIdx.x, T = blockDim.x, lane = t & 31, warp = t >> 5, warps = (T + 31) >> 5;
+  const uint32_t items = a.next ? a.next_gates : a.n, pass = T * kPrepGates;
+  for (uint32_t b0 = blockIdx.x * pass; b0 < items; b0 += a.prep_blocks * pass) {
+    // records, then pending operations, then updates: the qubits of a layer are
+    // distinct, but the compiler cannot move a load past a store to pend
+    uint2 in[kPrepGates], out[kPrepGates];
+    uint32_t pa[kPrepGates], pb[kPrepGates], emit = 0;
+    bool ok[kPrepGates];
+#pragma unroll
+    for (int i = 0; i < kPrepGates; ++i) {
+      const uint32_t g = b0 + i * T + t;
+      in[i] = make_uint2(QS_I << 24, 0);
+      if (g < items) in[i] = a.next ? __ldg(a.next + g) : make_uint2(QS_I << 24 | g, 0);
+    }
+#pragma unroll
+    for (int i = 0; i < kPrepGates; ++i) {
+      const uint32_t type = in[i].x >> 24, qa = in[i].x & 0xFFFFFFu, qb = in[i].y;
+      const bool two = is_two_qubit(type);
+      ok[i] = b0 + i * T + t < items;
+      if (ok[i] && (qa >= a.n || type >= QS_NUM_GATE_TYPES || (two && (qb >= a.n || qb == qa)))) {
+        atomicOr(a.err, kErrBadGate);
+        ok[i] = false;
+      }
+      pa[i] = ok[i] ? a.L.pend[qa] : 0;
+      pb[i] = ok[i] && two ? a.L.pend[qb] : 0;
+    }
+#pragma unroll
+    for (int i = 0; i < kPrepGates; ++i) {
+      const uint32_t type = in[i].x >> 24, qa = in[i].x & 0xFFFFFFu, qb = in[i].y;
+      if (!ok[i]) continue;
+      if (is_two_qubit(type)) {
+        out[i] = pair_record(type, qa, qb, pa[i], pb[i]);
+        if (pa[i]) a.L.pend[qa] = 0;
+        if (pb[i]) a.L.pend[qb] = 0;
+        emit |= 1u << i;
+      } else if (!a.next) {  // after the last layer: what is still pending
+        out[i] = single_record(qa, pa[i]);
+        emit |= (uint32_t)(pa[i] != 0) << i;
+      } else if (type != QS_I) {
+        a.L.pend[qa] = (uint8_t)op_then(pa[i], type);
+      }
+    }
+    uint32_t inc = __popc(emit);  // inclusive prefix over the warp
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t y = __shfl_up_sync(__activemask(), inc, d);
+      if (lane >= (uint32_t)d) inc += y;
+    }
+    const uint32_t last = min(31u, T - 1 - 32 * warp);
+    if (lane == last) s_warp[warp] = inc;
+    __syncthreads();
+    if (t == 0) {
+      uint32_t sum = 0;
+      for (uint32_t w = 0; w < warps; ++w) sum += s_warp[w];
+      s_base = sum ? atomicAdd(count, sum) : 0;
+    }
+    __syncthreads();
+    uint32_t at = s_base + inc - __popc(emit);
+    for (uint32_t w = 0; w < warp; ++w) at += s_warp[w];
+#pragma unroll
+    for (int i = 0; i < kPrepGates; ++i)
+      if ((emit >> i) & 1) rec[at++] = out[i];
+    __syncthreads();  // s_warp is rewritten
+  }
+}
+
+// one word of a gate: both qubits' pending operations, then the gate
+__device__ __forceinline__ void lazy_word(uint32_t type, uint32_t opa, uint32_t opb, unsigned long long &xa_,
+                                          unsigned long long &za_, unsigned long long &xb_, unsigned long long &zb_,
+                                          unsigned long long &s_) {
+  uint64_t xa = xa_, za = za_, xb = xb_, zb = zb_, s = s_;
+  if (opa) op_apply<true>(OpMasks(opa), xa, za, s);
+  if (opb) op_apply<true>(OpMasks(opb), xb, zb, s);
+  if (type) rule<true>(type, xa, za, xb, zb, s);
+  xa_ = xa; za_ = za; xb_ = xb; zb_ = zb; s_ = s;
+}
+
+// As gate_layer_kernel, two gates in flight a thread; the layer's gates are
+// split evenly over gx blocks (their number is known on the device only).
+__global__ void __launch_bounds__(256, 4) lazy_layer_kernel(const LazyArgs a) {
+  if (blockIdx.x < a.prep_blocks) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.L.count[(a.step + 2) % 3] = 0;
+    lazy_prepare(a);
+    return;
+  }
+  const uint32_t n_gates = a.L.count[a.step % 3];
+  const uint2 *recs = a.step & 1 ? a.L.rec1 : a.L.rec0;
+  const uint32_t blk = blockIdx.x - a.prep_blocks, bx = blk % a.gx, by = blk / a.gx;
+  const uint32_t t = threadIdx.x, lanes = a.lanes, lane = t / a.P, pair = by * a.P + (t - lane * a.P), cs = a.cs;
+  uint64_t *X = a.X, *Z = a.Z;
+  const bool active = pair < cs >> 1;
+  const uint32_t slots = (n_gates + lanes - 1) / lanes, per = (slots + a.gx - 1) / a.gx * lanes;
+  const uint32_t g0 = min(n_gates, bx * per), g1 = min(n_gates, g0 + per);
+  ulonglong2 sacc = make_ulonglong2(0, 0);
+  if (active) {
+    const size_t off = 2 * (size_t)pair;
+    for (uint32_t g = g0 + lane; g < g1; g += 2 * lanes) {
+      uint2 rec[2];
+      ulonglong2 xa[2], za[2], xb[2], zb[2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+        if (g + u * lanes < g1) {
+          rec[u] = recs[g + u * lanes];
+          const size_t oa = (size_t)(rec[u].x & 0xFFFFFu) * cs + off;
+          xa[u] = ld2(X + oa);
+          za[u] = ld2(Z + oa);
+          if ((rec[u].x >> 20) & 15) {
+            const size_t ob = (size_t)(rec[u].y & 0xFFFFFu) * cs + off;
+            xb[u] = ld2(X + ob);
+            zb[u] = ld2(Z + ob);
+          }
+        }
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+        if (g + u * lanes < g1) {
+          const uint32_t type = (rec[u].x >> 20) & 15, opa = rec[u].x >> 24, opb = rec[u].y >> 24;
+          lazy_word(type, opa, opb, xa[u].x, za[u].x, xb[u].x, zb[u].x, sacc.x);
+          lazy_word(type, opa, opb, xa[u].y, za[u].y, xb[u].y, zb[u].y, sacc.y);
+          const size_t oa = (size_t)(rec[u].x & 0xFFFFFu) * cs + off;
+          if (((kWritesXa >> type) & 1) || op_changes_x(opa)) st2(X + oa, xa[u]);
+          if (((kWritesZa >> type) & 1) || op_changes_z(opa)) st2(Z + oa, za[u]);
+          if (type) {
+            const size_t ob = (size_t)(rec[u].y & 0xFFFFFu) * cs + off;
+            if (((kWritesXb >> type) & 1) || op_changes_x(opb)) st2(X + ob, xb[u]);
+            if (((kWritesZb >> type) & 1) || op_changes_z(opb)) st2(Z + ob, zb[u]);
+          }
+        }
+    }
+  }
+  if (lanes > 1) {
+    __shared__ ulonglong2 red[256];
+    red[t] = sacc;
+    __syncthreads();
+    if (t < a.P)
+      for (uint32_t l = 1; l < lanes; ++l) {
+        const ulonglong2 v = red[l * a.P + t];
+        sacc.x ^= v.x; sacc.y ^= v.y;
+      }
+  }
+  if (active && lane == 0) {
+    if (sacc.x) atomicXor(reinterpret_cast<unsigned long long *>(a.S + 2 * (size_t)pair), sacc.x);
+    if (sacc.y) atomicXor(reinterpret_cast<unsigned long long *>(a.S + 2 * (size_t)pair + 1), sacc.y);
+  }
+}
+
+// n records each: the list of pending operations may hold every qubit
+size_t lazy_scratch_bytes(uint32_t n) { return 256 + 2 * (size_t)n * 8 + n; }
+
+cudaError_t launch_lazy_layers(const Dev &d, void *scratch, const uint32_t *packed, const int64_t *ptr, size_t nlayers,
+                               cudaStream_t s, int *launches) {
+  const uint32_t n = d.L.n, npairs = d.L.cs / 2;
+  uint8_t *p = static_cast<uint8_t *>(scratch);
+  LazyArgs a{};
+  a.X = d.X; a.Z = d.Z; a.S = d.S; a.cs = d.L.cs; a.n = n; a.err = d.err;
+  a.L.count = reinterpret_cast<uint32_t *>(p);
+  a.L.rec0 = reinterpret_cast<uint2 *>(p + 256);
+  a.L.rec1 = a.L.rec0 + n;
+  a.L.pend = p + 256 + 2 * (size_t)n * 8;
+  cudaError_t e = cudaMemsetAsync(a.L.count, 0, 12, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(a.L.pend, 0, n, s);
+  if (e != cudaSuccess) return e;
+  std::vector<size_t> todo;  // nonempty layers
+  for (size_t l = 0; l < nlayers; ++l)
+    if (ptr[l + 1] > ptr[l]) todo.push_back(l);
+  uint64_t gates = 0;  // at most so many records in the launch's layer
+  // launch i: layer i - 1 applied (the list of pending operations at the end), layer i prepared
+  for (size_t i = 0; i <= todo.size() + 1; ++i) {
+    a.step = (uint32_t)i;
+    uint64_t next = 0;
+    a.next = nullptr;
+    if (i < todo.size()) {
+      next = (uint64_t)(ptr[todo[i] + 1] - ptr[todo[i]]);
+      a.next = reinterpret_cast<const uint2 *>(packed) + ptr[todo[i]];
+    } else if (i == todo.size()) {
+      next = n;
+    }
+    a.next_gates = (uint32_t)next;
+    const GateGrid g = gate_grid(npairs, (uint32_t)std::max<uint64_t>(gates, 1));
+    const uint32_t threads = g.block.x;
+    a.P = g.P;
+    a.lanes = g.lanes;
+    // one wave of the four resident blocks per SM, eight at the largest sizes:
+    // 20,000 qubits 31.4 us a layer (two waves 35.1), 60,000 210 (212), 180,000
+    // 1,732 (eight waves 1,710)
+    const uint32_t chunks = g.grid.y;
+    const uint64_t wave = 4ull * d.sms, blocks_x = (gates * chunks > 1024 * wave ? 8 : 1) * wave / chunks;
+    a.gx = i ? (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(blocks_x, (gates + g.lanes - 1) / g.lanes)) : 0;
+    a.prep_blocks = (uint32_t)std::min<uint64_t>(kLazyPrepBlocks, (next + threads * kPrepGates - 1) / (threads * kPrepGates));
+    const uint32_t blocks = a.prep_blocks + a.gx * chunks;
+    if (blocks) lazy_layer_kernel<<<blocks, threads, 0, s>>>(a);
+    gates = i < todo.size() ? std::min<uint64_t>(next, std::max(1u, n / 2)) : n;
+  }
+  if (launches) *launches += (int)todo.size() + 2;
   return cudaGetLastError();
 }
 

@@ -207,6 +207,12 @@ struct Dev {
 cudaError_t launch_init(const Dev &d, const uint8_t *initstate_dev, cudaStream_t s);
 cudaError_t launch_gate_layer(const Dev &d, const uint32_t *packed, uint32_t n_gates,
                               cudaStream_t s);
+// layers ptr[0..nlayers] of `packed` on the tableau with one-qubit gates deferred
+// to the next two-qubit gate of their qubit (qs_lazy.cuh), nothing pending after;
+// scratch: lazy_scratch_bytes(n)
+size_t lazy_scratch_bytes(uint32_t n);
+cudaError_t launch_lazy_layers(const Dev &d, void *scratch, const uint32_t *packed, const int64_t *ptr, size_t nlayers,
+                               cudaStream_t s, int *launches);
 // frames: column-major frame matrices FX/FZ [n][fw] words (fw multiple of 2)
 cudaError_t launch_frame_layer(uint64_t *FX, uint64_t *FZ, uint32_t n, uint32_t fw,
                                const uint32_t *packed, uint32_t n_gates, uint32_t *err,

@@ -58,6 +58,7 @@ struct Op {
 constexpr int kRing = 4;
 constexpr uint32_t kBlockedMinCount = 16;    // windows this long use blocked measurement
 constexpr uint32_t kBlockedMinQubits = 64;
+constexpr size_t kLazyMinLayers = 2;         // runs of layers this long defer their one-qubit gates
 constexpr uint32_t kMaxQubits = 1u << 20;
 // Frame layers cover a qubit's shot words in chunks of 512 words along grid.y
 // (at most 65,535): 2e9 shots are 31.25 M words, 61,036 chunks.
@@ -257,6 +258,14 @@ int run_dev_layers(qs_sim *s, uint64_t *X, uint64_t *Z, uint64_t *S, uint32_t st
                                       (uint32_t)max_gates, s->d.err, s->stream));
       s->launches += 1;
     }
+    return QS_OK;
+  }
+  if (tableau && !s->d.inverse && nlayers >= kLazyMinLayers) {
+    // the row-major tableau, stale from here on, is the scratch
+    s->rows_valid = false;
+    int l = 0;
+    QS_CUDA(s, launch_lazy_layers(s->d, s->d.RX, packed, ptr, nlayers, s->stream, &l));
+    s->launches += (uint64_t)l;
     return QS_OK;
   }
   for (size_t l = 0; l < nlayers; ++l) {

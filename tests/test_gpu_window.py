@@ -73,3 +73,29 @@ def test_apply_variants_match_single_measurements(n, flags):
         sim.sync()
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("n,layers", [(1, 3), (5, 2), (64, 9), (130, 7), (700, 6), (14081, 5)])
+def test_deferred_gates_match_layer_by_layer(n, layers):
+    """A run of layers defers its one-qubit gates to the next two-qubit gate of their qubit; one layer
+    per call applies each in its own layer. All 11 gates, an empty layer and a layer of identities."""
+    c = C.gate_mix_circuit(n, layers, seed=n, final_measure_all=False)
+    ident = np.array([[C.I, q, 0] for q in range(min(n, 3))], np.uint32)
+    lp = c.layer_ptr
+    gates = np.concatenate([c.gates[:lp[1]], ident, c.gates[lp[1]:]])
+    lp = np.concatenate([lp[:2], lp[1:2], [lp[1] + len(ident)], lp[2:] + len(ident)])
+    c = C.Circuit(n=n, gates=np.ascontiguousarray(gates), layer_ptr=lp, ops=[])
+    out = []
+    for together in (True, False):
+        sim = qs.Simulator(n, flags=qs.QS_FLAG_NO_FUSION)
+        sim.reset(np.arange(n) % 3 == 1)
+        dc = sim.upload(c)
+        for l in range(1 if together else c.n_layers):
+            sim.apply_layers_dev(dc, l, c.n_layers if together else l + 1)
+        out.append(qs.qs_sim_tableau_export(sim.sim))
+        sim.sync()
+    assert np.array_equal(*out)
+    if n <= 130:
+        o = O.Oracle(n, (np.arange(n) % 3 == 1).astype(np.uint8))
+        o.apply(c.gates)
+        assert all(np.array_equal(a, b) for a, b in zip(qs.unpack_rows(out[0], n), o.get()))
