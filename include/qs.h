@@ -75,9 +75,9 @@ typedef struct qs_options {
   uint32_t reserved;
 } qs_options;
 
-/* qs_options.flags: apply every device-resident layer with its own kernel
- * instead of fusing a run of layers into one shared-memory pass (the fused
- * pass is used for n <= 14,080; results are identical either way). */
+/* qs_options.flags: never fuse a run of device-resident layers into one
+ * shared-memory pass (used for runs of 4 layers and more on n <= 14,080
+ * qubits; results are identical either way). */
 #define QS_FLAG_NO_FUSION 1u
 /* qs_options.flags: run every measurement as five separate launches (gather,
  * rowsum, deterministic partials, combine, finalize) instead of the pipelined

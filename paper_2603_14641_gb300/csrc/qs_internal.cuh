@@ -254,14 +254,16 @@ cudaError_t launch_measure_window(const Dev &d, const uint32_t *qubits, uint32_t
 size_t blocked_scratch_bytes(const Layout &L);
 cudaError_t launch_measure_blocks(const Dev &d, void *scratch, const uint32_t *window, uint32_t count, uint64_t m0,
                                   qs_key key, cudaStream_t s, int *launches);
-// fused segment of L layers on a word-sliced, shared-memory-resident tableau
-// (S == nullptr: frames, no signs); lptr: L + 1 device gate offsets
+// fused segment of L <= kFusedLayers layers on a word-sliced, shared-memory-resident
+// tableau (S == nullptr: frames, no signs), one-qubit gates deferred; nwords: the
+// words of a column that matter; lptr: L + 1 device gate offsets; max_gates: the
+// largest layer's gates; scratch: fused_scratch_bytes(n)
+constexpr uint32_t kFusedLayers = 128;
 bool fused_fits(uint32_t n);
-// max_gates: the largest layer of the segment (gates)
-cudaError_t launch_fused_segment(uint64_t *X, uint64_t *Z, uint64_t *S, uint32_t n, uint32_t stride,
-                                 uint32_t nwords, const uint32_t *packed, const int64_t *lptr,
-                                 uint32_t L, uint32_t max_gates, uint32_t *err, cudaStream_t s);
-
+size_t fused_scratch_bytes(uint32_t n);
+cudaError_t launch_fused_segment(uint64_t *X, uint64_t *Z, uint64_t *S, uint32_t n, uint32_t stride, uint32_t nwords,
+                                 const uint32_t *packed, const int64_t *lptr, uint32_t L, uint32_t max_gates, int sms,
+                                 void *scratch, uint32_t *err, cudaStream_t s);
 // device record of a simulator (one byte per measurement)
 const uint8_t *sim_record(const qs_sim *sim);
 

@@ -44,6 +44,27 @@ __host__ __device__ __forceinline__ uint32_t op_then(uint32_t op, uint32_t type)
   return (m0 ^ 1) | m1 << 1 | m2 << 2 | (m3 ^ 1) << 3 | a << 4 | b << 5 | c << 6;
 }
 
+// the one-qubit gate `type` followed by operation `op`
+__host__ __device__ __forceinline__ uint32_t op_after(uint32_t type, uint32_t op) {
+  uint32_t m0 = (op & 1) ^ 1, m1 = (op >> 1) & 1, m2 = (op >> 2) & 1, m3 = ((op >> 3) & 1) ^ 1;
+  uint32_t a = (op >> 4) & 1, b = (op >> 5) & 1, c = (op >> 6) & 1;
+  if (type == QS_H) {  // (x, z) -> (z, x), s += x z
+    uint32_t t = m0; m0 = m1; m1 = t;
+    t = m2; m2 = m3; m3 = t;
+    t = a; a = b; b = t;
+    c ^= 1;
+  } else if (type == QS_S || type == QS_SDG) {  // z -> x + z, s += x z, for S^dag + x; x (x + z) = x + x z
+    m0 ^= m1;
+    m2 ^= m3;
+    a ^= b ^ c ^ (type == QS_SDG);
+    c ^= 1;
+  } else {
+    a ^= type == QS_Z || type == QS_Y;  // s += x
+    b ^= type == QS_X || type == QS_Y;  // s += z
+  }
+  return (m0 ^ 1) | m1 << 1 | m2 << 2 | (m3 ^ 1) << 3 | a << 4 | b << 5 | c << 6;
+}
+
 // whether the operation changes the x (z) word
 __device__ __forceinline__ bool op_changes_x(uint32_t op) { return op & (kOpM0 | kOpM1); }
 __device__ __forceinline__ bool op_changes_z(uint32_t op) { return op & (kOpM2 | kOpM3); }
@@ -58,13 +79,14 @@ struct OpMasks {
   }
 };
 
-__device__ __forceinline__ uint64_t both(uint32_t m) { return ((uint64_t)m << 32) | m; }
+__device__ __forceinline__ uint32_t widen(uint32_t m, uint32_t) { return m; }
+__device__ __forceinline__ uint64_t widen(uint32_t m, uint64_t) { return ((uint64_t)m << 32) | m; }
 
-template <bool SIGNS>
-__device__ __forceinline__ void op_apply(const OpMasks &o, uint64_t &x, uint64_t &z, uint64_t &s) {
-  if (SIGNS) s ^= (x & ((z & both(o.c)) ^ both(o.a))) ^ (z & both(o.b));
-  const uint64_t nx = (x & both(o.m0)) ^ (z & both(o.m1));
-  z = (x & both(o.m2)) ^ (z & both(o.m3));
+template <bool SIGNS, typename W>
+__device__ __forceinline__ void op_apply(const OpMasks &o, W &x, W &z, W &s) {
+  if (SIGNS) s ^= (x & ((z & widen(o.c, x)) ^ widen(o.a, x))) ^ (z & widen(o.b, x));
+  const W nx = (x & widen(o.m0, x)) ^ (z & widen(o.m1, x));
+  z = (x & widen(o.m2, x)) ^ (z & widen(o.m3, x));
   x = nx;
 }
 

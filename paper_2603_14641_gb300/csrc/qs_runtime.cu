@@ -58,6 +58,7 @@ struct Op {
 constexpr int kRing = 4;
 constexpr uint32_t kBlockedMinCount = 16;    // windows this long use blocked measurement
 constexpr uint32_t kBlockedMinQubits = 64;
+constexpr size_t kFusedMinLayers = 4;        // shorter runs of layers take a launch each
 constexpr size_t kLazyMinLayers = 2;         // runs of layers this long defer their one-qubit gates
 constexpr uint32_t kMaxQubits = 1u << 20;
 // Frame layers cover a qubit's shot words in chunks of 512 words along grid.y
@@ -74,7 +75,7 @@ struct Carve {
 };
 
 struct Plan {
-  size_t X, Z, RX, RZ, S, colx, mst, detx, detz, dets, err, record, kinds, stage, blk, qsig, invp, total;
+  size_t X, Z, RX, RZ, S, colx, mst, detx, detz, dets, err, record, kinds, stage, blk, fused, qsig, invp, total;
   uint64_t record_cap;
   size_t stage_bytes;
 };
@@ -100,6 +101,7 @@ Plan make_plan(const Layout &L, const qs_options *opt) {
   p.kinds = c.take(p.record_cap);
   p.stage = c.take(p.stage_bytes);
   p.blk = c.take(blocked_scratch_bytes(L));
+  p.fused = c.take(fused_scratch_bytes(L.n));
   const bool inverse = opt && (opt->flags & QS_FLAG_INVERSE_TABLEAU);
   p.qsig = c.take(inverse ? 2ull * L.rs * 8 : 0);
   p.invp = c.take(inverse ? inv_scratch_words(L) * 8 : 0);
@@ -131,7 +133,8 @@ struct qs_sim {
   uint32_t stamp_id = 0;
   uint64_t launches = 0;
   uint32_t flags = 0;
-  void *blk = nullptr;  // scratch of the blocked measurement
+  void *blk = nullptr;    // scratch of the blocked measurement
+  void *fused = nullptr;  // scratch of the fused gate segments
   bool resumed = false; // state restored by qs_sim_tableau_import: no op log from |0...0>
   std::unique_ptr<KernelTimer> timer;  // qs_sim_set_timing
   // every noise op's targets, uploaded once for qs_sim_sample's replays (valid
@@ -233,18 +236,19 @@ int validate_pack(uint32_t n, const qs_gate *g, size_t count, std::vector<uint32
   return QS_OK;
 }
 
-// Enqueues layers [0, ptr.size() - 1) given by absolute gate offsets `ptr`
-// of device gate records `packed` on the tableau (S != nullptr) or on frames.
-// Runs of layers go through the fused shared-memory kernel when the word slice
-// fits, else one kernel per layer.
-int run_dev_layers(qs_sim *s, uint64_t *X, uint64_t *Z, uint64_t *S, uint32_t stride,
+// Enqueues layers [0, nlayers) given by absolute gate offsets `ptr` of device
+// gate records `packed` on the tableau (S != nullptr) or on frames. Runs of
+// layers go through the fused shared-memory kernels when a word slice fits (or,
+// on larger tableaus, with one-qubit gates deferred), else one kernel per layer.
+// nwords: the words of a column that matter (the rest is padding).
+int run_dev_layers(qs_sim *s, uint64_t *X, uint64_t *Z, uint64_t *S, uint32_t stride, uint32_t nwords,
                    const uint32_t *packed, const int64_t *ptr, size_t nlayers, bool tableau) {
   const uint32_t n = s->d.L.n;
   if (nlayers == 0) return QS_OK;
-  if (fused_fits(n) && !(s->flags & QS_FLAG_NO_FUSION) && !(tableau && s->d.inverse)) {
-    const size_t cap = s->plan.stage_bytes / 8 - 1;  // layers per staged offset table
-    for (size_t l0 = 0; l0 < nlayers; l0 += cap) {
-      const size_t L = std::min(cap, nlayers - l0);
+  if (nlayers >= kFusedMinLayers && fused_fits(n) && !(s->flags & QS_FLAG_NO_FUSION) && !(tableau && s->d.inverse)) {
+    // the staged offset table holds at least kFusedLayers + 1 entries
+    for (size_t l0 = 0; l0 < nlayers; l0 += kFusedLayers) {
+      const size_t L = std::min<size_t>(kFusedLayers, nlayers - l0);
       int slot;
       uint8_t *h = ring_slot(s, &slot);
       if (!h) return cuda_fail(s, cudaGetLastError(), "staging event");
@@ -253,14 +257,14 @@ int run_dev_layers(qs_sim *s, uint64_t *X, uint64_t *Z, uint64_t *S, uint32_t st
       if (rc) return rc;
       int64_t max_gates = 0;  // layers hold at most n gates (checked when they were added)
       for (size_t l = l0; l < l0 + L; ++l) max_gates = std::max<int64_t>(max_gates, ptr[l + 1] - ptr[l]);
-      QS_CUDA(s, launch_fused_segment(X, Z, S, n, stride, stride, packed,
+      QS_CUDA(s, launch_fused_segment(X, Z, S, n, stride, nwords, packed,
                                       reinterpret_cast<const int64_t *>(s->dstage), (uint32_t)L,
-                                      (uint32_t)max_gates, s->d.err, s->stream));
-      s->launches += 1;
+                                      (uint32_t)max_gates, s->d.sms, s->fused, s->d.err, s->stream));
+      s->launches += 3;
     }
     return QS_OK;
   }
-  if (tableau && !s->d.inverse && nlayers >= kLazyMinLayers) {
+  if (tableau && !s->d.inverse && nlayers >= kLazyMinLayers && (!fused_fits(n) || (s->flags & QS_FLAG_NO_FUSION))) {
     // the row-major tableau, stale from here on, is the scratch
     s->rows_valid = false;
     int l = 0;
@@ -352,6 +356,7 @@ int qs_sim_create(uint32_t n, const qs_options *opt, void *cuda_stream, void *wo
   s->d.record_cap = p.record_cap;
   s->dstage = b + p.stage;
   s->blk = b + p.blk;
+  s->fused = b + p.fused;
   s->d.qsig = s->d.inverse ? reinterpret_cast<uint64_t *>(b + p.qsig) : nullptr;
   s->d.inv_part = s->d.inverse ? reinterpret_cast<uint64_t *>(b + p.invp) : nullptr;
   int dev = 0;
@@ -503,7 +508,7 @@ int qs_sim_apply_layers_dev(qs_sim *s, const uint32_t *packed_dev, const int64_t
     if (cnt < 0 || cnt > (int64_t)s->d.L.n) return fail(QS_ERR_ARG, "bad layer_ptr");
   }
   tbegin(s->d.timer, QS_TIME_GATES, s->stream);
-  if ((rc = run_dev_layers(s, s->d.X, s->d.Z, s->d.S, s->d.L.cs, packed_dev, op.ptr.data(),
+  if ((rc = run_dev_layers(s, s->d.X, s->d.Z, s->d.S, s->d.L.cs, 2 * s->d.L.k, packed_dev, op.ptr.data(),
                            op.ptr.size() - 1, true)))
     return rc;
   tend(s->d.timer, QS_TIME_GATES, s->stream);
@@ -869,7 +874,7 @@ int qs_sim_sample(qs_sim *s, uint64_t shots, uint64_t seed, uint64_t *record, si
                                     (uint32_t)(op.packed.size() / 2), s->d.err, s->stream));
       s->launches += 1;
     } else if (op.kind == Op::kDevLayers) {
-      if ((rc = run_dev_layers(s, FX, FZ, nullptr, (uint32_t)fw, op.dev, op.ptr.data(),
+      if ((rc = run_dev_layers(s, FX, FZ, nullptr, (uint32_t)fw, (uint32_t)ow, op.dev, op.ptr.data(),
                                op.ptr.size() - 1, false)))
         return rc;
     } else if (op.kind == Op::kNoise) {
