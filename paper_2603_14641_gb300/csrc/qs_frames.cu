@@ -95,89 +95,221 @@ cudaError_t launch_frame_measure(uint64_t *FX, uint64_t *FZ, uint32_t n, uint32_
 }
 
 // Pauli noise channels on the frames (X_ERROR, Y_ERROR, Z_ERROR, DEPOLARIZE1,
-// DEPOLARIZE2; frames carry error events, Sec. 3). One thread per (target,
-// shot word j). The 64 shots' 32-bit draws u are bit-sliced: bit 31 - k of
-// every shot's u sits in random word W_k, so u < thr is decided for all 64
-// shots at once from the most significant bit down, and the loop stops as
-// soon as no shot is undecided (about 8 words on average instead of 32).
-// The fire mask applies X/Y/Z directly; only the shots that fired draw the
-// Pauli of a depolarising channel. Targets of one op are distinct, so every
-// frame word has one writer.
-__device__ __forceinline__ uint64_t noise_v(uint64_t e, uint64_t i, uint64_t s, uint64_t seed) {
-  return philox4x64_10(e, i, s, 4, seed, kNoiseKey).v[0];
-}
-__device__ __forceinline__ void add_pauli(int code, uint64_t bit, uint64_t &mx, uint64_t &mz) {
-  if (code == 1 || code == 2) mx |= bit;
-  if (code == 2 || code == 3) mz |= bit;
+// DEPOLARIZE2; frames carry error events, Sec. 3). An item is a (target, shot
+// word j). The 64 shots' 32-bit draws u are bit-sliced: bit 31 - k of every
+// shot's u sits in random word W_k, so u < thr is decided for all 64 shots at
+// once from the most significant bit down, four words (one Philox block) at a
+// time, and stops as soon as no shot is undecided. The fire mask applies X/Y/Z
+// directly; only the shots that fired draw the Pauli of a depolarising channel.
+// Targets of one op are distinct, so every frame word has one writer.
+//
+// What bounds it is Philox, and what it wastes is lanes: after two blocks (8
+// bits) 22 % of the items are undecided and at p = 1e-3 6 % have a shot that
+// fired, but nearly every warp has such an item, so warps ran 4.4 blocks per
+// item where 2.3 are needed. A block therefore takes 256 items through the first
+// two Philox blocks and then deals the undecided ones, and the shots that fired,
+// densely over its threads. (Passing in the first two rounds' uniform products
+// and the round keys from the host measured slower, as did a four-product 64 x 64
+// multiply in place of __umul64hi and the low product.) One launch takes up to
+// kNoiseGroupMax consecutive ops on distinct qubits (the depolarising ops after
+// one layer), so that their latencies overlap. 1,667 + 1,250 targets and 16,384
+// shots at p = 1e-3: 49 -> 35 us.
+
+// words of Philox(ctr = (e, i, ctr, tag), key)
+__device__ __forceinline__ P4 noise_philox(uint64_t e, uint64_t seed, uint32_t i, uint32_t ctr, int tag) {
+  return philox4x64_10(e, i, ctr, tag, seed, kNoiseKey);
 }
 
-__global__ void __launch_bounds__(256)
-frame_noise_kernel(uint64_t *__restrict__ FX, uint64_t *__restrict__ FZ, uint32_t fw, uint32_t ow,
-                   const uint32_t *__restrict__ targets, uint32_t count, uint32_t i0, int kind,
-                   uint64_t thr, uint64_t e, uint64_t seed) {
-  const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (tid >= (uint64_t)count * ow) return;
-  const uint32_t i = (uint32_t)(tid / ow), j = (uint32_t)(tid % ow);
-  const uint64_t gi = (uint64_t)i0 + i;
-  uint64_t fire = 0;
-  if (thr >> 32) {
-    fire = ~0ull;  // p >= 1
-  } else {
-    uint64_t undecided = ~0ull;
-    for (int t = 0; t < 8 && undecided; ++t) {
-      const P4 r = philox4x64_10(e, gi, 8ull * j + t, 3, seed, kNoiseKey);
+constexpr int kNoiseThreads = 128, kNoiseItems = 2 * kNoiseThreads;  // items per block
+
+// one more Philox block of an item's draws: 4 bits of u from bit 31 - 4 t down
+__device__ __forceinline__ void noise_bits(uint64_t e, uint64_t seed, uint32_t thr, uint32_t i, uint32_t j, int t,
+                                           uint64_t &fire, uint64_t &undecided) {
+  const P4 r = noise_philox(e, seed, i, 8 * j + t, 3);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const uint64_t w = r.v[q];  // bit 31 - (4 t + q) of every shot's u
-        if ((thr >> (31 - (4 * t + q))) & 1u) {
-          fire |= undecided & ~w;  // u has 0 where thr has 1: u < thr
-          undecided &= w;
-        } else {
-          undecided &= ~w;  // u has 1 where thr has 0: u > thr
-        }
-      }
+  for (int q = 0; q < 4; ++q) {
+    const uint64_t w = r.v[q];
+    if ((thr >> (31 - (4 * t + q))) & 1u) {
+      fire |= undecided & ~w;  // u has 0 where thr has 1: u < thr
+      undecided &= w;
+    } else {
+      undecided &= ~w;  // u has 1 where thr has 0: u > thr
     }
-    // shots still undecided after 32 bits have u == thr: no fire
-  }
-  if (!fire) return;
-  uint64_t ax = 0, az = 0, bx = 0, bz = 0;
-  if (kind == QS_NOISE_X) ax = fire;
-  else if (kind == QS_NOISE_Y) ax = az = fire;
-  else if (kind == QS_NOISE_Z) az = fire;
-  else {
-    uint64_t m = fire;
-    while (m) {
-      const int b = __ffsll((long long)m) - 1;
-      m &= m - 1;
-      const uint64_t v = noise_v(e, gi, 64ull * j + b, seed), bit = 1ull << b;
-      if (kind == QS_NOISE_DEPOLARIZE1) {
-        add_pauli(1 + (int)__umul64hi(v, 3), bit, ax, az);
-      } else {
-        const int idx = 1 + (int)__umul64hi(v, 15);
-        add_pauli(idx >> 2, bit, ax, az);
-        add_pauli(idx & 3, bit, bx, bz);
-      }
-    }
-  }
-  const uint64_t qa = kind == QS_NOISE_DEPOLARIZE2 ? targets[2 * i] : targets[i];
-  if (ax) FX[qa * fw + j] ^= ax;
-  if (az) FZ[qa * fw + j] ^= az;
-  if (kind == QS_NOISE_DEPOLARIZE2) {
-    const uint64_t qb = targets[2 * i + 1];
-    if (bx) FX[qb * fw + j] ^= bx;
-    if (bz) FZ[qb * fw + j] ^= bz;
   }
 }
 
-cudaError_t launch_frame_noise(uint64_t *FX, uint64_t *FZ, uint32_t fw, uint32_t ow,
-                               const uint32_t *targets, uint32_t count, uint32_t i0, int kind,
-                               uint64_t thr, uint64_t e, uint64_t seed, cudaStream_t s) {
-  if (count == 0 || ow == 0 || thr == 0) return cudaSuccess;  // never fires
-  const uint64_t threads = (uint64_t)count * ow;
-  const uint64_t blocks = (threads + 255) / 256;
-  if (blocks > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
-  frame_noise_kernel<<<(unsigned)blocks, 256, 0, s>>>(FX, FZ, fw, ow, targets, count, i0, kind, thr,
-                                                      e, seed);
+// one op of a launch; its blocks follow those of the ops before it
+struct NoiseLaunch {
+  const uint32_t *targets;
+  uint64_t items, thr, e;
+  uint32_t i0, first_block;
+  int kind;
+};
+struct NoiseGroup {
+  NoiseLaunch op[kNoiseGroupMax];
+  uint64_t seed;
+  int ops;
+};
+
+__global__ void __launch_bounds__(kNoiseThreads)
+frame_noise_kernel(uint64_t *__restrict__ FX, uint64_t *__restrict__ FZ, uint32_t fw, uint32_t ow,
+                   const __grid_constant__ NoiseGroup G) {
+  int o = 0;
+  while (o + 1 < G.ops && blockIdx.x >= G.op[o + 1].first_block) ++o;
+  const uint32_t *targets = G.op[o].targets;
+  const uint64_t items = G.op[o].items, thr = G.op[o].thr;
+  const uint32_t i0 = G.op[o].i0, blk = blockIdx.x - G.op[o].first_block;
+  const int kind = G.op[o].kind;
+  const uint64_t e = G.op[o].e, seed = G.seed;
+  __shared__ uint64_t s_fire[kNoiseItems], s_und[kNoiseItems];
+  __shared__ __align__(16) uint32_t s_pauli[kNoiseItems][8];  // x, z of the first and second target, as halves
+  __shared__ uint32_t s_first[kNoiseItems];     // draws before an item
+  __shared__ uint16_t s_queue[kNoiseItems];
+  __shared__ uint32_t s_n, s_warp[kNoiseThreads / 32], s_draws;
+  const uint32_t t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const uint64_t base = (uint64_t)blk * kNoiseItems;
+  const uint32_t n = (uint32_t)(items - base < kNoiseItems ? items - base : kNoiseItems);
+  const uint32_t b_i = (uint32_t)(base / ow), b_j = (uint32_t)(base % ow);  // uniform
+  // item x of the block: target index and shot word (x < 256: one 32-bit division)
+  auto place = [&](uint32_t x, uint32_t &i, uint32_t &j) {
+    const uint32_t d = (b_j + x) / ow;
+    i = b_i + d;
+    j = b_j + x - d * ow;
+  };
+  const bool draws = kind == QS_NOISE_DEPOLARIZE1 || kind == QS_NOISE_DEPOLARIZE2;
+  if (t == 0) s_n = 0;
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < kNoiseItems / kNoiseThreads; ++u) {
+    const uint32_t x = u * kNoiseThreads + t;
+    uint64_t fire = 0, und = 0;
+    if (x < n) {
+      if (thr >> 32) {
+        fire = ~0ull;  // p >= 1
+      } else {
+        uint32_t i, j;
+        place(x, i, j);
+        und = ~0ull;
+        noise_bits(e, seed, (uint32_t)thr, i0 + i, j, 0, fire, und);
+        noise_bits(e, seed, (uint32_t)thr, i0 + i, j, 1, fire, und);
+      }
+    }
+    s_fire[x] = fire;
+    s_und[x] = und;
+    const uint32_t ball = __ballot_sync(0xffffffffu, und != 0);
+    uint32_t at = 0;
+    if (lane == 0 && ball) at = atomicAdd(&s_n, (uint32_t)__popc(ball));
+    at = __shfl_sync(0xffffffffu, at, 0);
+    if (und) s_queue[at + __popc(ball & ((1u << lane) - 1))] = (uint16_t)x;
+  }
+  __syncthreads();
+  for (uint32_t k = t; k < s_n; k += kNoiseThreads) {
+    const uint32_t x = s_queue[k];
+    uint32_t i, j;
+    place(x, i, j);
+    uint64_t fire = s_fire[x], und = s_und[x];
+    for (int b = 2; b < 8 && und; ++b) noise_bits(e, seed, (uint32_t)thr, i0 + i, j, b, fire, und);
+    s_fire[x] = fire;  // shots still undecided after 32 bits have u == thr: no fire
+  }
+  __syncthreads();
+  if (draws) {
+    // the shots that fired, numbered through the block's items
+    const uint32_t f0 = __popcll(s_fire[2 * t]), f1 = __popcll(s_fire[2 * t + 1]);
+    uint32_t inc = f0 + f1;
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, inc, d);
+      if (lane >= (uint32_t)d) inc += y;
+    }
+    if (lane == 31) s_warp[warp] = inc;
+    __syncthreads();
+    uint32_t before = inc - f0 - f1, total = 0;
+    for (uint32_t w = 0; w < kNoiseThreads / 32; ++w) {
+      if (w < warp) before += s_warp[w];
+      total += s_warp[w];
+    }
+    s_first[2 * t] = before;
+    s_first[2 * t + 1] = before + f0;
+    if (t == 0) s_draws = total;
+    for (uint32_t k = t; k < kNoiseItems * 8; k += kNoiseThreads) s_pauli[k >> 3][k & 7] = 0;
+    __syncthreads();
+    total = s_draws;
+    for (uint32_t k = t; k < total; k += kNoiseThreads) {
+      uint32_t lo = 0, hi = kNoiseItems;  // last item with first <= k
+      while (hi - lo > 1) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (s_first[mid] <= k) lo = mid; else hi = mid;
+      }
+      uint64_t m = s_fire[lo];
+      for (uint32_t skip = k - s_first[lo]; skip; --skip) m &= m - 1;
+      const uint32_t b = (uint32_t)__ffsll((long long)m) - 1;
+      uint32_t i, j;
+      place(lo, i, j);
+      const uint64_t v = noise_philox(e, seed, i0 + i, 64 * j + b, 4).v[0];
+      uint32_t pa, pb = 0;  // 0 I, 1 X, 2 Y, 3 Z
+      if (kind == QS_NOISE_DEPOLARIZE1) {
+        pa = 1 + (uint32_t)__umul64hi(v, 3);
+      } else {
+        const uint32_t idx = 1 + (uint32_t)__umul64hi(v, 15);
+        pa = idx >> 2;
+        pb = idx & 3;
+      }
+      uint32_t *acc = s_pauli[lo] + (b >> 5);
+      const uint32_t bit = 1u << (b & 31);
+      if (pa == 1 || pa == 2) atomicOr(acc, bit);
+      if (pa >= 2) atomicOr(acc + 2, bit);
+      if (pb == 1 || pb == 2) atomicOr(acc + 4, bit);
+      if (pb >= 2) atomicOr(acc + 6, bit);
+    }
+    __syncthreads();
+  }
+  for (uint32_t x = t; x < n; x += kNoiseThreads) {
+    const uint64_t fire = s_fire[x];
+    if (!fire) continue;
+    uint32_t i, j;
+    place(x, i, j);
+    uint64_t ax = 0, az = 0, bx = 0, bz = 0;
+    if (draws) {
+      const uint64_t *acc = reinterpret_cast<const uint64_t *>(s_pauli[x]);
+      ax = acc[0]; az = acc[1]; bx = acc[2]; bz = acc[3];
+    } else {
+      if (kind != QS_NOISE_Z) ax = fire;
+      if (kind != QS_NOISE_X) az = fire;
+    }
+    const uint64_t qa = kind == QS_NOISE_DEPOLARIZE2 ? targets[2 * (uint64_t)i] : targets[i];
+    if (ax) FX[qa * fw + j] ^= ax;
+    if (az) FZ[qa * fw + j] ^= az;
+    if (kind == QS_NOISE_DEPOLARIZE2) {
+      const uint64_t qb = targets[2 * (uint64_t)i + 1];
+      if (bx) FX[qb * fw + j] ^= bx;
+      if (bz) FZ[qb * fw + j] ^= bz;
+    }
+  }
+}
+
+cudaError_t launch_frame_noise(uint64_t *FX, uint64_t *FZ, uint32_t fw, uint32_t ow, const NoiseOp *ops, int n,
+                               uint64_t seed, cudaStream_t s, int *launches) {
+  NoiseGroup G;
+  G.ops = 0;
+  G.seed = seed;
+  uint64_t blocks = 0;
+  for (int i = 0; i < n; ++i) {
+    const NoiseOp &x = ops[i];
+    if (x.count == 0 || ow == 0 || x.thr == 0) continue;  // never fires
+    if (G.ops == kNoiseGroupMax) return cudaErrorInvalidValue;
+    NoiseLaunch &l = G.op[G.ops++];
+    l.targets = x.targets;
+    l.items = (uint64_t)x.count * ow;
+    l.thr = x.thr;
+    l.i0 = x.i0;
+    l.kind = x.kind;
+    l.first_block = (uint32_t)blocks;
+    l.e = x.e;
+    blocks += (l.items + kNoiseItems - 1) / kNoiseItems;
+    if (blocks > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
+  }
+  if (G.ops == 0) return cudaSuccess;
+  frame_noise_kernel<<<(unsigned)blocks, kNoiseThreads, 0, s>>>(FX, FZ, fw, ow, G);
+  if (launches) *launches += 1;
   return cudaGetLastError();
 }
 

@@ -228,12 +228,19 @@ cudaError_t launch_frame_measure(uint64_t *FX, uint64_t *FZ, uint32_t n, uint32_
                                  const uint32_t *qubits, uint32_t count, uint64_t m0,
                                  const uint8_t *ref, uint64_t *out, uint64_t shots, uint64_t seed,
                                  uint32_t *err, cudaStream_t s);
-// noise op e (QS_NOISE_* kind) on targets[0..count) (pairs for DEPOLARIZE2,
-// count = number of pairs), global target index i0 + local index; shot words
-// 0..ow-1; a shot fires iff its 32-bit draw u < thr (thr = 2^32: always)
-cudaError_t launch_frame_noise(uint64_t *FX, uint64_t *FZ, uint32_t fw, uint32_t ow,
-                               const uint32_t *targets, uint32_t count, uint32_t i0, int kind,
-                               uint64_t thr, uint64_t e, uint64_t seed, cudaStream_t s);
+// noise op e (QS_NOISE_* kind) on targets[0..count) (pairs for DEPOLARIZE2, count =
+// number of pairs), global target index i0 + local index; a shot fires iff its
+// 32-bit draw u < thr (thr = 2^32: always)
+constexpr int kNoiseGroupMax = 4;
+struct NoiseOp {
+  const uint32_t *targets;
+  uint32_t count, i0;
+  int kind;
+  uint64_t thr, e;
+};
+// up to kNoiseGroupMax ops on pairwise distinct qubits, shot words 0..ow-1
+cudaError_t launch_frame_noise(uint64_t *FX, uint64_t *FZ, uint32_t fw, uint32_t ow, const NoiseOp *ops, int n,
+                               uint64_t seed, cudaStream_t s, int *launches);
 cudaError_t launch_reset_meas_state(const Dev &d, cudaStream_t s);
 // column q = qubits[i] of the row-major x part into colx, pivot by atomicMin into mst
 cudaError_t launch_gather(const Dev &d, const uint32_t *qubits, uint32_t i, cudaStream_t s);

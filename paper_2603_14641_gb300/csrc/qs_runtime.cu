@@ -53,6 +53,7 @@ struct Op {
   uint64_t thr = 0;              // kNoise: a shot fires iff its 32-bit draw u < thr
   uint64_t ordinal = 0;          // kNoise: index among the noise ops (the draw's e)
   uint64_t dev_off = 0;          // kNoise: offset of its targets in the sim's noise buffer (words)
+  bool joins = false;            // kNoise: launches with the noise op before it (distinct qubits)
 };
 
 constexpr int kRing = 4;
@@ -738,9 +739,10 @@ static int replay_noise(qs_sim *s, const Op &op, uint64_t *FX, uint64_t *FZ, uin
     memcpy(h, op.qubits.data() + (size_t)t0 * per, (size_t)c * per * 4);
     int rc = upload(s, slot, (size_t)c * per * 4);
     if (rc) return rc;
-    QS_CUDA(s, launch_frame_noise(FX, FZ, fw, ow, reinterpret_cast<uint32_t *>(s->dstage), c, t0,
-                                  op.noise_kind, op.thr, op.ordinal, seed, s->stream));
-    if (op.thr) s->launches += 1;
+    const NoiseOp one{reinterpret_cast<uint32_t *>(s->dstage), c, t0, op.noise_kind, op.thr, op.ordinal};
+    int l = 0;
+    QS_CUDA(s, launch_frame_noise(FX, FZ, fw, ow, &one, 1, seed, s->stream, &l));
+    s->launches += (uint64_t)l;
   }
   return QS_OK;
 }
@@ -760,6 +762,25 @@ static int upload_noise_targets(qs_sim *s) {
       if (!op.qubits.empty()) memcpy(host.data() + off, op.qubits.data(), op.qubits.size() * 4);
       off += op.qubits.size();
     }
+  // runs of noise ops on distinct qubits launch together
+  std::vector<uint32_t> seen(s->d.L.n, 0);
+  uint32_t run = 0;
+  int in_run = 0;
+  for (Op &op : s->ops) {
+    if (op.kind != Op::kNoise) {
+      in_run = 0;
+      continue;
+    }
+    bool distinct = in_run > 0 && in_run < kNoiseGroupMax;
+    for (size_t i = 0; i < op.qubits.size() && distinct; ++i) distinct = seen[op.qubits[i]] != run;
+    op.joins = distinct;
+    if (!distinct) {
+      ++run;
+      in_run = 0;
+    }
+    for (uint32_t q : op.qubits) seen[q] = run;
+    ++in_run;
+  }
   if (words > s->noise_dev_words) {
     if (s->noise_dev) {
       QS_CUDA(s, cudaStreamSynchronize(s->stream));  // earlier replays may still read it
@@ -781,14 +802,22 @@ static int upload_noise_targets(qs_sim *s) {
   return QS_OK;
 }
 
-// One noise op straight from the uploaded targets.
-static int replay_noise_dev(qs_sim *s, const Op &op, uint64_t *FX, uint64_t *FZ, uint32_t fw, uint32_t ow,
+// The noise op ops[i] and those that join it, straight from the uploaded
+// targets; i moves on to the last of them.
+static int replay_noise_dev(qs_sim *s, size_t *i, uint64_t *FX, uint64_t *FZ, uint32_t fw, uint32_t ow,
                             uint64_t seed) {
-  const uint32_t per = op.noise_kind == QS_NOISE_DEPOLARIZE2 ? 2 : 1;
-  const uint32_t total = (uint32_t)op.qubits.size() / per;
-  QS_CUDA(s, launch_frame_noise(FX, FZ, fw, ow, s->noise_dev + op.dev_off, total, 0, op.noise_kind, op.thr,
-                                op.ordinal, seed, s->stream));
-  if (op.thr && total) s->launches += 1;
+  NoiseOp group[kNoiseGroupMax];
+  int n = 0;
+  for (size_t k = *i;; ++k) {
+    const Op &op = s->ops[k];
+    const uint32_t per = op.noise_kind == QS_NOISE_DEPOLARIZE2 ? 2 : 1;
+    group[n++] = NoiseOp{s->noise_dev + op.dev_off, (uint32_t)op.qubits.size() / per, 0, op.noise_kind, op.thr, op.ordinal};
+    *i = k;
+    if (k + 1 >= s->ops.size() || s->ops[k + 1].kind != Op::kNoise || !s->ops[k + 1].joins) break;
+  }
+  int l = 0;
+  QS_CUDA(s, launch_frame_noise(FX, FZ, fw, ow, group, n, seed, s->stream, &l));
+  s->launches += (uint64_t)l;
   return QS_OK;
 }
 
@@ -863,7 +892,8 @@ int qs_sim_sample(qs_sim *s, uint64_t shots, uint64_t seed, uint64_t *record, si
   s->launches += 1;
   std::vector<uint32_t> qtmp, seen(n, 0);
   uint32_t sid = 0;
-  for (const Op &op : s->ops) {
+  for (size_t at = 0; at < s->ops.size(); ++at) {
+    const Op &op = s->ops[at];
     if (op.kind == Op::kHostLayer) {
       int slot;
       uint8_t *h = ring_slot(s, &slot);
@@ -878,7 +908,7 @@ int qs_sim_sample(qs_sim *s, uint64_t shots, uint64_t seed, uint64_t *record, si
                                op.ptr.size() - 1, false)))
         return rc;
     } else if (op.kind == Op::kNoise) {
-      if ((rc = replay_noise_dev(s, op, FX, FZ, (uint32_t)fw, (uint32_t)ow, seed))) return rc;
+      if ((rc = replay_noise_dev(s, &at, FX, FZ, (uint32_t)fw, (uint32_t)ow, seed))) return rc;
     } else {
       // measurement window: split into runs of distinct qubits (Sec. 5 processes
       // the measurements of one window in parallel)
