@@ -31,6 +31,7 @@ namespace qs {
 constexpr int kDetBlocks = 152;     // chunks of the deterministic product (one per SM)
 constexpr int kMeasStateWords = 16; // per-measurement device state
 constexpr int kInvChunks = 512;     // row chunks of the inverse-mode target pass
+constexpr uint32_t kInvColumnsMax = 16384;  // qubits up to which inverse-mode measurement goes by columns
 
 // device error flags (sticky, cleared by reset)
 enum : uint32_t {
@@ -201,7 +202,7 @@ struct Dev {
   KernelTimer *timer;      // CUDA-event timing of kernel classes, or nullptr (off)
   bool inverse;            // inverse-tableau mode (qubit-indexed signs, Alg. 1 measurement)
   uint64_t *qsig;          // inverse mode: S_S then S_D, rs words each
-  uint64_t *inv_part;      // inverse mode: measurement partials, 6 * kInvChunks * rs words
+  uint64_t *inv_part;      // inverse mode: measurement scratch, inv_scratch_words
 };
 
 cudaError_t launch_init(const Dev &d, const uint8_t *initstate_dev, cudaStream_t s);
@@ -250,6 +251,11 @@ cudaError_t launch_inv_gate_layer(const Dev &d, const uint32_t *packed, uint32_t
 size_t inv_scratch_words(const Layout &L);
 cudaError_t launch_inv_measure_one(const Dev &d, const uint32_t *qubits, uint32_t i, uint64_t midx,
                                    qs_key key, cudaStream_t s, int *launches);
+// the same for a window of measurements on the column-major tableau
+// (qs_inverse_columns.cu, n <= kInvColumnsMax)
+size_t inv_log_words(const Layout &L);
+cudaError_t launch_inv_measure_columns(const Dev &d, const uint32_t *qubits, uint32_t count, uint64_t m0, qs_key key,
+                                       cudaStream_t s, int *launches);
 // a window of measurements qubits[0..count) with record indices m0.., two
 // launches per measurement (plus two per window)
 bool measure_window_supported(const Layout &L);

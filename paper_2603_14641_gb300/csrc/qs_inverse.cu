@@ -21,7 +21,9 @@
 // shared memory, and thread 0 updates the sign bits with XOR atomics (gates
 // of a layer act on distinct qubits, which may share a sign word).
 //
-// Measurement (Alg. 1), four launches on the row-major tableau:
+// Measurement (Alg. 1) up to 16,384 qubits: by columns, up to 64 measurements
+// at once (qs_inverse_columns.cu). Beyond, where a column's words do not fit the
+// registers of one block, four launches per measurement on the row-major tableau:
 //  1. gather (shared with the CHP path): pivot p = smallest stabilizer with
 //     XS[p][q] = 1, and the column bits of every row.
 //  2. inv_targets: CX injections from the pivot into every later stabilizer t
@@ -442,7 +444,9 @@ inv_finalize_kernel(uint64_t *__restrict__ RX, uint64_t *__restrict__ RZ, uint64
   inv_finalize_block(RX, RZ, qsig, rs, k, q, mst[kMsPivot], mst, midx, seed, shot, record, kinds);
 }
 
-size_t inv_scratch_words(const Layout &L) { return (size_t)6 * kInvChunks * L.rs; }
+size_t inv_scratch_words(const Layout &L) {
+  return L.n <= kInvColumnsMax ? inv_log_words(L) : (size_t)6 * kInvChunks * L.rs;
+}
 
 cudaError_t launch_inv_measure_one(const Dev &d, const uint32_t *qubits, uint32_t i, uint64_t midx,
                                    qs_key key, cudaStream_t s, int *launches) {

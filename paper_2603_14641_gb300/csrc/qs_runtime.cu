@@ -518,9 +518,19 @@ int qs_sim_apply_layers_dev(qs_sim *s, const uint32_t *packed_dev, const int64_t
   return QS_OK;
 }
 
+// whether measurements work on the column-major tableau
+static bool measures_columns(const qs_sim *s) { return s->d.inverse && s->d.L.n <= kInvColumnsMax; }
+
 static int measure_staged(qs_sim *s, const uint32_t *qdev, uint32_t count, uint64_t m0, qs_key key) {
-  if (s->d.inverse) {  // Alg. 1, one measurement after another
+  if (s->d.inverse) {  // Alg. 1: blocks of steps by columns, or one measurement after another
     tbegin(s->d.timer, QS_TIME_MEASURE_SINGLE, s->stream);
+    if (measures_columns(s)) {
+      int l = 0;
+      QS_CUDA(s, launch_inv_measure_columns(s->d, qdev, count, m0, key, s->stream, &l));
+      s->launches += (uint64_t)l;
+      tend(s->d.timer, QS_TIME_MEASURE_SINGLE, s->stream);
+      return QS_OK;
+    }
     for (uint32_t i = 0; i < count; ++i) {
       int l = 0;
       QS_CUDA(s, launch_inv_measure_one(s->d, qdev, i, m0 + i, key, s->stream, &l));
@@ -567,7 +577,7 @@ int qs_sim_measure(qs_sim *s, const uint32_t *qubits, uint32_t count, qs_key key
   if (s->n_meas + count > s->d.record_cap)
     return fail(QS_ERR_SIZE, "record capacity exceeded (qs_options.record_capacity)");
   if (count == 0) return QS_OK;
-  if ((rc = ensure_rows(s))) return rc;
+  if ((rc = measures_columns(s) ? ensure_cols(s) : ensure_rows(s))) return rc;
   const uint64_t m0 = s->n_meas;
   const uint32_t chunk = (uint32_t)(s->plan.stage_bytes / 4);
   for (uint32_t off = 0; off < count; off += chunk) {
@@ -581,7 +591,7 @@ int qs_sim_measure(qs_sim *s, const uint32_t *qubits, uint32_t count, qs_key key
       return rc;
   }
   s->n_meas += count;
-  s->cols_valid = false;
+  (measures_columns(s) ? s->rows_valid : s->cols_valid) = false;
   Op op;
   op.kind = Op::kHostMeasure;
   op.qubits.assign(qubits, qubits + count);
@@ -602,11 +612,11 @@ int qs_sim_measure_dev(qs_sim *s, const uint32_t *qubits_dev, uint32_t count, qs
   if (s->n_meas + count > s->d.record_cap)
     return fail(QS_ERR_SIZE, "record capacity exceeded (qs_options.record_capacity)");
   if (count == 0) return QS_OK;
-  if ((rc = ensure_rows(s))) return rc;
+  if ((rc = measures_columns(s) ? ensure_cols(s) : ensure_rows(s))) return rc;
   const uint64_t m0 = s->n_meas;
   if ((rc = measure_staged(s, qubits_dev, count, m0, key))) return rc;
   s->n_meas += count;
-  s->cols_valid = false;
+  (measures_columns(s) ? s->rows_valid : s->cols_valid) = false;
   Op op;
   op.kind = Op::kDevMeasure;
   op.dev = qubits_dev;
