@@ -88,13 +88,11 @@ struct GateIn {
   ulonglong2 x1, z1, x2, z2;
 };
 
-// Reads the record of gate g and the column words it needs; false for an
+// Reads the column words the gate of record (w0, qb) needs; false for an
 // invalid record (flagged, skipped).
 template <bool SIGNS>
-__device__ __forceinline__ bool gate_load(GateIn &in, uint32_t g, const uint32_t *__restrict__ packed,
-                                          uint64_t *X, uint64_t *Z, uint32_t n, uint32_t cs,
-                                          size_t off, bool flag, uint32_t *err) {
-  const uint32_t w0 = __ldg(packed + 2 * g), qb = __ldg(packed + 2 * g + 1);
+__device__ __forceinline__ bool gate_load(GateIn &in, uint32_t w0, uint32_t qb, uint64_t *X, uint64_t *Z, uint32_t n,
+                                          uint32_t cs, size_t off, bool flag, uint32_t *err) {
   const uint32_t type = w0 >> 24, qa = w0 & 0xFFFFFFu;
   const bool two = is_two_qubit(type);
   if (qa >= n || type >= QS_NUM_GATE_TYPES || (two && (qb >= n || qb == qa))) {
@@ -149,19 +147,16 @@ __device__ __forceinline__ void gate_apply(GateIn &in, ulonglong2 &sacc, uint64_
   }
 }
 
-template <bool SIGNS, int INFLIGHT>
-__global__ void __launch_bounds__(256, INFLIGHT == 2 ? 4 : 6)
-gate_layer_kernel(uint64_t *__restrict__ X, uint64_t *__restrict__ Z, uint64_t *__restrict__ S,
-                  uint32_t n, uint32_t cs, const uint32_t *__restrict__ packed, uint32_t n_gates,
-                  uint32_t P, uint32_t lanes, uint32_t gpl, uint32_t *__restrict__ err) {
+// One thread block's gates [g0, g1) of a layer; record(g) gives gate g's two words.
+template <bool SIGNS, int INFLIGHT, class Record>
+__device__ __forceinline__ void gate_block(uint64_t *__restrict__ X, uint64_t *__restrict__ Z, uint64_t *__restrict__ S,
+                                           uint32_t n, uint32_t cs, Record record, uint32_t g0, uint32_t g1, uint32_t P,
+                                           uint32_t lanes, uint32_t *__restrict__ err) {
   const uint32_t npairs = cs >> 1;
   const uint32_t t = threadIdx.x;
   const uint32_t lane = t / P;
   const uint32_t pair = blockIdx.y * P + (t - lane * P);
   const bool active = pair < npairs;
-  const uint32_t group = lanes * gpl;
-  const uint32_t g0 = blockIdx.x * group;
-  const uint32_t g1 = min(g0 + group, n_gates);
   ulonglong2 sacc = make_ulonglong2(0, 0);
 
   if (active) {
@@ -171,9 +166,13 @@ gate_layer_kernel(uint64_t *__restrict__ X, uint64_t *__restrict__ Z, uint64_t *
       GateIn in[INFLIGHT];
       bool ok[INFLIGHT];
 #pragma unroll
-      for (int u = 0; u < INFLIGHT; ++u)
-        ok[u] = g + u * lanes < g1 &&
-                gate_load<SIGNS>(in[u], g + u * lanes, packed, X, Z, n, cs, off, flag, err);
+      for (int u = 0; u < INFLIGHT; ++u) {
+        ok[u] = g + u * lanes < g1;
+        if (ok[u]) {
+          const uint2 r = record(g + u * lanes);
+          ok[u] = gate_load<SIGNS>(in[u], r.x, r.y, X, Z, n, cs, off, flag, err);
+        }
+      }
 #pragma unroll
       for (int u = 0; u < INFLIGHT; ++u)
         if (ok[u]) gate_apply<SIGNS>(in[u], sacc, X, Z, cs, off);
@@ -196,6 +195,48 @@ gate_layer_kernel(uint64_t *__restrict__ X, uint64_t *__restrict__ Z, uint64_t *
       if (sacc.y) atomicXor(reinterpret_cast<unsigned long long *>(S + 2 * (size_t)pair + 1), sacc.y);
     }
   }
+}
+
+template <bool SIGNS, int INFLIGHT>
+__global__ void __launch_bounds__(256, INFLIGHT == 2 ? 4 : 6)
+gate_layer_kernel(uint64_t *__restrict__ X, uint64_t *__restrict__ Z, uint64_t *__restrict__ S,
+                  uint32_t n, uint32_t cs, const uint32_t *__restrict__ packed, uint32_t n_gates,
+                  uint32_t P, uint32_t lanes, uint32_t gpl, uint32_t *__restrict__ err) {
+  const uint32_t group = lanes * gpl, g0 = blockIdx.x * group;
+  gate_block<SIGNS, INFLIGHT>(
+      X, Z, S, n, cs, [&](uint32_t g) { return make_uint2(__ldg(packed + 2 * g), __ldg(packed + 2 * g + 1)); }, g0,
+      min(g0 + group, n_gates), P, lanes, err);
+}
+
+// A host layer whose records ride in the launch itself: one word a gate (type
+// << 28 | q0 << 14 | q1, up to 16,384 qubits), MAX of them in the kernel's
+// parameters. Staged, a layer is a copy and an event besides the launch, and
+// the kernel waits for the copy engine: 8.9 us a layer at 127 qubits from
+// back-to-back calls of the Python API, 5.9 with the records in the launch (host
+// time, both); 1,000 qubits 10.0 and 6.7. Limits: qubit numbers of 14 bits, and
+// beyond 2,048 gates (8 KB) the copy costs no more (4,000 qubits: 14.6 and 14.2).
+constexpr uint32_t kParamGroup = 512;  // gates of a block
+template <int MAX>
+struct ParamLayer {
+  uint32_t rec[MAX];
+};
+
+template <int MAX>
+__global__ void __launch_bounds__(256, 4)
+param_layer_kernel(uint64_t *__restrict__ X, uint64_t *__restrict__ Z, uint64_t *__restrict__ S, uint32_t n, uint32_t cs,
+                   uint32_t n_gates, uint32_t P, uint32_t lanes, uint32_t gpl, uint32_t *__restrict__ err,
+                   const __grid_constant__ ParamLayer<MAX> layer) {
+  __shared__ uint32_t rec[kParamGroup];
+  const uint32_t group = lanes * gpl, g0 = blockIdx.x * group, g1 = min(g0 + group, n_gates);
+  for (uint32_t i = threadIdx.x; g0 + i < g1; i += blockDim.x) rec[i] = layer.rec[g0 + i];
+  __syncthreads();
+  gate_block<true, 2>(
+      X, Z, S, n, cs,
+      [&](uint32_t g) {
+        const uint32_t r = rec[g - g0];
+        return make_uint2(r >> 28 << 24 | (r >> 14 & 0x3FFF), r & 0x3FFF);
+      },
+      g0, g1, P, lanes, err);
 }
 
 struct GateGrid {
@@ -228,6 +269,30 @@ cudaError_t launch_gate_layer(const Dev &d, const uint32_t *packed, uint32_t n_g
   GateGrid g = gate_grid(d.L.cs / 2, n_gates);
   gate_layer_kernel<true, 2><<<g.grid, g.block, 0, s>>>(d.X, d.Z, d.S, d.L.n, d.L.cs, packed, n_gates,
                                                      g.P, g.lanes, g.gpl, d.err);
+  return cudaGetLastError();
+}
+
+template <int MAX>
+static void launch_param(const Dev &d, const uint32_t *packed, uint32_t n_gates, cudaStream_t s) {
+  ParamLayer<MAX> layer;
+  for (uint32_t g = 0; g < n_gates; ++g)
+    layer.rec[g] = packed[2 * g] >> 24 << 28 | (packed[2 * g] & 0x3FFF) << 14 | packed[2 * g + 1];
+  GateGrid g = gate_grid(d.L.cs / 2, n_gates);
+  g.gpl = std::max(1u, std::min(g.gpl, kParamGroup / g.lanes));
+  g.grid.x = (n_gates + g.lanes * g.gpl - 1) / (g.lanes * g.gpl);
+  param_layer_kernel<MAX><<<g.grid, g.block, 0, s>>>(d.X, d.Z, d.S, d.L.n, d.L.cs, n_gates, g.P, g.lanes, g.gpl, d.err,
+                                                     layer);
+}
+
+bool param_layer_fits(uint32_t n, uint32_t n_gates) { return n <= 16384 && n_gates <= 2048; }
+
+cudaError_t launch_param_layer(const Dev &d, const uint32_t *packed, uint32_t n_gates, cudaStream_t s) {
+  if (n_gates <= 128)
+    launch_param<128>(d, packed, n_gates, s);
+  else if (n_gates <= 512)
+    launch_param<512>(d, packed, n_gates, s);
+  else
+    launch_param<2048>(d, packed, n_gates, s);
   return cudaGetLastError();
 }
 

@@ -208,6 +208,9 @@ struct Dev {
 cudaError_t launch_init(const Dev &d, const uint8_t *initstate_dev, cudaStream_t s);
 cudaError_t launch_gate_layer(const Dev &d, const uint32_t *packed, uint32_t n_gates,
                               cudaStream_t s);
+// the same for validated records in host memory, which go with the launch
+bool param_layer_fits(uint32_t n, uint32_t n_gates);
+cudaError_t launch_param_layer(const Dev &d, const uint32_t *packed, uint32_t n_gates, cudaStream_t s);
 // layers ptr[0..nlayers] of `packed` on the tableau with one-qubit gates deferred
 // to the next two-qubit gate of their qubit (qs_lazy.cuh), nothing pending after;
 // scratch: lazy_scratch_bytes(n)

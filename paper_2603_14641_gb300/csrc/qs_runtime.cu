@@ -451,13 +451,18 @@ int qs_sim_apply_layer(qs_sim *s, const qs_gate *gates, uint32_t n_gates) {
     return rc;
   if (n_gates == 0) return QS_OK;
   if ((rc = ensure_cols(s))) return rc;
-  int slot;
-  uint8_t *h = ring_slot(s, &slot);
-  if (!h) return cuda_fail(s, cudaGetLastError(), "staging event");
-  memcpy(h, op.packed.data(), op.packed.size() * 4);
-  if ((rc = upload(s, slot, op.packed.size() * 4))) return rc;
+  const bool with_launch = !s->d.inverse && param_layer_fits(s->d.L.n, n_gates);
+  if (!with_launch) {
+    int slot;
+    uint8_t *h = ring_slot(s, &slot);
+    if (!h) return cuda_fail(s, cudaGetLastError(), "staging event");
+    memcpy(h, op.packed.data(), op.packed.size() * 4);
+    if ((rc = upload(s, slot, op.packed.size() * 4))) return rc;
+  }
   tbegin(s->d.timer, QS_TIME_GATES, s->stream);
-  if (s->d.inverse)
+  if (with_launch)
+    QS_CUDA(s, launch_param_layer(s->d, op.packed.data(), n_gates, s->stream));
+  else if (s->d.inverse)
     QS_CUDA(s, launch_inv_gate_layer(s->d, reinterpret_cast<const uint32_t *>(s->dstage), n_gates,
                                      s->stream));
   else
