@@ -272,13 +272,12 @@ cudaError_t launch_measure_blocks(const Dev &d, void *scratch, const uint32_t *w
                                   qs_key key, cudaStream_t s, int *launches);
 // fused segment of L <= kFusedLayers layers on a word-sliced, shared-memory-resident
 // tableau (S == nullptr: frames, no signs), one-qubit gates deferred; nwords: the
-// words of a column that matter; lptr: L + 1 device gate offsets; max_gates: the
-// largest layer's gates; scratch: fused_scratch_bytes(n)
+// words of a column that matter; ptr: L + 1 gate offsets (host memory); scratch: fused_scratch_bytes(n)
 constexpr uint32_t kFusedLayers = 128;
 bool fused_fits(uint32_t n);
 size_t fused_scratch_bytes(uint32_t n);
 cudaError_t launch_fused_segment(uint64_t *X, uint64_t *Z, uint64_t *S, uint32_t n, uint32_t stride, uint32_t nwords,
-                                 const uint32_t *packed, const int64_t *lptr, uint32_t L, uint32_t max_gates, int sms,
+                                 const uint32_t *packed, const int64_t *ptr, uint32_t L, int sms,
                                  void *scratch, uint32_t *err, cudaStream_t s);
 // device record of a simulator (one byte per measurement)
 const uint8_t *sim_record(const qs_sim *sim);

@@ -247,20 +247,10 @@ int run_dev_layers(qs_sim *s, uint64_t *X, uint64_t *Z, uint64_t *S, uint32_t st
   const uint32_t n = s->d.L.n;
   if (nlayers == 0) return QS_OK;
   if (nlayers >= kFusedMinLayers && fused_fits(n) && !(s->flags & QS_FLAG_NO_FUSION) && !(tableau && s->d.inverse)) {
-    // the staged offset table holds at least kFusedLayers + 1 entries
     for (size_t l0 = 0; l0 < nlayers; l0 += kFusedLayers) {
       const size_t L = std::min<size_t>(kFusedLayers, nlayers - l0);
-      int slot;
-      uint8_t *h = ring_slot(s, &slot);
-      if (!h) return cuda_fail(s, cudaGetLastError(), "staging event");
-      memcpy(h, ptr + l0, (L + 1) * 8);
-      int rc = upload(s, slot, (L + 1) * 8);
-      if (rc) return rc;
-      int64_t max_gates = 0;  // layers hold at most n gates (checked when they were added)
-      for (size_t l = l0; l < l0 + L; ++l) max_gates = std::max<int64_t>(max_gates, ptr[l + 1] - ptr[l]);
-      QS_CUDA(s, launch_fused_segment(X, Z, S, n, stride, nwords, packed,
-                                      reinterpret_cast<const int64_t *>(s->dstage), (uint32_t)L,
-                                      (uint32_t)max_gates, s->d.sms, s->fused, s->d.err, s->stream));
+      QS_CUDA(s, launch_fused_segment(X, Z, S, n, stride, nwords, packed, ptr + l0, (uint32_t)L, s->d.sms, s->fused,
+                                      s->d.err, s->stream));
       s->launches += 3;
     }
     return QS_OK;
