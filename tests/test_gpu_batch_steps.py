@@ -1,0 +1,38 @@
+"""Batch circuits in shared memory: rounds of 7, 8, 9 and 17 measurements (passes of eight) with repeated
+qubits, and their frame samples, equal to a simulator of the circuit alone."""
+import numpy as np
+import pytest
+
+from paper_2603_14641_gb300 import qs
+from workloads import circuits as C
+
+pytestmark = pytest.mark.gpu
+
+
+def _circuit(n):
+    c = C.gate_mix_circuit(n, 10, seed=n, final_measure_all=False)
+    rng = np.random.default_rng(n)
+    c.ops = []
+    for i, m in enumerate((7, 8, 9, 17, 1)):
+        q = rng.integers(0, n, m).astype(np.uint32)
+        q[-1] = q[0]
+        c.ops += [("layers", 2 * i, 2 * i + 2), ("measure", q)]
+    return c
+
+
+def test_passes_of_eight_and_samples_equal_a_simulator():
+    sizes = [1, 2, 64, 65, 127, 129, 256, 257, 448, 512, 640, 700, 900]
+    circs = [_circuit(n) for n in sizes]
+    shots = [1, 64, 65, 130, 300, 200, 256, 257, 100, 513, 129, 128, 192]
+    b = qs.Batch(circs, list(range(len(sizes))))
+    b.run()
+    words = b.sample(shots, [7 + i for i in range(len(sizes))])
+    b.sync()
+    for i, c in enumerate(circs):
+        s = qs.Simulator(c.n)
+        assert np.array_equal(b.record(i), s.run(c, seed=i)), c.n
+        rows = np.arange(2 * c.n, dtype=np.uint32)
+        for u, v in zip(b.export_rows(i, rows), s.export_rows(rows)):
+            assert np.array_equal(u, v), c.n
+        want = s.sample(shots[i], 7 + i, on_device=False)
+        assert np.array_equal(words[i].cpu().numpy().view(np.uint64), want), c.n
