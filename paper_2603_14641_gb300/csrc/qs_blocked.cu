@@ -641,8 +641,6 @@ __global__ void __launch_bounds__(256, 4) blk_front_kernel(const FrontArgs a) {
   __shared__ uint32_t s_cnt[8];
   __shared__ uint64_t s_or[8];
   __shared__ bool s_last;
-  chain_next();
-  chain_wait();
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5, part = t % P;
   // the first blocks gather the next block's columns, the others sign the rows
   // of the previous one (nothing of which the symbolic pass needs)
@@ -973,8 +971,6 @@ __device__ __forceinline__ void list_rows(const MiddleArgs &a, uint32_t blk) {
 }
 
 __global__ void __launch_bounds__(kMidThreads) blk_middle_kernel(const MiddleArgs a) {
-  chain_next();
-  chain_wait();
   if (blockIdx.x < a.chunks) pivot_rows(a, blockIdx.x);
   else list_rows(a, blockIdx.x - a.chunks);
 }
@@ -1207,8 +1203,6 @@ blk_apply_kernel(uint64_t *__restrict__ RX, uint64_t *__restrict__ RZ, uint32_t 
                  uint8_t *__restrict__ Tp, const BlkState *st) {
   extern __shared__ ulonglong2 T[];  // [kSmemEntries][kCW] of (x word, z word)
   __shared__ uint32_t s_tmem;
-  chain_next();
-  chain_wait();
   const uint32_t cnt = st->ntouched;
   if (cnt == 0) return;  // every outcome of the block is deterministic
   const uint32_t u0 = blockIdx.x * kCW;  // first column word of the chunk
@@ -1352,8 +1346,6 @@ blk_apply_small_kernel(uint64_t *__restrict__ RX, uint64_t *__restrict__ RZ, uin
                        const uint64_t *__restrict__ VZ, const uint4 *__restrict__ list, uint8_t *__restrict__ Tp,
                        const BlkState *st) {
   __shared__ ulonglong2 T[16 * 16][CW];
-  chain_next();
-  chain_wait();
   const uint32_t cnt = st->ntouched;
   const uint32_t t = threadIdx.x, w = t % CW, word = blockIdx.x * CW + w;
   const uint32_t group = t / CW, units = gridDim.y * (kSmallThreads / CW);
@@ -1464,7 +1456,6 @@ __global__ void __launch_bounds__(kDetThreads) blk_det_kernel(const DetArgs a) {
   __shared__ uint32_t s_row[kDetThreads], s_d[kDetThreads];
   __shared__ uint32_t s_cnt[4];
   __shared__ int s_flag;
-  chain_wait();
   const uint32_t nd = a.win->ndet;
   if (nd == 0) return;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -1736,8 +1727,8 @@ static cudaError_t measure_window_cap(const Dev &d, void *scratch, const uint32_
     }
     const uint32_t blocks = (f.B ? ranges : 0) + (f.prev_B ? ranges : 0);
     const size_t off_bytes = f.lazy ? ranges * 4 : 0;
-    if (L.nrows <= kFrontSplitRows) launch_chained(blk_front_kernel<8>, blocks, 256, off_bytes, s, f);
-    else launch_chained(blk_front_kernel<1>, blocks, 256, off_bytes, s, f);
+    if (L.nrows <= kFrontSplitRows) blk_front_kernel<8><<<blocks, 256, off_bytes, s>>>(f);
+    else blk_front_kernel<1><<<blocks, 256, off_bytes, s>>>(f);
     ++nl;
     if (!f.lazy && f.B) {
       // the previous block's M and base are signed; C0 -> C1 -> C0 ...
@@ -1754,21 +1745,21 @@ static cudaError_t measure_window_cap(const Dev &d, void *scratch, const uint32_
     m.B = f.B;
     m.st = st;
     tbegin(d.timer, QS_TIME_BLK_PIVOT_ROWS, s);
-    launch_chained(blk_middle_kernel, mid_blocks, kMidThreads, 0, s, m);
+    blk_middle_kernel<<<mid_blocks, kMidThreads, 0, s>>>(m);
     tend(d.timer, QS_TIME_BLK_PIVOT_ROWS, s);
     tbegin(d.timer, QS_TIME_BLK_APPLY, s);
     if (words == 4)
-      launch_chained(
-          blk_apply_small_kernel<4>, dim3(chunks, rows_y), kSmallThreads, 0, s, d.RX, d.RZ, L.rs, (uint32_t)L.nrows, window + i0, (int)f.B, b.VX, b.VZ, b.list, b.Tp, st);
+      blk_apply_small_kernel<4><<<dim3(chunks, rows_y), kSmallThreads, 0, s>>>(
+          d.RX, d.RZ, L.rs, (uint32_t)L.nrows, window + i0, (int)f.B, b.VX, b.VZ, b.list, b.Tp, st);
     else if (words == 8)
-      launch_chained(
-          blk_apply_small_kernel<8>, dim3(chunks, rows_y), kSmallThreads, 0, s, d.RX, d.RZ, L.rs, (uint32_t)L.nrows, window + i0, (int)f.B, b.VX, b.VZ, b.list, b.Tp, st);
+      blk_apply_small_kernel<8><<<dim3(chunks, rows_y), kSmallThreads, 0, s>>>(
+          d.RX, d.RZ, L.rs, (uint32_t)L.nrows, window + i0, (int)f.B, b.VX, b.VZ, b.list, b.Tp, st);
     else if (!d.wide_offsets && (uint64_t)L.nrows * L.rs < (1ull << 32))
-      launch_chained(
-          blk_apply_kernel<uint32_t>, dim3(chunks, rows_y), kApplyThreads, smem, s, d.RX, d.RZ, L.rs, (uint32_t)L.nrows, window + i0, (int)f.B, b.VX, b.VZ, b.list, b.Tp, st);
+      blk_apply_kernel<uint32_t><<<dim3(chunks, rows_y), kApplyThreads, smem, s>>>(
+          d.RX, d.RZ, L.rs, (uint32_t)L.nrows, window + i0, (int)f.B, b.VX, b.VZ, b.list, b.Tp, st);
     else
-      launch_chained(
-          blk_apply_kernel<uint64_t>, dim3(chunks, rows_y), kApplyThreads, smem, s, d.RX, d.RZ, L.rs, (uint32_t)L.nrows, window + i0, (int)f.B, b.VX, b.VZ, b.list, b.Tp, st);
+      blk_apply_kernel<uint64_t><<<dim3(chunks, rows_y), kApplyThreads, smem, s>>>(
+          d.RX, d.RZ, L.rs, (uint32_t)L.nrows, window + i0, (int)f.B, b.VX, b.VZ, b.list, b.Tp, st);
     tend(d.timer, QS_TIME_BLK_APPLY, s);
     nl += 2;
     if (d.timer && (i0 & 4095) == 4032) d.timer->resolve();  // completed event pairs go back to the pool
@@ -1779,7 +1770,7 @@ static cudaError_t measure_window_cap(const Dev &d, void *scratch, const uint32_
   t.det_x = d.det_x; t.det_z = d.det_z; t.m0 = m0; t.record = d.record; t.err = d.err;
   // enough blocks for one outcome's ranges and for every group; blocks without an item leave at once
   const uint64_t most = std::max<uint64_t>(kDetBlocks, (count + kDetGroup - 1) / kDetGroup) * t.chunks;
-  launch_chained(blk_det_kernel, (unsigned)std::min<uint64_t>(most, 12ull * d.sms), kDetThreads, 0, s, t);
+  blk_det_kernel<<<(unsigned)std::min<uint64_t>(most, 12ull * d.sms), kDetThreads, 0, s>>>(t);
   if (launches) *launches += nl + 2;
   return cudaGetLastError();
 }

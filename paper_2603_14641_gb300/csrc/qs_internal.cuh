@@ -117,31 +117,6 @@ inline cudaError_t once_per_device(std::atomic<uint64_t> &done, F set) {
   return e;
 }
 
-// Chains of short kernels on one stream: a kernel launched with launch_chained may
-// become resident while the kernel before it still runs, so that its launch is
-// off the critical path. It calls chain_wait before it touches memory (all of the
-// earlier work in the stream is then complete and visible: every kernel of a
-// chain waits, so a chain is as ordered as plain launches), and chain_next as
-// early as it likes: its blocks are then all resident or done, and the next
-// kernel's blocks only take room that is free.
-__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
-template <class... P, class... A>
-inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
-  cudaLaunchAttribute attr{};
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t c{};
-  c.gridDim = grid;
-  c.blockDim = block;
-  c.dynamicSmemBytes = smem;
-  c.stream = s;
-  c.attrs = &attr;
-  c.numAttrs = 1;
-  return cudaLaunchKernelEx(&c, kernel, args...);
-}
-
 // Optional CUDA-event timing of kernel classes (qs_sim_set_timing): begin/end
 // record an event pair on the stream around a group of launches; pairs are
 // resolved into elapsed milliseconds once their end event has completed.

@@ -76,8 +76,6 @@ inv_lead_kernel(const uint64_t *__restrict__ X, const uint64_t *__restrict__ qsi
   __shared__ uint4 s_cand[2][32];  // per warp: first target row, the columns' parities
   __shared__ uint2 s_row[2][32];   // the columns' s at that row
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, warps = blockDim.x >> 5;
-  chain_next();
-  chain_wait();
   for (uint32_t i = tid; i < 64; i += blockDim.x) {
     s_q[i] = i < count ? qubits[i] : kNone;
     s_p[i] = kNone;
@@ -271,8 +269,6 @@ inv_apply_kernel(uint64_t *__restrict__ X, uint64_t *__restrict__ Z, uint64_t *_
   __shared__ uint64_t s_c[2 * kApplyWarps<W>];
   __shared__ uint32_t s_e[2 * kApplyWarps<W>];
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, warps = blockDim.x >> 5;
-  chain_next();
-  chain_wait();
   const uint32_t steps = log->steps;
   if (steps == 0) return;
   uint32_t *m = sm;                                                 // word w of mask j at w S + j
@@ -457,9 +453,9 @@ cudaError_t measure_columns(const Dev &d, const uint32_t *qubits, uint32_t count
   const uint32_t warps = std::max(4u, std::min(kApplyWarps<W>, (L.n + sms - 1) / sms));
   for (uint32_t off = 0; off < count; off += B) {
     const uint32_t c = std::min(B, count - off);
-    launch_chained(lead, 1, 32 * lead_warps, lead_smem, s, d.X, d.qsig, L.n, L.k, L.cs, 32 * W, qubits + off, c, m0 + off, key.seed,
+    lead<<<1, 32 * lead_warps, lead_smem, s>>>(d.X, d.qsig, L.n, L.k, L.cs, 32 * W, qubits + off, c, m0 + off, key.seed,
                                                key.shot, d.record, d.kinds, log, d.err);
-    launch_chained(inv_apply_kernel<W>, grid, 32 * warps, apply_smem(warps), s, d.X, d.Z, d.qsig, L.n, L.k, L.cs, L.rs, log);
+    inv_apply_kernel<W><<<grid, 32 * warps, apply_smem(warps), s>>>(d.X, d.Z, d.qsig, L.n, L.k, L.cs, L.rs, log);
     if (launches) *launches += 2;
   }
   return cudaGetLastError();
