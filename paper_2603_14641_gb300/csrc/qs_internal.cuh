@@ -206,6 +206,10 @@ struct Dev {
 };
 
 cudaError_t launch_init(const Dev &d, const uint8_t *initstate_dev, cudaStream_t s);
+// the same with the measurement state and the error flags, in one launch
+constexpr uint32_t kInitAllWords = 1u << 20;  // words of X up to which it is used
+bool init_all_fits(const Layout &L);
+cudaError_t launch_init_all(const Dev &d, const uint8_t *initstate_dev, cudaStream_t s);
 cudaError_t launch_gate_layer(const Dev &d, const uint32_t *packed, uint32_t n_gates,
                               cudaStream_t s);
 // the same for validated records in host memory, which go with the launch

@@ -406,17 +406,21 @@ int qs_sim_reset(qs_sim *s, const uint8_t *initstate) {
     if ((rc = upload(s, slot, n))) return rc;
     init_dev = s->dstage;
   }
-  QS_CUDA(s, cudaMemsetAsync(s->d.err, 0, 4, s->stream));
-  if (s->d.inverse) {
-    // same bits as the CHP mode, no per-row signs; the basis state sits in S_S
-    QS_CUDA(s, launch_init(s->d, nullptr, s->stream));
-    QS_CUDA(s, launch_inv_init_signs(s->d, init_dev, s->stream));
+  // inverse mode: same bits as the CHP mode, no per-row signs; the basis state sits in S_S
+  const uint8_t *row_signs = s->d.inverse ? nullptr : init_dev;
+  if (init_all_fits(s->d.L)) {
+    QS_CUDA(s, launch_init_all(s->d, row_signs, s->stream));
     s->launches += 1;
   } else {
-    QS_CUDA(s, launch_init(s->d, init_dev, s->stream));
+    QS_CUDA(s, cudaMemsetAsync(s->d.err, 0, 4, s->stream));
+    QS_CUDA(s, launch_init(s->d, row_signs, s->stream));
+    QS_CUDA(s, launch_reset_meas_state(s->d, s->stream));
+    s->launches += 3;
   }
-  QS_CUDA(s, launch_reset_meas_state(s->d, s->stream));
-  s->launches += 3;
+  if (s->d.inverse) {
+    QS_CUDA(s, launch_inv_init_signs(s->d, init_dev, s->stream));
+    s->launches += 1;
+  }
   s->cols_valid = true;
   s->rows_valid = false;
   s->n_meas = 0;
