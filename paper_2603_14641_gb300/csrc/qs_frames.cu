@@ -17,6 +17,8 @@
 //                             key = (seed, 0xE5505));
 //                             the Pauli of a depolarising channel comes from
 //                             word 0 of Philox(ctr = (e, i, s, 4), same key).
+#include <algorithm>
+
 #include "qs_internal.cuh"
 
 namespace qs {
@@ -45,8 +47,21 @@ cudaError_t launch_frame_init(uint64_t *FX, uint64_t *FZ, uint32_t n, uint32_t f
 
 // grid.x over shot-word quads, grid.y over the measurements of the window
 // (the qubits of one launch are distinct)
+// The measured qubits: a device list, or MAX of them in the launch's parameters.
+struct DeviceQubits {
+  const uint32_t *q;
+  __device__ __forceinline__ uint32_t operator[](uint32_t i) const { return q[i]; }
+};
+constexpr uint32_t kParamQubits = 1024;
+template <int MAX>
+struct ParamQubits {
+  uint32_t q[MAX];
+  __device__ __forceinline__ uint32_t operator[](uint32_t i) const { return q[i]; }
+};
+
+template <class Qubits>
 __global__ void frame_measure_kernel(const uint64_t *__restrict__ FX, uint64_t *__restrict__ FZ,
-                                     uint32_t n, uint32_t fw, const uint32_t *__restrict__ qubits,
+                                     uint32_t n, uint32_t fw, const __grid_constant__ Qubits qubits,
                                      uint64_t m0, const uint8_t *__restrict__ ref,
                                      uint64_t *__restrict__ out, uint64_t shots, uint64_t seed,
                                      uint32_t *__restrict__ err) {
@@ -77,19 +92,46 @@ __global__ void frame_measure_kernel(const uint64_t *__restrict__ FX, uint64_t *
   pz[1] = make_ulonglong2(r.v[2], r.v[3]);
 }
 
+template <class Qubits>
+static void frame_measure(uint64_t *FX, uint64_t *FZ, uint32_t n, uint32_t fw, const Qubits &qubits, uint32_t count,
+                          uint64_t m0, const uint8_t *ref, uint64_t *out, uint64_t shots, uint64_t seed,
+                          uint32_t *err, cudaStream_t s) {
+  const uint32_t quads = fw >> 2;
+  const uint32_t threads = quads < 128 ? ((quads + 31) / 32) * 32 : 128;
+  const dim3 grid((quads + threads - 1) / threads, count);
+  frame_measure_kernel<<<grid, threads, 0, s>>>(FX, FZ, n, fw, qubits, m0, ref, out, shots, seed, err);
+}
+
 cudaError_t launch_frame_measure(uint64_t *FX, uint64_t *FZ, uint32_t n, uint32_t fw,
                                  const uint32_t *qubits, uint32_t count, uint64_t m0,
                                  const uint8_t *ref, uint64_t *out, uint64_t shots, uint64_t seed,
                                  uint32_t *err, cudaStream_t s) {
-  if (count == 0) return cudaSuccess;
-  const uint32_t quads = fw >> 2;
-  const uint32_t threads = quads < 128 ? ((quads + 31) / 32) * 32 : 128;
   // grid.y is limited to 65535: split long windows
-  for (uint32_t off = 0; off < count; off += 65535) {
-    const uint32_t c = count - off < 65535 ? count - off : 65535;
-    dim3 grid((quads + threads - 1) / threads, c);
-    frame_measure_kernel<<<grid, threads, 0, s>>>(FX, FZ, n, fw, qubits + off, m0 + off, ref, out,
-                                                  shots, seed, err);
+  for (uint32_t off = 0; off < count; off += 65535)
+    frame_measure(FX, FZ, n, fw, DeviceQubits{qubits + off}, std::min(65535u, count - off), m0 + off, ref, out, shots,
+                  seed, err, s);
+  return cudaGetLastError();
+}
+
+// Staged, a list is a copy and an event besides the launch, and the kernel waits
+// for the copy engine; up to 2,048 qubits they go with one or two launches.
+bool param_qubits_fit(uint32_t count) { return count <= 2 * kParamQubits; }
+
+cudaError_t launch_frame_measure_host(uint64_t *FX, uint64_t *FZ, uint32_t n, uint32_t fw, const uint32_t *qubits,
+                                      uint32_t count, uint64_t m0, const uint8_t *ref, uint64_t *out, uint64_t shots,
+                                      uint64_t seed, uint32_t *err, cudaStream_t s, int *launches) {
+  for (uint32_t off = 0; off < count; off += kParamQubits) {
+    const uint32_t c = std::min(kParamQubits, count - off);
+    if (c <= 128) {
+      ParamQubits<128> list;
+      std::copy(qubits + off, qubits + off + c, list.q);
+      frame_measure(FX, FZ, n, fw, list, c, m0 + off, ref, out, shots, seed, err, s);
+    } else {
+      ParamQubits<kParamQubits> list;
+      std::copy(qubits + off, qubits + off + c, list.q);
+      frame_measure(FX, FZ, n, fw, list, c, m0 + off, ref, out, shots, seed, err, s);
+    }
+    ++*launches;
   }
   return cudaGetLastError();
 }

@@ -236,6 +236,11 @@ cudaError_t launch_frame_measure(uint64_t *FX, uint64_t *FZ, uint32_t n, uint32_
                                  const uint32_t *qubits, uint32_t count, uint64_t m0,
                                  const uint8_t *ref, uint64_t *out, uint64_t shots, uint64_t seed,
                                  uint32_t *err, cudaStream_t s);
+// the same for a list in host memory, which goes with the launch
+bool param_qubits_fit(uint32_t count);
+cudaError_t launch_frame_measure_host(uint64_t *FX, uint64_t *FZ, uint32_t n, uint32_t fw, const uint32_t *qubits,
+                                      uint32_t count, uint64_t m0, const uint8_t *ref, uint64_t *out, uint64_t shots,
+                                      uint64_t seed, uint32_t *err, cudaStream_t s, int *launches);
 // noise op e (QS_NOISE_* kind) on targets[0..count) (pairs for DEPOLARIZE2, count =
 // number of pairs), global target index i0 + local index; a shot fires iff its
 // 32-bit draw u < thr (thr = 2^32: always)

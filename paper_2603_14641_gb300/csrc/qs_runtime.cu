@@ -732,6 +732,28 @@ int qs_sim_sync(qs_sim *s) {
   return QS_OK;
 }
 
+// frame measurements of a host list of distinct qubits
+static int frame_measure_list(qs_sim *s, uint64_t *FX, uint64_t *FZ, uint32_t fw, const uint32_t *q, uint32_t count,
+                              uint64_t m0, uint64_t *out, uint64_t shots, uint64_t seed) {
+  if (param_qubits_fit(count)) {
+    int l = 0;
+    QS_CUDA(s, launch_frame_measure_host(FX, FZ, s->d.L.n, fw, q, count, m0, s->d.record, out, shots, seed, s->d.err,
+                                         s->stream, &l));
+    s->launches += (uint64_t)l;
+    return QS_OK;
+  }
+  int slot;
+  uint8_t *h = ring_slot(s, &slot);
+  if (!h) return cuda_fail(s, cudaGetLastError(), "staging event");
+  memcpy(h, q, (size_t)count * 4);
+  const int rc = upload(s, slot, (size_t)count * 4);
+  if (rc) return rc;
+  QS_CUDA(s, launch_frame_measure(FX, FZ, s->d.L.n, fw, reinterpret_cast<uint32_t *>(s->dstage), count, m0, s->d.record,
+                                  out, shots, seed, s->d.err, s->stream));
+  s->launches += (count + 65534) / 65535;
+  return QS_OK;
+}
+
 // Replays a noise op on the frames: targets staged through the pinned ring in
 // chunks (whole pairs for DEPOLARIZE2), target index continued across chunks.
 static int replay_noise(qs_sim *s, const Op &op, uint64_t *FX, uint64_t *FZ, uint32_t fw, uint32_t ow,
@@ -943,16 +965,8 @@ int qs_sim_sample(qs_sim *s, uint64_t shots, uint64_t seed, uint64_t *record, si
           if (qh[end] < n) seen[qh[end]] = sid;
           ++end;
         }
-        int slot;
-        uint8_t *h = ring_slot(s, &slot);
-        if (!h) return cuda_fail(s, cudaGetLastError(), "staging event");
-        memcpy(h, qh + start, (size_t)(end - start) * 4);
-        if ((rc = upload(s, slot, (size_t)(end - start) * 4))) return rc;
-        QS_CUDA(s, launch_frame_measure(FX, FZ, n, (uint32_t)fw,
-                                        reinterpret_cast<uint32_t *>(s->dstage), end - start,
-                                        op.m0 + start, s->d.record, out, shots, seed, s->d.err,
-                                        s->stream));
-        s->launches += (end - start + 65534) / 65535;
+        if ((rc = frame_measure_list(s, FX, FZ, (uint32_t)fw, qh + start, end - start, op.m0 + start, out, shots, seed)))
+          return rc;
         start = end;
       }
     }
@@ -1287,16 +1301,8 @@ extern "C" int qs_sim_sample_noalloc(qs_sim *s, uint64_t shots, uint64_t seed, u
           ++end;
         }
         for (uint32_t i = start; i < end; ++i) g_noalloc_seen[qh[i] >> 6] = 0;
-        int slot;
-        uint8_t *h = ring_slot(s, &slot);
-        if (!h) return cuda_fail(s, cudaGetLastError(), "staging event");
-        memcpy(h, qh + start, (size_t)(end - start) * 4);
-        if ((rc = upload(s, slot, (size_t)(end - start) * 4))) return rc;
-        QS_CUDA(s, launch_frame_measure(FX, FZ, n, (uint32_t)fw,
-                                        reinterpret_cast<uint32_t *>(s->dstage), end - start,
-                                        op.m0 + start, s->d.record, out, shots, seed, s->d.err,
-                                        s->stream));
-        s->launches += (end - start + 65534) / 65535;
+        if ((rc = frame_measure_list(s, FX, FZ, (uint32_t)fw, qh + start, end - start, op.m0 + start, out, shots, seed)))
+          return rc;
         start = end;
       }
     }
