@@ -286,6 +286,37 @@ finalize_kernel(uint64_t *__restrict__ RX, uint64_t *__restrict__ RZ, uint32_t r
 
 static std::atomic<uint64_t> g_rowsum_attr_set{0};
 
+// A measured list of host memory to the device inside a launch: no copy engine, no
+// event, and no slot of the staging ring to wait for.
+template <int MAX>
+struct ListParam {
+  uint32_t q[MAX];
+};
+
+template <int MAX>
+__global__ void __launch_bounds__(256)
+store_list_kernel(uint32_t *__restrict__ dst, uint32_t count, const __grid_constant__ ListParam<MAX> list) {
+  const uint32_t i = blockIdx.x * 256 + threadIdx.x;
+  if (i < count) dst[i] = list.q[i];
+}
+
+template <int MAX>
+static void store_list(uint32_t *dst, const uint32_t *q, uint32_t count, cudaStream_t s) {
+  ListParam<MAX> list;
+  std::copy(q, q + count, list.q);
+  store_list_kernel<MAX><<<(count + 255) / 256, 256, 0, s>>>(dst, count, list);
+}
+
+bool store_list_fits(uint32_t count) { return count <= 2048; }
+
+cudaError_t launch_store_list(uint32_t *dst, const uint32_t *q, uint32_t count, cudaStream_t s) {
+  if (count <= 256)
+    store_list<256>(dst, q, count, s);
+  else
+    store_list<2048>(dst, q, count, s);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_gather(const Dev &d, const uint32_t *qubits, uint32_t i, cudaStream_t s) {
   const Layout &L = d.L;
   gather_kernel<<<(uint32_t)((L.nrows + 255) / 256), 256, 0, s>>>(d.RX, L.rs, L.nrows, L.n, L.k, qubits,

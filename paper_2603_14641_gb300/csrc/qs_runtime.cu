@@ -581,11 +581,16 @@ int qs_sim_measure(qs_sim *s, const uint32_t *qubits, uint32_t count, qs_key key
   const uint32_t chunk = (uint32_t)(s->plan.stage_bytes / 4);
   for (uint32_t off = 0; off < count; off += chunk) {
     const uint32_t c = std::min(chunk, count - off);
-    int slot;
-    uint8_t *h = ring_slot(s, &slot);
-    if (!h) return cuda_fail(s, cudaGetLastError(), "staging event");
-    memcpy(h, qubits + off, (size_t)c * 4);
-    if ((rc = upload(s, slot, (size_t)c * 4))) return rc;
+    if (store_list_fits(c)) {
+      QS_CUDA(s, launch_store_list(reinterpret_cast<uint32_t *>(s->dstage), qubits + off, c, s->stream));
+      s->launches += 1;
+    } else {
+      int slot;
+      uint8_t *h = ring_slot(s, &slot);
+      if (!h) return cuda_fail(s, cudaGetLastError(), "staging event");
+      memcpy(h, qubits + off, (size_t)c * 4);
+      if ((rc = upload(s, slot, (size_t)c * 4))) return rc;
+    }
     if ((rc = measure_staged(s, reinterpret_cast<const uint32_t *>(s->dstage), c, m0 + off, key)))
       return rc;
   }

@@ -28,3 +28,19 @@ def test_windows_of_any_length_sample_the_same(n, count):
         sim.sync()
     for o in out[1:]:
         assert np.array_equal(np.asarray(o).view(np.uint64), out[0])
+
+
+@pytest.mark.parametrize("count", [1, 255, 256, 257, 2_048, 2_049])
+def test_host_lists_equal_device_lists(count):
+    import torch
+    n = 2_100
+    c = C.random_circuit(n, 6, 0.5, seed=n, final_measure_all=False)
+    q = np.random.default_rng(count).integers(0, n, count).astype(np.uint32)
+    a, b = qs.Simulator(n), qs.Simulator(n)
+    for s in (a, b):
+        s.apply_layers_dev(s.upload(c), 0, 6)
+    got = a.measure(q, seed=4)
+    b.measure_dev(torch.from_numpy(q.view(np.int32)).cuda(), seed=4)
+    assert np.array_equal(got, b.record())
+    for u, v in zip(a.export(), b.export()):
+        assert np.array_equal(u, v)
