@@ -117,6 +117,36 @@ inline cudaError_t once_per_device(std::atomic<uint64_t> &done, F set) {
   return e;
 }
 
+// Chains of short kernels on one stream: a kernel launched with launch_chained may
+// become resident while the kernel before it still runs, so that its launch is
+// off the critical path. Every thread calls chain_start before it touches memory:
+// it waits until the kernels before it are complete and their writes visible
+// (every kernel of a chain waits, so a chain is as ordered as plain launches) and
+// then lets the next kernel's blocks take the room that is left.
+// Such a kernel is alive while the one before it writes, so what an earlier
+// kernel of the stream may have written must not be read as read-only data: no
+// __ldg and no const __restrict__ pointers (they compile to loads that need not
+// see another kernel's writes), plain loads or __ldcg.
+__device__ __forceinline__ void chain_start() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <class... P, class... A>
+inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  c.attrs = &attr;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, kernel, args...);
+}
+
 // Optional CUDA-event timing of kernel classes (qs_sim_set_timing): begin/end
 // record an event pair on the stream around a group of launches; pairs are
 // resolved into elapsed milliseconds once their end event has completed.

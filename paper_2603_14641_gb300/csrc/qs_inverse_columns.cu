@@ -67,8 +67,8 @@ constexpr uint32_t kBlock = W <= 8 ? 64 : 32;  // measurements per block
 // before it is known which warp has the pivot, and a step takes one barrier.
 template <int V, int C>
 __global__ void __launch_bounds__(1024)
-inv_lead_kernel(const uint64_t *__restrict__ X, const uint64_t *__restrict__ qsig, uint32_t n, uint32_t k,
-                uint32_t cs, uint32_t stride, const uint32_t *__restrict__ qubits, uint32_t count, uint64_t m0,
+inv_lead_kernel(const uint64_t *X, const uint64_t *qsig, uint32_t n, uint32_t k,
+                uint32_t cs, uint32_t stride, const uint32_t *qubits, uint32_t count, uint64_t m0,
                 uint64_t seed, uint64_t shot, uint8_t *__restrict__ record, uint8_t *__restrict__ kinds,
                 InvLog *__restrict__ log, uint32_t *__restrict__ err) {
   extern __shared__ __align__(16) uint32_t masks[];  // stride words per step; at most 64 KB
@@ -76,6 +76,7 @@ inv_lead_kernel(const uint64_t *__restrict__ X, const uint64_t *__restrict__ qsi
   __shared__ uint4 s_cand[2][32];  // per warp: first target row, the columns' parities
   __shared__ uint2 s_row[2][32];   // the columns' s at that row
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, warps = blockDim.x >> 5;
+  chain_start();
   for (uint32_t i = tid; i < 64; i += blockDim.x) {
     s_q[i] = i < count ? qubits[i] : kNone;
     s_p[i] = kNone;
@@ -103,7 +104,7 @@ inv_lead_kernel(const uint64_t *__restrict__ X, const uint64_t *__restrict__ qsi
     for (int i = 0; i < V; i += 2) {
       const uint32_t w = (V * warp + i) / 2;
       const bool in = valid[c] && w < k;
-      const uint64_t dv = in ? col[w] : 0, sv = in ? col[k + w] : 0;
+      const uint64_t dv = in ? __ldcg(col + w) : 0, sv = in ? __ldcg(col + k + w) : 0;
       d[c][i] = (uint32_t)dv; d[c][i + 1] = (uint32_t)(dv >> 32);
       s[c][i] = (uint32_t)sv; s[c][i + 1] = (uint32_t)(sv >> 32);
       y += __popcll(sv & dv);
@@ -261,7 +262,7 @@ constexpr uint32_t kApplyWarps = W <= 8 ? 32 : 16;
 template <int W>
 __global__ void __launch_bounds__(32 * kApplyWarps<W>)
 inv_apply_kernel(uint64_t *__restrict__ X, uint64_t *__restrict__ Z, uint64_t *__restrict__ qsig, uint32_t n,
-                 uint32_t k, uint32_t cs, uint32_t rs, const InvLog *__restrict__ log) {
+                 uint32_t k, uint32_t cs, uint32_t rs, const InvLog *log) {
   constexpr uint32_t B = kBlock<W>, S = B + 1;  // odd stride: lanes over steps and over words both conflict-free
   extern __shared__ __align__(16) uint32_t sm[];
   __shared__ InvLog lg;
@@ -269,15 +270,16 @@ inv_apply_kernel(uint64_t *__restrict__ X, uint64_t *__restrict__ Z, uint64_t *_
   __shared__ uint64_t s_c[2 * kApplyWarps<W>];
   __shared__ uint32_t s_e[2 * kApplyWarps<W>];
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, warps = blockDim.x >> 5;
+  chain_start();
   const uint32_t steps = log->steps;
   if (steps == 0) return;
   uint32_t *m = sm;                                                 // word w of mask j at w S + j
   uint32_t *colbase = sm + (((size_t)32 * W * S + 3) & ~(size_t)3) + (size_t)warp * 4 * 32 * W;
   const uint32_t *gm = reinterpret_cast<const uint32_t *>(log + 1);
   for (uint32_t i = tid; i < sizeof(InvLog) / 4; i += blockDim.x)
-    reinterpret_cast<uint32_t *>(&lg)[i] = reinterpret_cast<const uint32_t *>(log)[i];
+    reinterpret_cast<uint32_t *>(&lg)[i] = __ldcg(reinterpret_cast<const uint32_t *>(log) + i);
 #pragma unroll 4
-  for (uint32_t i = tid; i < steps * 32 * W; i += blockDim.x) m[(size_t)(i % (32 * W)) * S + i / (32 * W)] = gm[i];
+  for (uint32_t i = tid; i < steps * 32 * W; i += blockDim.x) m[(size_t)(i % (32 * W)) * S + i / (32 * W)] = __ldcg(gm + i);
   for (uint32_t i = steps * 32 * W + tid; i < B * 32 * W; i += blockDim.x)
     m[(size_t)(i % (32 * W)) * S + i / (32 * W)] = 0;
   const uint32_t rounds = (n + gridDim.x * warps - 1) / (gridDim.x * warps);
@@ -453,9 +455,9 @@ cudaError_t measure_columns(const Dev &d, const uint32_t *qubits, uint32_t count
   const uint32_t warps = std::max(4u, std::min(kApplyWarps<W>, (L.n + sms - 1) / sms));
   for (uint32_t off = 0; off < count; off += B) {
     const uint32_t c = std::min(B, count - off);
-    lead<<<1, 32 * lead_warps, lead_smem, s>>>(d.X, d.qsig, L.n, L.k, L.cs, 32 * W, qubits + off, c, m0 + off, key.seed,
+    launch_chained(lead, 1, 32 * lead_warps, lead_smem, s, d.X, d.qsig, L.n, L.k, L.cs, 32 * W, qubits + off, c, m0 + off, key.seed,
                                                key.shot, d.record, d.kinds, log, d.err);
-    inv_apply_kernel<W><<<grid, 32 * warps, apply_smem(warps), s>>>(d.X, d.Z, d.qsig, L.n, L.k, L.cs, L.rs, log);
+    launch_chained(inv_apply_kernel<W>, grid, 32 * warps, apply_smem(warps), s, d.X, d.Z, d.qsig, L.n, L.k, L.cs, L.rs, log);
     if (launches) *launches += 2;
   }
   return cudaGetLastError();
