@@ -196,6 +196,7 @@ struct NoiseGroup {
 __global__ void __launch_bounds__(kNoiseThreads)
 frame_noise_kernel(uint64_t *__restrict__ FX, uint64_t *__restrict__ FZ, uint32_t fw, uint32_t ow,
                    const __grid_constant__ NoiseGroup G) {
+  chain_start();
   int o = 0;
   while (o + 1 < G.ops && blockIdx.x >= G.op[o + 1].first_block) ++o;
   const uint32_t *targets = G.op[o].targets;
@@ -350,7 +351,7 @@ cudaError_t launch_frame_noise(uint64_t *FX, uint64_t *FZ, uint32_t fw, uint32_t
     if (blocks > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
   }
   if (G.ops == 0) return cudaSuccess;
-  frame_noise_kernel<<<(unsigned)blocks, kNoiseThreads, 0, s>>>(FX, FZ, fw, ow, G);
+  launch_chained(frame_noise_kernel, (unsigned)blocks, kNoiseThreads, 0, s, FX, FZ, fw, ow, G);
   if (launches) *launches += 1;
   return cudaGetLastError();
 }

@@ -234,11 +234,12 @@ __device__ __forceinline__ void gate_block(uint64_t *__restrict__ X, uint64_t *_
 template <bool SIGNS, int INFLIGHT>
 __global__ void __launch_bounds__(256, INFLIGHT == 2 ? 4 : 6)
 gate_layer_kernel(uint64_t *__restrict__ X, uint64_t *__restrict__ Z, uint64_t *__restrict__ S,
-                  uint32_t n, uint32_t cs, const uint32_t *__restrict__ packed, uint32_t n_gates,
+                  uint32_t n, uint32_t cs, const uint32_t *packed, uint32_t n_gates,
                   uint32_t P, uint32_t lanes, uint32_t gpl, uint32_t *__restrict__ err) {
+  chain_start();
   const uint32_t group = lanes * gpl, g0 = blockIdx.x * group;
   gate_block<SIGNS, INFLIGHT>(
-      X, Z, S, n, cs, [&](uint32_t g) { return make_uint2(__ldg(packed + 2 * g), __ldg(packed + 2 * g + 1)); }, g0,
+      X, Z, S, n, cs, [&](uint32_t g) { return make_uint2(packed[2 * g], packed[2 * g + 1]); }, g0,
       min(g0 + group, n_gates), P, lanes, err);
 }
 
@@ -260,6 +261,7 @@ __global__ void __launch_bounds__(256, 4)
 param_layer_kernel(uint64_t *__restrict__ X, uint64_t *__restrict__ Z, uint64_t *__restrict__ S, uint32_t n, uint32_t cs,
                    uint32_t n_gates, uint32_t P, uint32_t lanes, uint32_t gpl, uint32_t *__restrict__ err,
                    const __grid_constant__ ParamLayer<MAX> layer) {
+  chain_start();
   __shared__ uint32_t rec[kParamGroup];
   const uint32_t group = lanes * gpl, g0 = blockIdx.x * group, g1 = min(g0 + group, n_gates);
   for (uint32_t i = threadIdx.x; g0 + i < g1; i += blockDim.x) rec[i] = layer.rec[g0 + i];
@@ -301,7 +303,7 @@ cudaError_t launch_gate_layer(const Dev &d, const uint32_t *packed, uint32_t n_g
                               cudaStream_t s) {
   if (n_gates == 0) return cudaSuccess;
   GateGrid g = gate_grid(d.L.cs / 2, n_gates);
-  gate_layer_kernel<true, 2><<<g.grid, g.block, 0, s>>>(d.X, d.Z, d.S, d.L.n, d.L.cs, packed, n_gates,
+  launch_chained(gate_layer_kernel<true, 2>, g.grid, g.block, 0, s, d.X, d.Z, d.S, d.L.n, d.L.cs, packed, n_gates,
                                                      g.P, g.lanes, g.gpl, d.err);
   return cudaGetLastError();
 }
@@ -314,7 +316,7 @@ static void launch_param(const Dev &d, const uint32_t *packed, uint32_t n_gates,
   GateGrid g = gate_grid(d.L.cs / 2, n_gates);
   g.gpl = std::max(1u, std::min(g.gpl, kParamGroup / g.lanes));
   g.grid.x = (n_gates + g.lanes * g.gpl - 1) / (g.lanes * g.gpl);
-  param_layer_kernel<MAX><<<g.grid, g.block, 0, s>>>(d.X, d.Z, d.S, d.L.n, d.L.cs, n_gates, g.P, g.lanes, g.gpl, d.err,
+  launch_chained(param_layer_kernel<MAX>, g.grid, g.block, 0, s, d.X, d.Z, d.S, d.L.n, d.L.cs, n_gates, g.P, g.lanes, g.gpl, d.err,
                                                      layer);
 }
 
@@ -336,10 +338,10 @@ cudaError_t launch_frame_layer(uint64_t *FX, uint64_t *FZ, uint32_t n, uint32_t 
   if (n_gates == 0) return cudaSuccess;
   GateGrid g = gate_grid(fw / 2, n_gates);
   if (g.lanes == 1)  // long frame columns (>= 512 shot words): as the tableau, two gates in flight
-    gate_layer_kernel<false, 2><<<g.grid, g.block, 0, s>>>(FX, FZ, nullptr, n, fw, packed, n_gates,
+    launch_chained(gate_layer_kernel<false, 2>, g.grid, g.block, 0, s, FX, FZ, nullptr, n, fw, packed, n_gates,
                                                         g.P, g.lanes, g.gpl, err);
   else
-    gate_layer_kernel<false, 1><<<g.grid, g.block, 0, s>>>(FX, FZ, nullptr, n, fw, packed, n_gates,
+    launch_chained(gate_layer_kernel<false, 1>, g.grid, g.block, 0, s, FX, FZ, nullptr, n, fw, packed, n_gates,
                                                         g.P, g.lanes, g.gpl, err);
   return cudaGetLastError();
 }
@@ -391,7 +393,7 @@ __device__ __forceinline__ void lazy_prepare(const LazyArgs &a) {
     for (int i = 0; i < kPrepGates; ++i) {
       const uint32_t g = b0 + i * T + t;
       in[i] = make_uint2(QS_I << 24, 0);
-      if (g < items) in[i] = a.next ? __ldg(a.next + g) : make_uint2(QS_I << 24 | g, 0);
+      if (g < items) in[i] = a.next ? __ldcg(a.next + g) : make_uint2(QS_I << 24 | g, 0);
     }
 #pragma unroll
     for (int i = 0; i < kPrepGates; ++i) {
@@ -458,6 +460,7 @@ __device__ __forceinline__ void lazy_word(uint32_t type, uint32_t opa, uint32_t 
 // As gate_layer_kernel, two gates in flight a thread; the layer's gates are
 // split evenly over gx blocks (their number is known on the device only).
 __global__ void __launch_bounds__(256, 4) lazy_layer_kernel(const LazyArgs a) {
+  chain_start();
   if (blockIdx.x < a.prep_blocks) {
     if (blockIdx.x == 0 && threadIdx.x == 0) a.L.count[(a.step + 2) % 3] = 0;
     lazy_prepare(a);
@@ -567,7 +570,7 @@ cudaError_t launch_lazy_layers(const Dev &d, void *scratch, const uint32_t *pack
     a.gx = i ? (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(blocks_x, (gates + g.lanes - 1) / g.lanes)) : 0;
     a.prep_blocks = (uint32_t)std::min<uint64_t>(kLazyPrepBlocks, (next + threads * kPrepGates - 1) / (threads * kPrepGates));
     const uint32_t blocks = a.prep_blocks + a.gx * chunks;
-    if (blocks) lazy_layer_kernel<<<blocks, threads, 0, s>>>(a);
+    if (blocks) launch_chained(lazy_layer_kernel, blocks, threads, 0, s, a);
     gates = i < todo.size() ? std::min<uint64_t>(next, std::max(1u, n / 2)) : n;
   }
   if (launches) *launches += (int)todo.size() + 2;

@@ -155,9 +155,10 @@ __device__ __forceinline__ void gate_signs(uint32_t type, Signs &g, const int *e
 __global__ void __launch_bounds__(256)
 inv_gate_layer_kernel(uint64_t *__restrict__ X, uint64_t *__restrict__ Z, uint64_t *__restrict__ qsig,
                       uint32_t n, uint32_t k, uint32_t cs, uint32_t rs,
-                      const uint32_t *__restrict__ packed, uint32_t *__restrict__ err) {
+                      const uint32_t *packed, uint32_t *__restrict__ err) {
+  chain_start();
   const uint32_t g = blockIdx.x;
-  const uint32_t w0 = __ldg(packed + 2 * g), qb = __ldg(packed + 2 * g + 1);
+  const uint32_t w0 = packed[2 * g], qb = packed[2 * g + 1];
   const uint32_t type = w0 >> 24, qa = w0 & 0xFFFFFFu;
   const bool two = inv_two(type);
   if (qa >= n || type >= QS_NUM_GATE_TYPES || (two && (qb >= n || qb == qa))) {
@@ -236,7 +237,7 @@ cudaError_t launch_inv_gate_layer(const Dev &d, const uint32_t *packed, uint32_t
   if (n_gates == 0) return cudaSuccess;
   const Layout &L = d.L;
   const uint32_t threads = L.k >= 256 ? 256 : (L.k >= 128 ? 128 : (L.k >= 64 ? 64 : 32));
-  inv_gate_layer_kernel<<<n_gates, threads, 0, s>>>(d.X, d.Z, d.qsig, L.n, L.k, L.cs, L.rs, packed, d.err);
+  launch_chained(inv_gate_layer_kernel, n_gates, threads, 0, s, d.X, d.Z, d.qsig, L.n, L.k, L.cs, L.rs, packed, d.err);
   return cudaGetLastError();
 }
 
