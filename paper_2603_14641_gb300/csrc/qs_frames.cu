@@ -25,6 +25,7 @@ namespace qs {
 
 // fw is a multiple of 4: one Philox block fills 4 consecutive shot words
 __global__ void frame_init_kernel(uint64_t *__restrict__ FZ, uint32_t n, uint32_t fw, uint64_t seed) {
+  chain_start();
   const uint64_t idx = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const uint32_t quads = fw >> 2;
   const uint64_t total = (uint64_t)n * quads;
@@ -41,7 +42,7 @@ cudaError_t launch_frame_init(uint64_t *FX, uint64_t *FZ, uint32_t n, uint32_t f
   cudaError_t e = cudaMemsetAsync(FX, 0, (size_t)n * fw * sizeof(uint64_t), s);
   if (e != cudaSuccess) return e;
   const uint64_t total = (uint64_t)n * (fw >> 2);
-  frame_init_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(FZ, n, fw, seed);
+  launch_chained(frame_init_kernel, (unsigned)((total + 255) / 256), 256, 0, s, FZ, n, fw, seed);
   return cudaGetLastError();
 }
 
@@ -60,11 +61,12 @@ struct ParamQubits {
 };
 
 template <class Qubits>
-__global__ void frame_measure_kernel(const uint64_t *__restrict__ FX, uint64_t *__restrict__ FZ,
+__global__ void frame_measure_kernel(const uint64_t *FX, uint64_t *__restrict__ FZ,
                                      uint32_t n, uint32_t fw, const __grid_constant__ Qubits qubits,
-                                     uint64_t m0, const uint8_t *__restrict__ ref,
+                                     uint64_t m0, const uint8_t *ref,
                                      uint64_t *__restrict__ out, uint64_t shots, uint64_t seed,
                                      uint32_t *__restrict__ err) {
+  chain_start();
   const uint32_t i = blockIdx.y;
   const uint32_t j4 = blockIdx.x * blockDim.x + threadIdx.x;
   if (j4 >= (fw >> 2)) return;
@@ -99,7 +101,7 @@ static void frame_measure(uint64_t *FX, uint64_t *FZ, uint32_t n, uint32_t fw, c
   const uint32_t quads = fw >> 2;
   const uint32_t threads = quads < 128 ? ((quads + 31) / 32) * 32 : 128;
   const dim3 grid((quads + threads - 1) / threads, count);
-  frame_measure_kernel<<<grid, threads, 0, s>>>(FX, FZ, n, fw, qubits, m0, ref, out, shots, seed, err);
+  launch_chained(frame_measure_kernel<Qubits>, grid, threads, 0, s, FX, FZ, n, fw, qubits, m0, ref, out, shots, seed, err);
 }
 
 cudaError_t launch_frame_measure(uint64_t *FX, uint64_t *FZ, uint32_t n, uint32_t fw,

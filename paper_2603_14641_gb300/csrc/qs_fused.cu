@@ -279,8 +279,9 @@ static cudaError_t launch_fused_r(const FusedArgs &a, uint32_t threads, uint32_t
 template <bool SIGNS, int R, int D>
 __global__ void __launch_bounds__(1024)
 fused_direct_kernel(uint64_t *__restrict__ X, uint64_t *__restrict__ Z, uint64_t *__restrict__ S, uint32_t n,
-                    uint32_t stride, const uint2 *__restrict__ packed, const __grid_constant__ LayerOffsets o,
+                    uint32_t stride, const uint2 *packed, const __grid_constant__ LayerOffsets o,
                     uint32_t layers, uint32_t *__restrict__ err) {
+  chain_start();
   extern __shared__ __align__(16) uint8_t fsm[];
   __shared__ uint32_t s_sign[2];
   uint64_t *sx = reinterpret_cast<uint64_t *>(fsm), *sz = sx + n;
@@ -331,7 +332,7 @@ fused_direct_kernel(uint64_t *__restrict__ X, uint64_t *__restrict__ Z, uint64_t
 #pragma unroll
     for (int i = 0; i < R; ++i)
       if (a + t + i * T < b) gate(ring[((l % D) * R + i) * T + t]);
-    for (uint32_t g = a + t + R * T; g < b; g += T) gate(__ldg(packed + g));
+    for (uint32_t g = a + t + R * T; g < b; g += T) gate(packed[g]);
     __syncthreads();
   }
   if (bad && blockIdx.x == 0) atomicOr(err, kErrBadGate);
@@ -361,8 +362,7 @@ static cudaError_t launch_direct_t(uint64_t *X, uint64_t *Z, uint64_t *S, uint32
                                 (int)kFusedSmemMax);
   });
   if (e != cudaSuccess) return e;
-  fused_direct_kernel<SIGNS, R, D>
-      <<<nwords, threads, direct_smem(n, threads, R, D), s>>>(X, Z, S, n, stride, gates, o, L, err);
+  launch_chained(fused_direct_kernel<SIGNS, R, D>, nwords, threads, direct_smem(n, threads, R, D), s, X, Z, S, n, stride, gates, o, L, err);
   return cudaGetLastError();
 }
 

@@ -70,8 +70,9 @@ __global__ void init_signs_kernel(uint64_t *__restrict__ S, const uint8_t *__res
 // which the reset call 14 -> 6.
 __global__ void __launch_bounds__(256)
 init_all_kernel(uint64_t *__restrict__ X, uint64_t *__restrict__ Z, uint64_t *__restrict__ S,
-                const uint8_t *__restrict__ init, uint32_t n, uint32_t k, uint32_t cs, uint32_t words,
+                const uint8_t *init, uint32_t n, uint32_t k, uint32_t cs, uint32_t words,
                 int64_t *__restrict__ mst, uint32_t *__restrict__ err) {
+  chain_start();
   const uint32_t t = blockIdx.x * 256 + threadIdx.x;
   for (uint32_t i = t; i < words; i += gridDim.x * 256) {
     const uint32_t q = i / cs, w = i - q * cs;
@@ -90,7 +91,7 @@ cudaError_t launch_init_all(const Dev &d, const uint8_t *initstate_dev, cudaStre
   const Layout &L = d.L;
   const uint32_t words = L.ncols * L.cs;  // at least cs and kMeasStateWords
   const uint32_t blocks = std::min<uint32_t>((words + 255) / 256, 16u * (uint32_t)d.sms);
-  init_all_kernel<<<blocks, 256, 0, s>>>(d.X, d.Z, d.S, initstate_dev, L.n, L.k, L.cs, words, d.mst, d.err);
+  launch_chained(init_all_kernel, blocks, 256, 0, s, d.X, d.Z, d.S, initstate_dev, L.n, L.k, L.cs, words, d.mst, d.err);
   return cudaGetLastError();
 }
 

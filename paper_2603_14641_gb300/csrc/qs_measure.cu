@@ -296,6 +296,7 @@ struct ListParam {
 template <int MAX>
 __global__ void __launch_bounds__(256)
 store_list_kernel(uint32_t *__restrict__ dst, uint32_t count, const __grid_constant__ ListParam<MAX> list) {
+  chain_start();
   const uint32_t i = blockIdx.x * 256 + threadIdx.x;
   if (i < count) dst[i] = list.q[i];
 }
@@ -304,7 +305,7 @@ template <int MAX>
 static void store_list(uint32_t *dst, const uint32_t *q, uint32_t count, cudaStream_t s) {
   ListParam<MAX> list;
   std::copy(q, q + count, list.q);
-  store_list_kernel<MAX><<<(count + 255) / 256, 256, 0, s>>>(dst, count, list);
+  launch_chained(store_list_kernel<MAX>, (count + 255) / 256, 256, 0, s, dst, count, list);
 }
 
 bool store_list_fits(uint32_t count) { return count <= 2048; }

@@ -67,8 +67,9 @@ __device__ __forceinline__ void transpose64(uint64_t &lo, uint64_t &hi, int lane
 // in:  rows_in x words_in (stride in_stride words); out: rows_out x words_out
 // grid.x = words_in / 4, grid.y = rows_in / 256 (both exact by construction)
 __global__ void __launch_bounds__(128)
-bit_transpose_kernel(const uint64_t *__restrict__ in, size_t in_stride, uint64_t *__restrict__ out,
+bit_transpose_kernel(const uint64_t *in, size_t in_stride, uint64_t *__restrict__ out,
                      size_t out_stride) {
+  chain_start();
   __shared__ uint64_t tile[256][5];  // [output row within block][output word], padded
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const size_t j0 = (size_t)blockIdx.x * 4;        // input word group
@@ -406,7 +407,7 @@ static cudaError_t transpose(const uint64_t *in, size_t in_stride, size_t rows_i
                                 err, s);
   // rows_in is a multiple of 256 and words_in of 4 by construction
   dim3 grid((unsigned)(words_in / 4), (unsigned)(rows_in / 256));
-  bit_transpose_kernel<<<grid, 128, 0, s>>>(in, in_stride, out, out_stride);
+  launch_chained(bit_transpose_kernel, grid, 128, 0, s, in, in_stride, out, out_stride);
   return cudaGetLastError();
 }
 
