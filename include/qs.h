@@ -107,11 +107,11 @@ typedef struct qs_options {
  * of the default (CHP) mode under gates, read by columns; per-row signs are
  * not kept (exports give 0 there). Measurements run Alg. 1 (pivot = smallest
  * anticommuting stabilizer, CX injections into the later ones, an H or H_YZ
- * and an X injection on the pivot), four launches each; records and
- * measurement kinds equal the CHP mode's under the same keys, and the state
+ * and an X injection on the pivot): up to 64 at once in two launches up to
+ * 16,384 qubits, four launches each beyond; records and measurement kinds
+ * equal the CHP mode's under the same keys, and the state
  * is the same, though the tableau bits after a measurement differ. Layers
- * run one launch each (no fused segments); measurements are never blocked;
- * qs_sim_tableau_import is refused. Fixed at create. */
+ * run one launch each (no fused segments); qs_sim_tableau_import is refused. Fixed at create. */
 #define QS_FLAG_INVERSE_TABLEAU 32u
 
 typedef struct qs_sim qs_sim;
@@ -376,7 +376,7 @@ int qs_sim_sample_noalloc(qs_sim *sim, uint64_t shots, uint64_t seed, uint64_t *
                           size_t record_words);
 
 /* ---------------------------------------------------------------------- */
-/* Batched persistent launch: many independent circuits, one kernel launch */
+/* Batched launch: many independent circuits at once                      */
 /* ---------------------------------------------------------------------- */
 
 /*

@@ -66,8 +66,7 @@ __global__ void init_signs_kernel(uint64_t *__restrict__ S, const uint8_t *__res
 }
 
 // Small tableaus: everything a reset writes in one launch, where three memsets and
-// three kernels are six launches: job of 256 qubits 311 -> 298 us of
-// which the reset call 14 -> 6.
+// three kernels are six launches: job of 256 qubits 311 -> 298 us (the call 14 -> 6).
 __global__ void __launch_bounds__(256)
 init_all_kernel(uint64_t *__restrict__ X, uint64_t *__restrict__ Z, uint64_t *__restrict__ S,
                 const uint8_t *init, uint32_t n, uint32_t k, uint32_t cs, uint32_t words,
