@@ -533,6 +533,7 @@ struct BSampleCirc {
   uint64_t *out;                  // [M][ow] words
 };
 
+constexpr uint64_t kPinnedRecordsMax = 64ull << 20;
 constexpr uint32_t kSampleStages = 3;
 
 __global__ void __launch_bounds__(128)
@@ -626,6 +627,21 @@ batch_sample_kernel(const BCirc *__restrict__ circs, const BSampleCirc *__restri
   }
 }
 
+// Every circuit's record into pinned host memory, a block each, at the end of a
+// run: a copy per record read took 16 us, 0.9 of the 3.2 ms of a batch of 56 circuits.
+struct RecordCopy {
+  const uint8_t *src;  // 16-byte aligned, as dst
+  uint8_t *dst;
+  uint64_t bytes;
+};
+
+__global__ void __launch_bounds__(256) batch_records_kernel(const RecordCopy *__restrict__ table) {
+  const RecordCopy c = table[blockIdx.x];
+  for (uint64_t i = threadIdx.x; i < c.bytes / 16; i += 256)
+    reinterpret_cast<uint4 *>(c.dst)[i] = reinterpret_cast<const uint4 *>(c.src)[i];
+  for (uint64_t i = c.bytes / 16 * 16 + threadIdx.x; i < c.bytes; i += 256) c.dst[i] = c.src[i];
+}
+
 }  // namespace qs
 
 using namespace qs;
@@ -692,6 +708,9 @@ struct qs_batch {
   bool pending = false;                 // work enqueued since the last successful qs_batch_sync
   bool persistent_ran = false;          // the last run gave a launch shape: n < kBatchSimMinQubits ran there
   std::vector<int32_t> sim_of;          // per circuit: index into sims, or -1
+  uint8_t *h_rec = nullptr;             // pinned: RecordCopy table, then every circuit's record
+  std::vector<uint64_t> rec_off;        // per circuit: its record in h_rec
+  bool rec_ready = false;               // h_rec holds (in stream order) the last run's records
   std::vector<BSim> sims;
   std::vector<cudaStream_t> wstreams;   // worker streams of the large circuits
   std::vector<cudaEvent_t> wevents;
@@ -1121,6 +1140,24 @@ int qs_batch_create(uint32_t count, const qs_batch_circuit *cc, void *stream, vo
     delete b;
     return rc;
   }
+  // without the pinned memory records are read one copy at a time
+  uint64_t bytes = ((uint64_t)count * sizeof(RecordCopy) + 255) / 256 * 256;
+  b->rec_off.resize(count);
+  for (uint32_t i = 0; i < count; ++i) {
+    b->rec_off[i] = bytes;
+    bytes += (b->meas_total[i] + 255) / 256 * 256;
+  }
+  if (bytes <= kPinnedRecordsMax && cudaMallocHost(reinterpret_cast<void **>(&b->h_rec), bytes) == cudaSuccess) {
+    memset(b->h_rec, 0, bytes);
+    RecordCopy *t = reinterpret_cast<RecordCopy *>(b->h_rec);
+    for (uint32_t i = 0; i < count; ++i) {
+      const BSim *x = b->sim_of[i] >= 0 ? &b->sims[b->sim_of[i]] : nullptr;
+      t[i] = {x && !x->mid ? sim_record(x->sim) : b->circs[i].record, b->h_rec + b->rec_off[i], b->meas_total[i]};
+    }
+  } else {
+    cudaGetLastError();
+    b->h_rec = nullptr;
+  }
   *out = b;
   return QS_OK;
 }
@@ -1129,6 +1166,7 @@ int qs_batch_destroy(qs_batch *b) {
   if (!b) return QS_OK;
   cudaStreamSynchronize(b->stream);
   free_sims(b);
+  if (b->h_rec) cudaFreeHost(b->h_rec);
   if (b->owns && b->ws) cudaFree(b->ws);
   delete b;
   return QS_OK;
@@ -1245,6 +1283,7 @@ static int batch_run(qs_batch *b, const qs_batch_tuning *tuning, uint32_t round_
   if (b->broken) return bfail(QS_ERR_STATE, "batch is unusable after an earlier device error");
   const bool persistent = tuning && tuning->threads != 0;
   b->pending = true;
+  b->rec_ready = false;
   size_t smem = 0;
   int rc = QS_OK;
   if (persistent && (rc = tuning_ok(b, *tuning, &smem))) return rc;
@@ -1264,8 +1303,17 @@ static int batch_run(qs_batch *b, const qs_batch_tuning *tuning, uint32_t round_
   } else if ((rc = run_resident(b, round_limit))) {
     return rc;
   }
-  if (sims) rc = run_sims(b, round_limit ? round_limit : 0xFFFFFFFFu);
-  return rc;
+  if (sims && (rc = run_sims(b, round_limit ? round_limit : 0xFFFFFFFFu))) return rc;
+  if (b->h_rec) {
+    batch_records_kernel<<<b->count, 256, 0, b->stream>>>(reinterpret_cast<const RecordCopy *>(b->h_rec));
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) {
+      b->broken = true;
+      return bfail(QS_ERR_CUDA, std::string("batch records: ") + cudaGetErrorString(e));
+    }
+    b->rec_ready = true;
+  }
+  return QS_OK;
 }
 
 static int run_kernel(qs_batch *b, const qs_batch_tuning &tuning, uint32_t round_limit) {
@@ -1354,7 +1402,12 @@ int qs_batch_record(qs_batch *b, uint32_t circuit, uint8_t *dst, size_t count) {
   if (count && !dst) return bfail(QS_ERR_ARG, "dst is NULL");
   int rc = qs_batch_sync(b);
   if (rc) return rc;
-  if (BSim *x = sim_of(b, circuit)) {
+  BSim *x = sim_of(b, circuit);
+  if (b->rec_ready && (!x || count <= qs_sim_num_measurements(x->sim))) {
+    if (count) memcpy(dst, b->h_rec + b->rec_off[circuit], count);
+    return QS_OK;
+  }
+  if (x) {
     rc = count ? qs_sim_record(x->sim, 0, count, dst) : QS_OK;
     return rc ? bfail(rc, qs_last_error()) : QS_OK;
   }

@@ -36,3 +36,21 @@ def test_passes_of_eight_and_samples_equal_a_simulator():
             assert np.array_equal(u, v), c.n
         want = s.sample(shots[i], 7 + i, on_device=False)
         assert np.array_equal(words[i].cpu().numpy().view(np.uint64), want), c.n
+
+
+def test_records_follow_the_last_run():
+    """Records after a partial run, a whole one and a partial one again; a count beyond what a
+    simulator's circuit has measured is refused."""
+    sizes = [50, 640, 700, 1_100]
+    circs = [_circuit(n) for n in sizes]
+    b = qs.Batch(circs, [1, 2, 3, 4])
+    want = [qs.Simulator(c.n).run(c, seed=i + 1) for i, c in enumerate(circs)]
+    lib, ptr = qs.lib(), qs.ctypes.c_void_p
+    for limit, m in ((2, 15), (0, 42), (1, 7)):
+        b.run(None, round_limit=limit)
+        for i in range(len(sizes)):
+            out = np.full(m, 9, np.uint8)
+            assert lib.qs_batch_record(ptr(b.h), i, out.ctypes.data, m) == 0
+            assert np.array_equal(out, want[i][:m]), (limit, sizes[i])
+        out = np.zeros(42, np.uint8)
+        assert (lib.qs_batch_record(ptr(b.h), 3, out.ctypes.data, 42) == 0) == (limit == 0)
