@@ -286,6 +286,8 @@ struct NoiseOp {
 cudaError_t launch_frame_noise(uint64_t *FX, uint64_t *FZ, uint32_t fw, uint32_t ow, const NoiseOp *ops, int n,
                                uint64_t seed, cudaStream_t s, int *launches);
 cudaError_t launch_reset_meas_state(const Dev &d, cudaStream_t s);
+// words [first, first + count) of the ROWS_PACKED export into out (device or pinned)
+cudaError_t launch_export_rows(const Dev &d, uint64_t *out, uint64_t first, uint64_t count, cudaStream_t s);
 // a list of up to 2,048 words from host memory to the device, in a launch
 bool store_list_fits(uint32_t count);
 cudaError_t launch_store_list(uint32_t *dst, const uint32_t *q, uint32_t count, cudaStream_t s);

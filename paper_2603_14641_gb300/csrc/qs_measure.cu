@@ -286,6 +286,36 @@ finalize_kernel(uint64_t *__restrict__ RX, uint64_t *__restrict__ RZ, uint32_t r
 
 static std::atomic<uint64_t> g_rowsum_attr_set{0};
 
+// ROWS_PACKED: 2n rows of k x words and k z words, then the 2n signs bit by bit
+__global__ void __launch_bounds__(256)
+export_rows_kernel(const uint64_t *RX, const uint64_t *RZ, const uint64_t *S, uint32_t rs, uint32_t n, uint32_t k,
+                   uint64_t *__restrict__ out, uint64_t first, uint64_t count) {
+  const uint64_t rows = 4ull * n * k;
+  for (uint64_t i = (uint64_t)blockIdx.x * 256 + threadIdx.x; i < count; i += (uint64_t)gridDim.x * 256) {
+    const uint64_t at = first + i;
+    if (at < rows) {
+      const uint64_t r = at / (2 * k), pr = r < n ? r : 64ull * k + (r - n);
+      const uint32_t u = (uint32_t)(at - r * 2 * k);
+      out[i] = u < k ? RX[pr * rs + u] : RZ[pr * rs + u - k];
+      continue;
+    }
+    uint64_t v = 0;
+    const uint64_t b0 = (at - rows) * 64;
+    for (uint64_t b = b0; b < b0 + 64 && b < 2ull * n; ++b) {
+      const uint64_t pr = b < n ? b : 64ull * k + (b - n);
+      v |= ((S[pr >> 6] >> (pr & 63)) & 1ull) << (b - b0);
+    }
+    out[i] = v;
+  }
+}
+
+cudaError_t launch_export_rows(const Dev &d, uint64_t *out, uint64_t first, uint64_t count, cudaStream_t s) {
+  const Layout &L = d.L;
+  const uint32_t blocks = (uint32_t)std::min<uint64_t>((count + 255) / 256, 8ull * d.sms);
+  export_rows_kernel<<<blocks, 256, 0, s>>>(d.RX, d.RZ, d.S, L.rs, L.n, L.k, out, first, count);
+  return cudaGetLastError();
+}
+
 // A measured list of host memory to the device inside a launch: no copy engine, no
 // event, and no slot of the staging ring to wait for.
 template <int MAX>

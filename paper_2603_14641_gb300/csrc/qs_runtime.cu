@@ -1014,6 +1014,19 @@ int qs_sim_tableau_export(qs_sim *s, int layout, void *dst, size_t dst_bytes, si
     return qs_sim_sync(s);
   }
   if ((rc = ensure_rows(s))) return rc;
+  const size_t row_words = 2ull * n * 2 * k, sign_words = (2ull * n + 63) / 64;
+  if (bytes <= s->plan.stage_bytes && !is_device_ptr(dst)) {
+    // small: packed straight into pinned memory, where five copies to pageable
+    // memory take a synchronisation each
+    int slot;
+    uint8_t *h = ring_slot(s, &slot);
+    if (!h) return cuda_fail(s, cudaGetLastError(), "staging event");
+    QS_CUDA(s, launch_export_rows(s->d, reinterpret_cast<uint64_t *>(h), 0, row_words + sign_words, s->stream));
+    s->launches += 1;
+    if ((rc = qs_sim_sync(s))) return rc;
+    memcpy(dst, h, bytes);
+    return QS_OK;
+  }
   const size_t dp = 2ull * k * 8, sp = (size_t)L.rs * 8, wb = (size_t)k * 8;
   QS_CUDA(s, cudaMemcpy2DAsync(o, dp, s->d.RX, sp, wb, n, cudaMemcpyDefault, s->stream));
   QS_CUDA(s, cudaMemcpy2DAsync(o + k, dp, s->d.RZ, sp, wb, n, cudaMemcpyDefault, s->stream));
@@ -1022,17 +1035,11 @@ int qs_sim_tableau_export(qs_sim *s, int layout, void *dst, size_t dst_bytes, si
                                s->stream));
   QS_CUDA(s, cudaMemcpy2DAsync(o + (size_t)n * 2 * k + k, dp, s->d.RZ + st, sp, wb, n,
                                cudaMemcpyDefault, s->stream));
-  std::vector<uint64_t> S(L.cs);
-  QS_CUDA(s, cudaMemcpyAsync(S.data(), s->d.S, (size_t)L.cs * 8, cudaMemcpyDeviceToHost, s->stream));
-  if ((rc = qs_sim_sync(s))) return rc;
-  const size_t sw = (2ull * n + 63) / 64;
-  std::vector<uint64_t> sig(sw, 0);
-  for (uint64_t i = 0; i < 2ull * n; ++i) {
-    const uint64_t pr = i < n ? i : 64ull * k + (i - n);
-    if ((S[pr >> 6] >> (pr & 63)) & 1u) sig[i >> 6] |= 1ull << (i & 63);
-  }
-  QS_CUDA(s, cudaMemcpy(o + 2ull * n * 2 * k, sig.data(), sw * 8, cudaMemcpyDefault));
-  return QS_OK;
+  // the signs of the 2n rows, next to each other (dst may be memory no kernel here can write)
+  QS_CUDA(s, launch_export_rows(s->d, reinterpret_cast<uint64_t *>(s->dstage), row_words, sign_words, s->stream));
+  s->launches += 1;
+  QS_CUDA(s, cudaMemcpyAsync(o + row_words, s->dstage, sign_words * 8, cudaMemcpyDefault, s->stream));
+  return qs_sim_sync(s);
 }
 
 // Words of a W-word NATIVE vector that hold bits belonging to no generator
