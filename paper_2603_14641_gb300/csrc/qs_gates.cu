@@ -365,7 +365,7 @@ struct LazyArgs {
   uint64_t *X, *Z, *S;
   uint32_t cs, n, P, lanes, gx;  // gx: blocks over the layer's gates
   uint32_t prep_blocks;          // first blocks of the grid: the next layer's records
-  const uint2 *next;             // its gates, or nullptr: list what is pending
+  const uint32_t *next;          // its gates (4-byte aligned), or nullptr: list what is pending
   uint32_t next_gates;
   uint32_t step;
   LazyScratch L;
@@ -393,7 +393,8 @@ __device__ __forceinline__ void lazy_prepare(const LazyArgs &a) {
     for (int i = 0; i < kPrepGates; ++i) {
       const uint32_t g = b0 + i * T + t;
       in[i] = make_uint2(QS_I << 24, 0);
-      if (g < items) in[i] = a.next ? __ldcg(a.next + g) : make_uint2(QS_I << 24 | g, 0);
+      if (g < items) in[i] = a.next ? make_uint2(__ldcg(a.next + 2 * (size_t)g), __ldcg(a.next + 2 * (size_t)g + 1))
+                                        : make_uint2(QS_I << 24 | g, 0);
     }
 #pragma unroll
     for (int i = 0; i < kPrepGates; ++i) {
@@ -553,7 +554,7 @@ cudaError_t launch_lazy_layers(const Dev &d, void *scratch, const uint32_t *pack
     a.next = nullptr;
     if (i < todo.size()) {
       next = (uint64_t)(ptr[todo[i] + 1] - ptr[todo[i]]);
-      a.next = reinterpret_cast<const uint2 *>(packed) + ptr[todo[i]];
+      a.next = packed + 2 * ptr[todo[i]];
     } else if (i == todo.size()) {
       next = n;
     }

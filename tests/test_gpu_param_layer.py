@@ -35,3 +35,19 @@ def test_host_layers_equal_device_layers(n, n_gates):
         qs.qs_sim_apply_layers_dev(b.sim, packed.data_ptr(), ptr, i, i + 1)
     for u, v in zip(a.export(), b.export()):
         assert np.array_equal(u, v)
+
+
+@pytest.mark.parametrize("n,flags", [(300, qs.QS_FLAG_NO_FUSION), (15_000, 0)])
+def test_unfused_device_records_need_four_byte_alignment_only(n, flags):
+    layers = [_layer(n, n // 2, i) for i in range(5)]
+    ptr = np.arange(6, dtype=np.int64) * (n // 2)
+    packed = qs.qs_pack_layers(n, np.concatenate(layers), ptr).view(np.int32)
+    out = []
+    for shift in (0, 1):
+        dev = torch.zeros(len(packed) + 1, dtype=torch.int32, device="cuda")
+        dev[shift:shift + len(packed)] = torch.from_numpy(packed).cuda()
+        sim = qs.Simulator(n, flags=flags)
+        qs.qs_sim_apply_layers_dev(sim.sim, dev.data_ptr() + 4 * shift, ptr, 0, 5)
+        out.append(qs.qs_sim_tableau_export(sim.sim))
+        sim.sync()
+    assert np.array_equal(*out)
