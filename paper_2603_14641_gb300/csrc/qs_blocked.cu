@@ -1755,18 +1755,18 @@ static cudaError_t measure_window_cap(const Dev &d, void *scratch, const uint32_
     launch_chained(blk_middle_kernel, mid_blocks, kMidThreads, 0, s, m);
     tend(d.timer, QS_TIME_BLK_PIVOT_ROWS, s);
     tbegin(d.timer, QS_TIME_BLK_APPLY, s);
+    auto apply = [&](auto kernel, int threads, size_t bytes) {
+      launch_chained(kernel, dim3(chunks, rows_y), threads, bytes, s, d.RX, d.RZ, L.rs, (uint32_t)L.nrows, window + i0,
+                     (int)f.B, b.VX, b.VZ, b.list, b.Tp, st);
+    };
     if (words == 4)
-      launch_chained(
-          blk_apply_small_kernel<4>, dim3(chunks, rows_y), kSmallThreads, 0, s, d.RX, d.RZ, L.rs, (uint32_t)L.nrows, window + i0, (int)f.B, b.VX, b.VZ, b.list, b.Tp, st);
+      apply(blk_apply_small_kernel<4>, kSmallThreads, 0);
     else if (words == 8)
-      launch_chained(
-          blk_apply_small_kernel<8>, dim3(chunks, rows_y), kSmallThreads, 0, s, d.RX, d.RZ, L.rs, (uint32_t)L.nrows, window + i0, (int)f.B, b.VX, b.VZ, b.list, b.Tp, st);
+      apply(blk_apply_small_kernel<8>, kSmallThreads, 0);
     else if (!d.wide_offsets && (uint64_t)L.nrows * L.rs < (1ull << 32))
-      launch_chained(
-          blk_apply_kernel<uint32_t>, dim3(chunks, rows_y), kApplyThreads, smem, s, d.RX, d.RZ, L.rs, (uint32_t)L.nrows, window + i0, (int)f.B, b.VX, b.VZ, b.list, b.Tp, st);
+      apply(blk_apply_kernel<uint32_t>, kApplyThreads, smem);
     else
-      launch_chained(
-          blk_apply_kernel<uint64_t>, dim3(chunks, rows_y), kApplyThreads, smem, s, d.RX, d.RZ, L.rs, (uint32_t)L.nrows, window + i0, (int)f.B, b.VX, b.VZ, b.list, b.Tp, st);
+      apply(blk_apply_kernel<uint64_t>, kApplyThreads, smem);
     tend(d.timer, QS_TIME_BLK_APPLY, s);
     nl += 2;
     if (d.timer && (i0 & 4095) == 4032) d.timer->resolve();  // completed event pairs go back to the pool

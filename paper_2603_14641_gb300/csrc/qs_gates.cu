@@ -316,8 +316,8 @@ static void launch_param(const Dev &d, const uint32_t *packed, uint32_t n_gates,
   GateGrid g = gate_grid(d.L.cs / 2, n_gates);
   g.gpl = std::max(1u, std::min(g.gpl, kParamGroup / g.lanes));
   g.grid.x = (n_gates + g.lanes * g.gpl - 1) / (g.lanes * g.gpl);
-  launch_chained(param_layer_kernel<MAX>, g.grid, g.block, 0, s, d.X, d.Z, d.S, d.L.n, d.L.cs, n_gates, g.P, g.lanes, g.gpl, d.err,
-                                                     layer);
+  launch_chained(param_layer_kernel<MAX>, g.grid, g.block, 0, s, d.X, d.Z, d.S, d.L.n, d.L.cs, n_gates, g.P, g.lanes,
+                 g.gpl, d.err, layer);
 }
 
 bool param_layer_fits(uint32_t n, uint32_t n_gates) { return n <= 16384 && n_gates <= 2048; }
