@@ -382,6 +382,8 @@ __device__ __forceinline__ void lazy_prepare(const LazyArgs &a) {
   uint2 *rec = a.step & 1 ? a.L.rec0 : a.L.rec1;
   uint32_t *count = a.L.count + (a.step + 1) % 3;
   const uint32_t t = threadIdx.x, T = blockDim.x, lane = t & 31, warp = t >> 5, warps = (T + 31) >> 5;
+  // the warp's last lane and its lanes: the last warp of a block need not be whole
+  const uint32_t last = min(31u, T - 1 - 32 * warp), members = 0xffffffffu >> (31 - last);
   const uint32_t items = a.next ? a.next_gates : a.n, pass = T * kPrepGates;
   for (uint32_t b0 = blockIdx.x * pass; b0 < items; b0 += a.prep_blocks * pass) {
     // records, then pending operations, then updates: the qubits of a layer are
@@ -424,12 +426,13 @@ __device__ __forceinline__ void lazy_prepare(const LazyArgs &a) {
         a.L.pend[qa] = (uint8_t)op_then(pa[i], type);
       }
     }
-    uint32_t inc = __popc(emit);  // inclusive prefix over the warp
+    // inclusive prefix over the warp; its lanes are named, so that they meet here
+    // whichever way they went through the branches above
+    uint32_t inc = __popc(emit);
     for (int d = 1; d < 32; d <<= 1) {
-      const uint32_t y = __shfl_up_sync(__activemask(), inc, d);
+      const uint32_t y = __shfl_up_sync(members, inc, d);
       if (lane >= (uint32_t)d) inc += y;
     }
-    const uint32_t last = min(31u, T - 1 - 32 * warp);
     if (lane == last) s_warp[warp] = inc;
     __syncthreads();
     if (t == 0) {
