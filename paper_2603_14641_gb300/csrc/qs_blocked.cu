@@ -1734,8 +1734,9 @@ static cudaError_t measure_window_cap(const Dev &d, void *scratch, const uint32_
     }
     const uint32_t blocks = (f.B ? ranges : 0) + (f.prev_B ? ranges : 0);
     const size_t off_bytes = f.lazy ? ranges * 4 : 0;
-    if (L.nrows <= kFrontSplitRows) launch_chained(blk_front_kernel<8>, blocks, 256, off_bytes, s, f);
-    else launch_chained(blk_front_kernel<1>, blocks, 256, off_bytes, s, f);
+    if ((e = launch_chained(L.nrows <= kFrontSplitRows ? blk_front_kernel<8> : blk_front_kernel<1>, blocks, 256, off_bytes,
+                            s, f)) != cudaSuccess)
+      return e;
     ++nl;
     if (!f.lazy && f.B) {
       // the previous block's M and base are signed; C0 -> C1 -> C0 ...
@@ -1745,6 +1746,7 @@ static cudaError_t measure_window_cap(const Dev &d, void *scratch, const uint32_
         blk_step_kernel<<<row_blocks, 256, 0, s>>>(L.nrows, L.n, L.k, j, (int)f.B, (j & 1) ? b.C1 : b.C0,
                                                (j & 1) ? b.C0 : b.C1, b.M, b.base, st);
       blk_step_finish_kernel<<<1, 64, 0, s>>>(st);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
       nl += (int)f.B + 1;
     }
     tend(d.timer, kind, s);
@@ -1752,21 +1754,22 @@ static cudaError_t measure_window_cap(const Dev &d, void *scratch, const uint32_
     m.B = f.B;
     m.st = st;
     tbegin(d.timer, QS_TIME_BLK_PIVOT_ROWS, s);
-    launch_chained(blk_middle_kernel, mid_blocks, kMidThreads, 0, s, m);
+    if ((e = launch_chained(blk_middle_kernel, mid_blocks, kMidThreads, 0, s, m)) != cudaSuccess) return e;
     tend(d.timer, QS_TIME_BLK_PIVOT_ROWS, s);
     tbegin(d.timer, QS_TIME_BLK_APPLY, s);
     auto apply = [&](auto kernel, int threads, size_t bytes) {
-      launch_chained(kernel, dim3(chunks, rows_y), threads, bytes, s, d.RX, d.RZ, L.rs, (uint32_t)L.nrows, window + i0,
-                     (int)f.B, b.VX, b.VZ, b.list, b.Tp, st);
+      return launch_chained(kernel, dim3(chunks, rows_y), threads, bytes, s, d.RX, d.RZ, L.rs, (uint32_t)L.nrows,
+                            window + i0, (int)f.B, b.VX, b.VZ, b.list, b.Tp, st);
     };
     if (words == 4)
-      apply(blk_apply_small_kernel<4>, kSmallThreads, 0);
+      e = apply(blk_apply_small_kernel<4>, kSmallThreads, 0);
     else if (words == 8)
-      apply(blk_apply_small_kernel<8>, kSmallThreads, 0);
+      e = apply(blk_apply_small_kernel<8>, kSmallThreads, 0);
     else if (!d.wide_offsets && (uint64_t)L.nrows * L.rs < (1ull << 32))
-      apply(blk_apply_kernel<uint32_t>, kApplyThreads, smem);
+      e = apply(blk_apply_kernel<uint32_t>, kApplyThreads, smem);
     else
-      apply(blk_apply_kernel<uint64_t>, kApplyThreads, smem);
+      e = apply(blk_apply_kernel<uint64_t>, kApplyThreads, smem);
+    if (e != cudaSuccess) return e;
     tend(d.timer, QS_TIME_BLK_APPLY, s);
     nl += 2;
     if (d.timer && (i0 & 4095) == 4032) d.timer->resolve();  // completed event pairs go back to the pool
@@ -1777,9 +1780,8 @@ static cudaError_t measure_window_cap(const Dev &d, void *scratch, const uint32_
   t.det_x = d.det_x; t.det_z = d.det_z; t.m0 = m0; t.record = d.record; t.err = d.err;
   // enough blocks for one outcome's ranges and for every group; blocks without an item leave at once
   const uint64_t most = std::max<uint64_t>(kDetBlocks, (count + kDetGroup - 1) / kDetGroup) * t.chunks;
-  launch_chained(blk_det_kernel, (unsigned)std::min<uint64_t>(most, 12ull * d.sms), kDetThreads, 0, s, t);
   if (launches) *launches += nl + 2;
-  return cudaGetLastError();
+  return launch_chained(blk_det_kernel, (unsigned)std::min<uint64_t>(most, 12ull * d.sms), kDetThreads, 0, s, t);
 }
 
 cudaError_t launch_measure_blocks(const Dev &d, void *scratch, const uint32_t *window, uint32_t count, uint64_t m0,

@@ -42,8 +42,7 @@ cudaError_t launch_frame_init(uint64_t *FX, uint64_t *FZ, uint32_t n, uint32_t f
   cudaError_t e = cudaMemsetAsync(FX, 0, (size_t)n * fw * sizeof(uint64_t), s);
   if (e != cudaSuccess) return e;
   const uint64_t total = (uint64_t)n * (fw >> 2);
-  launch_chained(frame_init_kernel, (unsigned)((total + 255) / 256), 256, 0, s, FZ, n, fw, seed);
-  return cudaGetLastError();
+  return launch_chained(frame_init_kernel, (unsigned)((total + 255) / 256), 256, 0, s, FZ, n, fw, seed);
 }
 
 // grid.x over shot-word quads, grid.y over the measurements of the window
@@ -95,13 +94,14 @@ __global__ void frame_measure_kernel(const uint64_t *FX, uint64_t *__restrict__ 
 }
 
 template <class Qubits>
-static void frame_measure(uint64_t *FX, uint64_t *FZ, uint32_t n, uint32_t fw, const Qubits &qubits, uint32_t count,
-                          uint64_t m0, const uint8_t *ref, uint64_t *out, uint64_t shots, uint64_t seed,
-                          uint32_t *err, cudaStream_t s) {
+static cudaError_t frame_measure(uint64_t *FX, uint64_t *FZ, uint32_t n, uint32_t fw, const Qubits &qubits, uint32_t count,
+                                 uint64_t m0, const uint8_t *ref, uint64_t *out, uint64_t shots, uint64_t seed,
+                                 uint32_t *err, cudaStream_t s) {
   const uint32_t quads = fw >> 2;
   const uint32_t threads = quads < 128 ? ((quads + 31) / 32) * 32 : 128;
   const dim3 grid((quads + threads - 1) / threads, count);
-  launch_chained(frame_measure_kernel<Qubits>, grid, threads, 0, s, FX, FZ, n, fw, qubits, m0, ref, out, shots, seed, err);
+  return launch_chained(frame_measure_kernel<Qubits>, grid, threads, 0, s, FX, FZ, n, fw, qubits, m0, ref, out, shots, seed,
+                        err);
 }
 
 cudaError_t launch_frame_measure(uint64_t *FX, uint64_t *FZ, uint32_t n, uint32_t fw,
@@ -109,10 +109,11 @@ cudaError_t launch_frame_measure(uint64_t *FX, uint64_t *FZ, uint32_t n, uint32_
                                  const uint8_t *ref, uint64_t *out, uint64_t shots, uint64_t seed,
                                  uint32_t *err, cudaStream_t s) {
   // grid.y is limited to 65535: split long windows
-  for (uint32_t off = 0; off < count; off += 65535)
-    frame_measure(FX, FZ, n, fw, DeviceQubits{qubits + off}, std::min(65535u, count - off), m0 + off, ref, out, shots,
-                  seed, err, s);
-  return cudaGetLastError();
+  cudaError_t e = cudaSuccess;
+  for (uint32_t off = 0; off < count && e == cudaSuccess; off += 65535)
+    e = frame_measure(FX, FZ, n, fw, DeviceQubits{qubits + off}, std::min(65535u, count - off), m0 + off, ref, out, shots,
+                      seed, err, s);
+  return e;
 }
 
 // Staged, a list is a copy and an event besides the launch, and the kernel waits
@@ -122,20 +123,21 @@ bool param_qubits_fit(uint32_t count) { return count <= 2 * kParamQubits; }
 cudaError_t launch_frame_measure_host(uint64_t *FX, uint64_t *FZ, uint32_t n, uint32_t fw, const uint32_t *qubits,
                                       uint32_t count, uint64_t m0, const uint8_t *ref, uint64_t *out, uint64_t shots,
                                       uint64_t seed, uint32_t *err, cudaStream_t s, int *launches) {
-  for (uint32_t off = 0; off < count; off += kParamQubits) {
+  cudaError_t e = cudaSuccess;
+  for (uint32_t off = 0; off < count && e == cudaSuccess; off += kParamQubits) {
     const uint32_t c = std::min(kParamQubits, count - off);
     if (c <= 128) {
       ParamQubits<128> list;
       std::copy(qubits + off, qubits + off + c, list.q);
-      frame_measure(FX, FZ, n, fw, list, c, m0 + off, ref, out, shots, seed, err, s);
+      e = frame_measure(FX, FZ, n, fw, list, c, m0 + off, ref, out, shots, seed, err, s);
     } else {
       ParamQubits<kParamQubits> list;
       std::copy(qubits + off, qubits + off + c, list.q);
-      frame_measure(FX, FZ, n, fw, list, c, m0 + off, ref, out, shots, seed, err, s);
+      e = frame_measure(FX, FZ, n, fw, list, c, m0 + off, ref, out, shots, seed, err, s);
     }
     ++*launches;
   }
-  return cudaGetLastError();
+  return e;
 }
 
 // Pauli noise channels on the frames (X_ERROR, Y_ERROR, Z_ERROR, DEPOLARIZE1,
@@ -353,9 +355,8 @@ cudaError_t launch_frame_noise(uint64_t *FX, uint64_t *FZ, uint32_t fw, uint32_t
     if (blocks > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
   }
   if (G.ops == 0) return cudaSuccess;
-  launch_chained(frame_noise_kernel, (unsigned)blocks, kNoiseThreads, 0, s, FX, FZ, fw, ow, G);
   if (launches) *launches += 1;
-  return cudaGetLastError();
+  return launch_chained(frame_noise_kernel, (unsigned)blocks, kNoiseThreads, 0, s, FX, FZ, fw, ow, G);
 }
 
 }  // namespace qs

@@ -362,9 +362,8 @@ static cudaError_t launch_direct_t(uint64_t *X, uint64_t *Z, uint64_t *S, uint32
                                 (int)kFusedSmemMax);
   });
   if (e != cudaSuccess) return e;
-  launch_chained(fused_direct_kernel<SIGNS, R, D>, nwords, threads, direct_smem(n, threads, R, D), s, X, Z, S, n, stride,
-                 gates, o, L, err);
-  return cudaGetLastError();
+  return launch_chained(fused_direct_kernel<SIGNS, R, D>, nwords, threads, direct_smem(n, threads, R, D), s, X, Z, S, n,
+                        stride, gates, o, L, err);
 }
 
 template <bool SIGNS>

@@ -90,8 +90,8 @@ cudaError_t launch_init_all(const Dev &d, const uint8_t *initstate_dev, cudaStre
   const Layout &L = d.L;
   const uint32_t words = L.ncols * L.cs;  // at least cs and kMeasStateWords
   const uint32_t blocks = std::min<uint32_t>((words + 255) / 256, 16u * (uint32_t)d.sms);
-  launch_chained(init_all_kernel, blocks, 256, 0, s, d.X, d.Z, d.S, initstate_dev, L.n, L.k, L.cs, words, d.mst, d.err);
-  return cudaGetLastError();
+  return launch_chained(init_all_kernel, blocks, 256, 0, s, d.X, d.Z, d.S, initstate_dev, L.n, L.k, L.cs, words, d.mst,
+                        d.err);
 }
 
 cudaError_t launch_init(const Dev &d, const uint8_t *initstate_dev, cudaStream_t s) {
@@ -303,33 +303,28 @@ cudaError_t launch_gate_layer(const Dev &d, const uint32_t *packed, uint32_t n_g
                               cudaStream_t s) {
   if (n_gates == 0) return cudaSuccess;
   GateGrid g = gate_grid(d.L.cs / 2, n_gates);
-  launch_chained(gate_layer_kernel<true, 2>, g.grid, g.block, 0, s, d.X, d.Z, d.S, d.L.n, d.L.cs, packed, n_gates,
-                                                     g.P, g.lanes, g.gpl, d.err);
-  return cudaGetLastError();
+  return launch_chained(gate_layer_kernel<true, 2>, g.grid, g.block, 0, s, d.X, d.Z, d.S, d.L.n, d.L.cs, packed, n_gates,
+                        g.P, g.lanes, g.gpl, d.err);
 }
 
 template <int MAX>
-static void launch_param(const Dev &d, const uint32_t *packed, uint32_t n_gates, cudaStream_t s) {
+static cudaError_t launch_param(const Dev &d, const uint32_t *packed, uint32_t n_gates, cudaStream_t s) {
   ParamLayer<MAX> layer;
   for (uint32_t g = 0; g < n_gates; ++g)
     layer.rec[g] = packed[2 * g] >> 24 << 28 | (packed[2 * g] & 0x3FFF) << 14 | packed[2 * g + 1];
   GateGrid g = gate_grid(d.L.cs / 2, n_gates);
   g.gpl = std::max(1u, std::min(g.gpl, kParamGroup / g.lanes));
   g.grid.x = (n_gates + g.lanes * g.gpl - 1) / (g.lanes * g.gpl);
-  launch_chained(param_layer_kernel<MAX>, g.grid, g.block, 0, s, d.X, d.Z, d.S, d.L.n, d.L.cs, n_gates, g.P, g.lanes,
-                 g.gpl, d.err, layer);
+  return launch_chained(param_layer_kernel<MAX>, g.grid, g.block, 0, s, d.X, d.Z, d.S, d.L.n, d.L.cs, n_gates, g.P,
+                        g.lanes, g.gpl, d.err, layer);
 }
 
 bool param_layer_fits(uint32_t n, uint32_t n_gates) { return n <= 16384 && n_gates <= 2048; }
 
 cudaError_t launch_param_layer(const Dev &d, const uint32_t *packed, uint32_t n_gates, cudaStream_t s) {
-  if (n_gates <= 128)
-    launch_param<128>(d, packed, n_gates, s);
-  else if (n_gates <= 512)
-    launch_param<512>(d, packed, n_gates, s);
-  else
-    launch_param<2048>(d, packed, n_gates, s);
-  return cudaGetLastError();
+  if (n_gates <= 128) return launch_param<128>(d, packed, n_gates, s);
+  if (n_gates <= 512) return launch_param<512>(d, packed, n_gates, s);
+  return launch_param<2048>(d, packed, n_gates, s);
 }
 
 cudaError_t launch_frame_layer(uint64_t *FX, uint64_t *FZ, uint32_t n, uint32_t fw,
@@ -338,12 +333,10 @@ cudaError_t launch_frame_layer(uint64_t *FX, uint64_t *FZ, uint32_t n, uint32_t 
   if (n_gates == 0) return cudaSuccess;
   GateGrid g = gate_grid(fw / 2, n_gates);
   if (g.lanes == 1)  // long frame columns (>= 512 shot words): as the tableau, two gates in flight
-    launch_chained(gate_layer_kernel<false, 2>, g.grid, g.block, 0, s, FX, FZ, nullptr, n, fw, packed, n_gates,
-                                                        g.P, g.lanes, g.gpl, err);
-  else
-    launch_chained(gate_layer_kernel<false, 1>, g.grid, g.block, 0, s, FX, FZ, nullptr, n, fw, packed, n_gates,
-                                                        g.P, g.lanes, g.gpl, err);
-  return cudaGetLastError();
+    return launch_chained(gate_layer_kernel<false, 2>, g.grid, g.block, 0, s, FX, FZ, nullptr, n, fw, packed, n_gates,
+                          g.P, g.lanes, g.gpl, err);
+  return launch_chained(gate_layer_kernel<false, 1>, g.grid, g.block, 0, s, FX, FZ, nullptr, n, fw, packed, n_gates,
+                        g.P, g.lanes, g.gpl, err);
 }
 
 // ---------------------------------------------------------------------
@@ -574,11 +567,11 @@ cudaError_t launch_lazy_layers(const Dev &d, void *scratch, const uint32_t *pack
     a.gx = i ? (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(blocks_x, (gates + g.lanes - 1) / g.lanes)) : 0;
     a.prep_blocks = (uint32_t)std::min<uint64_t>(kLazyPrepBlocks, (next + threads * kPrepGates - 1) / (threads * kPrepGates));
     const uint32_t blocks = a.prep_blocks + a.gx * chunks;
-    if (blocks) launch_chained(lazy_layer_kernel, blocks, threads, 0, s, a);
+    if (blocks && (e = launch_chained(lazy_layer_kernel, blocks, threads, 0, s, a)) != cudaSuccess) return e;
     gates = i < todo.size() ? std::min<uint64_t>(next, std::max(1u, n / 2)) : n;
   }
   if (launches) *launches += (int)todo.size() + 2;
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 
 }  // namespace qs

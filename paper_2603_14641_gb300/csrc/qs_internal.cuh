@@ -132,9 +132,11 @@ __device__ __forceinline__ void chain_start() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// The result is the only report of a failed launch (the last error is cleared, so
+// that event queries between launches cannot lose it): callers return it.
 template <class... P, class... A>
-inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                                  const A &...args) {
+[[nodiscard]] inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                                                cudaStream_t s, const A &...args) {
   cudaLaunchAttribute attr{};
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
@@ -145,7 +147,9 @@ inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, s
   c.stream = s;
   c.attrs = &attr;
   c.numAttrs = 1;
-  return cudaLaunchKernelEx(&c, kernel, args...);
+  const cudaError_t e = cudaLaunchKernelEx(&c, kernel, args...);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
 }
 
 // Optional CUDA-event timing of kernel classes (qs_sim_set_timing): begin/end
@@ -213,7 +217,7 @@ inline void tbegin(KernelTimer *t, int kind, cudaStream_t s) { if (t) t->begin(k
 inline void tend(KernelTimer *t, int kind, cudaStream_t s) { if (t) t->end(kind, s); }
 
 // ------------------------------------------------------------------------
-// Launchers (each returns cudaGetLastError() after the launch).
+// Launchers (each returns the first error of its launches).
 // ------------------------------------------------------------------------
 struct Dev {
   Layout L;

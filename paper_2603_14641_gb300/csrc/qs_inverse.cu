@@ -237,8 +237,8 @@ cudaError_t launch_inv_gate_layer(const Dev &d, const uint32_t *packed, uint32_t
   if (n_gates == 0) return cudaSuccess;
   const Layout &L = d.L;
   const uint32_t threads = L.k >= 256 ? 256 : (L.k >= 128 ? 128 : (L.k >= 64 ? 64 : 32));
-  launch_chained(inv_gate_layer_kernel, n_gates, threads, 0, s, d.X, d.Z, d.qsig, L.n, L.k, L.cs, L.rs, packed, d.err);
-  return cudaGetLastError();
+  return launch_chained(inv_gate_layer_kernel, n_gates, threads, 0, s, d.X, d.Z, d.qsig, L.n, L.k, L.cs, L.rs, packed,
+                        d.err);
 }
 
 // ---------------------------------------------------------------------------

@@ -455,13 +455,15 @@ cudaError_t measure_columns(const Dev &d, const uint32_t *qubits, uint32_t count
   const uint32_t warps = std::max(4u, std::min(kApplyWarps<W>, (L.n + sms - 1) / sms));
   for (uint32_t off = 0; off < count; off += B) {
     const uint32_t c = std::min(B, count - off);
-    launch_chained(lead, 1, 32 * lead_warps, lead_smem, s, d.X, d.qsig, L.n, L.k, L.cs, 32 * W, qubits + off, c,
-                   m0 + off, key.seed, key.shot, d.record, d.kinds, log, d.err);
-    launch_chained(inv_apply_kernel<W>, grid, 32 * warps, apply_smem(warps), s, d.X, d.Z, d.qsig, L.n, L.k, L.cs, L.rs,
-                   log);
+    e = launch_chained(lead, 1, 32 * lead_warps, lead_smem, s, d.X, d.qsig, L.n, L.k, L.cs, 32 * W, qubits + off, c,
+                       m0 + off, key.seed, key.shot, d.record, d.kinds, log, d.err);
+    if (e == cudaSuccess)
+      e = launch_chained(inv_apply_kernel<W>, grid, 32 * warps, apply_smem(warps), s, d.X, d.Z, d.qsig, L.n, L.k, L.cs,
+                         L.rs, log);
+    if (e != cudaSuccess) return e;
     if (launches) *launches += 2;
   }
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 
 }  // namespace

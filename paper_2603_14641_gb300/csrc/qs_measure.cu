@@ -332,20 +332,16 @@ store_list_kernel(uint32_t *__restrict__ dst, uint32_t count, const __grid_const
 }
 
 template <int MAX>
-static void store_list(uint32_t *dst, const uint32_t *q, uint32_t count, cudaStream_t s) {
+static cudaError_t store_list(uint32_t *dst, const uint32_t *q, uint32_t count, cudaStream_t s) {
   ListParam<MAX> list;
   std::copy(q, q + count, list.q);
-  launch_chained(store_list_kernel<MAX>, (count + 255) / 256, 256, 0, s, dst, count, list);
+  return launch_chained(store_list_kernel<MAX>, (count + 255) / 256, 256, 0, s, dst, count, list);
 }
 
 bool store_list_fits(uint32_t count) { return count <= 2048; }
 
 cudaError_t launch_store_list(uint32_t *dst, const uint32_t *q, uint32_t count, cudaStream_t s) {
-  if (count <= 256)
-    store_list<256>(dst, q, count, s);
-  else
-    store_list<2048>(dst, q, count, s);
-  return cudaGetLastError();
+  return count <= 256 ? store_list<256>(dst, q, count, s) : store_list<2048>(dst, q, count, s);
 }
 
 cudaError_t launch_gather(const Dev &d, const uint32_t *qubits, uint32_t i, cudaStream_t s) {

@@ -407,8 +407,7 @@ static cudaError_t transpose(const uint64_t *in, size_t in_stride, size_t rows_i
                                 err, s);
   // rows_in is a multiple of 256 and words_in of 4 by construction
   dim3 grid((unsigned)(words_in / 4), (unsigned)(rows_in / 256));
-  launch_chained(bit_transpose_kernel, grid, 128, 0, s, in, in_stride, out, out_stride);
-  return cudaGetLastError();
+  return launch_chained(bit_transpose_kernel, grid, 128, 0, s, in, in_stride, out, out_stride);
 }
 
 cudaError_t launch_to_rows(const Dev &d, cudaStream_t s) {
