@@ -1780,7 +1780,7 @@ static cudaError_t measure_window_cap(const Dev &d, void *scratch, const uint32_
   t.det_x = d.det_x; t.det_z = d.det_z; t.m0 = m0; t.record = d.record; t.err = d.err;
   // enough blocks for one outcome's ranges and for every group; blocks without an item leave at once
   const uint64_t most = std::max<uint64_t>(kDetBlocks, (count + kDetGroup - 1) / kDetGroup) * t.chunks;
-  if (launches) *launches += nl + 2;
+  if (launches) *launches += nl + 1;
   return launch_chained(blk_det_kernel, (unsigned)std::min<uint64_t>(most, 12ull * d.sms), kDetThreads, 0, s, t);
 }
 

@@ -435,7 +435,7 @@ static cudaError_t launch_slices(FusedArgs a, const FusedShape &f, uint32_t reco
 
 cudaError_t launch_fused_segment(uint64_t *X, uint64_t *Z, uint64_t *S, uint32_t n, uint32_t stride, uint32_t nwords,
                                  const uint32_t *packed, const int64_t *ptr, uint32_t L, int sms, void *scratch,
-                                 uint32_t *err, cudaStream_t s) {
+                                 uint32_t *err, cudaStream_t s, int *launches) {
   if (L == 0 || L > kFusedLayers) return cudaErrorInvalidValue;
   LayerOffsets o;
   uint32_t max_gates = 0;  // layers hold at most n gates (checked when they were added)
@@ -450,9 +450,12 @@ cudaError_t launch_fused_segment(uint64_t *X, uint64_t *Z, uint64_t *S, uint32_t
   // qubits 25 layers 52 / 51 (25,390) and 100 layers 104 / 152 (101,562), 1,000
   // qubits and 20,000 shots 25 layers 56 / 61 (30,468)
   const double cycles = 0.25 * n / 32 * 52 * ((nwords + sms - 1) / sms);
-  if (cycles * L < 28000)
+  if (cycles * L < 28000) {
+    *launches += 1;
     return S ? launch_direct<true>(X, Z, S, n, stride, nwords, gates, o, L, max_gates, err, s)
              : launch_direct<false>(X, Z, S, n, stride, nwords, gates, o, L, max_gates, err, s);
+  }
+  *launches += max_gates ? 3 : 2;
   uint8_t *p = static_cast<uint8_t *>(scratch);
   uint32_t *count = reinterpret_cast<uint32_t *>(p);
   uint8_t *act = p + act_offset();

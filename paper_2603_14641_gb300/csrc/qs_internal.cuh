@@ -327,7 +327,7 @@ bool fused_fits(uint32_t n);
 size_t fused_scratch_bytes(uint32_t n);
 cudaError_t launch_fused_segment(uint64_t *X, uint64_t *Z, uint64_t *S, uint32_t n, uint32_t stride, uint32_t nwords,
                                  const uint32_t *packed, const int64_t *ptr, uint32_t L, int sms,
-                                 void *scratch, uint32_t *err, cudaStream_t s);
+                                 void *scratch, uint32_t *err, cudaStream_t s, int *launches);
 // device record of a simulator (one byte per measurement)
 const uint8_t *sim_record(const qs_sim *sim);
 

@@ -249,9 +249,10 @@ int run_dev_layers(qs_sim *s, uint64_t *X, uint64_t *Z, uint64_t *S, uint32_t st
   if (nlayers >= kFusedMinLayers && fused_fits(n) && !(s->flags & QS_FLAG_NO_FUSION) && !(tableau && s->d.inverse)) {
     for (size_t l0 = 0; l0 < nlayers; l0 += kFusedLayers) {
       const size_t L = std::min<size_t>(kFusedLayers, nlayers - l0);
+      int l = 0;
       QS_CUDA(s, launch_fused_segment(X, Z, S, n, stride, nwords, packed, ptr + l0, (uint32_t)L, s->d.sms, s->fused,
-                                      s->d.err, s->stream));
-      s->launches += 3;
+                                      s->d.err, s->stream, &l));
+      s->launches += (uint64_t)l;
     }
     return QS_OK;
   }
