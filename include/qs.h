@@ -468,9 +468,10 @@ int qs_batch_export_rows(qs_batch *batch, uint32_t circuit, const uint32_t *rows
  * kernel on this batch's circuits of n < 1024 (the first round_limit rounds;
  * 0 = all; the simulators of the larger ones are idle
  * meanwhile) and returns the fastest. cache_path: NULL, or a text file
- * of "device|batch-signature|rounds threads blocks_per_sm words_per_block
- * fuse_depth" lines that is read first and appended to. Results do not depend
- * on the shape. */
+ * of "device|candidates|batch-signature|rounds threads blocks_per_sm
+ * words_per_block fuse_depth" lines that is read first and appended to
+ * (candidates: what was chosen from; lines of another choice are not answers).
+ * Results do not depend on the shape. */
 int qs_batch_autotune(qs_batch *batch, uint32_t round_limit, const char *cache_path,
                       qs_batch_tuning *best);
 

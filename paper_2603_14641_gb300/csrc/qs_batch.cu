@@ -52,6 +52,9 @@ constexpr int64_t kBNoPivot = LLONG_MAX;
 constexpr uint32_t kBatchSimMinQubits = 1024;
 constexpr uint32_t kBatchMaxWorkers = 16;
 constexpr uint32_t kBatchLimitQubits = 1u << 20;
+// What the autotuner chooses from, in its cache's keys: a line written when the
+// choice was another one (1: shapes of the persistent kernel alone) is no answer.
+constexpr uint32_t kTuneCandidates = 2;
 
 struct BAct {
   uint32_t c, l0, l1, q0, qn, pad;
@@ -1469,7 +1472,7 @@ int qs_batch_autotune(qs_batch *b, uint32_t round_limit, const char *cache_path,
       snprintf(dev_name, sizeof dev_name, "%s", prop.name);
   }
   char key[400];
-  snprintf(key, sizeof key, "%s|%016llx|%u", dev_name, (unsigned long long)b->signature, round_limit);
+  snprintf(key, sizeof key, "%s|%u|%016llx|%u", dev_name, kTuneCandidates, (unsigned long long)b->signature, round_limit);
   for (char *p = key; *p; ++p)
     if (*p == ' ') *p = '_';
   if (cache_path) {

@@ -1,0 +1,47 @@
+"""Host code of the batches on a CUDA runtime without a GPU: the autotuner's cache."""
+import ctypes
+
+import numpy as np
+
+from paper_2603_14641_gb300 import qs
+from tests import fake_cuda
+from workloads import circuits as C
+
+
+def _create(circs):
+    keep, arr = [], (qs.qs_batch_circuit * len(circs))()
+    for i, c in enumerate(circs):
+        g, lp = np.ascontiguousarray(c.gates, np.uint32), np.ascontiguousarray(c.layer_ptr, np.int64)
+        rl, rm, q = qs.circuit_rounds(c)
+        keep += [g, lp, rl, rm, q]
+        arr[i] = qs.qs_batch_circuit(c.n, c.n_layers, g.ctypes.data, lp.ctypes.data, len(rl) - 1, 0, rl.ctypes.data,
+                                     rm.ctypes.data, q.ctypes.data if q.size else None, i, 0)
+    h = ctypes.c_void_p()
+    assert qs.lib().qs_batch_create(len(circs), ctypes.byref(arr), None, None, 0, ctypes.byref(h)) == 0
+    return h
+
+
+def _circuits(sizes, depth=20, every=5):
+    return [C.random_circuit(n, depth, 0.5, seed=n, measure_every=every, measure_frac=0.2, final_measure_all=False)
+            for n in sizes]
+
+
+def test_autotune_takes_no_line_of_another_choice(monkeypatch, tmp_path):
+    """A line whose key lacks the set of candidates (the shapes of the persistent kernel alone) is not an answer."""
+    L = fake_cuda.use(monkeypatch)
+    circs = _circuits([50, 300, 900])
+    h = _create(circs)
+    sig, m64 = 1469598103934665603, (1 << 64) - 1
+    for v in [len(circs)] + [x for c in circs for x in (c.n, len(qs.circuit_rounds(c)[0]) - 1, len(c.gates), c.n_measurements)]:
+        sig = (sig ^ v) * 1099511628211 & m64
+    path = tmp_path / "tune.txt"
+    path.write_text(f"fake|{sig:016x}|0 512 1 1 0\n")
+    t = qs.qs_batch_tuning()
+    assert L.qs_batch_autotune(h, 0, str(path).encode(), ctypes.byref(t)) == 0
+    assert t.threads == 0  # every candidate takes the same time here: the first is kept
+    lines = path.read_text().splitlines()
+    assert len(lines) == 2
+    path.write_text(lines[1].split()[0] + " 256 2 1 1\n")  # a line of this choice is
+    assert L.qs_batch_autotune(h, 0, str(path).encode(), ctypes.byref(t)) == 0
+    assert (t.threads, t.blocks_per_sm, t.words_per_block, t.fuse_depth) == (256, 2, 1, 1)
+    L.qs_batch_destroy(h)
