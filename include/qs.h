@@ -412,8 +412,8 @@ typedef struct qs_batch_circuit {
 } qs_batch_circuit;
 
 /* Launch shape of the persistent kernel (qs_batch_autotune picks one).
- *   threads:         256, 512 or 1024 per CTA; 0 = the default path, without
- *                    the persistent kernel (the other members are not read)
+ *   threads:         256, 512 or 1024 per CTA; 0 = the default path, without the
+ *                    persistent kernel (the three members below are 0 then)
  *   blocks_per_sm:   CTAs per SM (0 = as many as fit)
  *   words_per_block: 64-row column words per shared-memory slice in the gate phase (1 or 2)
  *   fuse_depth:      layers per shared-memory pass in the gate phase (0 = whole round)

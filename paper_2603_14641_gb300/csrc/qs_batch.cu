@@ -1177,7 +1177,11 @@ int qs_batch_destroy(qs_batch *b) {
 
 static int tuning_ok(const qs_batch *b, const qs_batch_tuning &t, size_t *smem) {
   *smem = 0;
-  if (t.threads == 0) return QS_OK;  // the default: no persistent kernel
+  if (t.threads == 0) {  // the default: no persistent kernel
+    if (t.blocks_per_sm || t.words_per_block || t.fuse_depth)
+      return bfail(QS_ERR_ARG, "tuning.threads is 0 (the default path) and another member is not");
+    return QS_OK;
+  }
   if (t.threads != 256 && t.threads != 512 && t.threads != 1024)
     return bfail(QS_ERR_ARG, "tuning.threads must be 256, 512 or 1024");
   if (t.words_per_block != 1 && t.words_per_block != 2)
@@ -1285,11 +1289,12 @@ static int batch_run(qs_batch *b, const qs_batch_tuning *tuning, uint32_t round_
   if (!b) return bfail(QS_ERR_ARG, "batch is NULL");
   if (b->broken) return bfail(QS_ERR_STATE, "batch is unusable after an earlier device error");
   const bool persistent = tuning && tuning->threads != 0;
-  b->pending = true;
-  b->rec_ready = false;
   size_t smem = 0;
   int rc = QS_OK;
-  if (persistent && (rc = tuning_ok(b, *tuning, &smem))) return rc;
+  const bool small = b->any_small || b->sims.empty();  // the launch shape is for these
+  if (tuning && small && (rc = tuning_ok(b, *tuning, &smem))) return rc;
+  b->pending = true;
+  b->rec_ready = false;
   b->ran_full = (round_limit == 0 || round_limit >= b->nrounds) && !b->skip_sims;
   b->persistent_ran = persistent;
   bool sims = false;
@@ -1302,7 +1307,7 @@ static int batch_run(qs_batch *b, const qs_batch_tuning *tuning, uint32_t round_
       if (cudaStreamWaitEvent(st, b->start_ev, 0) != cudaSuccess)
         return bfail(QS_ERR_CUDA, "worker stream wait failed");
   if (persistent) {
-    if ((b->any_small || b->sims.empty()) && (rc = run_kernel(b, *tuning, round_limit))) return rc;
+    if (small && (rc = run_kernel(b, *tuning, round_limit))) return rc;
   } else if ((rc = run_resident(b, round_limit))) {
     return rc;
   }

@@ -1,4 +1,5 @@
-"""Host code of the batches on a CUDA runtime without a GPU: the autotuner's cache."""
+"""Host code of the batches on a CUDA runtime without a GPU: the autotuner's cache and
+the launch shapes that are refused."""
 import ctypes
 
 import numpy as np
@@ -45,3 +46,17 @@ def test_autotune_takes_no_line_of_another_choice(monkeypatch, tmp_path):
     assert L.qs_batch_autotune(h, 0, str(path).encode(), ctypes.byref(t)) == 0
     assert (t.threads, t.blocks_per_sm, t.words_per_block, t.fuse_depth) == (256, 2, 1, 1)
     L.qs_batch_destroy(h)
+
+
+def test_incomplete_launch_shapes_are_refused(monkeypatch):
+    """threads = 0 asks for the default path only where nothing else of a launch shape is given. A batch
+    without circuits for the persistent kernel does not look at the shape."""
+    L = fake_cuda.use(monkeypatch)
+    for sizes in ([50, 300], [1_024, 1_100]):
+        h = _create(_circuits(sizes))
+        for shape, ok in (((0, 0, 0, 0, 0), True), ((0, 0, 1, 0, 0), False), ((0, 2, 0, 0, 0), False),
+                          ((0, 0, 0, 1, 0), False), ((0, 0, 0, 0, 9), True), ((512, 1, 1, 0, 0), True),
+                          ((128, 1, 1, 0, 0), False)):
+            rc = L.qs_batch_run(h, ctypes.byref(qs.qs_batch_tuning(*shape)), 0)
+            assert rc == (0 if ok or sizes[0] > 1_000 else -1), (sizes, shape)
+        L.qs_batch_destroy(h)
