@@ -153,10 +153,10 @@ cudaError_t launch_frame_measure_host(uint64_t *FX, uint64_t *FZ, uint32_t n, ui
 // bits) 22 % of the items are undecided and at p = 1e-3 6 % have a shot that
 // fired, but nearly every warp has such an item, so warps ran 4.4 blocks per
 // item where 2.3 are needed. A block therefore takes 256 items through the first
-// two Philox blocks and then deals the undecided ones, and the shots that fired,
-// densely over its threads. (Passing in the first two rounds' uniform products
-// and the round keys from the host measured slower, as did a four-product 64 x 64
-// multiply in place of __umul64hi and the low product.) One launch takes up to
+// two Philox blocks and then deals the undecided ones, and the shots that fired (up
+// to kNoiseDense), densely over its threads. (Passing in the first two rounds'
+// uniform products and the round keys from the host measured slower, as did a
+// four-product 64 x 64 multiply in place of __umul64hi and the low product.) One launch takes up to
 // kNoiseGroupMax consecutive ops on distinct qubits (the depolarising ops after
 // one layer), so that their latencies overlap. 1,667 + 1,250 targets and 16,384
 // shots at p = 1e-3: 49 -> 35 us.
@@ -167,6 +167,13 @@ __device__ __forceinline__ P4 noise_philox(uint64_t e, uint64_t seed, uint32_t i
 }
 
 constexpr int kNoiseThreads = 128, kNoiseItems = 2 * kNoiseThreads;  // items per block
+// Fired shots of a block beyond which a thread draws those of its own two items, side
+// by side, instead of having all dealt out: dealing costs a search, a selection and
+// shared atomics a draw, which pay where lanes would wait for a few busy ones. 1,000
+// qubits x 20,000 shots, ten layers, dealt / own: p = 0.02 320 / 388 us, 0.1 575 / 642, 0.2
+// 881 / 807, 0.5 1,610 / 1,423, 1 3,273 / 1,905 (dealt with the bits of a shot word counted
+// off one by one 5,090, a thread per item throughout 1,885).
+constexpr uint32_t kNoiseDense = 16 * kNoiseItems;
 
 // one more Philox block of an item's draws: 4 bits of u from bit 31 - 4 t down
 __device__ __forceinline__ void noise_bits(uint64_t e, uint64_t seed, uint32_t thr, uint32_t i, uint32_t j, int t,
@@ -181,6 +188,30 @@ __device__ __forceinline__ void noise_bits(uint64_t e, uint64_t seed, uint32_t t
     } else {
       undecided &= ~w;  // u has 1 where thr has 0: u > thr
     }
+  }
+}
+
+// index of bit r (from 0) among the bits of m
+__device__ __forceinline__ uint32_t nth_bit(uint64_t m, uint32_t r) {
+  uint32_t w = (uint32_t)m, at = 0, c = __popc(w);
+  if (r >= c) { r -= c; w = (uint32_t)(m >> 32); at = 32; }
+#pragma unroll
+  for (int h = 16; h > 0; h >>= 1) {
+    c = __popc(w & ((1u << h) - 1));
+    if (r >= c) { r -= c; w >>= h; at += h; }
+  }
+  return at;
+}
+
+// the Pauli of a shot that fired: 0 I, 1 X, 2 Y, 3 Z on the first and second target
+__device__ __forceinline__ void noise_pauli(int kind, uint64_t v, uint32_t &pa, uint32_t &pb) {
+  pb = 0;
+  if (kind == QS_NOISE_DEPOLARIZE1) {
+    pa = 1 + (uint32_t)__umul64hi(v, 3);
+  } else {
+    const uint32_t idx = 1 + (uint32_t)__umul64hi(v, 15);
+    pa = idx >> 2;
+    pb = idx & 3;
   }
 }
 
@@ -212,7 +243,7 @@ frame_noise_kernel(uint64_t *__restrict__ FX, uint64_t *__restrict__ FZ, uint32_
   __shared__ __align__(16) uint32_t s_pauli[kNoiseItems][8];  // x, z of the first and second target, as halves
   __shared__ uint32_t s_first[kNoiseItems];     // draws before an item
   __shared__ uint16_t s_queue[kNoiseItems];
-  __shared__ uint32_t s_n, s_warp[kNoiseThreads / 32], s_draws;
+  __shared__ uint32_t s_n, s_warp[kNoiseThreads / 32];
   const uint32_t t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const uint64_t base = (uint64_t)blk * kNoiseItems;
   const uint32_t n = (uint32_t)(items - base < kNoiseItems ? items - base : kNoiseItems);
@@ -224,6 +255,7 @@ frame_noise_kernel(uint64_t *__restrict__ FX, uint64_t *__restrict__ FZ, uint32_
     j = b_j + x - d * ow;
   };
   const bool draws = kind == QS_NOISE_DEPOLARIZE1 || kind == QS_NOISE_DEPOLARIZE2;
+  bool dense = false;
   if (t == 0) s_n = 0;
   __syncthreads();
 #pragma unroll
@@ -276,30 +308,19 @@ frame_noise_kernel(uint64_t *__restrict__ FX, uint64_t *__restrict__ FZ, uint32_
     }
     s_first[2 * t] = before;
     s_first[2 * t + 1] = before + f0;
-    if (t == 0) s_draws = total;
-    for (uint32_t k = t; k < kNoiseItems * 8; k += kNoiseThreads) s_pauli[k >> 3][k & 7] = 0;
+    dense = total > kNoiseDense;
+    for (uint32_t k = t; k < kNoiseItems * 8 && !dense; k += kNoiseThreads) s_pauli[k >> 3][k & 7] = 0;
     __syncthreads();
-    total = s_draws;
-    for (uint32_t k = t; k < total; k += kNoiseThreads) {
+    for (uint32_t k = t; k < total && !dense; k += kNoiseThreads) {
       uint32_t lo = 0, hi = kNoiseItems;  // last item with first <= k
       while (hi - lo > 1) {
         const uint32_t mid = (lo + hi) >> 1;
         if (s_first[mid] <= k) lo = mid; else hi = mid;
       }
-      uint64_t m = s_fire[lo];
-      for (uint32_t skip = k - s_first[lo]; skip; --skip) m &= m - 1;
-      const uint32_t b = (uint32_t)__ffsll((long long)m) - 1;
-      uint32_t i, j;
+      const uint32_t b = nth_bit(s_fire[lo], k - s_first[lo]);
+      uint32_t i, j, pa, pb;
       place(lo, i, j);
-      const uint64_t v = noise_philox(e, seed, i0 + i, 64 * j + b, 4).v[0];
-      uint32_t pa, pb = 0;  // 0 I, 1 X, 2 Y, 3 Z
-      if (kind == QS_NOISE_DEPOLARIZE1) {
-        pa = 1 + (uint32_t)__umul64hi(v, 3);
-      } else {
-        const uint32_t idx = 1 + (uint32_t)__umul64hi(v, 15);
-        pa = idx >> 2;
-        pb = idx & 3;
-      }
+      noise_pauli(kind, noise_philox(e, seed, i0 + i, 64 * j + b, 4).v[0], pa, pb);
       uint32_t *acc = s_pauli[lo] + (b >> 5);
       const uint32_t bit = 1u << (b & 31);
       if (pa == 1 || pa == 2) atomicOr(acc, bit);
@@ -308,6 +329,37 @@ frame_noise_kernel(uint64_t *__restrict__ FX, uint64_t *__restrict__ FZ, uint32_
       if (pb >= 2) atomicOr(acc + 6, bit);
     }
     __syncthreads();
+  }
+  if (dense) {
+    // a thread's two items side by side: two Philox chains in flight
+    uint64_t m[2], acc[2][4] = {};
+    uint32_t i[2], j[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const uint32_t x = u * kNoiseThreads + t;
+      m[u] = x < n ? s_fire[x] : 0;
+      place(x, i[u], j[u]);
+    }
+    while (m[0] | m[1]) {
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const uint32_t b = (uint32_t)__ffsll((long long)m[u]) - 1;
+        const uint64_t bit = m[u] & (0 - m[u]);  // 0 for an item that is done
+        uint32_t pa, pb;
+        noise_pauli(kind, noise_philox(e, seed, i0 + i[u], 64 * j[u] + b, 4).v[0], pa, pb);
+        if (pa == 1 || pa == 2) acc[u][0] |= bit;
+        if (pa >= 2) acc[u][1] |= bit;
+        if (pb == 1 || pb == 2) acc[u][2] |= bit;
+        if (pb >= 2) acc[u][3] |= bit;
+        m[u] ^= bit;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      uint64_t *pauli = reinterpret_cast<uint64_t *>(s_pauli[u * kNoiseThreads + t]);
+#pragma unroll
+      for (int v = 0; v < 4; ++v) pauli[v] = acc[u][v];
+    }
   }
   for (uint32_t x = t; x < n; x += kNoiseThreads) {
     const uint64_t fire = s_fire[x];
