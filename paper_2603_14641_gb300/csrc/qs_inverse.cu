@@ -22,8 +22,9 @@
 // of a layer act on distinct qubits, which may share a sign word).
 //
 // Measurement (Alg. 1) up to 16,384 qubits: by columns, up to 64 measurements
-// at once (qs_inverse_columns.cu). Beyond, where a column's words do not fit the
-// registers of one block, four launches per measurement on the row-major tableau:
+// at once (qs_inverse_columns.cu), unless a call has so few that reading the whole
+// tableau costs more. Then, and beyond 16,384 qubits, where a column's words do not fit
+// the registers of one block, four launches per measurement on the row-major tableau:
 //  1. gather (shared with the CHP path): pivot p = smallest stabilizer with
 //     XS[p][q] = 1, and the column bits of every row.
 //  2. inv_targets: CX injections from the pivot into every later stabilizer t
@@ -446,7 +447,8 @@ inv_finalize_kernel(uint64_t *__restrict__ RX, uint64_t *__restrict__ RZ, uint64
 }
 
 size_t inv_scratch_words(const Layout &L) {
-  return L.n <= kInvColumnsMax ? inv_log_words(L) : (size_t)6 * kInvChunks * L.rs;
+  const size_t rows = (size_t)6 * kInvChunks * L.rs;
+  return L.n <= kInvColumnsMax ? std::max(rows, inv_log_words(L)) : rows;
 }
 
 cudaError_t launch_inv_measure_one(const Dev &d, const uint32_t *qubits, uint32_t i, uint64_t midx,

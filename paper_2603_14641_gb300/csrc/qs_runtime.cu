@@ -256,7 +256,7 @@ int run_dev_layers(qs_sim *s, uint64_t *X, uint64_t *Z, uint64_t *S, uint32_t st
     }
     return QS_OK;
   }
-  if (tableau && !s->d.inverse && nlayers >= kLazyMinLayers && (!fused_fits(n) || (s->flags & QS_FLAG_NO_FUSION))) {
+  if (tableau && !s->d.inverse && (!fused_fits(n) || (s->flags & QS_FLAG_NO_FUSION)) && nlayers >= kLazyMinLayers) {
     // the row-major tableau, stale from here on, is the scratch
     s->rows_valid = false;
     int l = 0;
@@ -518,13 +518,27 @@ int qs_sim_apply_layers_dev(qs_sim *s, const uint32_t *packed_dev, const int64_t
   return QS_OK;
 }
 
-// whether measurements work on the column-major tableau
-static bool measures_columns(const qs_sim *s) { return s->d.inverse && s->d.L.n <= kInvColumnsMax; }
+// Whether `count` measurements work on the column-major tableau. In inverse mode up
+// to kInvColumnsMax qubits both layouts can be measured (same bits). By columns a
+// block reads and writes the whole tableau however few its measurements are; by
+// rows each takes four launches of 31 us together. Calls that measure one qubit,
+// by rows / by columns without a layout switch: 4,000 qubits 29 / 17 us, 8,000
+// 31 / 51, 8,300 33 / 78, 16,000 37 / 203; the switch that a call needs first takes
+// about 5 + n^2 / 6e6 us.
+static bool measures_columns(const qs_sim *s, uint32_t count) {
+  const uint32_t n = s->d.L.n;
+  if (!s->d.inverse || n > kInvColumnsMax) return false;
+  const double blocks = (count + 31) / 32;  // of 64 up to 8,192 qubits
+  const double turn = 5 + (double)n * n / 6e6;
+  const double columns = blocks * (n <= 4096 ? 20 : n <= 8192 ? 20 + 0.008 * (n - 4096) : 78 + 0.016 * (n - 8300.0)) +
+                         (s->cols_valid ? 0 : turn);
+  return columns <= 31.0 * count + (s->rows_valid ? 0 : turn);
+}
 
-static int measure_staged(qs_sim *s, const uint32_t *qdev, uint32_t count, uint64_t m0, qs_key key) {
+static int measure_staged(qs_sim *s, const uint32_t *qdev, uint32_t count, uint64_t m0, qs_key key, bool columns) {
   if (s->d.inverse) {  // Alg. 1: blocks of steps by columns, or one measurement after another
     tbegin(s->d.timer, QS_TIME_MEASURE_SINGLE, s->stream);
-    if (measures_columns(s)) {
+    if (columns) {
       int l = 0;
       QS_CUDA(s, launch_inv_measure_columns(s->d, qdev, count, m0, key, s->stream, &l));
       s->launches += (uint64_t)l;
@@ -577,7 +591,8 @@ int qs_sim_measure(qs_sim *s, const uint32_t *qubits, uint32_t count, qs_key key
   if (s->n_meas + count > s->d.record_cap)
     return fail(QS_ERR_SIZE, "record capacity exceeded (qs_options.record_capacity)");
   if (count == 0) return QS_OK;
-  if ((rc = measures_columns(s) ? ensure_cols(s) : ensure_rows(s))) return rc;
+  const bool columns = measures_columns(s, count);
+  if ((rc = columns ? ensure_cols(s) : ensure_rows(s))) return rc;
   const uint64_t m0 = s->n_meas;
   const uint32_t chunk = (uint32_t)(s->plan.stage_bytes / 4);
   for (uint32_t off = 0; off < count; off += chunk) {
@@ -592,11 +607,11 @@ int qs_sim_measure(qs_sim *s, const uint32_t *qubits, uint32_t count, qs_key key
       memcpy(h, qubits + off, (size_t)c * 4);
       if ((rc = upload(s, slot, (size_t)c * 4))) return rc;
     }
-    if ((rc = measure_staged(s, reinterpret_cast<const uint32_t *>(s->dstage), c, m0 + off, key)))
+    if ((rc = measure_staged(s, reinterpret_cast<const uint32_t *>(s->dstage), c, m0 + off, key, columns)))
       return rc;
   }
   s->n_meas += count;
-  (measures_columns(s) ? s->rows_valid : s->cols_valid) = false;
+  (columns ? s->rows_valid : s->cols_valid) = false;
   Op op;
   op.kind = Op::kHostMeasure;
   op.qubits.assign(qubits, qubits + count);
@@ -617,11 +632,12 @@ int qs_sim_measure_dev(qs_sim *s, const uint32_t *qubits_dev, uint32_t count, qs
   if (s->n_meas + count > s->d.record_cap)
     return fail(QS_ERR_SIZE, "record capacity exceeded (qs_options.record_capacity)");
   if (count == 0) return QS_OK;
-  if ((rc = measures_columns(s) ? ensure_cols(s) : ensure_rows(s))) return rc;
+  const bool columns = measures_columns(s, count);
+  if ((rc = columns ? ensure_cols(s) : ensure_rows(s))) return rc;
   const uint64_t m0 = s->n_meas;
-  if ((rc = measure_staged(s, qubits_dev, count, m0, key))) return rc;
+  if ((rc = measure_staged(s, qubits_dev, count, m0, key, columns))) return rc;
   s->n_meas += count;
-  (measures_columns(s) ? s->rows_valid : s->cols_valid) = false;
+  (columns ? s->rows_valid : s->cols_valid) = false;
   Op op;
   op.kind = Op::kDevMeasure;
   op.dev = qubits_dev;
