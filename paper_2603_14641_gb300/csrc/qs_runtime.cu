@@ -59,7 +59,7 @@ struct Op {
 constexpr int kRing = 4;
 constexpr uint32_t kBlockedMinCount = 16;    // windows this long use blocked measurement
 constexpr uint32_t kBlockedMinQubits = 64;
-constexpr size_t kFusedMinLayers = 4;        // shorter runs of layers take a launch each
+constexpr uint32_t kFusedSmallQubits = 1024;
 constexpr size_t kLazyMinLayers = 2;         // runs of layers this long defer their one-qubit gates
 constexpr uint32_t kMaxQubits = 1u << 20;
 // Frame layers cover a qubit's shot words in chunks of 512 words along grid.y
@@ -237,6 +237,15 @@ int validate_pack(uint32_t n, const qs_gate *g, size_t count, std::vector<uint32
   return QS_OK;
 }
 
+// Shorter runs of layers take a launch a layer. Fusing pays from four layers on (3
+// layers one by one / 4 fused: 4,000 qubits 14 / 24 us, 10,000 31 / 124, a sampling of
+// 1,000 qubits and 200,000 shots 75 / 108), from two where a fused run is one short
+// launch and each block has an SM of its own (256 qubits, 2 layers 8.5 / 5.9, 3 layers
+// 12.2 / 6.0; 1,000 qubits 10.1 / 7.0, 15 / 7.6).
+size_t fused_min_layers(const qs_sim *s, uint32_t nwords) {
+  return s->d.L.n <= kFusedSmallQubits && nwords <= (uint32_t)s->d.sms ? 2 : 4;
+}
+
 // Enqueues layers [0, nlayers) given by absolute gate offsets `ptr` of device
 // gate records `packed` on the tableau (S != nullptr) or on frames. Runs of
 // layers go through the fused shared-memory kernels when a word slice fits (or,
@@ -246,7 +255,10 @@ int run_dev_layers(qs_sim *s, uint64_t *X, uint64_t *Z, uint64_t *S, uint32_t st
                    const uint32_t *packed, const int64_t *ptr, size_t nlayers, bool tableau) {
   const uint32_t n = s->d.L.n;
   if (nlayers == 0) return QS_OK;
-  if (nlayers >= kFusedMinLayers && fused_fits(n) && !(s->flags & QS_FLAG_NO_FUSION) && !(tableau && s->d.inverse)) {
+  // the fused kernels read a record as 8 bytes, the others as two words
+  const bool fused = nlayers >= fused_min_layers(s, nwords) && fused_fits(n) && !(s->flags & QS_FLAG_NO_FUSION) &&
+                     (reinterpret_cast<uintptr_t>(packed) & 7) == 0;
+  if (fused && !(tableau && s->d.inverse)) {
     for (size_t l0 = 0; l0 < nlayers; l0 += kFusedLayers) {
       const size_t L = std::min<size_t>(kFusedLayers, nlayers - l0);
       int l = 0;
