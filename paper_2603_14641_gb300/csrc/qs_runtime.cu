@@ -60,7 +60,6 @@ constexpr int kRing = 4;
 constexpr uint32_t kBlockedMinCount = 16;    // windows this long use blocked measurement
 constexpr uint32_t kBlockedMinQubits = 64;
 constexpr uint32_t kFusedSmallQubits = 1024;
-constexpr size_t kLazyMinLayers = 2;         // runs of layers this long defer their one-qubit gates
 constexpr uint32_t kMaxQubits = 1u << 20;
 // Frame layers cover a qubit's shot words in chunks of 512 words along grid.y
 // (at most 65,535): 2e9 shots are 31.25 M words, 61,036 chunks.
@@ -246,6 +245,24 @@ size_t fused_min_layers(const qs_sim *s, uint32_t nwords) {
   return s->d.L.n <= kFusedSmallQubits && nwords <= (uint32_t)s->d.sms ? 2 : 4;
 }
 
+// Whether the layers' one-qubit gates are deferred (larger tableaus). That costs two
+// launches and two memsets a run and the making of the records. Deferred / one by one,
+// half of the qubits in two-qubit gates, in us: 14,500 qubits 2 layers 52 / 41, 3 layers
+// 65 / 60, 4 layers 106 / 135; 20,000 qubits 111 / 102, 145 / 153, 187 / 243; 30,000
+// qubits 2 layers 194 / 198, 60,000 qubits 710 / 771. Layers in which every qubit is in a
+// two-qubit gate have nothing to defer (24.6 / 18.8 us a layer at 14,500 qubits, 60 / 52
+// at 20,000, 1,240 / 1,150 at 100,000). Types are in device memory; such layers are
+// known by their number of gates, half of the qubits (to 1 %).
+bool defers(uint32_t n, const int64_t *ptr, size_t nlayers) {
+  size_t layers = 0, pairs = 0;
+  for (size_t l = 0; l < nlayers; ++l) {
+    const int64_t gates = ptr[l + 1] - ptr[l];
+    layers += gates > 0;
+    pairs += 100 * gates >= 49 * (int64_t)n && 100 * gates <= 51 * (int64_t)n;
+  }
+  return layers >= (n < 24000 ? 4u : n < 40000 ? 3u : 2u) && 3 * pairs <= 2 * layers;
+}
+
 // Enqueues layers [0, nlayers) given by absolute gate offsets `ptr` of device
 // gate records `packed` on the tableau (S != nullptr) or on frames. Runs of
 // layers go through the fused shared-memory kernels when a word slice fits (or,
@@ -268,7 +285,7 @@ int run_dev_layers(qs_sim *s, uint64_t *X, uint64_t *Z, uint64_t *S, uint32_t st
     }
     return QS_OK;
   }
-  if (tableau && !s->d.inverse && (!fused_fits(n) || (s->flags & QS_FLAG_NO_FUSION)) && nlayers >= kLazyMinLayers) {
+  if (tableau && !s->d.inverse && (!fused_fits(n) || (s->flags & QS_FLAG_NO_FUSION)) && defers(n, ptr, nlayers)) {
     // the row-major tableau, stale from here on, is the scratch
     s->rows_valid = false;
     int l = 0;

@@ -1,4 +1,5 @@
-"""Which runs of device layers are fused, by the launches they take: one each, or one for a short fused run."""
+"""Which runs of device layers are fused or have their one-qubit gates deferred, by the launches they take: one
+each, one for a short fused run, and the layers plus two where gates are deferred."""
 import numpy as np
 import pytest
 
@@ -15,11 +16,30 @@ def _launches(sim, c, layers):
 
 
 @pytest.mark.parametrize("n,p,layers,launches", [
-    (256, 0.5, 1, 1), (256, 0.5, 2, 1), (1_024, 0.5, 3, 1), (1_025, 0.5, 3, 3), (1_025, 0.5, 4, 1)])
+    (256, 0.5, 1, 1), (256, 0.5, 2, 1), (1_024, 0.5, 3, 1), (1_025, 0.5, 3, 3), (1_025, 0.5, 4, 1),
+    (14_500, 0.5, 2, 2), (14_500, 0.5, 3, 3), (14_500, 0.5, 4, 6), (20_000, 0.8, 3, 3), (25_000, 0.5, 2, 2),
+    (25_000, 0.5, 3, 5), (41_000, 0.5, 2, 4),
+    (14_500, 1.0, 8, 8), (14_501, 1.0, 8, 8), (14_500, 0.0, 4, 6)])
 def test_runs(monkeypatch, n, p, layers, launches):
     fake_cuda.use(monkeypatch)
     s = qs.qs_sim_create(n)
     assert _launches(s, C.random_circuit(n, layers, p, seed=1, final_measure_all=False), layers) == launches
+    qs.qs_sim_destroy(s)
+
+
+def test_a_layer_of_one_qubit_gates_among_pairs(monkeypatch):
+    """H on every qubit and layers of pairs: deferred if a third of the layers may hold one-qubit gates."""
+    fake_cuda.use(monkeypatch)
+    n = 15_000
+    s = qs.qs_sim_create(n)
+    h = np.stack([np.full(n, C.H), np.arange(n), np.zeros(n)], 1).astype(np.uint32)
+    cz = np.stack([np.full(n // 2, C.CZ), np.arange(0, n, 2), np.arange(1, n, 2)], 1).astype(np.uint32)
+    for order, deferred in (("HCHC", True), ("HCCHCC", True), ("HCCCHCCC", False), ("C.C.C.H.H.", True), ("H..C.", False)):
+        gates = [{"H": h, "C": cz, ".": h[:0]}[k] for k in order]
+        lp = np.cumsum([0] + [len(g) for g in gates])
+        c = C.Circuit(n=n, gates=np.concatenate(gates), layer_ptr=lp, ops=[])
+        full = sum(len(g) > 0 for g in gates)
+        assert _launches(s, c, len(gates)) == full + 2 * deferred, order
     qs.qs_sim_destroy(s)
 
 
