@@ -157,11 +157,26 @@ int cuda_fail(qs_sim *s, cudaError_t e, const char *what) {
     if (e_ != cudaSuccess) return cuda_fail(sim, e_, #call); \
   } while (0)
 
-// Next pinned host slot, waiting until its previous copy has finished.
+// Next pinned host slot, waiting until its previous copy has finished. A slot is
+// allocated when it is first needed: most simulators stage nothing, and the four slots
+// were 0.2 of the 0.24 ms of a create and most of a destroy.
 uint8_t *ring_slot(qs_sim *s, int *slot) {
   int i = s->ring;
   s->ring = (s->ring + 1) % kRing;
-  if (cudaEventSynchronize(s->ev[i]) != cudaSuccess) return nullptr;
+  if (!s->hstage[i]) {
+    if (cudaHostAlloc(reinterpret_cast<void **>(&s->hstage[i]), s->plan.stage_bytes, cudaHostAllocDefault) != cudaSuccess) {
+      s->hstage[i] = nullptr;
+      return nullptr;
+    }
+    if (cudaEventCreateWithFlags(&s->ev[i], cudaEventDisableTiming) != cudaSuccess) {
+      cudaFreeHost(s->hstage[i]);
+      s->hstage[i] = nullptr;
+      s->ev[i] = nullptr;
+      return nullptr;
+    }
+  } else if (cudaEventSynchronize(s->ev[i]) != cudaSuccess) {
+    return nullptr;
+  }
   *slot = i;
   return s->hstage[i];
 }
@@ -391,15 +406,6 @@ int qs_sim_create(uint32_t n, const qs_options *opt, void *cuda_stream, void *wo
   }
   s->d.sms = 152;
   cudaDeviceGetAttribute(&s->d.sms, cudaDevAttrMultiProcessorCount, dev);
-  for (int i = 0; i < kRing; ++i) {
-    cudaError_t e = cudaHostAlloc(reinterpret_cast<void **>(&s->hstage[i]), p.stage_bytes,
-                                  cudaHostAllocDefault);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->ev[i], cudaEventDisableTiming);
-    if (e != cudaSuccess) {
-      qs_sim_destroy(s);
-      return fail(QS_ERR_OOM, std::string("pinned staging allocation failed: ") + cudaGetErrorString(e));
-    }
-  }
   int rc = qs_sim_reset(s, nullptr);
   if (rc != QS_OK) {
     std::string msg = g_last_error;
