@@ -536,7 +536,6 @@ struct BSampleCirc {
   uint64_t *out;                  // [M][ow] words
 };
 
-constexpr uint64_t kPinnedRecordsMax = 64ull << 20;
 constexpr uint32_t kSampleStages = 3;
 
 __global__ void __launch_bounds__(128)
@@ -630,21 +629,6 @@ batch_sample_kernel(const BCirc *__restrict__ circs, const BSampleCirc *__restri
   }
 }
 
-// Every circuit's record into pinned host memory, a block each, at the end of a
-// run: a copy per record read took 16 us, 0.9 of the 3.2 ms of a batch of 56 circuits.
-struct RecordCopy {
-  const uint8_t *src;  // 16-byte aligned, as dst
-  uint8_t *dst;
-  uint64_t bytes;
-};
-
-__global__ void __launch_bounds__(256) batch_records_kernel(const RecordCopy *__restrict__ table) {
-  const RecordCopy c = table[blockIdx.x];
-  for (uint64_t i = threadIdx.x; i < c.bytes / 16; i += 256)
-    reinterpret_cast<uint4 *>(c.dst)[i] = reinterpret_cast<const uint4 *>(c.src)[i];
-  for (uint64_t i = c.bytes / 16 * 16 + threadIdx.x; i < c.bytes; i += 256) c.dst[i] = c.src[i];
-}
-
 }  // namespace qs
 
 using namespace qs;
@@ -711,9 +695,13 @@ struct qs_batch {
   bool pending = false;                 // work enqueued since the last successful qs_batch_sync
   bool persistent_ran = false;          // the last run gave a launch shape: n < kBatchSimMinQubits ran there
   std::vector<int32_t> sim_of;          // per circuit: index into sims, or -1
-  uint8_t *h_rec = nullptr;             // pinned: RecordCopy table, then every circuit's record
-  std::vector<uint64_t> rec_off;        // per circuit: its record in h_rec
-  bool rec_ready = false;               // h_rec holds (in stream order) the last run's records
+  // All records lie side by side on the device and come to the host in one copy when
+  // the first is read: a copy per record took 16 us, 0.9 of the 3.2 ms of a batch of
+  // 56 circuits.
+  uint8_t *d_rec = nullptr;
+  std::vector<uint8_t> h_rec;           // the last run's records, once one has been read
+  size_t rec_bytes = 0;
+  bool rec_ready = false;               // d_rec holds (in stream order) the last run's records
   std::vector<BSim> sims;
   std::vector<cudaStream_t> wstreams;   // worker streams of the large circuits
   std::vector<cudaEvent_t> wevents;
@@ -749,12 +737,18 @@ static void layout_of(uint32_t n, uint32_t &k, uint32_t &cs, uint32_t &ncols, ui
 
 struct BatchPlan {
   std::vector<size_t> off_X, off_Z, off_S, off_RX, off_RZ, off_colx, off_mst, off_dx, off_dz,
-      off_ds, off_rec, off_g, off_lp, off_q, off_rt;
+      off_ds, off_rec, off_g, off_lp, off_q;
   size_t zero_end = 0, circs = 0, ids = 0, acts = 0, rounds = 0, pre_n = 0, bar = 0, err = 0, total = 0;
-  size_t acts_cap = 0;
+  size_t acts_cap = 0, rec = 0, rec_bytes = 0;
 };
 
-static int plan_batch(uint32_t count, const qs_batch_circuit *cc, BatchPlan &P, uint32_t &nrounds) {
+constexpr uint64_t kRecordsAtOnce = 64ull << 20;  // bytes of records up to which they are copied together
+
+static uint64_t measurements(const qs_batch_circuit &c) { return c.n_rounds ? c.round_meas[c.n_rounds] : 0; }
+
+// cc: the persistent kernel's view of the circuits orig
+static int plan_batch(uint32_t count, const qs_batch_circuit *cc, const qs_batch_circuit *orig, BatchPlan &P,
+                      uint32_t &nrounds) {
   Carve2 c;
   P.off_X.resize(count); P.off_Z.resize(count); P.off_S.resize(count);
   nrounds = 0;
@@ -771,7 +765,12 @@ static int plan_batch(uint32_t count, const qs_batch_circuit *cc, BatchPlan &P, 
   P.zero_end = c.off;
   P.off_RX.resize(count); P.off_RZ.resize(count); P.off_colx.resize(count); P.off_mst.resize(count);
   P.off_dx.resize(count); P.off_dz.resize(count); P.off_ds.resize(count); P.off_rec.resize(count);
-  P.off_g.resize(count); P.off_lp.resize(count); P.off_q.resize(count); P.off_rt.resize(count);
+  P.off_g.resize(count); P.off_lp.resize(count); P.off_q.resize(count);
+  for (uint32_t i = 0; i < count; ++i) {
+    P.off_rec[i] = P.rec_bytes;
+    P.rec_bytes += measurements(orig[i]);
+  }
+  P.rec = c.take(std::max<size_t>(P.rec_bytes, 1));
   for (uint32_t i = 0; i < count; ++i) {
     uint32_t k, cs, ncols, rs, nrows;
     layout_of(cc[i].n, k, cs, ncols, rs, nrows);
@@ -782,14 +781,11 @@ static int plan_batch(uint32_t count, const qs_batch_circuit *cc, BatchPlan &P, 
     P.off_dx[i] = c.take((size_t)k * rs * 8);
     P.off_dz[i] = c.take((size_t)k * rs * 8);
     P.off_ds[i] = c.take((size_t)k * 4);
-    const uint32_t nrr = cc[i].n_rounds;
-    const uint64_t M = nrr ? cc[i].round_meas[nrr] : 0;
-    P.off_rec[i] = c.take(std::max<uint64_t>(M, 1));
+    const uint64_t M = measurements(cc[i]);
     const int64_t G = cc[i].n_layers ? cc[i].layer_ptr[cc[i].n_layers] : 0;
     P.off_g[i] = c.take((size_t)std::max<int64_t>(G, 1) * 8);
-    P.off_lp[i] = c.take(((size_t)cc[i].n_layers + 1) * 8);
+    P.off_lp[i] = c.take(((size_t)cc[i].n_layers + 1 + cc[i].n_rounds + 1) * 8);  // layer offsets, round table
     P.off_q[i] = c.take((size_t)std::max<uint64_t>(M, 1) * 4);
-    P.off_rt[i] = c.take(2 * ((size_t)nrr + 1) * 4);
   }
   P.acts_cap = acts + 2 * (size_t)nrounds + 2;
   P.circs = c.take(count * sizeof(BCirc));
@@ -924,7 +920,7 @@ size_t qs_batch_required_bytes(uint32_t count, const qs_batch_circuit *circuits)
   const std::vector<qs_batch_circuit> kv = kernel_view(count, circuits);
   BatchPlan P;
   uint32_t nr;
-  plan_batch(count, kv.data(), P, nr);
+  plan_batch(count, kv.data(), circuits, P, nr);
   return P.total;
 }
 
@@ -942,7 +938,7 @@ int qs_batch_create(uint32_t count, const qs_batch_circuit *cc, void *stream, vo
   BatchPlan P;
   qs_batch *b = new (std::nothrow) qs_batch();
   if (!b) return bfail(QS_ERR_OOM, "host allocation failed");
-  plan_batch(count, cc, P, b->nrounds);
+  plan_batch(count, cc, orig, P, b->nrounds);
   b->stream = static_cast<cudaStream_t>(stream);
   b->count = count;
   if (workspace) {
@@ -983,7 +979,7 @@ int qs_batch_create(uint32_t count, const qs_batch_circuit *cc, void *stream, vo
     C.det_x = reinterpret_cast<uint64_t *>(base + P.off_dx[i]);
     C.det_z = reinterpret_cast<uint64_t *>(base + P.off_dz[i]);
     C.det_scal = reinterpret_cast<int32_t *>(base + P.off_ds[i]);
-    C.record = base + P.off_rec[i];
+    C.record = base + P.rec + P.off_rec[i];
     C.seed = c.seed;
     C.shot = c.shot;
     const int64_t G = c.n_layers ? c.layer_ptr[c.n_layers] : 0;
@@ -1002,10 +998,20 @@ int qs_batch_create(uint32_t count, const qs_batch_circuit *cc, void *stream, vo
     C.gates = reinterpret_cast<const uint32_t *>(base + P.off_g[i]);
     C.lptr = reinterpret_cast<const int64_t *>(base + P.off_lp[i]);
     C.qubits = reinterpret_cast<const uint32_t *>(base + P.off_q[i]);
-    C.rl = reinterpret_cast<const uint32_t *>(base + P.off_rt[i]);
+    C.rl = reinterpret_cast<const uint32_t *>(C.lptr + lp.size());
     C.rm = C.rl + c.n_rounds + 1;
     C.nrounds = c.n_rounds;
-    const uint64_t M = c.n_rounds ? c.round_meas[c.n_rounds] : 0;
+    const uint64_t M = measurements(c);
+    b->rl[i].assign(c.round_layers ? c.round_layers : nullptr,
+                    c.round_layers ? c.round_layers + c.n_rounds + 1 : nullptr);
+    b->rm[i].assign(c.round_meas ? c.round_meas : nullptr,
+                    c.round_meas ? c.round_meas + c.n_rounds + 1 : nullptr);
+    if (b->rl[i].empty()) b->rl[i].push_back(0);
+    if (b->rm[i].empty()) b->rm[i].push_back(0);
+    const size_t nl = lp.size(), rtb = b->rl[i].size() * 4;  // the round table goes with the layer offsets
+    lp.resize(nl + b->rl[i].size());
+    memcpy(lp.data() + nl, b->rl[i].data(), rtb);
+    memcpy(reinterpret_cast<uint8_t *>(lp.data() + nl) + rtb, b->rm[i].data(), rtb);
     e = cudaMemcpy(base + P.off_g[i], packed.data(), packed.size() * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
       e = cudaMemcpy(base + P.off_lp[i], lp.data(), lp.size() * 8, cudaMemcpyHostToDevice);
@@ -1013,14 +1019,6 @@ int qs_batch_create(uint32_t count, const qs_batch_circuit *cc, void *stream, vo
       e = cudaMemcpy(base + P.off_q[i], c.qubits, M * 4, cudaMemcpyHostToDevice);
     b->circs[i] = C;
     b->meas_total[i] = M;
-    b->rl[i].assign(c.round_layers ? c.round_layers : nullptr,
-                    c.round_layers ? c.round_layers + c.n_rounds + 1 : nullptr);
-    b->rm[i].assign(c.round_meas ? c.round_meas : nullptr,
-                    c.round_meas ? c.round_meas + c.n_rounds + 1 : nullptr);
-    if (b->rl[i].empty()) { b->rl[i].push_back(0); b->rm[i].push_back(0); }
-    const size_t rtb = b->rl[i].size() * 4;
-    if (e == cudaSuccess) e = cudaMemcpy(base + P.off_rt[i], b->rl[i].data(), rtb, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(base + P.off_rt[i] + rtb, b->rm[i].data(), rtb, cudaMemcpyHostToDevice);
     if (orig[i].n < kBatchSimMinQubits && (G > 0 || M > 0)) b->any_small = true;
     pre_n[i + 1] = pre_n[i] + c.n;
     b->n_max = std::max(b->n_max, c.n);
@@ -1035,6 +1033,8 @@ int qs_batch_create(uint32_t count, const qs_batch_circuit *cc, void *stream, vo
   b->d_err = reinterpret_cast<uint32_t *>(base + P.err);
   b->zero_begin = reinterpret_cast<uint64_t *>(base);
   b->zero_words = P.zero_end / 8;
+  b->d_rec = base + P.rec;
+  b->rec_bytes = P.rec_bytes;
   b->acts_cap = P.acts_cap;
   if (e == cudaSuccess)
     e = cudaMemcpy(b->d_circs, b->circs.data(), count * sizeof(BCirc), cudaMemcpyHostToDevice);
@@ -1143,24 +1143,6 @@ int qs_batch_create(uint32_t count, const qs_batch_circuit *cc, void *stream, vo
     delete b;
     return rc;
   }
-  // without the pinned memory records are read one copy at a time
-  uint64_t bytes = ((uint64_t)count * sizeof(RecordCopy) + 255) / 256 * 256;
-  b->rec_off.resize(count);
-  for (uint32_t i = 0; i < count; ++i) {
-    b->rec_off[i] = bytes;
-    bytes += (b->meas_total[i] + 255) / 256 * 256;
-  }
-  if (bytes <= kPinnedRecordsMax && cudaMallocHost(reinterpret_cast<void **>(&b->h_rec), bytes) == cudaSuccess) {
-    memset(b->h_rec, 0, bytes);
-    RecordCopy *t = reinterpret_cast<RecordCopy *>(b->h_rec);
-    for (uint32_t i = 0; i < count; ++i) {
-      const BSim *x = b->sim_of[i] >= 0 ? &b->sims[b->sim_of[i]] : nullptr;
-      t[i] = {x && !x->mid ? sim_record(x->sim) : b->circs[i].record, b->h_rec + b->rec_off[i], b->meas_total[i]};
-    }
-  } else {
-    cudaGetLastError();
-    b->h_rec = nullptr;
-  }
   *out = b;
   return QS_OK;
 }
@@ -1169,7 +1151,6 @@ int qs_batch_destroy(qs_batch *b) {
   if (!b) return QS_OK;
   cudaStreamSynchronize(b->stream);
   free_sims(b);
-  if (b->h_rec) cudaFreeHost(b->h_rec);
   if (b->owns && b->ws) cudaFree(b->ws);
   delete b;
   return QS_OK;
@@ -1218,9 +1199,9 @@ static int run_sims(qs_batch *b, uint32_t round_limit) {
           rc = qs_sim_measure(x.sim, x.qubits.data() + x.rm[r], x.rm[r + 1] - x.rm[r],
                               qs_key{x.seed, x.shot}, nullptr);
       }
-      // where qs_batch_sample looks for the records of n < kBatchSimMinQubits
+      // beside the other circuits' records, where the samples and the host look for it
       const uint64_t M = qs_sim_num_measurements(x.sim);
-      if (rc == QS_OK && x.mid && M &&
+      if (rc == QS_OK && M &&
           cudaMemcpyAsync(b->circs[x.index].record, sim_record(x.sim), M, cudaMemcpyDeviceToDevice,
                           b->wstreams[w]) != cudaSuccess)
         rc = QS_ERR_CUDA;
@@ -1295,6 +1276,7 @@ static int batch_run(qs_batch *b, const qs_batch_tuning *tuning, uint32_t round_
   if (tuning && small && (rc = tuning_ok(b, *tuning, &smem))) return rc;
   b->pending = true;
   b->rec_ready = false;
+  b->h_rec.clear();
   b->ran_full = (round_limit == 0 || round_limit >= b->nrounds) && !b->skip_sims;
   b->persistent_ran = persistent;
   bool sims = false;
@@ -1312,15 +1294,7 @@ static int batch_run(qs_batch *b, const qs_batch_tuning *tuning, uint32_t round_
     return rc;
   }
   if (sims && (rc = run_sims(b, round_limit ? round_limit : 0xFFFFFFFFu))) return rc;
-  if (b->h_rec) {
-    batch_records_kernel<<<b->count, 256, 0, b->stream>>>(reinterpret_cast<const RecordCopy *>(b->h_rec));
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) {
-      b->broken = true;
-      return bfail(QS_ERR_CUDA, std::string("batch records: ") + cudaGetErrorString(e));
-    }
-    b->rec_ready = true;
-  }
+  b->rec_ready = true;
   return QS_OK;
 }
 
@@ -1411,8 +1385,15 @@ int qs_batch_record(qs_batch *b, uint32_t circuit, uint8_t *dst, size_t count) {
   int rc = qs_batch_sync(b);
   if (rc) return rc;
   BSim *x = sim_of(b, circuit);
-  if (b->rec_ready && (!x || count <= qs_sim_num_measurements(x->sim))) {
-    if (count) memcpy(dst, b->h_rec + b->rec_off[circuit], count);
+  if (b->rec_ready && b->rec_bytes <= kRecordsAtOnce && (!x || count <= qs_sim_num_measurements(x->sim))) {
+    if (b->h_rec.empty() && b->rec_bytes) {
+      b->h_rec.resize(b->rec_bytes);
+      if (cudaMemcpy(b->h_rec.data(), b->d_rec, b->rec_bytes, cudaMemcpyDeviceToHost) != cudaSuccess) {
+        b->broken = true;
+        return bfail(QS_ERR_CUDA, "record copy failed");
+      }
+    }
+    if (count) memcpy(dst, b->h_rec.data() + (b->circs[circuit].record - b->d_rec), count);
     return QS_OK;
   }
   if (x) {

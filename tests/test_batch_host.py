@@ -1,5 +1,5 @@
-"""Host code of the batches on a CUDA runtime without a GPU: the autotuner's cache and
-the launch shapes that are refused."""
+"""Host code of the batches on a CUDA runtime without a GPU: the autotuner's cache, the
+launch shapes that are refused, and what creating a batch and reading its records costs."""
 import ctypes
 
 import numpy as np
@@ -60,3 +60,19 @@ def test_incomplete_launch_shapes_are_refused(monkeypatch):
             rc = L.qs_batch_run(h, ctypes.byref(qs.qs_batch_tuning(*shape)), 0)
             assert rc == (0 if ok or sizes[0] > 1_000 else -1), (sizes, shape)
         L.qs_batch_destroy(h)
+
+
+def test_create_uploads_a_circuit_in_three_copies(monkeypatch):
+    """Gates, offsets and qubits; nothing is pinned, and all records come to the host in one copy."""
+    L = fake_cuda.use(monkeypatch)
+    circs = _circuits([5, 64, 640, 300, 17, 2])
+    h = _create(circs)
+    assert fake_cuda.count("pinned") == 0
+    assert fake_cuda.count("copy") <= 3 * len(circs) + 4
+    assert L.qs_batch_run(h, None, 0) == 0
+    L.fake_reset(-1, 0)
+    for i, c in enumerate(circs):
+        out = np.zeros(max(c.n_measurements, 1), np.uint8)
+        assert L.qs_batch_record(h, i, out.ctypes.data, c.n_measurements) == 0
+    assert fake_cuda.count("copy") <= 2  # the error flags, the records
+    L.qs_batch_destroy(h)
