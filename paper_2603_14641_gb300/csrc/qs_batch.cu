@@ -658,7 +658,8 @@ struct BSim {
   uint32_t index = 0;
   qs_sim *sim = nullptr;
   bool mid = false;                // n < kBatchSimMinQubits: runs here unless a launch shape is given
-  uint32_t *packed_dev = nullptr;  // qs_pack_layers records, device
+  const uint32_t *gates = nullptr; // qs_pack_layers records, device: the batch's (mid), or
+  uint32_t *packed_dev = nullptr;  // its own
   std::vector<int64_t> lp;         // layer offsets
   std::vector<uint32_t> rl, rm, qubits;
   uint64_t seed = 0, shot = 0;
@@ -703,6 +704,7 @@ struct qs_batch {
   size_t rec_bytes = 0;
   bool rec_ready = false;               // d_rec holds (in stream order) the last run's records
   std::vector<BSim> sims;
+  void *sim_ws = nullptr;               // the simulators' device memory, one allocation
   std::vector<cudaStream_t> wstreams;   // worker streams of the large circuits
   std::vector<cudaEvent_t> wevents;
   cudaEvent_t start_ev = nullptr;       // worker streams start after the batch stream's earlier work
@@ -716,6 +718,8 @@ static void free_sims(qs_batch *b) {
     if (x.packed_dev) cudaFree(x.packed_dev);
   }
   b->sims.clear();
+  if (b->sim_ws) cudaFree(b->sim_ws);
+  b->sim_ws = nullptr;
   for (cudaEvent_t e : b->wevents) cudaEventDestroy(e);
   for (cudaStream_t st : b->wstreams) cudaStreamDestroy(st);
   if (b->start_ev) cudaEventDestroy(b->start_ev);
@@ -1097,6 +1101,22 @@ int qs_batch_create(uint32_t count, const qs_batch_circuit *cc, void *stream, vo
     b->wstreams.push_back(st);
     b->wevents.push_back(ev);
   }
+  auto options = [&](uint32_t i) {
+    qs_options opt{};
+    opt.record_capacity = std::max<uint64_t>(measurements(orig[i]), 1);
+    return opt;
+  };
+  size_t sim_bytes = 0;
+  for (uint32_t i : large) {
+    const qs_options opt = options(i);
+    sim_bytes += qs_sim_required_bytes(orig[i].n, &opt);
+  }
+  if (rc == QS_OK && sim_bytes && cudaMalloc(&b->sim_ws, sim_bytes) != cudaSuccess) {
+    cudaGetLastError();
+    b->sim_ws = nullptr;
+    rc = bfail(QS_ERR_OOM, "cudaMalloc of the batch's simulators failed");
+  }
+  uint8_t *sim_at = static_cast<uint8_t *>(b->sim_ws);
   for (size_t j = 0; j < large.size() && rc == QS_OK; ++j) {
     const uint32_t i = large[j];
     const qs_batch_circuit &c = orig[i];
@@ -1115,25 +1135,31 @@ int qs_batch_create(uint32_t count, const qs_batch_circuit *cc, void *stream, vo
     const int64_t G = c.n_layers ? c.layer_ptr[c.n_layers] : 0;
     x.lp.assign(c.layer_ptr ? c.layer_ptr : nullptr, c.layer_ptr ? c.layer_ptr + c.n_layers + 1 : nullptr);
     if (x.lp.empty()) x.lp.push_back(0);
-    std::vector<uint32_t> packed(2 * (size_t)std::max<int64_t>(G, 1), 0);
-    if (c.n_layers && (rc = qs_pack_layers(c.n, c.gates, c.layer_ptr, c.n_layers, packed.data()))) {
-      rc = bfail(rc, std::string("circuit ") + std::to_string(i) + ": " + qs_last_error());
-      break;
+    if (x.mid) {
+      x.gates = b->circs[i].gates;
+    } else {
+      std::vector<uint32_t> packed(2 * (size_t)std::max<int64_t>(G, 1), 0);
+      if (c.n_layers && (rc = qs_pack_layers(c.n, c.gates, c.layer_ptr, c.n_layers, packed.data()))) {
+        rc = bfail(rc, std::string("circuit ") + std::to_string(i) + ": " + qs_last_error());
+        break;
+      }
+      if (cudaMalloc(&x.packed_dev, packed.size() * 4) != cudaSuccess ||
+          cudaMemcpy(x.packed_dev, packed.data(), packed.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess) {
+        cudaGetLastError();
+        if (x.packed_dev) cudaFree(x.packed_dev);
+        rc = bfail(QS_ERR_OOM, "gate records of a large circuit");
+        break;
+      }
+      x.gates = x.packed_dev;
     }
-    if (cudaMalloc(&x.packed_dev, packed.size() * 4) != cudaSuccess ||
-        cudaMemcpy(x.packed_dev, packed.data(), packed.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess) {
-      cudaGetLastError();
+    const qs_options opt = options(i);
+    const size_t bytes = qs_sim_required_bytes(c.n, &opt);
+    if ((rc = qs_sim_create(c.n, &opt, b->wstreams[j % nw], sim_at, bytes, &x.sim))) {
       if (x.packed_dev) cudaFree(x.packed_dev);
-      rc = bfail(QS_ERR_OOM, "gate records of a large circuit");
-      break;
-    }
-    qs_options opt{};
-    opt.record_capacity = std::max<uint64_t>(M, 1);
-    if ((rc = qs_sim_create(c.n, &opt, b->wstreams[j % nw], nullptr, 0, &x.sim))) {
-      cudaFree(x.packed_dev);
       rc = bfail(rc, std::string("circuit ") + std::to_string(i) + ": " + qs_last_error());
       break;
     }
+    sim_at += bytes;  // a multiple of 256
     b->sim_of[i] = (int32_t)b->sims.size();
     b->sims.push_back(std::move(x));
   }
@@ -1194,7 +1220,7 @@ static int run_sims(qs_batch *b, uint32_t round_limit) {
       const uint32_t lim = std::min(nr, round_limit);
       for (uint32_t r = 0; r < lim && rc == QS_OK; ++r) {
         if (x.rl[r + 1] > x.rl[r])
-          rc = qs_sim_apply_layers_dev(x.sim, x.packed_dev, x.lp.data(), x.rl[r], x.rl[r + 1]);
+          rc = qs_sim_apply_layers_dev(x.sim, x.gates, x.lp.data(), x.rl[r], x.rl[r + 1]);
         if (rc == QS_OK && x.rm[r + 1] > x.rm[r])
           rc = qs_sim_measure(x.sim, x.qubits.data() + x.rm[r], x.rm[r + 1] - x.rm[r],
                               qs_key{x.seed, x.shot}, nullptr);

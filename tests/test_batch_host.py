@@ -76,3 +76,15 @@ def test_create_uploads_a_circuit_in_three_copies(monkeypatch):
         assert L.qs_batch_record(h, i, out.ctypes.data, c.n_measurements) == 0
     assert fake_cuda.count("copy") <= 2  # the error flags, the records
     L.qs_batch_destroy(h)
+
+
+def test_simulators_of_a_batch_share_an_allocation(monkeypatch):
+    """Circuits of 641 to 1,023 qubits run through simulators: one allocation for all, the batch's gate records."""
+    L = fake_cuda.use(monkeypatch)
+    circs = _circuits([700, 641, 1_023, 900, 800])
+    h = _create(circs)
+    assert fake_cuda.count("pinned") == 0
+    assert fake_cuda.count("cudaMalloc") == 2  # the batch's workspace, the simulators
+    assert fake_cuda.count("copy") <= 3 * len(circs) + 4
+    assert L.qs_batch_run(h, None, 0) == 0
+    L.qs_batch_destroy(h)
