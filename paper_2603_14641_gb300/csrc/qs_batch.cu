@@ -658,6 +658,7 @@ struct BSim {
   uint32_t index = 0;
   qs_sim *sim = nullptr;
   bool mid = false;                // n < kBatchSimMinQubits: runs here unless a launch shape is given
+  bool pending = false;            // work since its flags were last read (12 us a simulator)
   const uint32_t *gates = nullptr; // qs_pack_layers records, device: the batch's (mid), or
   uint32_t *packed_dev = nullptr;  // its own
   std::vector<int64_t> lp;         // layer offsets
@@ -1306,7 +1307,8 @@ static int batch_run(qs_batch *b, const qs_batch_tuning *tuning, uint32_t round_
   b->ran_full = (round_limit == 0 || round_limit >= b->nrounds) && !b->skip_sims;
   b->persistent_ran = persistent;
   bool sims = false;
-  for (const BSim &x : b->sims) sims |= !(x.mid ? persistent : b->skip_sims);
+  for (BSim &x : b->sims)
+    if (!(x.mid ? persistent : b->skip_sims)) sims = x.pending = true;
   // the worker streams start after the batch stream's earlier work, beside its kernels
   if (sims && cudaEventRecord(b->start_ev, b->stream) != cudaSuccess)
     return bfail(QS_ERR_CUDA, "batch event record failed");
@@ -1390,8 +1392,10 @@ int qs_batch_sync(qs_batch *b) {
     return bfail(QS_ERR_INTERNAL, buf);
   }
   for (BSim &x : b->sims) {
+    if (!x.pending) continue;
     const int rc = qs_sim_sync(x.sim);
     if (rc) return bfail(rc, std::string("circuit ") + std::to_string(x.index) + ": " + qs_last_error());
+    x.pending = false;
   }
   b->pending = false;
   return QS_OK;
@@ -1649,6 +1653,7 @@ int qs_batch_sample(qs_batch *b, const uint64_t *shots, const uint64_t *seeds, u
     for (uint32_t c = 0; c < b->count; ++c) {
       if (!(shots[c] > 0 && is_large(b, c))) continue;
       BSim &x = b->sims[b->sim_of[c]];
+      x.pending = true;
       const uint64_t ow = (shots[c] + 63) / 64;
       const int rc = qs_sim_sample(x.sim, shots[c], seeds[c], records[c], b->meas_total[c] * ow, nullptr, 0);
       if (rc) return bfail(rc, std::string("circuit ") + std::to_string(c) + ": " + qs_last_error());

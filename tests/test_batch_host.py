@@ -88,3 +88,22 @@ def test_simulators_of_a_batch_share_an_allocation(monkeypatch):
     assert fake_cuda.count("copy") <= 3 * len(circs) + 4
     assert L.qs_batch_run(h, None, 0) == 0
     L.qs_batch_destroy(h)
+
+
+def test_sync_reads_the_flags_of_simulators_with_work(monkeypatch):
+    """After a run those of every simulator, after sampling those of the circuits that sample through theirs."""
+    L = fake_cuda.use(monkeypatch)
+    circs = _circuits([700, 641, 1_023, 1_024, 1_100, 50])
+    h = _create(circs)
+    k, ow = len(circs), 2
+    out = [np.zeros((c.n_measurements, ow), np.uint64) for c in circs]
+    ptrs = (ctypes.c_void_p * k)(*[o.ctypes.data for o in out])
+    for want, call in ((1 + 5, lambda: L.qs_batch_run(h, None, 0)),
+                       (1 + 2, lambda: L.qs_batch_sample(h, np.full(k, 128, np.uint64).ctypes.data,
+                                                         np.zeros(k, np.uint64).ctypes.data, ctypes.cast(ptrs, ctypes.c_void_p))),
+                       (0, lambda: 0)):
+        assert call() == 0
+        L.fake_reset(-1, 0)
+        assert L.qs_batch_sync(h) == 0
+        assert fake_cuda.count("copy") == want
+    L.qs_batch_destroy(h)
