@@ -98,9 +98,10 @@ def test_sync_reads_the_flags_of_simulators_with_work(monkeypatch):
     k, ow = len(circs), 2
     out = [np.zeros((c.n_measurements, ow), np.uint64) for c in circs]
     ptrs = (ctypes.c_void_p * k)(*[o.ctypes.data for o in out])
+    shots, seeds = np.full(k, 128, np.uint64), np.zeros(k, np.uint64)
     for want, call in ((1 + 5, lambda: L.qs_batch_run(h, None, 0)),
-                       (1 + 2, lambda: L.qs_batch_sample(h, np.full(k, 128, np.uint64).ctypes.data,
-                                                         np.zeros(k, np.uint64).ctypes.data, ctypes.cast(ptrs, ctypes.c_void_p))),
+                       (1 + 2, lambda: L.qs_batch_sample(h, shots.ctypes.data, seeds.ctypes.data,
+                                                         ctypes.cast(ptrs, ctypes.c_void_p))),
                        (0, lambda: 0)):
         assert call() == 0
         L.fake_reset(-1, 0)
