@@ -72,6 +72,11 @@ def footprint_bytes(n: int, n_gates: int, n_meas: int, shots: int) -> int:
             + 2 * max(n_meas, 1) * ow * 8 + n_gates * 8 + n_meas * 4 + 3 * 4096)
 
 
+# Circuits above this size hold a simulator in a batch (include/qs.h, qs_batch_circuit)
+# besides their share of the batch's own workspace, which is less than a simulator's.
+BATCH_SIMULATOR_ABOVE = 640
+
+
 class Scheduler:
     """FIFO admission by slots and a byte budget, with worker threads.
 
@@ -83,14 +88,17 @@ class Scheduler:
     def __init__(self, slots: int, budget_bytes: int, footprint: Callable[[Request], int],
                  execute: Callable[[Request, int, float, int], Result],
                  execute_batch: Optional[Callable] = None,
-                 batchable: Optional[Callable[[Request], bool]] = None, max_batch: int = 64):
+                 batchable: Optional[Callable[[Request], bool]] = None, max_batch: int = 64,
+                 batch_footprint: Optional[Callable[[Request], int]] = None):
         self.slots = slots
         self.budget = budget_bytes
         self.footprint = footprint
         self.execute = execute
         # execute_batch(requests, slot, admit_s, footprints) -> [Result]; requests
-        # for which batchable() holds are grouped when they wait together
+        # for which batchable() holds are grouped when they wait together, and
+        # count with batch_footprint() then
         self.execute_batch = execute_batch
+        self.batch_footprint = batch_footprint or footprint
         self.batchable = batchable
         self.max_batch = max_batch
         self.batches = 0          # batches of two or more requests run
@@ -130,12 +138,15 @@ class Scheduler:
                             if self.execute_batch is not None and self.batchable(req):
                                 while (self.pending and len(group) < self.max_batch
                                        and self.batchable(self.pending[0])):
-                                    f2 = self.footprint(self.pending[0])
-                                    if self.in_use + f2 > self.budget:
+                                    f2 = self.batch_footprint(self.pending[0])
+                                    # with the second one the head is in a batch, too
+                                    head = self.batch_footprint(req) - fp if len(group) == 1 else 0
+                                    if self.in_use + head + f2 > self.budget:
                                         break
+                                    fps[0] += head
                                     group.append(self.pending.popleft())
                                     fps.append(f2)
-                                    self.in_use += f2
+                                    self.in_use += head + f2
                             self.peak_in_use = max(self.peak_in_use, self.in_use)
                             self.active += len(group)
                             self.peak_active = max(self.peak_active, self.active)
@@ -208,6 +219,10 @@ class GpuExecutor:
     def footprint(self, req: Request) -> int:
         c = req.circuit
         return footprint_bytes(c.n, c.n_gates, c.n_measurements, req.shots)
+
+    def batch_footprint(self, req: Request) -> int:
+        n = req.circuit.n
+        return self.footprint(req) + (self.qs.qs_sim_required_bytes(n) if n > BATCH_SIMULATOR_ABOVE else 0)
 
     @staticmethod
     def batchable(req: Request) -> bool:
@@ -299,7 +314,7 @@ def serve(requests: List[Request], slots: int = 8, budget_bytes: int = 64 << 30,
     ex = GpuExecutor(slots, device, keep_samples)
     sch = Scheduler(slots, budget_bytes, ex.footprint, ex,
                     execute_batch=ex.execute_batch if batching else None,
-                    batchable=ex.batchable, max_batch=max_batch)
+                    batchable=ex.batchable, max_batch=max_batch, batch_footprint=ex.batch_footprint)
     t = time.perf_counter()
     res = sch.run(requests, realtime=realtime)
     makespan = time.perf_counter() - t
