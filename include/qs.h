@@ -76,8 +76,13 @@ typedef struct qs_options {
 } qs_options;
 
 /* qs_options.flags: never fuse a run of device-resident layers into one
- * shared-memory pass (used for runs of 4 layers and more on n <= 14,080
- * qubits; results are identical either way). */
+ * shared-memory pass (used on n <= 14,080 qubits for runs of 4 layers and more,
+ * 2 and more up to 1,024 qubits). With the flag, and above that size, runs of
+ * layers defer their one-qubit gates to the next two-qubit gate of their qubit,
+ * one launch a layer, except short runs (2 or 3 layers) and layers that are all
+ * two-qubit gates; a run of one layer is its own launch. Results are identical
+ * either way. Gate records at addresses that are multiples of 4 but not of 8 are
+ * never fused. */
 #define QS_FLAG_NO_FUSION 1u
 /* qs_options.flags: run every measurement as five separate launches (gather,
  * rowsum, deterministic partials, combine, finalize) instead of the pipelined
@@ -108,7 +113,8 @@ typedef struct qs_options {
  * not kept (exports give 0 there). Measurements run Alg. 1 (pivot = smallest
  * anticommuting stabilizer, CX injections into the later ones, an H or H_YZ
  * and an X injection on the pivot): up to 64 at once in two launches up to
- * 16,384 qubits, four launches each beyond; records and measurement kinds
+ * 16,384 qubits, four launches each beyond and where a call has only a few on
+ * more than about 5,000 qubits (same bits); records and measurement kinds
  * equal the CHP mode's under the same keys, and the state
  * is the same, though the tableau bits after a measurement differ. Layers
  * run one launch each (no fused segments); qs_sim_tableau_import is refused. Fixed at create. */

@@ -6,9 +6,11 @@
 // to 640 qubits with one block each, tableau in shared memory
 // (qs_batch_resident.cu), and the larger ones through one simulator each on
 // worker streams. With a launch shape given (qs_batch_tuning) the circuits of
-// n < 1024 run in the persistent kernel below instead: a cooperative launch that
-// walks every circuit's program in lock-step rounds (a round = a segment of gate
-// layers followed by a list of Z-measurements) and spreads each phase of a round
+// n < 1024 run in the persistent kernel below instead, slower on every batch
+// measured (1.3 to 14 times) and kept because callers may ask for it: a
+// cooperative launch that walks every circuit's program in lock-step rounds (a
+// round = a segment of gate layers followed by a list of Z-measurements) and
+// spreads each phase of a round
 // over all CTAs through flattened work lists (a work queue built on the host
 // from the circuits' sizes; items are taken grid-stride):
 //   init      zero X/Z/S, set D_i = X_i, S_i = Z_i               (Alg. 2 init)
@@ -48,7 +50,8 @@ namespace qs {
 constexpr int64_t kBNoPivot = LLONG_MAX;
 // Circuits of at least this many qubits always run through per-circuit
 // simulators (blocked measurement, 64 measurements per tableau pass) on worker
-// streams; the persistent kernel takes the smaller ones.
+// streams. Smaller ones do so above kResidentMaxQubits, unless a launch shape
+// sends them to the persistent kernel.
 constexpr uint32_t kBatchSimMinQubits = 1024;
 constexpr uint32_t kBatchMaxWorkers = 16;
 constexpr uint32_t kBatchLimitQubits = 1u << 20;
@@ -517,8 +520,8 @@ __global__ void __launch_bounds__(1024) batch_kernel(BProg P, uint32_t round_lim
 }
 
 // ---------------------------------------------------------------------------
-// Batched Pauli-frame sampling (Sec. 5, Alg. 9) of the persistent part's
-// circuits, one launch for all of them: an item is (circuit, 64-shot word);
+// Batched Pauli-frame sampling (Sec. 5, Alg. 9) of the circuits of n < 1024,
+// one launch for all of them: an item is (circuit, 64-shot word);
 // a block runs the circuit's whole program on that word's frame slice held
 // in shared memory (X~, Z~ of every qubit, 16 n bytes): frame init from the
 // keyed Philox words, every layer's gates without signs (barrier between

@@ -510,7 +510,7 @@ class Simulator:
 
 
 # ----------------------------------------------------------------------
-# Batched persistent launch
+# Batched launch
 # ----------------------------------------------------------------------
 
 def _bcheck(rc: int, where: str) -> None:
@@ -546,7 +546,7 @@ def circuit_rounds(circuit):
 
 
 class Batch:
-    """Many circuits in one persistent launch (qs_batch_* of include/qs.h)."""
+    """Many circuits at once (qs_batch_* of include/qs.h)."""
 
     def __init__(self, circuits, seeds, shot: int = 0, device: str = "cuda", stream=None):
         import torch

@@ -17,8 +17,8 @@ built around its method:
     channels) that wait together are served together: when a slot admits one,
     it also takes the small requests queued right behind it (in arrival order,
     within the memory budget, up to max_batch) and runs them as one batch --
-    all their reference shots in one persistent launch (qs_batch_run) and all
-    their shots in one sampling launch (qs_batch_sample);
+    all their reference shots in one batch run (qs_batch_run, up to 640 qubits a
+    block per circuit) and all their shots in one sampling launch (qs_batch_sample);
   * results do not depend on the mix: each request owns its tableau and its
     coins and frames are keyed by (seed, shot, index), so a request's record is
     bit-identical alone and among others.
@@ -226,12 +226,12 @@ class GpuExecutor:
 
     @staticmethod
     def batchable(req: Request) -> bool:
-        """Small noiseless circuits run in the batch's persistent kernel."""
+        """Small noiseless circuits run together as a batch."""
         c = req.circuit
         return c.n < 1024 and not any(op[0] == "noise" for op in c.ops)
 
     def execute_batch(self, reqs: List[Request], slot: int, admit_s: float, fps) -> List[Result]:
-        """Serves requests together: reference shots in one persistent launch
+        """Serves requests together: reference shots in one batch run
         (qs_batch_run), shots in one sampling launch (qs_batch_sample); the
         coins are keyed (seed, 0) and the frames by seed + 1, as for a request
         served alone, so the results are the same."""
