@@ -1420,7 +1420,11 @@ int qs_batch_record(qs_batch *b, uint32_t circuit, uint8_t *dst, size_t count) {
   BSim *x = sim_of(b, circuit);
   if (b->rec_ready && b->rec_bytes <= kRecordsAtOnce && (!x || count <= qs_sim_num_measurements(x->sim))) {
     if (b->h_rec.empty() && b->rec_bytes) {
-      b->h_rec.resize(b->rec_bytes);
+      try {
+        b->h_rec.resize(b->rec_bytes);
+      } catch (const std::bad_alloc &) {
+        return bfail(QS_ERR_OOM, "host allocation failed");
+      }
       if (cudaMemcpy(b->h_rec.data(), b->d_rec, b->rec_bytes, cudaMemcpyDeviceToHost) != cudaSuccess) {
         b->broken = true;
         return bfail(QS_ERR_CUDA, "record copy failed");

@@ -159,12 +159,18 @@ int cuda_fail(qs_sim *s, cudaError_t e, const char *what) {
 
 // Next pinned host slot, waiting until its previous copy has finished. A slot is
 // allocated when it is first needed: most simulators stage nothing, and the four slots
-// were 0.2 of the 0.24 ms of a create and most of a destroy.
+// were 0.2 of the 0.24 ms of a create and most of a destroy. The call may be part of
+// a stream capture, which allocating would end unless the thread allows it.
 uint8_t *ring_slot(qs_sim *s, int *slot) {
   int i = s->ring;
   s->ring = (s->ring + 1) % kRing;
   if (!s->hstage[i]) {
-    if (cudaHostAlloc(reinterpret_cast<void **>(&s->hstage[i]), s->plan.stage_bytes, cudaHostAllocDefault) != cudaSuccess) {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    const cudaError_t e =
+        cudaHostAlloc(reinterpret_cast<void **>(&s->hstage[i]), s->plan.stage_bytes, cudaHostAllocDefault);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) {
       s->hstage[i] = nullptr;
       return nullptr;
     }

@@ -1,7 +1,6 @@
 """The library's host code on a CUDA runtime without a GPU (runtime.cpp): its objects linked with the fake
 instead of CUDA's runtime. `load()` gives the C ABI, `use(monkeypatch)` lets the qs module call it."""
 import ctypes
-import glob
 import os
 import subprocess
 
@@ -15,10 +14,9 @@ def load():
     global _lib
     if _lib is None:
         build.build()
-        objs = sorted(glob.glob(os.path.join(build.LIBDIR, "obj", "*.o")))
-        if not objs:
+        objs = [os.path.join(build.LIBDIR, "obj", os.path.basename(s) + ".o") for s in build._sources()]
+        if not all(os.path.exists(o) for o in objs):
             build.build(force=True)
-            objs = sorted(glob.glob(os.path.join(build.LIBDIR, "obj", "*.o")))
         out = os.path.join(build.LIBDIR, f"libqs_fake.{os.getpid()}.so")
         cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(build._nvcc()))), "include")
         subprocess.run(["g++", "-std=c++17", "-O1", "-fPIC", "-shared", "-Wl,-Bsymbolic", "-I", cuda,
