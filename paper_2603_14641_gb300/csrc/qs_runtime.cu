@@ -562,10 +562,11 @@ int qs_sim_apply_layers_dev(qs_sim *s, const uint32_t *packed_dev, const int64_t
 // Whether `count` measurements work on the column-major tableau. In inverse mode up
 // to kInvColumnsMax qubits both layouts can be measured (same bits). By columns a
 // block reads and writes the whole tableau however few its measurements are; by
-// rows each takes four launches of 31 us together. Calls that measure one qubit,
-// by rows / by columns without a layout switch: 4,000 qubits 29 / 17 us, 8,000
-// 31 / 51, 8,300 33 / 78, 16,000 37 / 203; the switch that a call needs first takes
-// about 5 + n^2 / 6e6 us.
+// rows each takes four launches, 27 + 0.0006 n us together. Calls that measure one
+// qubit, by rows / by columns without a layout switch: 4,000 qubits 29 / 17 us, 8,000
+// 31 / 51, 8,300 33 / 78, 16,000 37 / 203 (a deterministic outcome, which cannot be
+// known here, 10 to 16 us by rows and 6 by columns, where nothing is to be applied);
+// the switch that a call needs first takes about 5 + n^2 / 6e6 us.
 static bool measures_columns(const qs_sim *s, uint32_t count) {
   const uint32_t n = s->d.L.n;
   if (!s->d.inverse || n > kInvColumnsMax) return false;
@@ -573,7 +574,7 @@ static bool measures_columns(const qs_sim *s, uint32_t count) {
   const double turn = 5 + (double)n * n / 6e6;
   const double columns = blocks * (n <= 4096 ? 20 : n <= 8192 ? 20 + 0.008 * (n - 4096) : 78 + 0.016 * (n - 8300.0)) +
                          (s->cols_valid ? 0 : turn);
-  return columns <= 31.0 * count + (s->rows_valid ? 0 : turn);
+  return columns <= (27 + 0.0006 * n) * count + (s->rows_valid ? 0 : turn);
 }
 
 static int measure_staged(qs_sim *s, const uint32_t *qdev, uint32_t count, uint64_t m0, qs_key key, bool columns) {

@@ -33,7 +33,7 @@ def test_mixed_calls_equal_one_window(n):
             assert np.array_equal(a, b)
 
 
-@pytest.mark.parametrize("n,few,many", [(2_000, 0, 1), (9_000, 2, 3), (16_000, 6, 7), (16_385, 70, 0)])
+@pytest.mark.parametrize("n,few,many", [(2_000, 0, 1), (9_000, 2, 3), (16_000, 5, 6), (16_385, 70, 0)])
 def test_few_measurements_take_rows(monkeypatch, n, few, many):
     """With both layouts at hand: four launches a measurement against two a block."""
     fake_cuda.use(monkeypatch)
