@@ -776,7 +776,7 @@ static int plan_batch(uint32_t count, const qs_batch_circuit *cc, const qs_batch
   P.off_g.resize(count); P.off_lp.resize(count); P.off_q.resize(count);
   for (uint32_t i = 0; i < count; ++i) {
     P.off_rec[i] = P.rec_bytes;
-    P.rec_bytes += measurements(orig[i]);
+    P.rec_bytes += (measurements(orig[i]) + 31) & ~size_t(31);
   }
   P.rec = c.take(std::max<size_t>(P.rec_bytes, 1));
   for (uint32_t i = 0; i < count; ++i) {
@@ -1302,7 +1302,9 @@ static int batch_run(qs_batch *b, const qs_batch_tuning *tuning, uint32_t round_
   const bool persistent = tuning && tuning->threads != 0;
   size_t smem = 0;
   int rc = QS_OK;
-  const bool small = b->any_small || b->sims.empty();  // the launch shape is for these
+  bool large = false;
+  for (const BSim &x : b->sims) large |= !x.mid;
+  const bool small = b->any_small || !large;  // the launch shape is for these
   if (tuning && small && (rc = tuning_ok(b, *tuning, &smem))) return rc;
   b->pending = true;
   b->rec_ready = false;
