@@ -673,7 +673,8 @@ struct qs_batch {
   cudaStream_t stream = nullptr;
   void *ws = nullptr;
   bool owns = false, broken = false;
-  uint32_t count = 0, nrounds = 0, n_max = 0;
+  uint32_t count = 0, nrounds = 0, n_max = 0;  // nrounds: of the persistent kernel's circuits
+  uint32_t most_rounds = 0;                    // of any circuit
   std::vector<BCirc> circs;            // host copy, device pointers
   std::vector<uint64_t> meas_total;    // per circuit
   std::vector<std::vector<uint32_t>> rl, rm;  // per circuit round layer / measurement offsets
@@ -947,6 +948,7 @@ int qs_batch_create(uint32_t count, const qs_batch_circuit *cc, void *stream, vo
   qs_batch *b = new (std::nothrow) qs_batch();
   if (!b) return bfail(QS_ERR_OOM, "host allocation failed");
   plan_batch(count, cc, orig, P, b->nrounds);
+  for (uint32_t i = 0; i < count; ++i) b->most_rounds = std::max(b->most_rounds, orig[i].n_rounds);
   b->stream = static_cast<cudaStream_t>(stream);
   b->count = count;
   if (workspace) {
@@ -1309,7 +1311,7 @@ static int batch_run(qs_batch *b, const qs_batch_tuning *tuning, uint32_t round_
   b->pending = true;
   b->rec_ready = false;
   b->h_rec.clear();
-  b->ran_full = (round_limit == 0 || round_limit >= b->nrounds) && !b->skip_sims;
+  b->ran_full = (round_limit == 0 || round_limit >= b->most_rounds) && !b->skip_sims;
   b->persistent_ran = persistent;
   bool sims = false;
   for (BSim &x : b->sims)

@@ -108,3 +108,19 @@ def test_sync_reads_the_flags_of_simulators_with_work(monkeypatch):
         assert L.qs_batch_sync(h) == 0
         assert fake_cuda.count("copy") == want
     L.qs_batch_destroy(h)
+
+
+def test_a_run_that_stops_within_a_large_circuit_is_not_complete(monkeypatch):
+    """Sampling needs the records of a complete run of every circuit, the large ones included."""
+    L = fake_cuda.use(monkeypatch)
+    circs = _circuits([50], every=10) + _circuits([1_100], every=2)
+    assert [len(qs.circuit_rounds(c)[0]) - 1 for c in circs] == [2, 10]
+    h = _create(circs)
+    out = [np.zeros((c.n_measurements, 1), np.uint64) for c in circs]
+    ptrs = (ctypes.c_void_p * 2)(*[o.ctypes.data for o in out])
+    shots, seeds = np.full(2, 10, np.uint64), np.zeros(2, np.uint64)
+    for limit, rc in ((3, -6), (9, -6), (10, 0), (0, 0)):
+        assert L.qs_batch_run(h, None, limit) == 0
+        got = L.qs_batch_sample(h, shots.ctypes.data, seeds.ctypes.data, ctypes.cast(ptrs, ctypes.c_void_p))
+        assert got == rc, limit
+    L.qs_batch_destroy(h)
