@@ -69,13 +69,10 @@ struct BlkState {
   uint64_t G[64];      // G[s] bit t = parity(z_{V_s} . x_{V_t})
 };
 
-constexpr uint32_t kDetChunks = 512;  // 32-word column chunks of the largest row (n = 2^20)
-
 // state of one window; zeroed before its first block together with the
 // accumulators behind it
 struct BlkWindow {
   uint32_t front_arrived, middle_arrived, ndet, pad;
-  uint32_t det_chunk[3 * kDetChunks];  // row ranges of blk_det that have arrived, per group and column chunk
   BlkState st[2];
 };
 
@@ -1453,6 +1450,7 @@ struct DetArgs {
   BlkWindow *win;
   int32_t *acc;         // phase exponent per outcome
   uint32_t *arrived;    // items of a group that are done
+  uint32_t *ranges;     // row ranges that are done, per group (three at most) and column chunk
   uint64_t *det_x, *det_z;
   uint64_t m0;
   uint8_t *record;
@@ -1557,7 +1555,7 @@ __global__ void __launch_bounds__(kDetThreads) blk_det_kernel(const DetArgs a) {
     __threadfence();
     __syncthreads();
     if (R > 1) {
-      if (t == 0) s_flag = atomicAdd(&a.win->det_chunk[g * a.chunks + ch], 1u) == R - 1;
+      if (t == 0) s_flag = atomicAdd(a.ranges + g * a.chunks + ch, 1u) == R - 1;
       __syncthreads();
       if (!s_flag) continue;
       __threadfence();
@@ -1605,11 +1603,11 @@ static uint32_t apply_chunks(const Layout &L) { return (L.rs + apply_words(L) - 
 
 // device scratch of the blocked measurement
 struct BlkScratch {
-  uint8_t *zero;       // start of the part zeroed per window: win, acc, arrived
+  uint8_t *zero;       // start of the part zeroed per window: win, acc, arrived, det_ranges
   size_t zero_bytes;
   BlkWindow *win;
   int32_t *acc;
-  uint32_t *arrived;
+  uint32_t *arrived, *det_ranges;
   uint64_t *C0, *C1, *M, *orC, *VX, *VZ;
   uint32_t *listRow, *cnt, *done, *det;
   int32_t *base;
@@ -1617,6 +1615,9 @@ struct BlkScratch {
   uint4 *list;
   size_t total;
 };
+
+// column chunks of blk_det
+static uint32_t det_chunks(const Layout &L) { return (L.k + 31) / 32; }
 
 // measurements per window (the capacity of det and acc)
 static uint32_t blk_window_cap(const Layout &L) { return (uint32_t)L.nrows; }
@@ -1638,6 +1639,7 @@ static BlkScratch blk_scratch(const Layout &L, void *scratch) {
   b.win = reinterpret_cast<BlkWindow *>(take(sizeof(BlkWindow)));
   b.acc = reinterpret_cast<int32_t *>(take(cap * 4));
   b.arrived = reinterpret_cast<uint32_t *>(take((cap / kDetGroup + 1) * 4));
+  b.det_ranges = reinterpret_cast<uint32_t *>(take(3 * (size_t)det_chunks(L) * 4));
   b.zero_bytes = off;
   b.C0 = reinterpret_cast<uint64_t *>(take(L.nrows * 8));
   b.C1 = reinterpret_cast<uint64_t *>(take(L.nrows * 8));
@@ -1777,8 +1779,8 @@ static cudaError_t measure_window_cap(const Dev &d, void *scratch, const uint32_
     if (d.timer && (i0 & 4095) == 4032) d.timer->resolve();  // completed event pairs go back to the pool
   }
   DetArgs t{};
-  t.RX = d.RX; t.RZ = d.RZ; t.S = d.S; t.rs = L.rs; t.n = L.n; t.k = L.k; t.chunks = (L.k + 31) / 32;
-  t.window = window; t.det = b.det; t.win = b.win; t.acc = b.acc; t.arrived = b.arrived;
+  t.RX = d.RX; t.RZ = d.RZ; t.S = d.S; t.rs = L.rs; t.n = L.n; t.k = L.k; t.chunks = det_chunks(L);
+  t.window = window; t.det = b.det; t.win = b.win; t.acc = b.acc; t.arrived = b.arrived; t.ranges = b.det_ranges;
   t.det_x = d.det_x; t.det_z = d.det_z; t.m0 = m0; t.record = d.record; t.err = d.err;
   // enough blocks for one outcome's ranges and for every group; blocks without an item leave at once
   const uint64_t most = std::max<uint64_t>(kDetBlocks, (count + kDetGroup - 1) / kDetGroup) * t.chunks;
